@@ -110,7 +110,7 @@ void free_handle(hps_handle* h) {
   cudaSetDevice(h->dev);
   if (h->stream) cudaStreamSynchronize(h->stream);
   krylov_free(h);
-  void* ptrs[] = {h->tables, h->R64, h->R32, h->H64, h->H32, h->R16lo, h->R16ls, h->H16lo, h->H16ls, h->lambda, h->lambda_q, h->Kc64, h->Kc32, h->B64,
+  void* ptrs[] = {h->tables, h->ftab, h->R64, h->R32, h->H64, h->H32, h->R16lo, h->R16ls, h->H16lo, h->H16ls, h->lambda, h->lambda_q, h->Kc64, h->Kc32, h->B64,
                   h->B32, h->pc_scratch, h->Kc16, h->Kc16s, h->B16, h->B16s, h->tc_error, h->cdiag,
                   h->dct.slot_lf, h->dct.slot_cluster, h->dct.cl_slot_begin, h->dct.cl_kc_off, h->dct.lf_slot,
                   h->dct.int_mask, h->dct.b_off, h->dct.leaf_bcls, h->dct.bc_rep, h->dct.kc_off,
@@ -144,6 +144,7 @@ void init_fields(hps_handle* h, const hps_grid* g, double kappa, double eta, con
   h->h[1] = 1.0 / g->ny;
   h->h[2] = 1.0 / g->nz;
   h->tl = TableLayout(g->p);
+  h->ft = FaceTables(h->n1);
   h->ldR = (int)rup4(h->nb);
   h->ldH = (int)rup4(h->ni);
 }
@@ -277,6 +278,7 @@ int hps_setup(const hps_grid* g, double kappa, double eta, const double* b, cons
     const bool want32 = (o.forms & HPS_FORM_MIXED) != 0;
     int r;
     if ((r = dalloc(h, (void**)&h->tables, h->tl.total * sizeof(double)))) return r;
+    if ((r = dalloc(h, (void**)&h->ftab, (size_t)3 * h->ft.per_axis * sizeof(double2)))) return r;
     const size_t rel = (size_t)h->nl * h->nb * h->ldR;
     const size_t hel = (size_t)h->nl * h->nb * h->ldH;
     if (!o.lean && (r = dalloc(h, (void**)&h->R64, rel * sizeof(double2)))) return r;
@@ -307,6 +309,7 @@ int hps_setup(const hps_grid* g, double kappa, double eta, const double* b, cons
     else
       HPS_CUDA_TRY(cudaMemsetAsync(db, 0, (size_t)h->nint * sizeof(double2), st));
     HPS_CUDA_TRY(launch_tables(h->tables, h->tl, h->h[0], h->h[1], h->h[2], st));
+    HPS_CUDA_TRY(launch_face_tables(h, st));
     HPS_CUDA_TRY(launch_cdiag(db, kappa, h->nint, dc, st));
     if ((r = build_exact_maps(h, dc, st))) return r;
     if (o.cluster == 2) {
@@ -383,7 +386,7 @@ size_t hps_setup_bytes(const hps_grid* g, const hps_options* opt, int nrhs) {
   const size_t c16 = sizeof(double2), c8 = sizeof(float2);
   const size_t rel = (size_t)h.nl * h.nb * h.ldR;
   const size_t hel = (size_t)h.nl * h.nb * h.ldH;
-  size_t bytes = h.tl.total * sizeof(double) + (o.lean ? 0 : rel * c16) + (want32 ? rel * c8 : 0) +
+  size_t bytes = h.tl.total * sizeof(double) + (size_t)3 * h.ft.per_axis * c16 + (o.lean ? 0 : rel * c16) + (want32 ? rel * c8 : 0) +
                  hel * (o.lean ? c8 : c16) + (size_t)h.nl * c16;
   if (want32)  // FP16 remainders of R and H and their row scales; FP32 H beside FP64 H
     bytes += (rel + hel) * sizeof(__half2) + (size_t)2 * h.nl * h.nb * sizeof(float) + (o.lean ? 0 : hel * c8);

@@ -52,6 +52,19 @@ struct TableLayout {
   }
 };
 
+// Offsets (in complex doubles) of the tables of the line-wise face elimination (setup.cu),
+// one block of per_axis values per axis.
+struct FaceTables {
+  int T, G, L, Pi, per_axis;
+  explicit FaceTables(int n1 = 2) {
+    T = 0;                // n1 x n1
+    G = T + n1 * n1;      // 2 x n1: Gamma
+    L = G + 2 * n1;       // n1 x 2: Lambda
+    Pi = L + 2 * n1;      // 2 x 2: Phi^{-1}
+    per_axis = Pi + 4;
+  }
+};
+
 // Cluster (block-Jacobi) bookkeeping, built on the host from integer grid
 // arithmetic and uploaded once.
 //
@@ -341,6 +354,8 @@ struct hps_handle {
 
   double* tables = nullptr;
   hps::TableLayout tl;
+  double2* ftab = nullptr;  // 3 x per_axis: face elimination tables
+  hps::FaceTables ft;
 
   // exact leaf maps (Gauss basis)
   int ldR = 0, ldH = 0;
@@ -356,6 +371,7 @@ struct hps_handle {
   float* H16ls = nullptr;
   double2* lambda = nullptr;    // nl: homogenized constants lambda^tau
   double2* lambda_q = nullptr;  // nl: lambda^tau after binning (opt.lambda_bin), used by the preconditioner
+  std::vector<double2> lambda_q_host;
   double2* cdiag = nullptr;   // nl x ni: C = kappa^2 (1 - b) at interior nodes (kept for recovery)
 
   // the paper's global-system path (options.full_system)
@@ -394,7 +410,26 @@ struct hps_handle {
 
 namespace hps {
 
+// ---- inverse.cu ----
+// nbatch complex matrices of N rows and ncols columns (row-major, leading dimension ld), matrix i
+// at A + i * stride (i = ids[0..nbatch-1] when given).  ncols == N: in-place inverse with
+// interchanged columns, A^{-1}[:, perm[i]] = X[:, i]; ncols > N: the columns [N, ncols) become
+// A^{-1} times them.  U: ustride >= gj_scratch_elems(ncols) elements per matrix; perm: pstride >=
+// N ints per matrix.  *status = 1 when a pivot is zero or not a number.  N <= 3072.
+template <class T> size_t gj_scratch_elems(int ncols);
+template <class T>
+cudaError_t batched_gj(T* A, long long stride, int ld, int N, int ncols, int nbatch, T* U, long long ustride, int* perm,
+                       int pstride, int* status, cudaStream_t st, const int* ids = nullptr);
+
+// nbatch augmented matrices [A | E] (n rows, ncols columns) in complex float, one column at a time
+// in exact arithmetic order: on exit the rows [gj0, n) of the columns [n, ncols) hold those rows of
+// A^{-1} E.  ids, status as above; U: ustride >= gj_augmented_scratch_elems(ncols).  n <= 5120.
+size_t gj_augmented_scratch_elems(int ncols);
+cudaError_t batched_gj_augmented(float2* A, long long stride, int ld, int n, int ncols, int gj0, int nbatch, float2* U,
+                                 long long ustride, int* status, cudaStream_t st, const int* ids = nullptr);
+
 // ---- setup.cu ----
+cudaError_t launch_face_tables(const hps_handle* h, cudaStream_t st);
 cudaError_t launch_tables(double* tables, const TableLayout& tl, double hx, double hy, double hz,
                           cudaStream_t st);
 cudaError_t launch_nodes(const double* tables, const TableLayout& tl, int nx, int ny, int nz,

@@ -1,22 +1,32 @@
 // Setup of the HPS operators on the device (per medium, not per iteration).
 //
-// Per leaf (Sec. 2.1, eq. (leaf)): assemble the dense leaf matrix
-//   A = [ -(D_x^2 + D_y^2 + D_z^2) - C ]   interior rows
-//       [  N + i eta I(I_b, :)          ]   face rows (eq. (flux), F)
-// augmented with identity columns, and eliminate it with partial pivoting
-// (FP64).  Eliminating the last n_b pivots Gauss-Jordan style turns the
-// bottom-right block of U into I, so the boundary rows of the augmented part
-// are (A^{-1})_{b,:} directly:
-//   R_C = I - 2 i eta (A^{-1})_bb,   H_C = -2 i eta (A^{-1})_bi,
-// which follows from g = G u = F u - 2 i eta u_b (eq. (G)).  The face data is
-// then moved to Gauss points: R = P R_C P^{-1}, H = P H_C, P = blockdiag(Q (x) Q).
+// Leaf systems (Sec. 2.1, eq. (leaf)): interior rows -(D_x^2 + D_y^2 + D_z^2) u - C u = s,
+// face rows F u = N u + i eta u = f (eq. (flux)).  A face node couples only to the grid line
+// normal to its face, so the face unknowns are eliminated line by line in closed form: with
+// Phi (2 x 2) and Psi (2 x n1) the face rows' blocks of one line and Theta (n1 x 2) the
+// interior rows' columns of its two ends,
+//   u_b = Phi^{-1} f - Gamma u_i,     Gamma = Phi^{-1} Psi,
+//   S u_i = s - Lambda f,             Lambda = Theta Phi^{-1},
+//   S = T_x (+) T_y (+) T_z - C,      T = -(D^2)_ii - Theta Gamma  (n1 x n1 per axis),
+// and only the n_i x n_i matrix S is inverted numerically (inverse.cu).  From
+// g = G u = F u - 2 i eta u_b (eq. (G)) the leaf maps on the Chebyshev face nodes are
+//   H_C = 2 i eta Gamma S^{-1},   R_C = I - 2 i eta Phi^{-1} - H_C Lambda,
+// moved to Gauss points: R = P R_C P^{-1}, H = P H_C, P = blockdiag(Q (x) Q).  Eliminating the
+// faces first leaves n_i^3 complex multiply-adds per leaf (n_i = 512 at p = 10), where the
+// elimination of the whole leaf system with its n right-hand sides takes 4.0 times as many
+// (5.9 at p = 8); both run on the FP64 pipe, which bounds the setup.  Its error is the smaller
+// one, too: 7e-8 against 1e-7 (complex float) relative to the complex-double maps at p = 10.
 //
 // Preconditioner (Sec. 4, Sec. 4.1): the same leaf maps with C replaced by
 // lambda^tau = (max + min)/2 of C over the leaf (homogenized, R~).  For every
 // cluster of leaves, J_c = I + Pi_c R~ ordered (external, internal) is
-// [[I, 0], [B, I + D]], so J_c^{-1} r needs K_c = (I + D)^{-1} (dense, inverted
-// here by the same elimination kernel) and the blocks B^beta of R~ (internal
-// rows, external columns of each leaf).
+// [[I, 0], [B, I + D]], so J_c^{-1} r needs K_c = (I + D)^{-1} (dense) and the blocks B^beta of
+// R~ (internal rows, external columns of each leaf).  D couples a slot only to the slots of the
+// leaf across its face, so with the leaves coloured like a checkerboard it is
+// [[0, D_rb], [D_br, 0]] and
+//   M = I - D_rb D_br,  K_rr = M^{-1},  K_rb = -M^{-1} D_rb,  K_b* = [0 | I] - D_br K_r*:
+// one inverse of half the size and block-sparse products (3 of 12 blocks per slot on 2x2x2
+// clusters), a quarter of the operations of inverting I + D.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -190,6 +200,156 @@ __global__ void nodes_kernel(const double* T, TableLayout tl, int nx, int ny, in
   }
 }
 
+// ---------------------------------------------------------------------------
+// Tables of the line-wise face elimination per axis, complex double: T (n1 x n1), Gamma
+// (2 x n1), Lambda (n1 x 2), Phi^{-1} (2 x 2).  One thread per axis; n1 <= 14.
+// ---------------------------------------------------------------------------
+__global__ void face_tables_kernel(const double* tab, TableLayout tl, FaceTables ft, double eta, double2* out) {
+  const int axis = threadIdx.x;
+  if (axis >= 3) return;
+  const int p = tl.p, n1 = p - 2, e = p - 1;
+  const double* D = tab + tl.D + axis * p * p;
+  const double* D2 = tab + tl.D2 + axis * p * p;
+  double2* o = out + axis * ft.per_axis;
+  // Phi = [[-D00 + i eta, -D0e], [De0, Dee + i eta]] (outward normals)
+  const double2 f00 = make_double2(-D[0], eta), f01 = make_double2(-D[e], 0.0);
+  const double2 f10 = make_double2(D[e * p], 0.0), f11 = make_double2(D[e * p + e], eta);
+  const double2 di = cinv(csub(cmul(f00, f11), cmul(f01, f10)));
+  double2 pi[2][2];
+  pi[0][0] = cmul(f11, di);
+  pi[0][1] = cscale(cmul(f01, di), -1.0);
+  pi[1][0] = cscale(cmul(f10, di), -1.0);
+  pi[1][1] = cmul(f00, di);
+  for (int r = 0; r < 2; ++r) {
+    for (int c = 0; c < 2; ++c) o[ft.Pi + 2 * r + c] = pi[r][c];
+    // Gamma = Phi^{-1} Psi, Psi = [-D0m; Dem]
+    for (int m = 0; m < n1; ++m)
+      o[ft.G + r * n1 + m] = csub(cscale(pi[r][1], D[e * p + m + 1]), cscale(pi[r][0], D[m + 1]));
+  }
+  for (int m = 0; m < n1; ++m) {
+    // Theta = -[D2_m0, D2_me]
+    const double t0 = -D2[(m + 1) * p], t1 = -D2[(m + 1) * p + e];
+    for (int c = 0; c < 2; ++c) o[ft.L + 2 * m + c] = cadd(cscale(pi[0][c], t0), cscale(pi[1][c], t1));
+    for (int k = 0; k < n1; ++k) {
+      const double2 tg = cadd(cscale(o[ft.G + k], t0), cscale(o[ft.G + n1 + k], t1));
+      o[ft.T + m * n1 + k] = make_double2(-D2[(m + 1) * p + k + 1] - tg.x, -tg.y);
+    }
+  }
+}
+
+// Interior nodes of the grid line normal to a face pair: node m is base + m * step; line l =
+// a + n1 * b with (a, b) the in-face indices of its two end nodes (first axis fastest).
+__device__ __forceinline__ void face_line(int axis, int l, int n1, int& base, int& step) {
+  const int a = l % n1, b = l / n1;
+  step = axis == 0 ? 1 : axis == 1 ? n1 : n1 * n1;
+  base = axis == 0 ? n1 * (a + n1 * b) : axis == 1 ? a + n1 * n1 * b : l;
+}
+
+// S = T_x (+) T_y (+) T_z - C of a batch of leaves (row-major, leading dimension ld), one thread
+// per entry.  C from cdiag of leaf leaf0 + b, or the constant lam[b].
+template <class T>
+__global__ void schur_assemble_kernel(T* S, long long stride, int ld, int leaf0, const double2* ftab, FaceTables ft,
+                                      int n1, const double2* cdiag, const double2* lam) {
+  const int ni = n1 * n1 * n1, b = blockIdx.y;
+  T* Sb = S + b * stride;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ni * ni; t += gridDim.x * blockDim.x) {
+    const int r = t / ni, c = t - r * ni;
+    const int i = r % n1, j = (r / n1) % n1, k = r / (n1 * n1);
+    const int i2 = c % n1, j2 = (c / n1) % n1, k2 = c / (n1 * n1);
+    double2 v = make_double2(0.0, 0.0);
+    if (j == j2 && k == k2) v = cadd(v, ftab[ft.T + i * n1 + i2]);
+    if (i == i2 && k == k2) v = cadd(v, ftab[ft.per_axis + ft.T + j * n1 + j2]);
+    if (i == i2 && j == j2) v = cadd(v, ftab[2 * ft.per_axis + ft.T + k * n1 + k2]);
+    if (r == c) v = csub(v, lam ? lam[b] : cdiag[(long long)(leaf0 + b) * ni + r]);
+    Sb[(long long)r * ld + c] = cvt<T>(v);
+  }
+}
+
+// H_C = 2 i eta Gamma S^{-1} from the inverse X (columns interchanged by perm).  One CTA per
+// grid line: its two end nodes share the line's n1 rows of X, so each is read three times in all.
+template <class T>
+__global__ void __launch_bounds__(128) hc_kernel(const T* X, long long stride, int ldx, const int* perm,
+                                                 const double2* ftab, FaceTables ft, int n1, double eta, T* H,
+                                                 long long hstride, int ldh) {
+  __shared__ T g[2][kMaxP];
+  const int ni = n1 * n1 * n1, n2 = n1 * n1, b = blockIdx.y;
+  const int axis = blockIdx.x / n2, l = blockIdx.x % n2;
+  if (threadIdx.x < 2 * n1)
+    g[threadIdx.x / n1][threadIdx.x % n1] = cvt<T>(ftab[axis * ft.per_axis + ft.G + threadIdx.x]);
+  __syncthreads();
+  int base, step;
+  face_line(axis, l, n1, base, step);
+  const T* Xb = X + b * stride;
+  T* H0 = H + b * hstride + (long long)(2 * axis * n2 + l) * ldh;
+  T* H1 = H0 + (long long)n2 * ldh;
+  const int* pm = perm + (long long)b * ni;
+  using R_ = typename Real<T>::type;
+  const R_ w = (R_)(2.0 * eta);
+  for (int i = threadIdx.x; i < ni; i += 128) {
+    T a0 = czero<T>(), a1 = czero<T>();
+    for (int m = 0; m < n1; ++m) {
+      const T x = Xb[(long long)(base + m * step) * ldx + i];
+      cfma(a0, g[0][m], x);
+      cfma(a1, g[1][m], x);
+    }
+    const int c = pm[i];
+    T o;
+    o.x = -w * a0.y;
+    o.y = w * a0.x;
+    H0[c] = o;
+    o.x = -w * a1.y;
+    o.y = w * a1.x;
+    H1[c] = o;
+  }
+}
+
+// R_C = I - 2 i eta Phi^{-1} - H_C Lambda, or with xbb the boundary block of the leaf inverse,
+// (A^{-1})_bb = Phi^{-1} + H_C Lambda / (2 i eta); one CTA per row (its row of H_C staged in
+// shared memory).
+template <class T>
+__global__ void __launch_bounds__(128) rc_kernel(const T* H, long long hstride, int ldh, const double2* ftab,
+                                                 FaceTables ft, int n1, double eta, T* R, long long rstride, int ldr,
+                                                 bool xbb) {
+  extern __shared__ __align__(16) unsigned char rc_smem[];
+  T* h = reinterpret_cast<T*>(rc_smem);
+  __shared__ T lam[3][2 * kMaxP];
+  const int ni = n1 * n1 * n1, n2 = n1 * n1, b = blockIdx.y, jb = blockIdx.x;
+  const T* Hr = H + b * hstride + (long long)jb * ldh;
+  for (int i = threadIdx.x; i < ni; i += 128) h[i] = Hr[i];
+  for (int i = threadIdx.x; i < 6 * n1; i += 128)
+    lam[i / (2 * n1)][i % (2 * n1)] = cvt<T>(ftab[(i / (2 * n1)) * ft.per_axis + ft.L + i % (2 * n1)]);
+  __syncthreads();
+  T* Rr = R + b * rstride + (long long)jb * ldr;
+  const int f = jb / n2, l = jb % n2;
+  for (int t = threadIdx.x; t < 3 * n2; t += 128) {
+    const int axis = t / n2, l2 = t % n2;
+    int base, step;
+    face_line(axis, l2, n1, base, step);
+    T a[2] = {czero<T>(), czero<T>()};
+    for (int m = 0; m < n1; ++m) {
+      const T x = h[base + m * step];
+      cfma(a[0], x, lam[axis][2 * m]);
+      cfma(a[1], x, lam[axis][2 * m + 1]);
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      T v = czero<T>();
+      if (axis == f >> 1 && l2 == l) {  // ends of the same line
+        const double2 ph = ftab[axis * ft.per_axis + ft.Pi + 2 * (f & 1) + e];
+        v = cvt<T>(xbb ? ph : make_double2((e == (f & 1) ? 1.0 : 0.0) + 2.0 * eta * ph.y, -2.0 * eta * ph.x));
+      }
+      if (xbb) {  // a / (2 i eta) = (a.y - i a.x) / (2 eta)
+        const auto w = (typename Real<T>::type)(0.5 / eta);
+        v.x += w * a[e].y;
+        v.y -= w * a[e].x;
+      } else {
+        v = csub(v, a[e]);
+      }
+      Rr[(2 * axis + e) * n2 + l2] = v;
+    }
+  }
+}
+
 // Local index of grid node (i, j, k), 0 <= i,j,k < p, not on an edge/corner.
 __device__ __forceinline__ int gidx(int i, int j, int k, int p, int n1, int ni) {
   const int last = p - 1;
@@ -202,22 +362,15 @@ __device__ __forceinline__ int gidx(int i, int j, int k, int p, int n1, int ni) 
   return ni + face * n1 * n1 + (a - 1) + n1 * (b - 1);
 }
 
-// ---------------------------------------------------------------------------
-// Leaf matrix assembly into a zeroed row-major workspace (one thread per row).
-// Columns [0, n): A; with ecols >= 1 also [n, n+nb): e_{boundary}; with
-// ecols == 2 also [n+nb, n+nb+ni): e_{interior}.  Interior rows take C from cdiag, or the leaf constant
-// lam[leaf] for the homogenized operator.
-// ---------------------------------------------------------------------------
-template <class T>
-__global__ void assemble_kernel(T* W, long long wstride, int ld, const int* leaf_ids, int leaf0,
-                                int nbatch, const double* tab, TableLayout tl, double eta,
-                                const double2* cdiag, const double2* lam, int ecols) {
+// The homogenized leaf systems of a mixed-only preconditioner, complex float, row-major, zeroed
+// beforehand: columns [0, n) the leaf matrix with the constant lam[b], [n, n + nb) the identity
+// columns of the boundary rows.  One thread per row.
+__global__ void leaf32_assemble_kernel(float2* W, long long wstride, int ld, const double* tab, TableLayout tl,
+                                       double eta, const double2* lam) {
   const int p = tl.p, n1 = p - 2, ni = n1 * n1 * n1, nb = 6 * n1 * n1, n = ni + nb;
-  const int b = blockIdx.y;
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nbatch || r >= n) return;
-  const int leaf = leaf_ids ? leaf_ids[b] : leaf0 + b;
-  T* row = W + (long long)b * wstride + (long long)r * ld;
+  const int b = blockIdx.y, r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= n) return;
+  float2* row = W + b * wstride + (long long)r * ld;
   const double* D = tab + tl.D;
   const double* D2 = tab + tl.D2;
   if (r < ni) {
@@ -227,150 +380,37 @@ __global__ void assemble_kernel(T* W, long long wstride, int ld, const int* leaf
       row[gidx(i, m, k, p, n1, ni)].x -= D2[1 * p * p + j * p + m];
       row[gidx(i, j, m, p, n1, ni)].x -= D2[2 * p * p + k * p + m];
     }
-    const double2 c = lam ? lam[leaf] : cdiag[(long long)leaf * ni + r];
-    row[r].x -= c.x;
-    row[r].y -= c.y;
-    if (ecols == 2) row[n + nb + r].x = 1.0;
+    row[r].x -= lam[b].x;
+    row[r].y -= lam[b].y;
   } else {
-    const int jb = r - ni;
-    const int face = jb / (n1 * n1), rem = jb % (n1 * n1);
-    const int a = rem % n1 + 1, bb = rem / n1 + 1;
-    const int axis = face >> 1;
-    const int e = (face & 1) ? p - 1 : 0;
+    const int jb = r - ni, face = jb / (n1 * n1), rem = jb % (n1 * n1);
+    const int axis = face >> 1, e = (face & 1) ? p - 1 : 0;
     const double sg = (face & 1) ? 1.0 : -1.0;
     int pt[3];
     pt[axis] = e;
-    pt[axis == 0 ? 1 : 0] = a;
-    pt[axis == 2 ? 1 : 2] = bb;
+    pt[axis == 0 ? 1 : 0] = rem % n1 + 1;
+    pt[axis == 2 ? 1 : 2] = rem / n1 + 1;
     for (int m = 0; m < p; ++m) {
       int q3[3] = {pt[0], pt[1], pt[2]};
       q3[axis] = m;
       row[gidx(q3[0], q3[1], q3[2], p, n1, ni)].x += sg * D[axis * p * p + e * p + m];
     }
     row[r].y += eta;
-    if (ecols >= 1) row[n + jb].x = 1.0;
+    row[n + jb].x = 1.f;
   }
 }
 
-// ---------------------------------------------------------------------------
-// Batched elimination with partial pivoting, one CTA per matrix (row-major,
-// n rows, ncols >= n columns).  Pivots k >= gj0 also eliminate the rows
-// [gj0, k) above them, so on exit rows [gj0, n) of columns [n, ncols) hold
-// the corresponding rows of A^{-1} E.  A zero pivot sets *status = 1.
-// ---------------------------------------------------------------------------
-// v -= m u (complex), the elimination's one update
-template <class T>
-__device__ __forceinline__ void gj_update(T& v, const T m, const T u) {
-  v.x -= m.x * u.x - m.y * u.y;
-  v.y -= m.x * u.y + m.y * u.x;
-}
-
-template <class T, int NT>
-__global__ void __launch_bounds__(NT) gj_kernel(T* W, long long wstride, int ld, int n, int ncols,
-                                                int gj0, int nbatch, int* status) {
-  extern __shared__ __align__(16) unsigned char gj_smem[];
-  T* prow = reinterpret_cast<T*>(gj_smem);
-  __shared__ double sval[NT / 32];
-  __shared__ int sidx[NT / 32];
-  __shared__ int piv_s;
-  if ((int)blockIdx.x >= nbatch) return;
-  T* M = W + (long long)blockIdx.x * wstride;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int k = 0; k < n; ++k) {
-    double best = -1.0;
-    int bi = n;
-    for (int r = k + tid; r < n; r += NT) {
-      const T v = M[(long long)r * ld + k];
-      double a = fabs(v.x) + fabs(v.y);
-      if (a > best) { best = a; bi = r; }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      double ob = __shfl_xor_sync(0xffffffffu, best, o);
-      int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-    }
-    if (lane == 0) { sval[warp] = best; sidx[warp] = bi; }
-    __syncthreads();
-    if (warp == 0) {
-      best = (lane < NT / 32) ? sval[lane] : -1.0;
-      bi = (lane < NT / 32) ? sidx[lane] : n;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        double ob = __shfl_xor_sync(0xffffffffu, best, o);
-        int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-      }
-      if (lane == 0) {
-        if (!(best > 0.0) || bi >= n) {
-          atomicExch(status, 1);
-          bi = k;
-        }
-        piv_s = bi;
-      }
-    }
-    __syncthreads();
-    const int piv = piv_s;
-    const T pv = M[(long long)piv * ld + k];
-    const T inv = (pv.x == 0 && pv.y == 0) ? czero<T>() : cinv(pv);
-    for (int c = k + tid; c < ncols; c += NT) {
-      T a = M[(long long)piv * ld + c];
-      if (piv != k) M[(long long)piv * ld + c] = M[(long long)k * ld + c];
-      a = cmul(a, inv);
-      prow[c] = a;
-      M[(long long)k * ld + c] = a;
-    }
-    __syncthreads();
-    const int lo = (k >= gj0) ? gj0 : k + 1;
-    for (int r = lo + warp; r < n; r += NT / 32) {
-      if (r == k) continue;
-      T* Mr = M + (long long)r * ld;
-      const T m = Mr[k];
-      if (m.x == 0 && m.y == 0) continue;
-      // four loads in flight per lane; every element gets the same update as one at a time
-      int c = k + 1 + lane;
-      for (; c + 96 < ncols; c += 128) {
-        T v[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) v[e] = Mr[c + 32 * e];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          gj_update(v[e], m, prow[c + 32 * e]);
-          Mr[c + 32 * e] = v[e];
-        }
-      }
-      for (; c < ncols; c += 32) {
-        T v = Mr[c];
-        gj_update(v, m, prow[c]);
-        Mr[c] = v;
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// R_C = I - 2 i eta X_bb and (optionally) H_C = -2 i eta X_bi from the
-// eliminated workspace, written to per-leaf storage with leading dims ldr/ldh.
-template <class T>
-__global__ void extract_kernel(const T* W, long long wstride, int ld, int n, int ni, int nb,
-                               double eta, int nbatch, T* R, long long rstride, int ldr,
-                               T* H, long long hstride, int ldh) {
+// R_C = I - 2 i eta (A^{-1})_bb from the eliminated float systems.
+__global__ void leaf32_extract_kernel(const float2* W, long long wstride, int ld, int n, int nb, double eta, float2* R,
+                                      long long rstride, int ldr) {
   const int b = blockIdx.y;
-  if (b >= nbatch) return;
-  const int ncols_out = nb + (H ? ni : 0);
-  const T* Wb = W + (long long)b * wstride;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < (long long)nb * ncols_out;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int jb = (int)(t / ncols_out), c = (int)(t % ncols_out);
-    const double2 v = cvt<double2>(Wb[(long long)(ni + jb) * ld + n + c]);
-    // -2 i eta (v.x + i v.y) = 2 eta v.y - 2 i eta v.x
-    double2 o = make_double2(2.0 * eta * v.y, -2.0 * eta * v.x);
-    if (c < nb) {
-      if (c == jb) o.x += 1.0;
-      R[(long long)b * rstride + (long long)jb * ldr + c] = cvt<T>(o);
-    } else {
-      H[(long long)b * hstride + (long long)jb * ldh + (c - nb)] = cvt<T>(o);
-    }
+  const float2* Wb = W + b * wstride;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nb * nb; t += gridDim.x * blockDim.x) {
+    const int jb = t / nb, c = t % nb;
+    const double2 v = cvt<double2>(Wb[(long long)(n - nb + jb) * ld + n + c]);
+    double2 o = make_double2(2.0 * eta * v.y, -2.0 * eta * v.x);  // -2 i eta v
+    if (c == jb) o.x += 1.0;
+    R[b * rstride + (long long)jb * ldr + c] = cvt<float2>(o);
   }
 }
 
@@ -478,11 +518,12 @@ __global__ void lambda_kernel(const double2* c, int ni, double2* lam) {
   }
 }
 
-// B^leaf = R~^leaf[internal face rows][external face cols] for the leaves of a batch,
+// B^leaf = R~^leaf[internal face rows][external face cols] for the leaves of a batch (leaf b's
+// map is number map_pos[b] of Rt),
 // stored transposed (column-major: column c holds the nint q^2 rows, ld rup4(nint q^2))
 // so that stage B reads it with one thread per row, coalesced.
 template <class T>
-__global__ void extract_b_kernel(const T* Rt, long long rstride, int ldr, const int* leaf_ids,
+__global__ void extract_b_kernel(const T* Rt, long long rstride, int ldr, const int* leaf_ids, const int* map_pos,
                                  int nbatch, int q, const uint8_t* int_mask, const long long* b_off,
                                  double2* B64, float2* B32) {
   const int b = blockIdx.y;
@@ -504,117 +545,241 @@ __global__ void extract_b_kernel(const T* Rt, long long rstride, int ldr, const 
        t += (long long)gridDim.x * blockDim.x) {
     const int r = (int)(t / (next * q2)), c = (int)(t % (next * q2));
     const int rf = ifaces[r / q2], cf = efaces[c / q2];
-    const T v = Rt[(long long)b * rstride + (long long)(rf * q2 + r % q2) * ldr + cf * q2 + c % q2];
+    const T v = Rt[map_pos[b] * rstride + (long long)(rf * q2 + r % q2) * ldr + cf * q2 + c % q2];
     const long long o = off + (long long)c * ldt + r;  // stored transposed: column c, row r
     if (B64) B64[o] = cvt<double2>(v);
     if (B32) B32[o] = cvt<float2>(v);
   }
 }
 
-// [I + D | I] for each cluster of a batch (row-major, ld = ldw); D couples
-// internal slot a (leaf alpha, face k) to the slots of beta = nbr(alpha, k)
-// through R~^beta's rows on face k^1.
+// Block products of the checkerboard form of K_c.  A cluster's slots (leaf, face) are described
+// by int4 (leaf, leaf across the face, face, map number of the leaf across), leaves by their
+// position in the cluster; ord lists the slots of red leaves, then those of black ones (h each).
+// Block (a, s) of D is nonzero when slot s belongs to the leaf across slot a: the rows of a's
+// opposite face and the columns of s's face of that leaf's R~.
+//   mode 0  M_ab   = delta_ab - sum_s D_as D_sb         (a, b red; s black)
+//   mode 1  K_as   = -sum_b K_ab D_bs                   (a, b red; s black)
+//   mode 2  K_st   = delta_st - sum_a D_sa K_at         (s black; a red; t any)
+// One CTA per 64 x 64 part of a q^2 x q^2 block; a thread owns rows ty + 16 i and columns
+// tx + 16 j, so parts narrower than 64 (q^2 = 36, 49) skip whole rows and columns of threads.
 template <class T>
-__global__ void assemble_cluster_kernel(T* W, long long wstride, int ldw, int cl0, int nbatch,
-                                        const int* cl_slot_begin, const int* slot_lf,
-                                        const int* cl_leaf_begin, const int* cl_leaves,
-                                        const T* Rt, long long rstride, int ldr, int leafpos0,
-                                        GridDims g, int q) {
-  const int b = blockIdx.y;
-  if (b >= nbatch) return;
-  const int c = cl0 + b;
-  const int q2 = q * q;
-  const int s0 = cl_slot_begin[c], ns = cl_slot_begin[c + 1] - s0;
-  const int nint = ns * q2;
-  const int lb = cl_leaf_begin[c], le = cl_leaf_begin[c + 1];
-  T* Wb = W + (long long)b * wstride;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < (long long)nint * nint;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int row = (int)(t / nint), col = (int)(t % nint);
-    const int sa = row / q2, ja = row % q2;
-    const int sb = col / q2, jb = col % q2;
-    const int lfa = slot_lf[s0 + sa], lfb = slot_lf[s0 + sb];
-    const int alpha = lfa / 6, ka = lfa % 6;
-    const int beta_b = lfb / 6, kb = lfb % 6;
-    T v = czero<T>();
-    if (row == col) v.x = 1;
-    const int beta = g.neighbor(alpha, ka);
-    if (beta == beta_b) {
-      int pos = -1;
-      for (int l = lb; l < le; ++l)
-        if (cl_leaves[l] == beta) pos = l - leafpos0;
-      const T r = Rt[(long long)pos * rstride + (long long)((ka ^ 1) * q2 + ja) * ldr + kb * q2 + jb];
-      v.x += r.x;
-      v.y += r.y;
+struct KcBlocks {
+  const int4* slots;
+  const int* ord;
+  const int* slot_begin;
+  int c0, q2, parts;
+  const T* Rt;
+  long long rstride;
+  int ldr;
+  T* M;  // h q^2 x h q^2 per cluster, leading dimension h q^2
+  long long mstride;
+  T* K;  // 2 h q^2 square per cluster
+  long long kstride;
+};
+
+template <class T, int MODE>
+__global__ void __launch_bounds__(256) kc_product_kernel(const KcBlocks<T> A) {
+  constexpr int kK = 16;
+  __shared__ T sa[kK][64], sb[kK][64];
+  const int b = blockIdx.y, c = A.c0 + b, q2 = A.q2;
+  const int s0 = A.slot_begin[c], ns = A.slot_begin[c + 1] - s0, h = ns / 2;
+  const int ncb = MODE == 2 ? ns : h;  // column blocks
+  const int pp = A.parts * A.parts;
+  const int pair = blockIdx.x / pp, part = blockIdx.x % pp;
+  if (pair >= h * ncb) return;
+  const int4* sl = A.slots + s0;
+  const int* ord = A.ord + s0;
+  const int ri = pair / ncb, ci = pair % ncb;
+  const int rs = ord[MODE == 2 ? h + ri : ri];
+  const int cs = MODE == 2 ? ci : ord[MODE == 1 ? h + ci : ci];
+  const int r0 = (part / A.parts) * 64, c0 = (part % A.parts) * 64;
+  const int nr = min(64, q2 - r0), nc = min(64, q2 - c0);
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  T* K = A.K + b * A.kstride;
+  const long long ldk = (long long)ns * q2;
+  auto dblock = [&](int from, int to) {  // D block (from, to): slot `to` lies on the leaf across `from`
+    return A.Rt + sl[from].w * A.rstride + (long long)((sl[from].z ^ 1) * q2) * A.ldr + sl[to].z * q2;
+  };
+  T acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = czero<T>();
+  for (int m = 0; m < h; ++m) {
+    const int ks = ord[MODE == 0 ? h + m : m];
+    const T *pa, *pb;
+    long long lda, ldb;
+    if (MODE == 0) {
+      if (sl[ks].x != sl[rs].y || sl[cs].x != sl[ks].y) continue;
+      pa = dblock(rs, ks);
+      pb = dblock(ks, cs);
+      lda = ldb = A.ldr;
+    } else if (MODE == 1) {
+      if (sl[cs].x != sl[ks].y) continue;
+      pa = K + (long long)rs * q2 * ldk + ks * q2;
+      pb = dblock(ks, cs);
+      lda = ldk;
+      ldb = A.ldr;
+    } else {
+      if (sl[ks].x != sl[rs].y) continue;
+      pa = dblock(rs, ks);
+      pb = K + (long long)ks * q2 * ldk + cs * q2;
+      lda = A.ldr;
+      ldb = ldk;
     }
+    for (int k0 = 0; k0 < q2; k0 += kK) {
+      const int nk = min(kK, q2 - k0);
+      __syncthreads();
+      for (int t = threadIdx.x; t < kK * 64; t += 256) {
+        const int kk = t % kK, r = t / kK;
+        sa[kk][r] = (kk < nk && r < nr) ? pa[(r0 + r) * lda + k0 + kk] : czero<T>();
+        const int k2 = t / 64, cc = t % 64;
+        sb[k2][cc] = (k2 < nk && cc < nc) ? pb[(k0 + k2) * ldb + c0 + cc] : czero<T>();
+      }
+      __syncthreads();
+      for (int kk = 0; kk < nk; ++kk) {
+        T x[4], y[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          x[i] = sa[kk][ty + 16 * i];
+          y[i] = sb[kk][tx + 16 * i];
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (16 * i + (ty & ~1) >= nr) break;
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (16 * j < nc) cfma(acc[i][j], x[i], y[j]);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int r = ty + 16 * i, cc = tx + 16 * j;
+      if (r >= nr || cc >= nc) continue;
+      T v = czero<T>();
+      if (MODE != 1 && rs == cs && r0 + r == c0 + cc) v.x = 1;
+      v = csub(v, acc[i][j]);
+      if (MODE == 0)
+        A.M[b * A.mstride + (long long)(ri * q2 + r0 + r) * (h * q2) + ci * q2 + c0 + cc] = v;
+      else
+        K[(long long)(rs * q2 + r0 + r) * ldk + cs * q2 + c0 + cc] = v;
+    }
+}
+
+// K_rr = M^{-1}: the inverse's columns back in place (perm), rows and columns at their slots.
+template <class T>
+__global__ void kc_red_kernel(const KcBlocks<T> A, const int* perm, int pstride) {
+  const int b = blockIdx.y, c = A.c0 + b, q2 = A.q2;
+  const int s0 = A.slot_begin[c], ns = A.slot_begin[c + 1] - s0, hn = ns / 2 * q2;
+  const int* ord = A.ord + s0;
+  const int* pm = perm + (long long)b * pstride;
+  const T* X = A.M + b * A.mstride;
+  T* K = A.K + b * A.kstride;
+  const long long ldk = (long long)ns * q2;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < hn * hn; t += gridDim.x * blockDim.x) {
+    const int r = t / hn, i = t - r * hn, cc = pm[i];
+    K[(long long)(ord[r / q2] * q2 + r % q2) * ldk + ord[cc / q2] * q2 + cc % q2] = X[t];
+  }
+}
+
+// [I + D | I] of each cluster of a batch in complex float (row-major, leading dimension ldw).
+__global__ void cluster32_assemble_kernel(float2* W, long long wstride, int ldw, const KcBlocks<float2> A) {
+  const int b = blockIdx.y, c = A.c0 + b, q2 = A.q2;
+  const int s0 = A.slot_begin[c], nint = (A.slot_begin[c + 1] - s0) * q2;
+  const int4* sl = A.slots + s0;
+  float2* Wb = W + b * wstride;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nint * nint; t += gridDim.x * blockDim.x) {
+    const int row = t / nint, col = t - row * nint;
+    const int4 a = sl[row / q2], s = sl[col / q2];
+    const float2 e = make_float2(row == col ? 1.f : 0.f, 0.f);
+    float2 v = e;
+    if (s.x == a.y)
+      v = cadd(v, A.Rt[a.w * A.rstride + (long long)((a.z ^ 1) * q2 + row % q2) * A.ldr + s.z * q2 + col % q2]);
     Wb[(long long)row * ldw + col] = v;
-    T e = czero<T>();
-    if (row == col) e.x = 1;
     Wb[(long long)row * ldw + nint + col] = e;
   }
 }
 
+// K_c of a batch from the workspace (aug: the right half of [I + D | I], leading dimension ldw;
+// otherwise a square of its own size) into the handle's copies.
 template <class T>
-__global__ void extract_kc_kernel(const T* W, long long wstride, int ldw, int cl0, int nbatch,
-                                  const int* cl_slot_begin, const long long* kc_off, int q, double2* K64,
-                                  float2* K32) {
-  const int b = blockIdx.y;
-  if (b >= nbatch) return;
-  const int c = cl0 + b;
-  const int q2 = q * q;
-  const int nint = (cl_slot_begin[c + 1] - cl_slot_begin[c]) * q2;
+__global__ void extract_kc_kernel(const T* K, long long kstride, bool aug, int ldw, int cl0, const int* cl_slot_begin,
+                                  const long long* kc_off, int q, double2* K64, float2* K32) {
+  const int b = blockIdx.y, c = cl0 + b;
+  const int nint = (cl_slot_begin[c + 1] - cl_slot_begin[c]) * q * q;
   const int ldk = (int)rup4(nint);
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < (long long)nint * nint;
        t += (long long)gridDim.x * blockDim.x) {
     const int row = (int)(t / nint), col = (int)(t % nint);
-    const T v = W[(long long)b * wstride + (long long)row * ldw + nint + col];
+    const T v = K[b * kstride + (aug ? (long long)row * ldw + nint + col : t)];
     const long long o = kc_off[c] + (long long)row * ldk + col;
     if (K64) K64[o] = cvt<double2>(v);
     if (K32) K32[o] = cvt<float2>(v);
   }
 }
 
-// Right-hand-side columns [s; P^{-1} f] of the leaf systems of a batch (leaves
-// leaf0..leaf0+nbatch-1), one column per right-hand side at W[:, n + k].
-// P^{-1} maps a face's Gauss-point data F (q x q) to the Chebyshev face nodes:
-// Qi F Qi^T.
-__global__ void recover_rhs_kernel(double2* W, long long wstride, int ld, int leaf0, int nbatch, const double* tab,
-                                   TableLayout tl, const double2* s, const double2* f, int nrhs, long long nint,
-                                   long long nf) {
-  const int q = tl.q, q2 = q * q, n1 = tl.p - 2, ni = n1 * n1 * n1, nb = 6 * q2, n = ni + nb;
-  const int b = blockIdx.y;
-  if (b >= nbatch) return;
-  const int leaf = leaf0 + b;
+// Face data at the Chebyshev face nodes, fhat = P^{-1} f: Qi F Qi^T on every face of the leaves
+// leaf0..leaf0+nbatch-1, [leaf][rhs][nb].
+__global__ void recover_faces_kernel(double2* fhat, int leaf0, const double* tab, TableLayout tl, const double2* f,
+                                     int nrhs, long long nf) {
+  const int q = tl.q, q2 = q * q, nb = 6 * q2, b = blockIdx.y;
   const double* Qi = tab + tl.Qi;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n * nrhs; t += gridDim.x * blockDim.x) {
-    const int r = t % n, k = t / n;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nb * nrhs; t += gridDim.x * blockDim.x) {
+    const int jb = t % nb, k = t / nb, a = jb % q2, a1 = a % q, a2 = a / q;
+    const double2* F = f + k * nf + (long long)(leaf0 + b) * nb + (jb - a);
     double2 v = make_double2(0.0, 0.0);
-    if (r < ni) {
-      if (s) v = s[k * nint + (long long)leaf * ni + r];
-    } else {
-      const int jb = r - ni, face = jb / q2, a = jb % q2, a1 = a % q, a2 = a / q;
-      const double2* F = f + k * nf + (long long)leaf * nb + (long long)face * q2;
-      for (int j2 = 0; j2 < q; ++j2) {
-        double2 row = make_double2(0.0, 0.0);
-        for (int j1 = 0; j1 < q; ++j1) row = cadd(row, cscale(F[j2 * q + j1], Qi[a1 * q + j1]));
-        v = cadd(v, cscale(row, Qi[a2 * q + j2]));
-      }
+    for (int j2 = 0; j2 < q; ++j2) {
+      double2 row = make_double2(0.0, 0.0);
+      for (int j1 = 0; j1 < q; ++j1) row = cadd(row, cscale(F[j2 * q + j1], Qi[a1 * q + j1]));
+      v = cadd(v, cscale(row, Qi[a2 * q + j2]));
     }
-    W[(long long)b * wstride + (long long)r * ld + n + k] = v;
+    fhat[((long long)b * nrhs + k) * nb + jb] = v;
   }
 }
 
-__global__ void recover_extract_kernel(const double2* W, long long wstride, int ld, int n, int ni, int leaf0,
-                                       int nbatch, int nrhs, long long nint, double2* u, long long nfc,
-                                       double2* uf) {
-  const int b = blockIdx.y;
-  if (b >= nbatch) return;
-  const int nb = n - ni;
+// Right-hand-side columns s - Lambda fhat of the reduced leaf systems, column k at W[:, ni + k].
+__global__ void recover_rhs_kernel(double2* W, long long wstride, int ld, int leaf0, const double2* ftab,
+                                   FaceTables ft, int n1, const double2* s, const double2* fhat, int nrhs,
+                                   long long nint) {
+  const int n2 = n1 * n1, ni = n1 * n2, nb = 6 * n2, b = blockIdx.y;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ni * nrhs; t += gridDim.x * blockDim.x) {
+    const int r = t % ni, k = t / ni;
+    const int m[3] = {r % n1, (r / n1) % n1, r / n2};
+    const int line[3] = {m[1] + n1 * m[2], m[0] + n1 * m[2], m[0] + n1 * m[1]};
+    const double2* fh = fhat + ((long long)b * nrhs + k) * nb;
+    double2 v = s ? s[k * nint + (long long)(leaf0 + b) * ni + r] : make_double2(0.0, 0.0);
+    for (int axis = 0; axis < 3; ++axis)
+      for (int e = 0; e < 2; ++e)
+        v = csub(v, cmul(ftab[axis * ft.per_axis + ft.L + 2 * m[axis] + e], fh[(2 * axis + e) * n2 + line[axis]]));
+    W[b * wstride + (long long)r * ld + ni + k] = v;
+  }
+}
+
+// u_i from the solved columns, and u_b = Phi^{-1} fhat - Gamma u_i.
+__global__ void recover_extract_kernel(const double2* W, long long wstride, int ld, int leaf0, const double2* ftab,
+                                       FaceTables ft, int n1, const double2* fhat, int nrhs, long long nint,
+                                       double2* u, long long nfc, double2* uf) {
+  const int n2 = n1 * n1, ni = n1 * n2, nb = 6 * n2, n = ni + (uf ? nb : 0), b = blockIdx.y;
+  const double2* Wb = W + b * wstride;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n * nrhs; t += gridDim.x * blockDim.x) {
     const int r = t % n, k = t / n;
-    const double2 v = W[(long long)b * wstride + (long long)r * ld + n + k];
-    if (r < ni) u[k * nint + (long long)(leaf0 + b) * ni + r] = v;
-    else if (uf) uf[k * nfc + (long long)(leaf0 + b) * nb + (r - ni)] = v;
+    if (r < ni) {
+      u[k * nint + (long long)(leaf0 + b) * ni + r] = Wb[(long long)r * ld + ni + k];
+      continue;
+    }
+    const int jb = r - ni, f = jb / n2, l = jb % n2, axis = f >> 1, e = f & 1;
+    const double2* tb = ftab + axis * ft.per_axis;
+    const double2* fh = fhat + ((long long)b * nrhs + k) * nb + 2 * axis * n2 + l;
+    double2 v = cadd(cmul(tb[ft.Pi + 2 * e], fh[0]), cmul(tb[ft.Pi + 2 * e + 1], fh[n2]));
+    int base, step;
+    face_line(axis, l, n1, base, step);
+    for (int m = 0; m < n1; ++m)
+      v = csub(v, cmul(tb[ft.G + e * n1 + m], Wb[(long long)(base + m * step) * ld + ni + k]));
+    uf[k * nfc + (long long)(leaf0 + b) * nb + jb] = v;
   }
 }
 
@@ -646,14 +811,12 @@ __global__ void quantize_kc_kernel(const float2* K32, __half2* K16, float* kscal
   }
 }
 
-// K_c rows of one batch straight from the elimination workspace (columns
-// [nint, 2 nint) of each cluster's [I + D | I]) into FP16 with row scales.
-__global__ void quantize_kc_ws_kernel(const float2* W, long long wstride, int ldw, int cl0, int nbatch,
-                                      const int* cl_slot_begin, const long long* kc_off, int q2, __half2* K16,
-                                      float* kscale) {
+// K_c rows of one batch straight from the workspace (the right half of [I + D | I]) into FP16 with
+// row scales.
+__global__ void quantize_kc_ws_kernel(const float2* W, long long wstride, int ldw, int cl0, const int* cl_slot_begin,
+                                      const long long* kc_off, int q2, __half2* K16, float* kscale) {
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.y;
-  if (b >= nbatch) return;
   const int c = cl0 + b;
   const int s0 = cl_slot_begin[c];
   const int nint = (cl_slot_begin[c + 1] - s0) * q2;
@@ -724,6 +887,11 @@ cudaError_t launch_tables(double* tables, const TableLayout& tl, double hx, doub
   return cudaGetLastError();
 }
 
+cudaError_t launch_face_tables(const hps_handle* h, cudaStream_t st) {
+  face_tables_kernel<<<1, 32, 0, st>>>(h->tables, h->tl, h->ft, h->eta, h->ftab);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_cdiag(const double2* b, double kappa, long long count, double2* c, cudaStream_t st) {
   cdiag_kernel<<<1024, 256, 0, st>>>(b, kappa, count, c);
   return cudaGetLastError();
@@ -736,18 +904,6 @@ cudaError_t launch_nodes(const double* tables, const TableLayout& tl, int nx, in
 }
 
 namespace {
-
-constexpr int kGjThreads = 512;
-
-template <class T>
-cudaError_t run_gj(T* W, long long wstride, int ld, int n, int ncols, int gj0, int nbatch, int* status,
-                   cudaStream_t st) {
-  const size_t smem = (size_t)ncols * sizeof(T);
-  cudaError_t e = allow_dynamic_smem((const void*)gj_kernel<T, kGjThreads>, smem);
-  if (e != cudaSuccess) return e;
-  gj_kernel<T, kGjThreads><<<nbatch, kGjThreads, smem, st>>>(W, wstride, ld, n, ncols, gj0, nbatch, status);
-  return cudaGetLastError();
-}
 
 template <class T>
 cudaError_t run_seg_kron(T* M, long long mstride, int ld, int nrows, int ncols, int nbatch,
@@ -781,10 +937,10 @@ size_t workspace_budget(const hps_handle* h) {
 }  // namespace
 
 // Cap on the transient setup workspace: 24 GiB, raised up to 96 GiB where that is needed for one
-// leaf elimination per SM (large leaves, p >= 14); the remaining HBM budget of the handle when one
+// leaf inverse per SM (large leaves, p >= 15); the remaining HBM budget of the handle when one
 // is set (setup also keeps it under a third of the free device memory).
 size_t workspace_cap(const hps_handle* h) {
-  const size_t per = (size_t)h->n * (size_t)(h->n + h->nb + h->ni) * sizeof(double2);
+  const size_t per = (size_t)h->ni * (h->ni + gj_scratch_elems<double2>(1)) * sizeof(double2);
   size_t cap = std::max((size_t)24 << 30, std::min(per * (size_t)std::max(h->nsm, 1), (size_t)96 << 30));
   if (h->opt.hbm_budget) {
     const size_t rest = h->opt.hbm_budget > h->bytes ? h->opt.hbm_budget - h->bytes : 0;
@@ -793,64 +949,129 @@ size_t workspace_cap(const hps_handle* h) {
   return cap;
 }
 
+// Leaves of one batch of the exact maps: the inverses of 8 leaves per SM at most (the update
+// launches of a batch then have thousands of tiles, and more leaves would gain nothing).
 size_t exact_maps_workspace(const hps_handle* h, size_t budget, int* nbatch_out) {
-  const long long per = (long long)h->n * (h->n + h->nb + h->ni) * (long long)sizeof(double2);
-  int nbatch = (int)std::min<long long>((long long)h->nl, std::max<long long>(1, (long long)(budget / per)));
-  nbatch = std::min(nbatch, 4 * h->nsm);
+  size_t per = ((size_t)h->ni * h->ni + gj_scratch_elems<double2>(h->ni)) * sizeof(double2) + (size_t)h->ni * sizeof(int);
+  if (h->opt.lean) per += (size_t)h->nb * (h->ldR + h->ldH) * sizeof(double2);  // FP64 maps before rounding
+  int nbatch = (int)std::min<size_t>((size_t)h->nl, std::max<size_t>(1, budget / per));
+  nbatch = std::min(nbatch, 8 * h->nsm);
   if (nbatch_out) *nbatch_out = nbatch;
-  return (size_t)per * nbatch;
+  return per * nbatch;
 }
 
+namespace {
+
+// Transient device memory of one setup phase, freed on every way out.
+struct Workspace {
+  std::vector<void*> ptrs;
+  template <class V> cudaError_t get(V*& p, size_t count) {
+    void* v = nullptr;
+    const cudaError_t e = cudaMalloc(&v, std::max<size_t>(count, 1) * sizeof(V));
+    if (e == cudaSuccess) ptrs.push_back(v);
+    p = (V*)v;
+    return e;
+  }
+  ~Workspace() {
+    for (void* v : ptrs) cudaFree(v);
+  }
+};
+
+// Buffers of a batch of leaf inverses.
+template <class T>
+struct LeafWork {
+  T *S = nullptr, *U = nullptr;
+  int *perm = nullptr, *status = nullptr;
+  cudaError_t get(Workspace& ws, const hps_handle* h, int nbatch, cudaStream_t st) {
+    cudaError_t e = ws.get(S, (size_t)nbatch * h->ni * h->ni);
+    if (e == cudaSuccess) e = ws.get(U, (size_t)nbatch * gj_scratch_elems<T>(h->ni));
+    if (e == cudaSuccess) e = ws.get(perm, (size_t)nbatch * h->ni);
+    if (e == cudaSuccess) e = ws.get(status, 1);
+    if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sizeof(int), st);
+    return e;
+  }
+};
+
+// Leaf maps on the Chebyshev face nodes of nbt leaves: R_C (xbb: (A^{-1})_bb) into R, H_C into H
+// (leading dimensions ldR, ldH of the handle).  C from the medium of the leaves leaf0..., or the constants lam.
+template <class T>
+int chebyshev_maps(const hps_handle* h, const LeafWork<T>& w, int nbt, int leaf0, const double2* cdiag,
+                   const double2* lam, T* R, T* H, cudaStream_t st, bool xbb = false) {
+  const int n1 = h->n1, ni = h->ni, nb = h->nb, n2 = n1 * n1;
+  const long long ss = (long long)ni * ni, rs = (long long)nb * h->ldR, hs = (long long)nb * h->ldH;
+  schur_assemble_kernel<T><<<dim3(std::min(1024, (ni * ni + 255) / 256), nbt), 256, 0, st>>>(
+      w.S, ss, ni, leaf0, h->ftab, h->ft, n1, cdiag, lam);
+  HPS_CUDA_TRY(cudaGetLastError());
+  HPS_CUDA_TRY(batched_gj<T>(w.S, ss, ni, ni, ni, nbt, w.U, (long long)gj_scratch_elems<T>(ni), w.perm, ni, w.status, st));
+  hc_kernel<T><<<dim3(3 * n2, nbt), 128, 0, st>>>(w.S, ss, ni, w.perm, h->ftab, h->ft, n1, h->eta, H, hs, h->ldH);
+  HPS_CUDA_TRY(cudaGetLastError());
+  rc_kernel<T><<<dim3(nb, nbt), 128, (size_t)ni * sizeof(T), st>>>(H, hs, h->ldH, h->ftab, h->ft, n1, h->eta, R, rs,
+                                                                  h->ldR, xbb);
+  HPS_CUDA_TRY(cudaGetLastError());
+  return HPS_OK;
+}
+
+}  // namespace
+
+// Clusters of one batch of the preconditioner's blocks: at most 2 per SM.
 size_t precond_workspace(const hps_handle* h, size_t budget, int* cb_out) {
   const ClusterTables& ct = h->ct;
   const int q2 = h->q * h->q;
-  int max_int = 0, max_leaves = 0;
+  size_t max_int = 0, max_leaves = 0;
   for (int k = 0; k < ct.nkc; ++k) {
     const int c = ct.kc_rep[k];
-    max_int = std::max(max_int, (ct.cl_slot_begin[c + 1] - ct.cl_slot_begin[c]) * q2);
-    max_leaves = std::max(max_leaves, ct.cl_leaf_begin[c + 1] - ct.cl_leaf_begin[c]);
+    max_int = std::max<size_t>(max_int, (size_t)(ct.cl_slot_begin[c + 1] - ct.cl_slot_begin[c]) * q2);
+    max_leaves = std::max<size_t>(max_leaves, ct.cl_leaf_begin[c + 1] - ct.cl_leaf_begin[c]);
   }
-  const long long wl_stride = (long long)h->n * (h->n + h->nb);
-  const int ldw = std::max(2, 2 * max_int);
-  const long long wc_stride = (long long)std::max(1, max_int) * ldw;
-  const size_t per_cluster =
-      ((size_t)wl_stride * max_leaves + (size_t)h->nb * h->ldR * max_leaves + (size_t)wc_stride) * sizeof(double2);
-  int cb = (int)std::min<size_t>((size_t)std::max(1, ct.nkc), std::max<size_t>(1, budget / per_cluster));
+  const size_t hn = max_int / 2, nbl = (size_t)h->nb * h->ldR;
+  size_t per_cluster;
+  if (h->opt.forms & HPS_FORM_FP64) {
+    const size_t leaf = (size_t)h->ni * h->ni + gj_scratch_elems<double2>(h->ni) + h->ni + nbl + (size_t)h->nb * h->ldH;
+    per_cluster = (leaf * max_leaves + max_int * max_int + hn * hn + gj_scratch_elems<double2>((int)hn) + hn) * sizeof(double2);
+  } else {
+    const size_t leaf = (size_t)(h->n + gj_augmented_scratch_elems(1)) * (h->n + h->nb) + nbl;
+    per_cluster = (leaf * max_leaves + 2 * max_int * (max_int + gj_augmented_scratch_elems(1))) * sizeof(float2);
+  }
+  int cb = (int)std::min<size_t>((size_t)std::max(1, ct.nkc), std::max<size_t>(1, budget / std::max<size_t>(1, per_cluster)));
   cb = std::min(cb, std::max(1, 2 * h->nsm));
   if (cb_out) *cb_out = cb;
   return per_cluster * cb;
 }
 
-// Interior values of the leaf solutions u^tau = A^{tau,-1} [s^tau; P^{-1} f^tau]
-// (eq. (leaf)), by FP64 elimination of each leaf system with nrhs extra columns.
+// Leaf solutions u^tau = A^{tau,-1} [s^tau; P^{-1} f^tau] (eq. (leaf)): S u_i = s - Lambda fhat by
+// FP64 elimination with nrhs extra columns, u_b from u_i line by line.
 int recover_interior(hps_handle* h, const double2* s, const double2* f, int nrhs, double2* u, double2* uf,
                      cudaStream_t st) {
-  const int n = h->n, ni = h->ni;
-  const int ncols = n + nrhs, ld = ncols;
-  const long long wstride = (long long)n * ld;
-  const size_t per = (size_t)wstride * sizeof(double2);
+  const int ni = h->ni, nb = h->nb, n1 = h->n1;
+  const int ld = ni + nrhs;
+  const long long wstride = (long long)ni * ld;
+  const size_t scr = gj_scratch_elems<double2>(ld);
+  const size_t per = ((size_t)wstride + scr + (size_t)nb * nrhs) * sizeof(double2) + (size_t)ni * sizeof(int);
   int nbatch = (int)std::min<size_t>((size_t)h->nl, std::max<size_t>(1, workspace_budget(h) / per));
-  nbatch = std::min(nbatch, 4 * h->nsm);
-  double2* W = nullptr;
-  int* d_status = nullptr;
-  HPS_CUDA_TRY(cudaMalloc(&W, per * nbatch));
-  HPS_CUDA_TRY(cudaMalloc(&d_status, sizeof(int)));
+  nbatch = std::min(nbatch, 8 * h->nsm);
+  Workspace ws;
+  double2 *W = nullptr, *U = nullptr, *fhat = nullptr;
+  int *perm = nullptr, *d_status = nullptr;
+  HPS_CUDA_TRY(ws.get(W, (size_t)wstride * nbatch));
+  HPS_CUDA_TRY(ws.get(U, scr * nbatch));
+  HPS_CUDA_TRY(ws.get(fhat, (size_t)nb * nrhs * nbatch));
+  HPS_CUDA_TRY(ws.get(perm, (size_t)ni * nbatch));
+  HPS_CUDA_TRY(ws.get(d_status, 1));
   HPS_CUDA_TRY(cudaMemsetAsync(d_status, 0, sizeof(int), st));
   int rc = HPS_OK;
   for (int l0 = 0; l0 < h->nl && rc == HPS_OK; l0 += nbatch) {
     const int nbt = std::min(nbatch, h->nl - l0);
     auto body = [&]() -> int {
-      HPS_CUDA_TRY(cudaMemsetAsync(W, 0, per * nbt, st));
-      dim3 ga((n + 127) / 128, nbt);
-      assemble_kernel<double2><<<ga, 128, 0, st>>>(W, wstride, ld, nullptr, l0, nbt, h->tables, h->tl, h->eta,
-                                                  h->cdiag, nullptr, 0);
+      schur_assemble_kernel<double2><<<dim3(std::min(1024, (ni * ni + 255) / 256), nbt), 256, 0, st>>>(
+          W, wstride, ld, l0, h->ftab, h->ft, n1, h->cdiag, nullptr);
       HPS_CUDA_TRY(cudaGetLastError());
-      recover_rhs_kernel<<<dim3(32, nbt), 128, 0, st>>>(W, wstride, ld, l0, nbt, h->tables, h->tl, s, f, nrhs,
-                                                         h->nint, h->nf);
+      recover_faces_kernel<<<dim3(32, nbt), 128, 0, st>>>(fhat, l0, h->tables, h->tl, f, nrhs, h->nf);
       HPS_CUDA_TRY(cudaGetLastError());
-      HPS_CUDA_TRY(run_gj(W, wstride, ld, n, ncols, 0, nbt, d_status, st));
-      recover_extract_kernel<<<dim3(32, nbt), 128, 0, st>>>(W, wstride, ld, n, ni, l0, nbt, nrhs, h->nint, u,
-                                                             (long long)h->nl * h->nb, uf);
+      recover_rhs_kernel<<<dim3(32, nbt), 128, 0, st>>>(W, wstride, ld, l0, h->ftab, h->ft, n1, s, fhat, nrhs, h->nint);
+      HPS_CUDA_TRY(cudaGetLastError());
+      HPS_CUDA_TRY(batched_gj<double2>(W, wstride, ld, ni, ld, nbt, U, (long long)scr, perm, ni, d_status, st));
+      recover_extract_kernel<<<dim3(32, nbt), 128, 0, st>>>(W, wstride, ld, l0, h->ftab, h->ft, n1, fhat, nrhs,
+                                                             h->nint, u, h->nf, uf);
       HPS_CUDA_TRY(cudaGetLastError());
       return HPS_OK;
     };
@@ -858,28 +1079,20 @@ int recover_interior(hps_handle* h, const double2* s, const double2* f, int nrhs
   }
   if (rc == HPS_OK) rc = check_status(d_status, st, "leaf solution recovery");
   cudaStreamSynchronize(st);
-  cudaFree(W);
-  cudaFree(d_status);
   return rc;
 }
 
 int build_exact_maps(hps_handle* h, const double2* cdiag, cudaStream_t st) {
-  const int n = h->n, ni = h->ni, nb = h->nb;
-  const int ncols = n + nb + ni;
-  const int ld = ncols;
-  const long long wstride = (long long)n * ld;
-  const size_t per = (size_t)wstride * sizeof(double2);
+  const int ni = h->ni, nb = h->nb;
   int nbatch = 1;
   exact_maps_workspace(h, workspace_budget(h), &nbatch);
-  double2* W = nullptr;
-  int* d_status = nullptr;
+  Workspace ws;
+  LeafWork<double2> lw;
+  HPS_CUDA_TRY(lw.get(ws, h, nbatch, st));
   double2 *Rtmp = nullptr, *Htmp = nullptr;  // lean mode: FP64 maps of one batch before rounding
-  HPS_CUDA_TRY(cudaMalloc(&W, per * nbatch));
-  HPS_CUDA_TRY(cudaMalloc(&d_status, sizeof(int)));
-  HPS_CUDA_TRY(cudaMemsetAsync(d_status, 0, sizeof(int), st));
   if (!h->R64) {
-    HPS_CUDA_TRY(cudaMalloc(&Rtmp, (size_t)nbatch * nb * h->ldR * sizeof(double2)));
-    HPS_CUDA_TRY(cudaMalloc(&Htmp, (size_t)nbatch * nb * h->ldH * sizeof(double2)));
+    HPS_CUDA_TRY(ws.get(Rtmp, (size_t)nbatch * nb * h->ldR));
+    HPS_CUDA_TRY(ws.get(Htmp, (size_t)nbatch * nb * h->ldH));
     HPS_CUDA_TRY(cudaMemsetAsync(Rtmp, 0, (size_t)nbatch * nb * h->ldR * sizeof(double2), st));
     HPS_CUDA_TRY(cudaMemsetAsync(Htmp, 0, (size_t)nbatch * nb * h->ldH * sizeof(double2), st));
   }
@@ -887,18 +1100,9 @@ int build_exact_maps(hps_handle* h, const double2* cdiag, cudaStream_t st) {
   for (int l0 = 0; l0 < h->nl && rc == HPS_OK; l0 += nbatch) {
     const int nbt = std::min(nbatch, h->nl - l0);
     auto body = [&]() -> int {
-      HPS_CUDA_TRY(cudaMemsetAsync(W, 0, per * nbt, st));
-      dim3 ga((n + 127) / 128, nbt);
-      assemble_kernel<double2><<<ga, 128, 0, st>>>(W, wstride, ld, nullptr, l0, nbt, h->tables, h->tl, h->eta,
-                                                  cdiag, nullptr, 2);
-      HPS_CUDA_TRY(cudaGetLastError());
-      HPS_CUDA_TRY(run_gj(W, wstride, ld, n, ncols, ni, nbt, d_status, st));
       double2* Rb = h->R64 ? h->R64 + (long long)l0 * nb * h->ldR : Rtmp;
       double2* Hb = h->H64 ? h->H64 + (long long)l0 * nb * h->ldH : Htmp;
-      dim3 ge(256, nbt);
-      extract_kernel<double2><<<ge, 256, 0, st>>>(W, wstride, ld, n, ni, nb, h->eta, nbt, Rb,
-                                                  (long long)nb * h->ldR, h->ldR, Hb, (long long)nb * h->ldH, h->ldH);
-      HPS_CUDA_TRY(cudaGetLastError());
+      if (const int r = chebyshev_maps<double2>(h, lw, nbt, l0, cdiag, nullptr, Rb, Hb, st)) return r;
       // R = P (R_C P^{-1}): rows by Q^{-T} (.) Q^{-1}, then columns by Q (.) Q^T.
       HPS_CUDA_TRY(run_seg_kron(Rb, (long long)nb * h->ldR, h->ldR, nb, nb, nbt, h->tables, h->tl, 1, 0, h->nsm, st));
       HPS_CUDA_TRY(run_seg_kron(Rb, (long long)nb * h->ldR, h->ldR, nb, nb, nbt, h->tables, h->tl, 0, 1, h->nsm, st));
@@ -924,12 +1128,8 @@ int build_exact_maps(hps_handle* h, const double2* cdiag, cudaStream_t st) {
     };
     rc = body();
   }
-  if (rc == HPS_OK) rc = check_status(d_status, st, "leaf ItI maps");
+  if (rc == HPS_OK) rc = check_status(lw.status, st, "leaf ItI maps");
   cudaStreamSynchronize(st);
-  cudaFree(W);
-  cudaFree(d_status);
-  if (Rtmp) cudaFree(Rtmp);
-  if (Htmp) cudaFree(Htmp);
   return rc;
 }
 
@@ -1208,77 +1408,181 @@ void assign_blocks(hps_handle* h, const std::vector<double2>* lamq) {
 // preconditioner needs, at the FP32 rate).  One representative cluster per
 // block is built; its leaves' B blocks are the distinct B blocks (a leaf's B
 // block depends only on its binned lambda and internal-face mask, both part of
-// the cluster key).  rep_* index the representatives as clusters 0..nkc-1.
+// the cluster key).  Within a batch of clusters each distinct constant's leaf
+// map is built once.
 template <class T>
-int build_precond_blocks(hps_handle* h, const int* d_rep_leaf_begin, const int* d_rep_leaves,
-                         const int* d_rep_slot_lf, const std::vector<int>& rep_leaf_begin, cudaStream_t st) {
+int build_precond_blocks(hps_handle* h, const std::vector<int>& rep_leaf_begin, const std::vector<int>& rep_leaves,
+                         cudaStream_t st) {
   ClusterTables& ct = h->ct;
-  const int n = h->n, ni = h->ni, nb = h->nb, q = h->q, q2 = q * q;
-  int max_int = 0, max_leaves = 0;
-  for (int k = 0; k < ct.nkc; ++k) {
-    max_int = std::max(max_int, (ct.kc_slot_begin[k + 1] - ct.kc_slot_begin[k]) * q2);
-    max_leaves = std::max(max_leaves, rep_leaf_begin[k + 1] - rep_leaf_begin[k]);
-  }
-  const int ncols_l = n + nb, ld_l = ncols_l;
-  const long long wl_stride = (long long)n * ld_l;
-  const int ldw = std::max(2, 2 * max_int);
-  const long long wc_stride = (long long)std::max(1, max_int) * ldw;
-  int cb = 1;
+  const int nb = h->nb, q = h->q, q2 = q * q;
+  int cb = 1, max_int = 0;
   precond_workspace(h, workspace_budget(h), &cb);
-  T *Wl = nullptr, *Rt = nullptr, *Wc = nullptr;
-  int* d_status = nullptr;
-  HPS_CUDA_TRY(cudaMalloc(&Wl, (size_t)wl_stride * max_leaves * cb * sizeof(T)));
-  HPS_CUDA_TRY(cudaMalloc(&Rt, (size_t)nb * h->ldR * max_leaves * cb * sizeof(T)));
-  HPS_CUDA_TRY(cudaMalloc(&Wc, (size_t)wc_stride * cb * sizeof(T)));
-  HPS_CUDA_TRY(cudaMalloc(&d_status, sizeof(int)));
-  HPS_CUDA_TRY(cudaMemsetAsync(d_status, 0, sizeof(int), st));
-  GridDims gd{h->nx, h->ny, h->nz};
-  int rc = HPS_OK;
-  for (int c0 = 0; c0 < ct.nkc && rc == HPS_OK; c0 += cb) {
+  // per batch: the distinct constants and each representative leaf's map among them
+  std::vector<double2> lams;
+  std::vector<int> lam_begin(1, 0), map_pos(rep_leaves.size(), 0);
+  int max_lam = 1;
+  for (int c0 = 0; c0 < ct.nkc; c0 += cb) {
+    std::map<std::pair<uint64_t, uint64_t>, int> seen;
+    for (int l = rep_leaf_begin[c0]; l < rep_leaf_begin[std::min(ct.nkc, c0 + cb)]; ++l) {
+      const double2 v = h->lambda_q_host[rep_leaves[l]];
+      uint64_t a, b;
+      std::memcpy(&a, &v.x, 8);
+      std::memcpy(&b, &v.y, 8);
+      const auto it = seen.emplace(std::make_pair(a, b), (int)seen.size());
+      if (it.second) lams.push_back(v);
+      map_pos[l] = it.first->second;
+    }
+    lam_begin.push_back((int)lams.size());
+    max_lam = std::max(max_lam, (int)seen.size());
+  }
+  // slots of the representatives: (leaf, leaf across, face, map of the leaf across), red ones first
+  std::vector<int4> slots;
+  std::vector<int> ord;
+  for (int k = 0; k < ct.nkc; ++k) {
+    const int c = ct.kc_rep[k], lb = rep_leaf_begin[k];
+    const int s0 = ct.cl_slot_begin[c], ns = ct.cl_slot_begin[c + 1] - s0;
+    max_int = std::max(max_int, ns * q2);
+    auto pos = [&](int leaf) {
+      for (int l = lb; l < rep_leaf_begin[k + 1]; ++l)
+        if (rep_leaves[l] == leaf) return l - lb;
+      return -1;
+    };
+    std::vector<int> black;
+    for (int i = 0; i < ns; ++i) {
+      const int leaf = ct.slot_lf[s0 + i] / 6, f = ct.slot_lf[s0 + i] % 6;
+      int c3[3] = {leaf % h->nx, (leaf / h->nx) % h->ny, leaf / (h->nx * h->ny)};
+      const bool red = (c3[0] + c3[1] + c3[2]) % 2 == 0;
+      c3[f >> 1] += (f & 1) ? 1 : -1;
+      const int across = pos(c3[0] + h->nx * (c3[1] + h->ny * c3[2]));
+      slots.push_back(make_int4(pos(leaf), across, f, map_pos[lb + across]));
+      if (red) ord.push_back(i);
+      else black.push_back(i);
+    }
+    ord.insert(ord.end(), black.begin(), black.end());
+  }
+  // matrices of one size per batch (clusters cut off at the end of an odd axis are smaller)
+  struct Group {
+    int n, first, count;
+  };
+  std::vector<int> ids;
+  std::vector<std::vector<Group>> groups;
+  for (int c0 = 0; c0 < ct.nkc; c0 += cb) {
+    std::map<int, std::vector<int>> by_size;
+    for (int k = c0; k < std::min(ct.nkc, c0 + cb); ++k)
+      by_size[(ct.kc_slot_begin[k + 1] - ct.kc_slot_begin[k]) * q2].push_back(k - c0);
+    std::vector<Group> g;
+    for (const auto& e : by_size) {
+      if (e.first > 0) g.push_back({e.first, (int)ids.size(), (int)e.second.size()});
+      ids.insert(ids.end(), e.second.begin(), e.second.end());
+    }
+    groups.push_back(std::move(g));
+  }
+  constexpr bool k64 = std::is_same<T, double2>::value;
+  const int n = h->n, hmax = max_int / 2, ldl = n + nb, ldw = 2 * max_int;
+  const long long rs = (long long)nb * h->ldR, hs = (long long)nb * h->ldH, ls = (long long)n * ldl;
+  const long long ms = (long long)hmax * hmax, kst = k64 ? (long long)max_int * max_int : (long long)max_int * ldw;
+  Workspace ws;
+  LeafWork<double2> lw;            // FP64: leaf inverses
+  double2* Ht = nullptr;
+  T *Wl = nullptr, *Ul = nullptr;  // complex float: augmented leaf systems
+  T *Rt = nullptr, *M = nullptr, *K = nullptr, *U = nullptr;
+  int *perm = nullptr, *d_ids = nullptr, *d_ord = nullptr, *d_pos = nullptr, *d_leaves = nullptr;
+  int4* d_slots = nullptr;
+  double2* d_lam = nullptr;
+  HPS_CUDA_TRY(ws.get(Rt, (size_t)rs * max_lam));
+  HPS_CUDA_TRY(ws.get(K, (size_t)kst * cb));
+  if constexpr (k64) {
+    HPS_CUDA_TRY(lw.get(ws, h, max_lam, st));
+    HPS_CUDA_TRY(ws.get(Ht, (size_t)hs * max_lam));
+    HPS_CUDA_TRY(ws.get(M, (size_t)ms * cb));
+    HPS_CUDA_TRY(ws.get(U, gj_scratch_elems<double2>(hmax) * cb));
+    HPS_CUDA_TRY(ws.get(perm, (size_t)hmax * cb));
+  } else {
+    HPS_CUDA_TRY(ws.get(lw.status, 1));
+    HPS_CUDA_TRY(cudaMemsetAsync(lw.status, 0, sizeof(int), st));
+    HPS_CUDA_TRY(ws.get(Wl, (size_t)ls * max_lam));
+    HPS_CUDA_TRY(ws.get(Ul, gj_augmented_scratch_elems(ldl) * max_lam));
+    HPS_CUDA_TRY(ws.get(U, gj_augmented_scratch_elems(ldw) * cb));
+  }
+  auto put = [&](auto*& d, const auto& v) -> cudaError_t {
+    cudaError_t e = ws.get(d, v.size());
+    if (e == cudaSuccess && !v.empty())
+      e = cudaMemcpyAsync(d, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice, st);
+    return e;
+  };
+  HPS_CUDA_TRY(put(d_ids, ids));
+  HPS_CUDA_TRY(put(d_ord, ord));
+  HPS_CUDA_TRY(put(d_pos, map_pos));
+  HPS_CUDA_TRY(put(d_leaves, rep_leaves));
+  HPS_CUDA_TRY(put(d_slots, slots));
+  HPS_CUDA_TRY(put(d_lam, lams));
+  int rc = HPS_OK, batch = 0;
+  for (int c0 = 0; c0 < ct.nkc && rc == HPS_OK; c0 += cb, ++batch) {
     const int nc = std::min(cb, ct.nkc - c0);
-    const int lb = rep_leaf_begin[c0], le = rep_leaf_begin[c0 + nc];
-    const int nlb = le - lb;
-    const int* leaf_ids = d_rep_leaves + lb;
+    const int lb = rep_leaf_begin[c0], nlb = rep_leaf_begin[c0 + nc] - lb;
+    const int nlam = lam_begin[batch + 1] - lam_begin[batch];
     auto body = [&]() -> int {
-      HPS_CUDA_TRY(cudaMemsetAsync(Wl, 0, (size_t)wl_stride * nlb * sizeof(T), st));
-      dim3 ga((n + 127) / 128, nlb);
-      assemble_kernel<T><<<ga, 128, 0, st>>>(Wl, wl_stride, ld_l, leaf_ids, 0, nlb, h->tables, h->tl, h->eta,
-                                             nullptr, h->lambda_q, 1);
-      HPS_CUDA_TRY(cudaGetLastError());
-      HPS_CUDA_TRY(run_gj(Wl, wl_stride, ld_l, n, ncols_l, ni, nlb, d_status, st));
-      dim3 ge(256, nlb);
-      extract_kernel<T><<<ge, 256, 0, st>>>(Wl, wl_stride, ld_l, n, ni, nb, h->eta, nlb, Rt, (long long)nb * h->ldR,
-                                            h->ldR, nullptr, 0, 0);
-      HPS_CUDA_TRY(cudaGetLastError());
-      HPS_CUDA_TRY(run_seg_kron(Rt, (long long)nb * h->ldR, h->ldR, nb, nb, nlb, h->tables, h->tl, 1, 0, h->nsm, st));
-      HPS_CUDA_TRY(run_seg_kron(Rt, (long long)nb * h->ldR, h->ldR, nb, nb, nlb, h->tables, h->tl, 0, 1, h->nsm, st));
-      extract_b_kernel<T><<<dim3(64, nlb), 256, 0, st>>>(Rt, (long long)nb * h->ldR, h->ldR, leaf_ids, nlb, q,
-                                                         h->dct.int_mask, h->dct.b_off, h->B64, h->B32);
-      HPS_CUDA_TRY(cudaGetLastError());
-      assemble_cluster_kernel<T><<<dim3(256, nc), 256, 0, st>>>(Wc, wc_stride, ldw, c0, nc, h->dct.kc_slot_begin,
-                                                                d_rep_slot_lf, d_rep_leaf_begin, d_rep_leaves, Rt,
-                                                                (long long)nb * h->ldR, h->ldR, lb, gd, q);
-      HPS_CUDA_TRY(cudaGetLastError());
-      // blocks of one size are eliminated in one launch
-      int cstart = c0;
-      while (cstart < c0 + nc) {
-        const int sz = (ct.kc_slot_begin[cstart + 1] - ct.kc_slot_begin[cstart]) * q2;
-        int cend = cstart + 1;
-        while (cend < c0 + nc && (ct.kc_slot_begin[cend + 1] - ct.kc_slot_begin[cend]) * q2 == sz) ++cend;
-        if (sz > 0)
-          HPS_CUDA_TRY(run_gj(Wc + (long long)(cstart - c0) * wc_stride, wc_stride, ldw, sz, 2 * sz, 0, cend - cstart,
-                              d_status, st));
-        cstart = cend;
-      }
-      if (h->Kc64 || h->Kc32) {
-        extract_kc_kernel<T><<<dim3(256, nc), 256, 0, st>>>(Wc, wc_stride, ldw, c0, nc, h->dct.kc_slot_begin,
-                                                            h->dct.kc_off, q, h->Kc64, h->Kc32);
+      const double2* lam = d_lam + lam_begin[batch];
+      if constexpr (k64) {
+        if (const int r = chebyshev_maps(h, lw, nlam, 0, nullptr, lam, Rt, Ht, st)) return r;
+      } else {
+        HPS_CUDA_TRY(cudaMemsetAsync(Wl, 0, (size_t)ls * nlam * sizeof(T), st));
+        leaf32_assemble_kernel<<<dim3((n + 127) / 128, nlam), 128, 0, st>>>(Wl, ls, ldl, h->tables, h->tl, h->eta, lam);
+        HPS_CUDA_TRY(cudaGetLastError());
+        HPS_CUDA_TRY(batched_gj_augmented(Wl, ls, ldl, n, ldl, h->ni, nlam, Ul,
+                                          (long long)gj_augmented_scratch_elems(ldl), lw.status, st));
+        leaf32_extract_kernel<<<dim3(64, nlam), 256, 0, st>>>(Wl, ls, ldl, n, nb, h->eta, Rt, rs, h->ldR);
         HPS_CUDA_TRY(cudaGetLastError());
       }
-      if constexpr (std::is_same<T, float2>::value) {
+      HPS_CUDA_TRY(run_seg_kron(Rt, rs, h->ldR, nb, nb, nlam, h->tables, h->tl, 1, 0, h->nsm, st));
+      HPS_CUDA_TRY(run_seg_kron(Rt, rs, h->ldR, nb, nb, nlam, h->tables, h->tl, 0, 1, h->nsm, st));
+      extract_b_kernel<T><<<dim3(64, nlb), 256, 0, st>>>(Rt, rs, h->ldR, d_leaves + lb, d_pos + lb, nlb, q,
+                                                         h->dct.int_mask, h->dct.b_off, h->B64, h->B32);
+      HPS_CUDA_TRY(cudaGetLastError());
+      if (hmax == 0) return HPS_OK;
+      KcBlocks<T> A;
+      A.slots = d_slots;
+      A.ord = d_ord;
+      A.slot_begin = h->dct.kc_slot_begin;
+      A.c0 = c0;
+      A.q2 = q2;
+      A.parts = (q2 + 63) / 64;
+      A.Rt = Rt;
+      A.rstride = rs;
+      A.ldr = h->ldR;
+      A.M = M;
+      A.mstride = ms;
+      A.K = K;
+      A.kstride = kst;
+      if constexpr (k64) {
+        const int hsl = hmax / q2, pp = A.parts * A.parts;
+        kc_product_kernel<T, 0><<<dim3(hsl * hsl * pp, nc), 256, 0, st>>>(A);
+        HPS_CUDA_TRY(cudaGetLastError());
+        for (const Group& g : groups[batch])
+          HPS_CUDA_TRY(batched_gj<T>(M, ms, g.n / 2, g.n / 2, g.n / 2, g.count, U, (long long)gj_scratch_elems<T>(hmax),
+                                     perm, hmax, lw.status, st, d_ids + g.first));
+        kc_red_kernel<T><<<dim3(128, nc), 256, 0, st>>>(A, perm, hmax);
+        HPS_CUDA_TRY(cudaGetLastError());
+        kc_product_kernel<T, 1><<<dim3(hsl * hsl * pp, nc), 256, 0, st>>>(A);
+        HPS_CUDA_TRY(cudaGetLastError());
+        kc_product_kernel<T, 2><<<dim3(2 * hsl * hsl * pp, nc), 256, 0, st>>>(A);
+        HPS_CUDA_TRY(cudaGetLastError());
+      } else {
+        cluster32_assemble_kernel<<<dim3(256, nc), 256, 0, st>>>(K, kst, ldw, A);
+        HPS_CUDA_TRY(cudaGetLastError());
+        for (const Group& g : groups[batch])
+          HPS_CUDA_TRY(batched_gj_augmented(K, kst, ldw, g.n, 2 * g.n, 0, g.count, U,
+                                            (long long)gj_augmented_scratch_elems(ldw), lw.status, st, d_ids + g.first));
+      }
+      if (h->Kc64 || h->Kc32) {
+        extract_kc_kernel<T><<<dim3(256, nc), 256, 0, st>>>(K, kst, !k64, ldw, c0, h->dct.kc_slot_begin, h->dct.kc_off, q,
+                                                            h->Kc64, h->Kc32);
+        HPS_CUDA_TRY(cudaGetLastError());
+      }
+      if constexpr (!k64) {
         if (!h->Kc32 && h->Kc16) {
-          quantize_kc_ws_kernel<<<dim3(64, nc), 256, 0, st>>>(Wc, wc_stride, ldw, c0, nc, h->dct.kc_slot_begin,
-                                                              h->dct.kc_off, q2, h->Kc16, h->Kc16s);
+          quantize_kc_ws_kernel<<<dim3(64, nc), 256, 0, st>>>(K, kst, ldw, c0, h->dct.kc_slot_begin, h->dct.kc_off, q2,
+                                                              h->Kc16, h->Kc16s);
           HPS_CUDA_TRY(cudaGetLastError());
         }
       }
@@ -1286,12 +1590,8 @@ int build_precond_blocks(hps_handle* h, const int* d_rep_leaf_begin, const int* 
     };
     rc = body();
   }
-  if (rc == HPS_OK) rc = check_status(d_status, st, "preconditioner blocks");
+  if (rc == HPS_OK) rc = check_status(lw.status, st, "preconditioner blocks");
   cudaStreamSynchronize(st);
-  cudaFree(Wl);
-  cudaFree(Rt);
-  cudaFree(Wc);
-  cudaFree(d_status);
   return rc;
 }
 
@@ -1344,6 +1644,7 @@ int classify_preconditioner(hps_handle* h, const double2* cdiag, cudaStream_t st
   std::vector<double2> lamq;
   if ((rc = compute_lambdas(h, cdiag, st, lamq))) return rc;
   assign_blocks(h, &lamq);
+  h->lambda_q_host = lamq;
   if ((rc = upload(h, h->dct.slot_lf, ct.slot_lf, st))) return rc;
   if ((rc = upload(h, h->dct.slot_cluster, ct.slot_cluster, st))) return rc;
   if ((rc = upload(h, h->dct.cl_slot_begin, ct.cl_slot_begin, st))) return rc;
@@ -1377,30 +1678,14 @@ int build_preconditioner(hps_handle* h, const double2* cdiag, cudaStream_t st) {
   (void)cdiag;
   const ClusterTables& ct = h->ct;
   // the representative cluster of every distinct K block, as clusters 0..nkc-1
-  std::vector<int> rep_leaf_begin(1, 0), rep_leaves, rep_slot_lf;
+  std::vector<int> rep_leaf_begin(1, 0), rep_leaves;
   for (int k = 0; k < ct.nkc; ++k) {
     const int c = ct.kc_rep[k];
     for (int l = ct.cl_leaf_begin[c]; l < ct.cl_leaf_begin[c + 1]; ++l) rep_leaves.push_back(ct.cl_leaves[l]);
     rep_leaf_begin.push_back((int)rep_leaves.size());
-    for (int sl = ct.cl_slot_begin[c]; sl < ct.cl_slot_begin[c + 1]; ++sl) rep_slot_lf.push_back(ct.slot_lf[sl]);
   }
-  int *d_leaf_begin = nullptr, *d_leaves = nullptr, *d_slot_lf = nullptr;
-  auto dev = [&](int*& d, const std::vector<int>& v) -> int {
-    HPS_CUDA_TRY(cudaMalloc(&d, std::max<size_t>(1, v.size()) * sizeof(int)));
-    if (!v.empty()) HPS_CUDA_TRY(cudaMemcpyAsync(d, v.data(), v.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-    return HPS_OK;
-  };
-  int rc = dev(d_leaf_begin, rep_leaf_begin);
-  if (!rc) rc = dev(d_leaves, rep_leaves);
-  if (!rc) rc = dev(d_slot_lf, rep_slot_lf);
-  if (!rc)
-    rc = h->Kc64 ? build_precond_blocks<double2>(h, d_leaf_begin, d_leaves, d_slot_lf, rep_leaf_begin, st)
-                 : build_precond_blocks<float2>(h, d_leaf_begin, d_leaves, d_slot_lf, rep_leaf_begin, st);
-  cudaStreamSynchronize(st);
-  if (d_leaf_begin) cudaFree(d_leaf_begin);
-  if (d_leaves) cudaFree(d_leaves);
-  if (d_slot_lf) cudaFree(d_slot_lf);
-  return rc;
+  return h->Kc64 ? build_precond_blocks<double2>(h, rep_leaf_begin, rep_leaves, st)
+                 : build_precond_blocks<float2>(h, rep_leaf_begin, rep_leaves, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -1412,15 +1697,14 @@ int build_preconditioner(hps_handle* h, const double2* cdiag, cudaStream_t st) {
 // ---------------------------------------------------------------------------
 namespace {
 
-__global__ void extract_sinv_kernel(const double2* W, long long wstride, int ld, int n, int ni, int nb, int nbatch,
-                                    const int* cls, double2* S64, float2* S32) {
+// S~^{-1} = (A~^{-1})_bb of a batch into the handle's copies.
+__global__ void extract_sinv_kernel(const double2* X, long long xstride, int ldx, int nb, int first, double2* S64,
+                                    float2* S32) {
   const int b = blockIdx.y;
-  if (b >= nbatch) return;
-  const long long off = (long long)cls[b] * nb * nb;
+  const long long off = (long long)(first + b) * nb * nb;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < (long long)nb * nb;
        t += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(t / nb), c = (int)(t % nb);
-    const double2 v = W[(long long)b * wstride + (long long)(ni + r) * ld + n + c];
+    const double2 v = X[b * xstride + (t / nb) * ldx + t % nb];
     if (S64) S64[off + t] = v;
     if (S32) S32[off + t] = make_float2((float)v.x, (float)v.y);
   }
@@ -1579,7 +1863,7 @@ bool axis_eig(int n, const double* M, double* V, double* Vinv, double* E) {
 
 int build_full_system(hps_handle* h, const double2* cdiag, cudaStream_t st) {
   FullSystem& fs = h->fs;
-  const int n = h->n, ni = h->ni, nb = h->nb, n1 = h->n1, p = h->p;
+  const int nb = h->nb, n1 = h->n1, p = h->p;
   int rc = HPS_OK;
   std::vector<double2> lamq;
   if ((rc = compute_lambdas(h, cdiag, st, lamq))) return rc;
@@ -1611,45 +1895,35 @@ int build_full_system(hps_handle* h, const double2* cdiag, cudaStream_t st) {
   if (want32 && (rc = dal((void**)&fs.Sinv32, per * fs.ncls * sizeof(float2)))) return rc;
   if ((rc = dal((void**)&fs.d_cls, (size_t)h->nl * sizeof(int)))) return rc;
   HPS_CUDA_TRY(cudaMemcpyAsync(fs.d_cls, fs.cls.data(), (size_t)h->nl * sizeof(int), cudaMemcpyHostToDevice, st));
-  // S~^{-1} of every distinct constant from the elimination of its homogenized leaf matrix
+  // S~^{-1} of every distinct constant from its homogenized leaf map
   {
-    const int ncols = n + nb, ld = ncols;
-    const long long wstride = (long long)n * ld;
-    const size_t perw = (size_t)wstride * sizeof(double2);
-    int nbatch = (int)std::min<size_t>((size_t)fs.ncls, std::max<size_t>(1, workspace_budget(h) / perw));
+    const size_t perl = ((size_t)h->ni * h->ni + gj_scratch_elems<double2>(h->ni) + (size_t)nb * (h->ldR + h->ldH)) *
+                            sizeof(double2) + (size_t)h->ni * sizeof(int);
+    int nbatch = (int)std::min<size_t>((size_t)fs.ncls, std::max<size_t>(1, workspace_budget(h) / perl));
     nbatch = std::min(nbatch, 4 * h->nsm);
-    double2* W = nullptr;
-    int *d_status = nullptr, *d_leaves = nullptr, *d_seq = nullptr;
-    HPS_CUDA_TRY(cudaMalloc(&W, perw * nbatch));
-    HPS_CUDA_TRY(cudaMalloc(&d_status, sizeof(int)));
-    HPS_CUDA_TRY(cudaMalloc(&d_leaves, (size_t)fs.ncls * sizeof(int)));
-    HPS_CUDA_TRY(cudaMalloc(&d_seq, (size_t)fs.ncls * sizeof(int)));
-    std::vector<int> seq(fs.ncls);
-    for (int k = 0; k < fs.ncls; ++k) seq[k] = k;
-    HPS_CUDA_TRY(cudaMemsetAsync(d_status, 0, sizeof(int), st));
-    HPS_CUDA_TRY(cudaMemcpyAsync(d_leaves, rep.data(), (size_t)fs.ncls * sizeof(int), cudaMemcpyHostToDevice, st));
-    HPS_CUDA_TRY(cudaMemcpyAsync(d_seq, seq.data(), (size_t)fs.ncls * sizeof(int), cudaMemcpyHostToDevice, st));
+    Workspace ws;
+    LeafWork<double2> lw;
+    double2 *Rt = nullptr, *Ht = nullptr, *d_lam = nullptr;
+    const long long rs = (long long)nb * h->ldR, hs = (long long)nb * h->ldH;
+    HPS_CUDA_TRY(lw.get(ws, h, nbatch, st));
+    HPS_CUDA_TRY(ws.get(Rt, (size_t)rs * nbatch));
+    HPS_CUDA_TRY(ws.get(Ht, (size_t)hs * nbatch));
+    HPS_CUDA_TRY(ws.get(d_lam, (size_t)fs.ncls));
+    std::vector<double2> lams(fs.ncls);
+    for (int k = 0; k < fs.ncls; ++k) lams[k] = lamq[rep[k]];
+    HPS_CUDA_TRY(cudaMemcpyAsync(d_lam, lams.data(), (size_t)fs.ncls * sizeof(double2), cudaMemcpyHostToDevice, st));
     for (int k0 = 0; k0 < fs.ncls && rc == HPS_OK; k0 += nbatch) {
       const int nbt = std::min(nbatch, fs.ncls - k0);
       auto body = [&]() -> int {
-        HPS_CUDA_TRY(cudaMemsetAsync(W, 0, perw * nbt, st));
-        assemble_kernel<double2><<<dim3((n + 127) / 128, nbt), 128, 0, st>>>(
-            W, wstride, ld, d_leaves + k0, 0, nbt, h->tables, h->tl, h->eta, nullptr, h->lambda_q, 1);
-        HPS_CUDA_TRY(cudaGetLastError());
-        HPS_CUDA_TRY(run_gj(W, wstride, ld, n, ncols, ni, nbt, d_status, st));
-        extract_sinv_kernel<<<dim3(64, nbt), 256, 0, st>>>(W, wstride, ld, n, ni, nb, nbt, d_seq + k0, fs.Sinv64,
-                                                          fs.Sinv32);
+        if (const int r = chebyshev_maps<double2>(h, lw, nbt, 0, nullptr, d_lam + k0, Rt, Ht, st, true)) return r;
+        extract_sinv_kernel<<<dim3(64, nbt), 256, 0, st>>>(Rt, rs, h->ldR, nb, k0, fs.Sinv64, fs.Sinv32);
         HPS_CUDA_TRY(cudaGetLastError());
         return HPS_OK;
       };
       rc = body();
     }
-    if (rc == HPS_OK) rc = check_status(d_status, st, "homogenized leaf systems");
+    if (rc == HPS_OK) rc = check_status(lw.status, st, "homogenized leaf systems");
     cudaStreamSynchronize(st);
-    cudaFree(W);
-    cudaFree(d_status);
-    cudaFree(d_leaves);
-    cudaFree(d_seq);
     if (rc) return rc;
   }
   // Algorithm 3 tables: L1 = (D~^2)[1..p-2][1..p-2] = V E V^{-1} per axis
