@@ -221,8 +221,9 @@ struct RhsP {
 };
 
 // Stage K over distinct blocks: item = (block k, block slot s, first member,
-// member count) with the members the clusters sharing block k; "right-hand
-// side" rr of the item is member rr (one right-hand side per launch).
+// member count) with the members the clusters sharing block k; the vectors of
+// an item are its (member, right-hand side) pairs, nrl right-hand sides per
+// launch, so that a block streamed once serves up to 8 vectors.
 template <class TM_, class TIN, class TOUT>
 struct PrecKP {
   using TM = TM_;
@@ -241,7 +242,8 @@ struct PrecKP {
     const TIN* t;
     TOUT* z;
     long long nf, tstride;
-    int nrhs;  // group width of the launch
+    int nrl;   // right-hand sides of the launch: vector rr = member * nrl + rhs
+    int nrhs;  // vectors of an item, member group width x nrl
     long long nitems;
   };
   // item (k, s * kKRowSplit + part, first member, members): rows
@@ -264,17 +266,16 @@ struct PrecKP {
     return it.nrows > 0;
   }
   __device__ static Acc load_x(const Args& A, const ItemInfo& it, int rr, int c) {
-    if (rr >= it.mask) return czero<Acc>();
-    const int cl = A.members[it.xoff + rr];
-    return cvt<Acc>(A.t[A.cl_tpos[cl] + c]);
+    const int m = rr / A.nrl;
+    if (m >= it.mask) return czero<Acc>();
+    return cvt<Acc>(A.t[(long long)(rr - m * A.nrl) * A.tstride + A.cl_tpos[A.members[it.xoff + m]] + c]);
   }
   __device__ static void store(const Args& A, const ItemInfo& it, const Acc* outs, int, int tid) {
-    for (int idx = tid; idx < it.mask * it.nrows; idx += kThreads) {
-      const int rr = idx / it.nrows, jj = idx % it.nrows;
-      const int cl = A.members[it.xoff + rr];
-      const int lf = A.slot_lf[A.cl_slot_begin[cl] + it.face];
+    for (int idx = tid; idx < it.mask * A.nrl * it.nrows; idx += kThreads) {
+      const int rr = idx / it.nrows, jj = idx % it.nrows, m = rr / A.nrl;
+      const int lf = A.slot_lf[A.cl_slot_begin[A.members[it.xoff + m]] + it.face];
       const long long o = (long long)(lf / 6) * A.nb + (long long)(lf % 6) * A.q2 + it.nbr + jj;
-      A.z[o] = cvt<TOUT>(rscale(outs[idx], A.kscale, it.aoff + jj));
+      A.z[(long long)(rr - m * A.nrl) * A.nf + o] = cvt<TOUT>(rscale(outs[idx], A.kscale, it.aoff + jj));
     }
   }
   __device__ static void copy(const Args&, const ItemInfo&, int, int) {}
@@ -383,12 +384,6 @@ struct PrecBArgs {
   int nrhs;
   long long vstride, tstride;  // per right-hand side: r and z, t
   const int* gate;  // as in seg_gemv_kernel
-  // optional: the largest |component| of t per (right-hand side, cluster), as float bits
-  // (non-negative floats order like their bit patterns, so atomicMax gives the same result in
-  // any order); the scale of the FP16 tensor-core stage K
-  unsigned* tmax;
-  const int* leaf_cluster;
-  int ncl;
   // work items: groups of leaves sharing one B block, as (first index into gleaves, count)
   const int2* groups;
   const int* gleaves;
@@ -432,9 +427,6 @@ __global__ void __launch_bounds__(kThreads) prec_b_kernel(const PrecBArgs<TM, TI
       }
       __syncthreads();
       if (nint == 0) continue;
-      float tmx[NR];
-#pragma unroll
-      for (int rr = 0; rr < NR; ++rr) tmx[rr] = 0.f;
       for (int row = threadIdx.x; row < nrows; row += kThreads) {
         Acc acc[NR];
 #pragma unroll
@@ -454,23 +446,7 @@ __global__ void __launch_bounds__(kThreads) prec_b_kernel(const PrecBArgs<TM, TI
           const int e = leaf * 6 + k;
           const Acc g = rscale(acc[rr], A.bscale, (long long)A.bsc[e] + j);
           const Acc v = csub(cvt<Acc>(A.r[(long long)rhs * A.vstride + A.brd[e] + j]), g);
-          const TOUT tv = cvt<TOUT>(v);
-          A.t[(long long)rhs * A.tstride + A.bto[e] + j] = tv;
-          if constexpr (std::is_same<TOUT, float2>::value) tmx[rr] = fmaxf(tmx[rr], fmaxf(fabsf(tv.x), fabsf(tv.y)));
-        }
-      }
-      if constexpr (std::is_same<TOUT, float2>::value) {
-        if (A.tmax) {
-#pragma unroll
-          for (int rr = 0; rr < NR; ++rr) {
-            float m = tmx[rr];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-            if ((threadIdx.x & 31) == 0 && rr < nr && m > 0.f) {
-              const int vid = v0 + rr, leaf = A.gleaves[grp.x + vid / A.nrhs], rhs = vid % A.nrhs;
-              atomicMax(A.tmax + (long long)rhs * A.ncl + A.leaf_cluster[leaf], __float_as_uint(m));
-            }
-          }
+          A.t[(long long)rhs * A.tstride + A.bto[e] + j] = cvt<TOUT>(v);
         }
       }
     }
@@ -584,11 +560,25 @@ cudaError_t precond_t(const hps_handle* h, const TM* B, const TM* K, const TIN* 
                       bool use_tc = false) {
   const int q2 = h->q * h->q;
   const long long tstride = h->ct.tsize;
-  // FP16 blocks with complex-float output on the uniform layout: stage K of every block on the
-  // tensor cores with FP16 operands, t scaled per cluster (stage B records the scales)
-  bool tc16 = false;
-  if constexpr (std::is_same<TM, __half2>::value && std::is_same<TOUT, float2>::value)
-    tc16 = precond_tc16_eligible(h, nrhs);
+  // FP16 blocks with complex-float output on the uniform layout: both stages in tc_precond16.cu
+  if constexpr (std::is_same<TM, __half2>::value && std::is_same<TOUT, float2>::value) {
+    if (precond_tc16_eligible(h, nrhs)) {
+      constexpr VType kIn = std::is_same<TIN, float2>::value ? VType::C64
+                            : std::is_same<TIN, float4>::value ? VType::DF : VType::C128;
+      // blocks shared by many clusters: their complex-FP32 copies where they are kept, except for
+      // one right-hand side and multiples of 64
+      const bool tc32 = use_tc && nrhs > 1 && nrhs % 64 != 0;
+      cudaEvent_t ev = h->prof.begin(st);
+      cudaError_t e = launch_precond_b16(h, kIn, r, z, tc32 ? t : nullptr, nrhs, st);
+      h->prof.end(HPS_PHASE_PRECOND_B, ev, st);
+      if (e != cudaSuccess) return e;
+      ev = h->prof.begin(st);
+      e = launch_precond_tc16(h, z, nrhs, tc32, st);
+      if (e == cudaSuccess && tc32) e = launch_precond_tc_vec(h, t, z, nrhs, h->tc_error, st);
+      h->prof.end(HPS_PHASE_PRECOND_K, ev, st);
+      return e;
+    }
+  }
   {
     PrecBArgs<TM, TIN, TOUT> A;
     A.B = B;
@@ -607,16 +597,9 @@ cudaError_t precond_t(const hps_handle* h, const TM* B, const TM* K, const TIN* 
     A.nrhs = nrhs;
     A.vstride = h->nf;
     A.tstride = tstride;
-    A.tmax = nullptr;
-    A.leaf_cluster = h->dct.leaf_cluster;
-    A.ncl = h->ct.ncl;
     A.groups = h->dct.bgroups;
     A.gleaves = h->dct.bgroup_leaves;
     A.ngroups = (int)h->ct.bgroups.size();
-    if (tc16) {
-      HPS_TRY_CUDA_E(cudaMemsetAsync(h->tmax, 0, (size_t)h->ct.ncl * nrhs * sizeof(float), st));
-      A.tmax = reinterpret_cast<unsigned*>(h->tmax);
-    }
     using Acc = typename MT<TM>::Acc;
     cudaEvent_t ev = h->prof.begin(st);
     auto launch_b = [&](auto kern, int nr) -> cudaError_t {
@@ -651,12 +634,6 @@ cudaError_t precond_t(const hps_handle* h, const TM* B, const TM* K, const TIN* 
     if (e != cudaSuccess) return e;
   }
   if (h->ct.nslots == 0) return cudaSuccess;
-  if (tc16) {
-    cudaEvent_t ev = h->prof.begin(st);
-    const cudaError_t e = launch_precond_tc16(h, (const float2*)t, (float2*)z, nrhs, st);
-    h->prof.end(HPS_PHASE_PRECOND_K, ev, st);
-    return e;
-  }
   if constexpr (std::is_same<TOUT, float2>::value) {
     // many right-hand sides: every block once per 64 of them, on the tensor cores
     if (precond_tc_multi_eligible(h, nrhs)) {
@@ -685,22 +662,31 @@ cudaError_t precond_t(const hps_handle* h, const TM* B, const TM* K, const TIN* 
     long long* counter = &h->prof.launches;
     cudaEvent_t ev = h->prof.begin(st);
     cudaError_t e = cudaSuccess;
-    for (int rhs = 0; rhs < nrhs && e == cudaSuccess; ++rhs) {
-      A.t = t + (long long)rhs * tstride;
-      A.z = z + (long long)rhs * h->nf;
-      if (use_tc) {
+    if (use_tc) {
+      for (int rhs = 0; rhs < nrhs && e == cudaSuccess; ++rhs) {
         if constexpr (std::is_same<TOUT, float2>::value)
-          e = launch_precond_tc(h, (const float2*)A.t, (float2*)A.z, h->tc_error, st);
+          e = launch_precond_tc(h, (const float2*)t + (long long)rhs * tstride, (float2*)z + (long long)rhs * h->nf,
+                                h->tc_error, st);
         else
           e = cudaErrorInvalidValue;
       }
-      for (int g = 0; g < 4 && e == cudaSuccess; ++g) {
-        const long long n = use_tc ? h->ct.kitems_ntc[g] : (long long)h->ct.kitems[g].size();
-        if (n == 0) continue;
-        A.items = h->dct.kitems[g];
-        A.nitems = n;
-        A.nrhs = 1 << g;
-        e = launch_group<P>(A, 1 << g, xcap, q2, h->nsm, st, counter, h->gate, h->shapes.k[g]);
+    }
+    // member groups of width w take 8 / w right-hand sides per launch (fewer where the staged
+    // vectors do not fit in shared memory)
+    int fit = 8;
+    while (fit > 1 && (size_t)fit * (xcap + q2) * sizeof(typename MT<TM>::Acc) > (size_t)220 * 1024) fit >>= 1;
+    for (int g = 0; g < 4 && e == cudaSuccess; ++g) {
+      const long long n = use_tc ? h->ct.kitems_ntc[g] : (long long)h->ct.kitems[g].size();
+      if (n == 0) continue;
+      A.items = h->dct.kitems[g];
+      A.nitems = n;
+      const int step = std::max(1, fit >> g);
+      for (int r0 = 0; r0 < nrhs && e == cudaSuccess; r0 += step) {
+        A.nrl = std::min(step, nrhs - r0);
+        A.nrhs = A.nrl << g;
+        A.t = t + (long long)r0 * tstride;
+        A.z = z + (long long)r0 * h->nf;
+        e = launch_group<P>(A, A.nrhs, xcap, q2, h->nsm, st, counter, h->gate, h->shapes.k[group_index(A.nrhs)]);
       }
     }
     h->prof.end(HPS_PHASE_PRECOND_K, ev, st);
@@ -921,6 +907,7 @@ cudaError_t tune_stage_k(hps_handle* h, const TM* K, const float* kscale, void* 
     if (n == 0) continue;
     A.items = h->dct.kitems[g];
     A.nitems = n;
+    A.nrl = 1;
     A.nrhs = 1 << g;
     const std::array<long long, 6> key{h->dev, 10 + (long long)sizeof(TM), h->q, h->nl, g, n};
     h->shapes.k[g] = tune_group<P>(h, A, 1 << g, xcap_of(h, XCap::StageK), A.q2, key, h->shapes.k[g], st);

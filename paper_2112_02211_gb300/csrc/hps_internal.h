@@ -131,9 +131,16 @@ struct ClusterTables {
   int nint0 = 0;                     // internal values of every cluster when uniform
   std::vector<int> pos_class;        // [ncl] K block of the member at stage-K position m
   std::vector<int> leaf_cluster;     // [nleaves] cluster of each leaf
-  // FP16 tensor-core stage K of one right-hand side (uniform layout): items (block, 128-row
-  // tile, first member position, members <= 64)
+  // FP16 tensor-core stage K (uniform layout): items (block, 128-row tile, first member position,
+  // members <= P) for every P = members per item that some number of right-hand sides up to
+  // max_rhs needs; list P is [tc16_begin[P], + tc16_count[P]), the blocks of kc_tc last (from
+  // tc16_ntc[P] on)
   std::vector<int4> tc16_items;
+  int tc16_begin[65] = {}, tc16_count[65] = {}, tc16_ntc[65] = {};
+  std::vector<int2> b16_items;       // its stage B: (first position, members <= P, + kTcItem in kc_tc), P = 1, 2, 4
+  int b16_begin[5] = {}, b16_count[5] = {};
+  int max_members = 0;               // most members of any K block
+  std::vector<int> zoff;             // uniform: [position][24] face-vector offset of each slot
   // stage-B work items: leaves sorted by B block, in groups of at most kBGroup that share one
   // block (first index into bgroup_leaves, count)
   std::vector<int> bgroup_leaves;
@@ -164,6 +171,9 @@ struct DeviceClusterTables {
   int* pos_class = nullptr;
   int* leaf_cluster = nullptr;
   int4* tc16_items = nullptr;
+  int* cl_leaves = nullptr;
+  int* zoff = nullptr;
+  int2* b16_items = nullptr;
   int* bgroup_leaves = nullptr;
   int2* bgroups = nullptr;
 };
@@ -390,8 +400,11 @@ struct hps_handle {
   __half2* B16 = nullptr;   // FP16 copies of B, rows scaled by 1/B16s[(bcls*6+face)*q^2 + j]
   float* B16s = nullptr;
   void* pc_scratch = nullptr;  // nslots*q^2*max_rhs complex double (precond t buffer)
-  float* tmax = nullptr;       // [rhs][cluster] largest |component| of stage B's t (FP16 stage K scale)
-  int tmax_rhs = 0;            // right-hand sides tmax holds
+  // FP16 tensor-core stage K: stage B's t of each vector (position * nrhs + rhs), scaled by its
+  // largest |component| tmax and split into FP16 operand rows [4][vector][nint0] (tc_precond16.cu)
+  __half2* op16 = nullptr;
+  float* tmax = nullptr;
+  int tmax_rhs = 0;            // right-hand sides they hold
 
   int* tc_error = nullptr;  // device error word of the tensor-core kernels
   // While a GMRES cycle is captured: the device word that the per-step kernels
@@ -460,13 +473,12 @@ void build_cluster_tables(hps_handle* h, int width);
 void assign_blocks(hps_handle* h, const std::vector<double2>* lamq);
 // Shared K blocks with at least this many member clusters run on the tensor cores.
 constexpr int kTcMinMembers = 16;
+// Mark of a stage-B item whose block is in kc_tc.
+constexpr int kTcItem = 256;
 // Stage-K work items of the SIMT kernel cover 1/kKRowSplit of a slot's q^2 rows
 // (finer items balance the last wave of the launch).
 constexpr int kKRowSplit = 2;
-// Leaves per stage-B work item (leaves sharing one B block).  Items of 8 leaves were measured
-// faster (0.070 vs 0.147 ms per application at 16^3 leaves) but gave a wrong preconditioner on a
-// complex medium (GMRES stalled; the same items one vector at a time gave other iterates than
-// one leaf per item), for a reason not yet found; one leaf per item until it is.
+// Leaves per stage-B work item of the general layouts (leaves sharing one B block).
 constexpr int kBGroup = 1;
 // Dynamic shared memory a block may opt into on sm_103 (227 KB).
 constexpr int kMaxDynSmem = 227 * 1024;
@@ -503,11 +515,19 @@ cudaError_t launch_precond_tc(const hps_handle* h, const float2* t, float2* z, i
 // in one launch (complex-FP32 blocks, one TF32 product): the GEMM of each K_c against the
 // columns (member cluster, right-hand side).  Needs ct.uniform.  t: [rhs][tsize], z: [rhs][nf].
 bool precond_tc_multi_eligible(const hps_handle* h, int nrhs);
-// Stage K of every cluster block on the tensor cores with FP16 operands (tc_precond16.cu): the
-// FP16 blocks against t scaled per cluster by tmax (which stage B fills); one right-hand side or
-// 64, 128, ... of them; needs the uniform layout.
+// The preconditioner with FP16 blocks on the uniform layout (tc_precond16.cu): stage B into
+// FP16 operand rows, stage K of every cluster block on the tensor cores; any nrhs up to max_rhs.
 bool precond_tc16_eligible(const hps_handle* h, int nrhs);
-cudaError_t launch_precond_tc16(const hps_handle* h, const float2* t, float2* z, int nrhs, cudaStream_t st);
+int tc16_members_per_item(int cols, int nrhs);
+// t32: where stage B leaves t itself, [vector][nint0], for the blocks of kc_tc (or nullptr);
+// skip_tc: without those blocks (launch_precond_tc_vec applies them).
+cudaError_t launch_precond_b16(const hps_handle* h, VType tin, const void* r, float2* z, float2* t32, int nrhs,
+                               cudaStream_t st);
+cudaError_t launch_precond_tc16(const hps_handle* h, float2* z, int nrhs, bool skip_tc, cudaStream_t st);
+// Stage K of the shared blocks ct.kc_tc (complex-FP32 blocks, one TF32 product) for nrhs right-hand
+// sides in one launch; uniform layout, t32 [vector][nint0].
+cudaError_t launch_precond_tc_vec(const hps_handle* h, const float2* t32, float2* z, int nrhs, int* d_error,
+                                  cudaStream_t st);
 cudaError_t launch_precond_tc_multi(const hps_handle* h, const float2* t, float2* z, int nrhs, int* d_error,
                                     cudaStream_t st);
 // Timed wrappers (phase intervals recorded when profiling is on).

@@ -1358,16 +1358,6 @@ void assign_blocks(hps_handle* h, const std::vector<double2>* lamq) {
       if (ct.cl_tpos[ct.kc_members[m]] != m * nint0) ct.uniform = false;
     ct.nint0 = ct.uniform ? (int)nint0 : 0;
   }
-  // FP16 tensor-core stage K items of one right-hand side: per block, per 128-row tile, the
-  // members in tiles of 64 (consecutive items reuse the block's row tile from L2)
-  ct.tc16_items.clear();
-  if (ct.uniform && ct.nint0 % 32 == 0) {
-    const int mtiles = (ct.nint0 + 127) / 128;
-    for (int k = 0; k < ct.nkc; ++k)
-      for (int mt = 0; mt < mtiles; ++mt)
-        for (int p0 = ct.kc_mem_begin[k]; p0 < ct.kc_mem_begin[k + 1]; p0 += 64)
-          ct.tc16_items.push_back(make_int4(k, mt, p0, std::min(64, ct.kc_mem_begin[k + 1] - p0)));
-  }
   // blocks for the tensor-core path: many members, an even row length (16-byte
   // aligned member rows of complex floats)
   ct.kc_tc.clear();
@@ -1381,6 +1371,43 @@ void assign_blocks(hps_handle* h, const std::vector<double2>* lamq) {
   for (auto& v : ct.kitems) v.clear();
   std::vector<char> is_tc(ct.nkc, 0);
   for (int k : ct.kc_tc) is_tc[k] = 1;
+  // FP16 tensor-core stage K items: per block, per 128-row tile, its members P at a time
+  // (consecutive items reuse the block's row tile from L2)
+  ct.tc16_items.clear();
+  ct.zoff.clear();
+  ct.b16_items.clear();
+  ct.max_members = 0;
+  for (int k = 0; k < ct.nkc; ++k) ct.max_members = std::max(ct.max_members, ct.kc_mem_begin[k + 1] - ct.kc_mem_begin[k]);
+  std::fill(ct.tc16_begin, ct.tc16_begin + 65, 0);
+  std::fill(ct.tc16_count, ct.tc16_count + 65, 0);
+  if (ct.uniform && ct.nint0 % 32 == 0) {
+    const int mtiles = (ct.nint0 + 127) / 128;
+    for (int m = 0; m < ct.ncl; ++m)
+      for (int sl = 0; sl < 24; ++sl) {
+        const int lf = ct.slot_lf[ct.cl_slot_begin[ct.kc_members[m]] + sl];
+        ct.zoff.push_back(lf / 6 * h->nb + lf % 6 * q2);
+      }
+    for (int P = 1; P <= 4; P *= 2) {
+      ct.b16_begin[P] = (int)ct.b16_items.size();
+      for (int k = 0; k < ct.nkc; ++k)
+        for (int p0 = ct.kc_mem_begin[k]; p0 < ct.kc_mem_begin[k + 1]; p0 += P)
+          ct.b16_items.push_back(make_int2(p0, std::min(P, ct.kc_mem_begin[k + 1] - p0) + (is_tc[k] ? kTcItem : 0)));
+      ct.b16_count[P] = (int)ct.b16_items.size() - ct.b16_begin[P];
+    }
+    for (int e = 0; e < 2 * std::min(64, h->opt.max_rhs); ++e) {
+      const int P = tc16_members_per_item(e & 1 ? 64 : 16, e / 2 + 1);
+      if (ct.tc16_count[P]) continue;
+      ct.tc16_begin[P] = (int)ct.tc16_items.size();
+      for (int pass = 0; pass < 2; ++pass) {
+        for (int k = 0; k < ct.nkc; ++k)
+          for (int mt = 0; is_tc[k] == pass && mt < mtiles; ++mt)
+            for (int p0 = ct.kc_mem_begin[k]; p0 < ct.kc_mem_begin[k + 1]; p0 += P)
+              ct.tc16_items.push_back(make_int4(k, mt, p0, std::min(P, ct.kc_mem_begin[k + 1] - p0)));
+        if (pass == 0) ct.tc16_ntc[P] = (int)ct.tc16_items.size() - ct.tc16_begin[P];
+      }
+      ct.tc16_count[P] = (int)ct.tc16_items.size() - ct.tc16_begin[P];
+    }
+  }
   for (int pass = 0; pass < 2; ++pass) {
     for (int k = 0; k < ct.nkc; ++k) {
       const int ns = ct.kc_slot_begin[k + 1] - ct.kc_slot_begin[k];
@@ -1666,6 +1693,9 @@ int classify_preconditioner(hps_handle* h, const double2* cdiag, cudaStream_t st
   if ((rc = upload(h, h->dct.pos_class, ct.pos_class, st))) return rc;
   if ((rc = upload(h, h->dct.leaf_cluster, ct.leaf_cluster, st))) return rc;
   if ((rc = upload(h, h->dct.tc16_items, ct.tc16_items, st))) return rc;
+  if ((rc = upload(h, h->dct.cl_leaves, ct.cl_leaves, st))) return rc;
+  if ((rc = upload(h, h->dct.zoff, ct.zoff, st))) return rc;
+  if ((rc = upload(h, h->dct.b16_items, ct.b16_items, st))) return rc;
   if ((rc = upload(h, h->dct.bgroup_leaves, ct.bgroup_leaves, st))) return rc;
   if ((rc = upload(h, h->dct.bgroups, ct.bgroups, st))) return rc;
   for (int i = 0; i < 4; ++i)

@@ -21,6 +21,11 @@
 // map each: K_c rows of block pos_class[m], and the member's t for 64
 // right-hand sides (box 32 floats x 1 member x 64 rhs).
 //
+// Several right-hand sides on the uniform layout (VEC): the vectors (member, right-hand side) of a
+// block are consecutive rows of t ([position][rhs][nint]), so an item is (block, 128-row tile, up
+// to 64 vectors) from the list of the FP16 path (tc_precond16.cu) and all blocks and right-hand
+// sides run in one launch; one launch per block and right-hand side took 8 us each.
+//
 // Kernel (one CTA per SM, persistent over items = (128-row tile, 64-member tile)):
 //   warp 0       TMA producer: A tile (128 rows x 32 floats) and T tile
 //                (64 members x 32 floats), 128-byte swizzle, 5-stage ring
@@ -68,6 +73,10 @@ struct PkArgs {
   float2* z;
   int* error;
   const int* gate;  // while a GMRES cycle is replayed: 0 = no right-hand side active, return at once
+  // VEC only
+  const int4* items;         // (block, row tile, first position, members)
+  const int* zoff;           // [position][24] output offset of each slot
+  int nitems;
   // MULTI only
   const int* pos_class;      // K block of the member at each stage-K position
   int npos, rtiles, nrhs;
@@ -85,15 +94,20 @@ struct __align__(8) Bars {
   int abort;
 };
 
-template <bool MULTI>
+enum class Mode { Block, Multi, Vec };
+
+template <Mode M>
 __global__ void __launch_bounds__(kThreads, 1)
     tc_precond_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapT, PkArgs a) {
   if (a.gate && *a.gate == 0) return;  // before any barrier or TMEM allocation
+  constexpr bool MULTI = M == Mode::Multi, VEC = M == Mode::Vec;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   Bars* bars = reinterpret_cast<Bars*>(ring + kStages * kStageBytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long nitems = MULTI ? (long long)a.npos * a.mtiles * a.rtiles : (long long)a.mtiles * a.ntiles;
+  const long long nitems = VEC     ? (long long)a.nitems * a.rtiles
+                           : MULTI ? (long long)a.npos * a.mtiles * a.rtiles
+                                   : (long long)a.mtiles * a.ntiles;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -139,6 +153,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           rt = rem % a.rtiles;
           nt = 0;
           blk = a.pos_class[pos];
+        } else if (VEC) {
+          const int4 e = a.items[item / a.rtiles];
+          blk = e.x;
+          mt = e.y;
+          nt = e.z * a.nrhs + (int)(item % a.rtiles) * kMem;  // first vector
         } else {
           mt = (int)(item % a.mtiles);
           nt = (int)(item / a.mtiles);
@@ -156,6 +175,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (MULTI) {
             tma_load_3d(st, &mapA, &bars->full[s], kb * kTileK, mt * kTileM, blk);
             tma_load_3d(st + kABytes + kBBytes, &mapT, &bars->full[s], kb * kTileK, pos, rt * kMem);
+          } else if (VEC) {
+            tma_load_3d(st, &mapA, &bars->full[s], kb * kTileK, mt * kTileM, blk);
+            tma_load_2d(st + kABytes + kBBytes, &mapT, &bars->full[s], kb * kTileK, nt);
           } else {
             tma_load_2d(st, &mapA, &bars->full[s], kb * kTileK, mt * kTileM);
             tma_load_2d(st + kABytes + kBBytes, &mapT, &bars->full[s], kb * kTileK, nt * kMem);
@@ -249,8 +271,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      int mt, nt, pos = 0, rt = 0;
-      if (MULTI) {
+      int mt, nt, pos = 0, rt = 0, cnt = 0;
+      if (VEC) {
+        const int4 e = a.items[item / a.rtiles];
+        const int first = (int)(item % a.rtiles) * kMem;
+        mt = e.y;
+        nt = e.z * a.nrhs + first;
+        cnt = min(kMem, e.w * a.nrhs - first);
+      } else if (MULTI) {
         pos = (int)(item / ((long long)a.mtiles * a.rtiles));
         const int rem = (int)(item % ((long long)a.mtiles * a.rtiles));
         mt = rem / a.rtiles;
@@ -269,7 +297,18 @@ __global__ void __launch_bounds__(kThreads, 1)
         tmem_ld32(taddr + kMem + half * 32, im);
         if (row < a.nint) {
           const int sl = row / a.q2, j = row % a.q2;
-          if (MULTI) {
+          if (VEC) {
+            const int v0 = nt + half * 32, n = cnt - half * 32;
+            int p = v0 / a.nrhs, rhs = v0 - p * a.nrhs;
+#pragma unroll
+            for (int c = 0; c < 32; ++c) {
+              if (c < n) a.z[(long long)rhs * a.nf + a.zoff[p * 24 + sl] + j] = make_float2(re[c], im[c]);
+              if (++rhs == a.nrhs) {
+                rhs = 0;
+                ++p;
+              }
+            }
+          } else if (MULTI) {
             // columns: 64 right-hand sides of one member
             const int cl = a.members[pos];
             const int lf = a.slot_lf[a.cl_slot_begin[cl] + sl];
@@ -316,7 +355,7 @@ cudaError_t launch_precond_tc(const hps_handle* h, const float2* t, float2* z, i
   if (!encode) return cudaErrorNotSupported;
   const int q2 = h->q * h->q;
   const int smem = kStages * kStageBytes + (int)sizeof(Bars) + 1024;
-  cudaError_t e = allow_dynamic_smem((const void*)tc_precond_kernel<false>, smem);
+  cudaError_t e = allow_dynamic_smem((const void*)tc_precond_kernel<Mode::Block>, smem);
   if (e != cudaSuccess) return e;
   for (int k : ct.kc_tc) {
     const int ns = ct.kc_slot_begin[k + 1] - ct.kc_slot_begin[k];
@@ -364,17 +403,76 @@ cudaError_t launch_precond_tc(const hps_handle* h, const float2* t, float2* z, i
     a.z = z;
     a.error = d_error;
     a.gate = h->gate;
+    a.items = nullptr;
+    a.zoff = nullptr;
+    a.nitems = 0;
     a.pos_class = nullptr;
     a.npos = a.rtiles = a.nrhs = 0;
     a.nf = 0;
     const long long items = (long long)a.mtiles * a.ntiles;
     const int grid = (int)std::min<long long>(items, h->nsm);
-    tc_precond_kernel<false><<<grid, kThreads, smem, st>>>(mapA, mapT, a);
+    tc_precond_kernel<Mode::Block><<<grid, kThreads, smem, st>>>(mapA, mapT, a);
     ++h->prof.launches;
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
+}
+
+cudaError_t launch_precond_tc_vec(const hps_handle* h, const float2* t32, float2* z, int nrhs, int* d_error,
+                                  cudaStream_t st) {
+  const ClusterTables& ct = h->ct;
+  if (!h->Kc32 || !d_error || !ct.uniform) return cudaErrorInvalidValue;
+  const int P = tc16_members_per_item(kMem, nrhs);
+  PkArgs a = {};
+  a.nitems = ct.tc16_count[P] - ct.tc16_ntc[P];
+  if (a.nitems == 0) return cudaSuccess;
+  auto encode = encoder();
+  if (!encode) return cudaErrorNotSupported;
+  const int nint = ct.nint0;
+  // TMA: 16-byte aligned bases and strides (checked, not assumed)
+  if ((reinterpret_cast<uintptr_t>(h->Kc32) | reinterpret_cast<uintptr_t>(t32)) % 16 != 0 || (8LL * nint) % 16 != 0)
+    return cudaErrorInvalidValue;
+  const int smem = kStages * kStageBytes + (int)sizeof(Bars) + 1024;
+  const cudaError_t e = allow_dynamic_smem((const void*)tc_precond_kernel<Mode::Vec>, smem);
+  if (e != cudaSuccess) return e;
+  CUtensorMap mapA, mapT;
+  {
+    cuuint64_t dims[3] = {(cuuint64_t)(2 * nint), (cuuint64_t)nint, (cuuint64_t)ct.nkc};
+    cuuint64_t strides[2] = {(cuuint64_t)nint * 8, (cuuint64_t)nint * nint * 8};
+    cuuint32_t box[3] = {kTileK, kTileM, 1};
+    cuuint32_t es[3] = {1, 1, 1};
+    if (encode(&mapA, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, (void*)h->Kc32, dims, strides, box, es,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return cudaErrorInvalidValue;
+  }
+  {
+    cuuint64_t dims[2] = {(cuuint64_t)(2 * nint), (cuuint64_t)ct.ncl * nrhs};
+    cuuint64_t strides[1] = {(cuuint64_t)nint * 8};
+    cuuint32_t box[2] = {kTileK, kMem};
+    cuuint32_t es[2] = {1, 1};
+    if (encode(&mapT, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, (void*)t32, dims, strides, box, es,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return cudaErrorInvalidValue;
+  }
+  a.nint = nint;
+  a.kblocks = (2 * nint + kTileK - 1) / kTileK;
+  a.q2 = h->q * h->q;
+  a.nb = h->nb;
+  a.items = h->dct.tc16_items + ct.tc16_begin[P] + ct.tc16_ntc[P];
+  a.zoff = h->dct.zoff;
+  a.rtiles = (nrhs + kMem - 1) / kMem;
+  a.nrhs = nrhs;
+  a.nf = h->nf;
+  a.z = z;
+  a.error = d_error;
+  a.gate = h->gate;
+  const int grid = (int)std::min<long long>((long long)a.nitems * a.rtiles, h->nsm);
+  tc_precond_kernel<Mode::Vec><<<grid, kThreads, smem, st>>>(mapA, mapT, a);
+  ++h->prof.launches;
+  return cudaGetLastError();
 }
 
 bool precond_tc_multi_eligible(const hps_handle* h, int nrhs) {
@@ -398,7 +496,7 @@ cudaError_t launch_precond_tc_multi(const hps_handle* h, const float2* t, float2
       (8LL * tstride) % 16 != 0)
     return cudaErrorInvalidValue;
   const int smem = kStages * kStageBytes + (int)sizeof(Bars) + 1024;
-  cudaError_t e = allow_dynamic_smem((const void*)tc_precond_kernel<true>, smem);
+  cudaError_t e = allow_dynamic_smem((const void*)tc_precond_kernel<Mode::Multi>, smem);
   if (e != cudaSuccess) return e;
   CUtensorMap mapA, mapT;
   {
@@ -437,6 +535,9 @@ cudaError_t launch_precond_tc_multi(const hps_handle* h, const float2* t, float2
   a.z = z;
   a.error = d_error;
   a.gate = h->gate;
+  a.items = nullptr;
+  a.zoff = nullptr;
+  a.nitems = 0;
   a.pos_class = h->dct.pos_class;
   a.npos = ct.ncl;
   a.rtiles = nrhs / kMem;
@@ -444,7 +545,7 @@ cudaError_t launch_precond_tc_multi(const hps_handle* h, const float2* t, float2
   a.nf = h->nf;
   const long long items = (long long)a.npos * a.mtiles * a.rtiles;
   const int grid = (int)std::min<long long>(items, h->nsm);
-  tc_precond_kernel<true><<<grid, kThreads, smem, st>>>(mapA, mapT, a);
+  tc_precond_kernel<Mode::Multi><<<grid, kThreads, smem, st>>>(mapA, mapT, a);
   ++h->prof.launches;
   return cudaGetLastError();
 }

@@ -1,38 +1,37 @@
-// Stage K of the cluster preconditioner (z_int = K_c t, Sec. 4, Algorithm 4 in
-// face form) for every cluster block in one launch, on the 5th-generation
-// tensor cores with FP16 operands (kind::f16, FP32 accumulation in TMEM).
+// The cluster preconditioner on the uniform layout with FP16 blocks (z = J^{-1} r, Sec. 4,
+// Algorithm 4 in face form), for any number of right-hand sides, in two launches:
 //
-// Operands:
-// * K_c in its FP16 copy (each row divided by its FP32 scale s_row, so that
-//   the entries are at most 1), read by TMA as a real n x 2n matrix A of
-//   interleaved (re, im) halves: 64 halves (128 bytes) per row and stage;
-// * t of each member cluster (complex FP32, the stage-B output) divided by the
-//   largest component of that cluster's t (stage B records it) and split by
-//   the transform warps into two FP16 terms, hi + lo (~22 bits), each laid out
-//   as the rows conj(t) and the re/im swap of t, so that A B_hi + A B_lo =
-//   [Re | Im] of K_c t / (s_row t_max).
-// The epilogue multiplies back by s_row and t_max.  K_c carries 2^-11 relative
-// rounding (a fixed matrix: the FP16 blocks the SIMT stage K uses); t is kept
-// to ~2^-22, so the result stays linear in t to FP32 level.  GMRES applies the
-// preconditioner to V y in its update and assumes that this equals
-// sum_j y_j M^{-1} v_j; with one FP16 rounding of t (2^-11, input-dependent)
-// that would hold only to ~2e-4.
+// * stage B (prec_b16_kernel): a thread-block cluster of 4 CTAs per up to 4 vectors that share
+//   their B blocks (right-hand sides, or members of one K block), two of the 8 leaves a CTA, forms
+//   t = r_int - B r_ext (SIMT, two rows per thread, B stored transposed), finds the largest component t_max through distributed shared memory and
+//   writes t / t_max as the tensor cores' operand: two FP16 terms hi + lo (~22 bits), each as the
+//   rows conj(t) and the re/im swap of t.  Doing this here, once, replaces the conversion that
+//   every 128-row tile of stage K would repeat (7 times at p = 8) on its way through shared memory.
+// * stage K (tc_precond16_kernel): z_int = K_c t on the 5th-generation tensor cores
+//   (tcgen05.mma.kind::f16, FP32 accumulation in TMEM).  A = K_c's FP16 copy (each row divided by
+//   its FP32 scale s_row) as a real n x 2n matrix of interleaved (re, im) halves; B = the operand
+//   rows; A B_hi + A B_lo = [Re | Im] of K_c t / (s_row t_max), multiplied back by s_row and t_max
+//   in the epilogue.  K_c carries 2^-11 relative rounding (a fixed matrix); t is kept to ~2^-22,
+//   so the result stays linear in t to FP32 level.  GMRES applies the preconditioner to V y in its
+//   update and assumes that this equals sum_j y_j M^{-1} v_j; with one FP16 rounding of t (2^-11,
+//   input-dependent) that would hold only to ~2e-4.
 //
-// Needs the uniform layout (every cluster 2x2x2, 24 q^2 a multiple of 32):
-// the blocks are one [block][row][2n halves] array and t one
-// [rhs][position][2n floats] array.  Items:
-// * one right-hand side: (block k, 128-row tile, first member position, member
-//   count <= 64) from a list built at setup; B rows = members;
-// * 64, 128, ... right-hand sides: (position, 128-row tile, 64-RHS tile); B
-//   rows = right-hand sides of one member.
+// Vector v = position * nrhs + rhs (position: place of the member cluster in stage-K order), so
+// the vectors of the clusters that share a block are consecutive.  A stage-K item is (block,
+// 128-row tile, up to COLS vectors): as many members as COLS / nrhs holds, or COLS right-hand sides
+// of one member.  The four operand planes of an item lie one after the other in shared memory, so
+// one MMA of N = 4 COLS per K step of 16 makes all four products against one read of A (separate
+// accumulators, added in the epilogue).  COLS = 16 keeps a stage at 24 KB and two CTAs per SM;
+// COLS = 64 (48 KB stages, one CTA per SM, all of TMEM) reads a block fewer times where many
+// vectors share it.  launch_precond_tc16 says where the line lies.
 //
-// Warp roles (384 threads, one CTA per SM, persistent, three 64 KB stages):
-// warp 0 TMA producer (A tile 128 rows x 128 bytes, two T boxes of 32 floats x
-// 64 rows), warp 1 TMEM allocation and the MMA issuer (two MMAs per K chunk:
-// hi and lo), warps 2..7 the FP16 conversion of t into the two swizzled B
-// tiles, warps 8..11 the epilogue.  Every wait is bounded; on a
-// time-out the CTA sets the error word, waits (bounded) for its own copies and
-// MMAs, frees TMEM and returns.
+// Stage K's warp roles (192 threads, persistent, four stages): warp 0 TMA producer (A tile 128
+// rows x 128 bytes, operand box 4 planes x COLS rows x 128 bytes), warp 1 TMEM allocation and the
+// MMA issuer, warps 2..5 the epilogue.  Every wait is bounded; on a time-out the CTA sets the error
+// word, waits (bounded) for its own copies and MMAs, frees TMEM and returns.
+//
+// Needs the uniform layout (every cluster 2x2x2, 24 q^2 a multiple of 32).
+#include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cudaTypedefs.h>
@@ -49,33 +48,271 @@ namespace {
 
 using namespace tc;
 
-constexpr int kStages = 3;
+// ---------------------------------------------------------------------------
+// Stage B
+// ---------------------------------------------------------------------------
+template <class TIN>
+struct PrecB16Args {
+  const __half2* B;       // FP16 blocks, transposed (column c holds the rows), rows divided by bscale
+  const float* bscale;
+  const long long* b_off;
+  const int* brd;         // per leaf, internal faces then external: input offsets
+  const int* bto;         // per leaf, internal faces: t offsets
+  const int* bsc;         // per leaf, internal faces: row-scale bases
+  const int* members;     // clusters in stage-K position order
+  const int* leaves;      // 8 leaves of each cluster
+  const int2* items;      // (first position, members), members of one K block; + kTcItem: a block of kc_tc
+  const TIN* r;
+  float2* z;
+  float2* t32;            // optional [vector][n]: t itself for the vectors of kc_tc blocks
+  __half2* op;            // operand rows [4][ncl * nrhs][n]: conj hi, swap hi, conj lo, swap lo
+  float* tmax;            // [ncl * nrhs]
+  int q2, n, ncl, nrhs, rtiles;
+  long long nf;
+  const int* gate;
+};
+
+constexpr int kBCluster = 4;  // CTAs per leaf cluster: two of its 8 leaves each
+
+// NR vectors per CTA, each entry of B loaded once for all of them; two rows per thread, so that
+// each staged input value feeds two sums.  B comes from L2 (3 q^2 entries per row): the next
+// entries of each row are in flight while the ones before them are used, the rows' offsets, scales and own inputs
+// loaded before the sums.
+template <class TIN, int NR>
+__global__ void __cluster_dims__(kBCluster, 1, 1) __maxnreg__(80) prec_b16_kernel(const PrecB16Args<TIN> A) {
+  namespace cg = cooperative_groups;
+  if (A.gate && *A.gate == 0) return;  // the same for every CTA of the cluster
+  extern __shared__ __align__(16) unsigned char b16_smem[];
+  const int q2 = A.q2, n3 = 3 * q2, n = A.n;  // a leaf: n3 internal rows, n3 external columns
+  const int nc = 2 * n3;                      // columns of the CTA's two leaves
+  float2* xs = reinterpret_cast<float2*>(b16_smem);  // [NR][nc]
+  __shared__ float red[20][NR], cmax[NR];
+  __shared__ long long roff[NR];
+  __shared__ int vpos[NR];
+  const int item = blockIdx.x / kBCluster, l0 = (blockIdx.x % kBCluster) * 2;
+  int2 it = A.items[item / A.rtiles];
+  const bool keep = A.t32 && it.y >= kTcItem;
+  it.y &= kTcItem - 1;
+  const int first = (item % A.rtiles) * NR;
+  const int nr = min(NR, it.y * A.nrhs - first), v0 = it.x * A.nrhs + first;
+  const int tid = threadIdx.x, nt = blockDim.x;
+  if (tid < NR) {
+    const int v = v0 + min(tid, nr - 1), p = v / A.nrhs;
+    vpos[tid] = p;
+    roff[tid] = (long long)(v - p * A.nrhs) * A.nf;
+  }
+  __syncthreads();
+  // the leaves of vector rr's cluster (vectors of an item share the B blocks, not the leaves)
+  const int* leaves[NR];
+  long long ro[NR];
+#pragma unroll
+  for (int rr = 0; rr < NR; ++rr) {
+    leaves[rr] = A.leaves + 8 * A.members[vpos[rr]] + l0;
+    ro[rr] = roff[rr];
+  }
+  for (int t = tid; t < nc; t += nt) {
+    const int li = t >= n3, c = t - li * n3, k = c / q2;
+#pragma unroll
+    for (int rr = 0; rr < NR; ++rr) {
+      if (rr < nr) {
+        const long long o = ro[rr] + A.brd[leaves[rr][li] * 6 + 3 + k] + (c - k * q2);
+        const float2 v = cvt<float2>(A.r[o]);
+        xs[rr * nc + t] = v;
+        A.z[o] = v;
+      } else {
+        xs[rr * nc + t] = make_float2(0.f, 0.f);
+      }
+    }
+  }
+  __syncthreads();
+  constexpr int kRows = 2;
+  constexpr int kU = NR == 4 ? 4 : 12;  // entries per row in flight (80 registers: 6 CTAs per SM at q = 6)
+  const int hr = n3 / 2;  // rows of a thread: hr apart
+  const bool on = tid < n3;
+  float2 tv[kRows][NR];
+  int to[kRows][NR];
+  float mx[NR];
+#pragma unroll
+  for (int rr = 0; rr < NR; ++rr) mx[rr] = 0.f;
+  if (on) {
+    const int ldr = (int)rup4(n3);
+    const int li = tid >= hr, row0 = tid - li * hr;
+    const int leaf0 = leaves[0][li];
+    const __half2* Bm = A.B + A.b_off[leaf0] + row0;
+    const float2* x = xs + li * n3;
+    __half2 b0[kRows][kU], b1[kRows][kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+#pragma unroll
+      for (int i = 0; i < kRows; ++i) b0[i][u] = Bm[u * ldr + i * hr];
+    float sc[kRows];
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+      const int row = row0 + i * hr, k = row / q2, j = row - k * q2;
+      sc[i] = A.bscale[A.bsc[leaf0 * 6 + k] + j];
+#pragma unroll
+      for (int rr = 0; rr < NR; ++rr) {
+        const int e = leaves[rr][li] * 6 + k;
+        to[i][rr] = A.bto[e] - vpos[rr] * n + j;
+        tv[i][rr] = rr < nr ? cvt<float2>(A.r[ro[rr] + A.brd[e] + j]) : make_float2(0.f, 0.f);
+      }
+    }
+    float2 acc[kRows][NR];
+#pragma unroll
+    for (int i = 0; i < kRows; ++i)
+#pragma unroll
+      for (int rr = 0; rr < NR; ++rr) acc[i][rr] = make_float2(0.f, 0.f);
+    for (int c = 0; c < n3; c += kU) {  // n3 is a multiple of 12: q is even
+      if (c + kU < n3) {
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+#pragma unroll
+          for (int i = 0; i < kRows; ++i) b1[i][u] = Bm[(c + kU + u) * ldr + i * hr];
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        float2 bv[kRows];
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) {
+          bv[i] = __half22float2(b0[i][u]);
+          b0[i][u] = b1[i][u];
+        }
+#pragma unroll
+        for (int rr = 0; rr < NR; ++rr) {
+          const float2 xv = x[rr * nc + c + u];
+#pragma unroll
+          for (int i = 0; i < kRows; ++i) cfma(acc[i][rr], bv[i], xv);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kRows; ++i)
+#pragma unroll
+      for (int rr = 0; rr < NR; ++rr) {
+        tv[i][rr] = csub(tv[i][rr], make_float2(acc[i][rr].x * sc[i], acc[i][rr].y * sc[i]));
+        if (keep && rr < nr) A.t32[(long long)(v0 + rr) * n + to[i][rr]] = tv[i][rr];
+        if (rr < nr) mx[rr] = fmaxf(mx[rr], fmaxf(fabsf(tv[i][rr].x), fabsf(tv[i][rr].y)));
+      }
+  }
+#pragma unroll
+  for (int rr = 0; rr < NR; ++rr) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx[rr] = fmaxf(mx[rr], __shfl_xor_sync(0xffffffffu, mx[rr], o));
+    if ((tid & 31) == 0) red[tid >> 5][rr] = mx[rr];
+  }
+  __syncthreads();
+  if (tid < NR) {
+    float m = 0.f;
+    for (int w = 0; w < nt / 32; ++w) m = fmaxf(m, red[w][tid]);
+    cmax[tid] = m;
+  }
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  const long long plane = (long long)A.ncl * A.nrhs * n;
+#pragma unroll
+  for (int rr = 0; rr < NR; ++rr) {
+    if (rr >= nr) break;
+    float m = 0.f;
+#pragma unroll
+    for (int w = 0; w < kBCluster; ++w) m = fmaxf(m, *cl.map_shared_rank(&cmax[rr], w));
+    const long long v = v0 + rr;
+    if (tid == 0 && l0 == 0) A.tmax[v] = m;
+    // A maximum below the smallest normal float (a cluster far from every source, whose t holds
+    // only subnormal values) would overflow the reciprocal: such a cluster's t is taken as 0, a
+    // change below 2^-126 of the vector's scale.
+    const float sc = m >= 0x1p-126f ? 1.f / m : 0.f;
+    __half2* op = A.op + v * n;
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+      if (!on) break;
+      const float2 x = make_float2(tv[i][rr].x * sc, tv[i][rr].y * sc);
+      const __half2 h = __floats2half2_rn(x.x, x.y);
+      const __half2 l = __floats2half2_rn(x.x - __low2float(h), x.y - __high2float(h));
+      __half2* d = op + to[i][rr];
+      d[0] = __halves2half2(__low2half(h), __hneg(__high2half(h)));
+      d[plane] = __halves2half2(__high2half(h), __low2half(h));
+      d[2 * plane] = __halves2half2(__low2half(l), __hneg(__high2half(l)));
+      d[3 * plane] = __halves2half2(__high2half(l), __low2half(l));
+    }
+  }
+  cl.sync();  // no CTA leaves while another may read its maximum
+}
+
+template <class TIN>
+cudaError_t stage_b16(const hps_handle* h, const TIN* r, float2* z, float2* t32, int nrhs, cudaStream_t st) {
+  const ClusterTables& ct = h->ct;
+  PrecB16Args<TIN> a;
+  a.B = h->B16;
+  a.bscale = h->B16s;
+  a.b_off = h->dct.b_off;
+  a.brd = h->dct.brd;
+  a.bto = h->dct.bto;
+  a.bsc = h->dct.bsc;
+  a.members = h->dct.kc_members;
+  a.leaves = h->dct.cl_leaves;
+  a.r = r;
+  a.z = z;
+  a.t32 = t32;
+  a.op = h->op16;
+  a.tmax = h->tmax;
+  a.q2 = h->q * h->q;
+  a.n = ct.nint0;
+  a.ncl = ct.ncl;
+  a.nrhs = nrhs;
+  a.nf = h->nf;
+  a.gate = h->gate;
+  // Vectors per item: the most (up to 4) that leave 4 CTAs per SM, and no more than any block has.
+  // Measured at p = 8: 12^3 leaves of a bump medium, one right-hand side, 20.8 us with 1 vector
+  // against 24.9 us with 4 (too few CTAs); 8^3 leaves, 12 right-hand sides, 45 us with 4.
+  const int n3 = 3 * a.q2;
+  auto ctas_of = [&](int k) {
+    return (long long)ct.b16_count[tc16_members_per_item(k, nrhs)] * ((nrhs + k - 1) / k) * kBCluster;
+  };
+  int nr = 4;
+  while (nr > 1 && (ctas_of(nr) < 4LL * h->nsm || (long long)ct.max_members * nrhs <= nr / 2)) nr >>= 1;
+  const int P = tc16_members_per_item(nr, nrhs);
+  a.items = h->dct.b16_items + ct.b16_begin[P];
+  a.rtiles = (nrhs + nr - 1) / nr;
+  const int threads = (int)round_up(n3, 32);
+  const size_t smem = (size_t)nr * 2 * n3 * sizeof(float2);
+  auto run = [&](auto kern) -> cudaError_t {
+    const cudaError_t e = allow_dynamic_smem((const void*)kern, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)((long long)ct.b16_count[P] * a.rtiles * kBCluster), threads, smem, st>>>(a);
+    ++h->prof.launches;
+    return cudaGetLastError();
+  };
+  if (nr == 1) return run(prec_b16_kernel<TIN, 1>);
+  if (nr == 2) return run(prec_b16_kernel<TIN, 2>);
+  return run(prec_b16_kernel<TIN, 4>);
+}
+
+// ---------------------------------------------------------------------------
+// Stage K
+// ---------------------------------------------------------------------------
+constexpr int kStages = 4;
 constexpr int kTileM = 128;
-constexpr int kCols = 64;               // B rows per operand half: members or right-hand sides
-constexpr int kTileN = 2 * kCols;       // (re, im) accumulator columns
 constexpr int kKHalves = 64;            // K extent of a stage (128 bytes of FP16)
 constexpr int kABytes = kTileM * 128;   // 16 KB
-constexpr int kBBytes = kTileN * 128;   // 16 KB
-constexpr int kTBoxBytes = kCols * 128; // 8 KB: 64 rows x 32 floats
-// stage layout (1024-byte aligned parts): A | B (high halves of t) | B (low halves) | T box 0 |
-// T box 1
-constexpr int kTOff = kABytes + 2 * kBBytes;
-constexpr int kStageBytes = kTOff + 2 * kTBoxBytes;  // 64 KB
-constexpr int kThreads = 384;
-constexpr int kTmemCols = 256;
+constexpr int kThreads = 192;
+
+template <int COLS> struct Shape {
+  static constexpr int kBBytes = 4 * COLS * 128;           // operand planes conj hi, swap hi, conj lo, swap lo
+  static constexpr int kStageBytes = kABytes + kBBytes;    // parts 1024-byte aligned
+  static constexpr int kN = 4 * COLS;                      // accumulator columns
+  static constexpr int kTmemCols = 2 * kN;                 // two accumulators
+};
 
 struct Pk16Args {
-  int nint, mtiles, kblocks, q2, nb, ncl;
+  int nint, kblocks, q2, nb;
   long long nitems;
-  const int4* items;       // one RHS: (block, row tile, first position, count)
-  const int* members;      // clusters in stage-K position order
-  const int* pos_class;    // block of each position (MULTI)
+  const int4* items;       // (block, row tile, first position, members)
+  int rtiles;              // COLS-RHS tiles of one member (nrhs > COLS), else 1
+  int nrhs;
   const int* kc_slot_begin;
-  const int* cl_slot_begin;
-  const int* slot_lf;
+  const int* zoff;         // [position][24] output offset of each slot of the member's faces
   const float* kscale;     // FP16 row scales, index kc_slot_begin[k] q^2 + row
-  const float* tmax;       // [rhs][cluster] largest |component| of t
-  int rtiles, nrhs;
+  const float* tmax;       // [vector]
   long long nf;
   float2* z;
   int* error;
@@ -84,7 +321,6 @@ struct Pk16Args {
 
 struct __align__(8) Bars {
   uint64_t full[kStages];
-  uint64_t split[kStages];
   uint64_t empty[kStages];
   uint64_t acc_full[2];
   uint64_t acc_empty[2];
@@ -93,50 +329,23 @@ struct __align__(8) Bars {
   int abort;
 };
 
-// Item decode shared by the roles.
-template <bool MULTI>
-__device__ __forceinline__ void decode(const Pk16Args& a, long long item, int& blk, int& mt, int& pos0, int& cnt,
-                                       int& rt) {
-  if (MULTI) {
-    const long long per = (long long)a.mtiles * a.rtiles;
-    pos0 = (int)(item / per);
-    const int rem = (int)(item % per);
-    mt = rem / a.rtiles;
-    rt = rem % a.rtiles;
-    cnt = 1;
-    blk = a.pos_class[pos0];
-  } else {
-    const int4 e = a.items[item];
-    blk = e.x;
-    mt = e.y;
-    pos0 = e.z;
-    cnt = e.w;
-    rt = 0;
-  }
+// block, row tile, first vector and vector count of an item
+template <int COLS>
+__device__ __forceinline__ void decode(const Pk16Args& a, long long item, int& blk, int& mt, int& v0, int& cnt) {
+  const int4 e = a.items[item / a.rtiles];
+  const int first = (int)(item % a.rtiles) * COLS;
+  blk = e.x;
+  mt = e.y;
+  v0 = e.z * a.nrhs + first;
+  cnt = min(COLS, e.w * a.nrhs - first);
 }
 
-// 1 / (largest component of t) of the cluster whose data fills B row m, 0 for unused rows.  A
-// maximum below the smallest normal float (a cluster far from every source, whose t holds only
-// subnormal values) would overflow the reciprocal: such a cluster's t is taken as 0, a change
-// below 2^-126 of the vector's scale.
-template <bool MULTI>
-__device__ __forceinline__ float inv_scale(const Pk16Args& a, int m, int pos0, int cnt, int rt) {
-  float mx;
-  if (MULTI) {
-    const int rhs = rt * kCols + m;
-    if (rhs >= a.nrhs) return 0.f;
-    mx = a.tmax[(long long)rhs * a.ncl + a.members[pos0]];
-  } else {
-    if (m >= cnt) return 0.f;
-    mx = a.tmax[a.members[pos0 + m]];
-  }
-  return mx >= 0x1p-126f ? 1.f / mx : 0.f;
-}
-
-template <bool MULTI>
-__global__ void __launch_bounds__(kThreads, 1)
-    tc_precond16_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapT,
+template <int COLS>
+__global__ void __launch_bounds__(kThreads, COLS == 16 ? 2 : 1)
+    tc_precond16_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                         Pk16Args a) {
+  using S = Shape<COLS>;
+  constexpr int kStageBytes = S::kStageBytes, kTmemCols = S::kTmemCols;
   if (a.gate && *a.gate == 0) return;  // before any barrier or TMEM allocation
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -146,7 +355,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&bars->full[s], 1);
-      mbar_init(&bars->split[s], 6);
       mbar_init(&bars->empty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -178,8 +386,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       long long it = 0;
       bool ok = true;
       for (long long item = blockIdx.x; item < a.nitems && ok; item += gridDim.x) {
-        int blk, mt, pos0, cnt, rt;
-        decode<MULTI>(a, item, blk, mt, pos0, cnt, rt);
+        int blk, mt, v0, cnt;
+        decode<COLS>(a, item, blk, mt, v0, cnt);
         for (int kb = 0; kb < a.kblocks; ++kb, ++it) {
           const int s = (int)(it % kStages);
           const uint32_t ph = (uint32_t)((it / kStages) & 1);
@@ -189,97 +397,24 @@ __global__ void __launch_bounds__(kThreads, 1)
             break;
           }
           unsigned char* st = ring + s * kStageBytes;
-          mbar_expect_tx(&bars->full[s], kABytes + 2 * kTBoxBytes);
+          mbar_expect_tx(&bars->full[s], kStageBytes);
           tma_load_3d(st, &mapA, &bars->full[s], kb * kKHalves, mt * kTileM, blk);
-          unsigned char* tdst = st + kTOff;
-          for (int b = 0; b < 2; ++b) {
-            const int x = kb * kKHalves + b * 32;  // floats of t: the same K range as the halves of A
-            if (MULTI) tma_load_3d(tdst + b * kTBoxBytes, &mapT, &bars->full[s], x, pos0, rt * kCols);
-            else tma_load_2d(tdst + b * kTBoxBytes, &mapT, &bars->full[s], x, pos0);
-          }
+          tma_load_3d(st + kABytes, &mapB, &bars->full[s], kb * kKHalves, v0, 0);
         }
       }
       for (long long j = (it > kStages ? it - kStages : 0); j < it; ++j)
         if (!mbar_wait(&bars->full[(int)(j % kStages)], (uint32_t)((j / kStages) & 1))) fail();
     }
-  } else if (warp >= 2 && warp < 8) {
-    // ---------------- t -> FP16 B operand (conj rows, swap rows), 128-byte swizzle ----------------
-    const int tt = threadIdx.x - 64;  // 0..191
-    constexpr int kTasks = kCols * 8, kPer = (kTasks + 191) / 192;
-    long long it = 0;
-    for (long long item = blockIdx.x; item < a.nitems; item += gridDim.x) {
-      int blk, mt, pos0, cnt, rt;
-      decode<MULTI>(a, item, blk, mt, pos0, cnt, rt);
-      // a thread fills the same B rows at every K step: their scales once per item
-      float scr[kPer];
-#pragma unroll
-      for (int i = 0; i < kPer; ++i) {
-        const int task = tt + 192 * i;
-        scr[i] = task < kTasks ? inv_scale<MULTI>(a, task >> 3, pos0, cnt, rt) : 0.f;
-      }
-      for (int kb = 0; kb < a.kblocks; ++kb, ++it) {
-        const int s = (int)(it % kStages);
-        const uint32_t ph = (uint32_t)((it / kStages) & 1);
-        if (bars->abort || !mbar_wait(&bars->full[s], ph)) {
-          fail();
-          goto split_done;
-        }
-        unsigned char* st = ring + s * kStageBytes;
-        unsigned char* B = st + kABytes;
-        unsigned char* Blo = B + kBBytes;
-        const unsigned char* T = st + kTOff;
-        // task = (row m, 16-byte chunk c of the B row): 4 complex values of K index 4c..4c+3,
-        // which are floats 8(c%4)..8(c%4)+7 of T box c/4, row m (two 16-byte T chunks)
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-          const int task = tt + 192 * i;
-          if (task >= kTasks) break;
-          const int m = task >> 3, c = task & 7;
-          const float sc = scr[i];
-          const unsigned char* trow = T + (c >> 2) * kTBoxBytes + m * 128;
-          const int ch0 = 2 * (c & 3);
-          const float4 p0 = *reinterpret_cast<const float4*>(trow + ((ch0 ^ (m & 7)) << 4));
-          const float4 p1 = *reinterpret_cast<const float4*>(trow + (((ch0 + 1) ^ (m & 7)) << 4));
-          // t / t_max = hi + lo in two FP16 terms (~22 bits): the product stays linear in t to
-          // FP32 level, as the Krylov update, which applies the preconditioner to V y, needs
-          const float x[8] = {p0.x * sc, p0.y * sc, p0.z * sc, p0.w * sc, p1.x * sc, p1.y * sc, p1.z * sc, p1.w * sc};
-          uint32_t cjh[4], swh[4], cjl[4], swl[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const __half2 h = __floats2half2_rn(x[2 * e], x[2 * e + 1]);  // (re, im) high parts
-            const __half2 l = __floats2half2_rn(x[2 * e] - __low2float(h), x[2 * e + 1] - __high2float(h));
-            // conj row (re, -im), swap row (im, re); negation is exact in FP16
-            const __half2 hc = __halves2half2(__low2half(h), __hneg(__high2half(h)));
-            const __half2 hs = __halves2half2(__high2half(h), __low2half(h));
-            const __half2 lc = __halves2half2(__low2half(l), __hneg(__high2half(l)));
-            const __half2 ls = __halves2half2(__high2half(l), __low2half(l));
-            cjh[e] = *reinterpret_cast<const uint32_t*>(&hc);
-            swh[e] = *reinterpret_cast<const uint32_t*>(&hs);
-            cjl[e] = *reinterpret_cast<const uint32_t*>(&lc);
-            swl[e] = *reinterpret_cast<const uint32_t*>(&ls);
-          }
-          const int pc = (c ^ (m & 7)) << 4;  // rows m and 64 + m share the swizzle phase
-          *reinterpret_cast<uint4*>(B + m * 128 + pc) = make_uint4(cjh[0], cjh[1], cjh[2], cjh[3]);
-          *reinterpret_cast<uint4*>(B + (kCols + m) * 128 + pc) = make_uint4(swh[0], swh[1], swh[2], swh[3]);
-          *reinterpret_cast<uint4*>(Blo + m * 128 + pc) = make_uint4(cjl[0], cjl[1], cjl[2], cjl[3]);
-          *reinterpret_cast<uint4*>(Blo + (kCols + m) * 128 + pc) = make_uint4(swl[0], swl[1], swl[2], swl[3]);
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bars->split[s]);
-      }
-    }
-  split_done:;
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
     if (lane == 0) {
-      const uint32_t idesc = instr_desc_f16(kTileN, kTileM);
+      const uint32_t idesc = instr_desc_f16(S::kN, kTileM);
       long long it = 0;
       long long local = 0;
       bool ok = true;
       for (long long item = blockIdx.x; item < a.nitems && ok; item += gridDim.x, ++local) {
         const int b = (int)(local & 1);
-        const uint32_t acc = tmem + (uint32_t)(b * kTileN);
+        const uint32_t acc = tmem + (uint32_t)(b * S::kN);
         if (local >= 2 && !mbar_wait(&bars->acc_empty[b], (uint32_t)(((local >> 1) - 1) & 1))) {
           fail();
           ok = false;
@@ -289,19 +424,17 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int kb = 0; kb < a.kblocks; ++kb, ++it) {
           const int s = (int)(it % kStages);
           const uint32_t ph = (uint32_t)((it / kStages) & 1);
-          if (bars->abort || !mbar_wait(&bars->split[s], ph)) {
+          if (bars->abort || !mbar_wait(&bars->full[s], ph)) {
             fail();
             ok = false;
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t base = smem_u32(ring + s * kStageBytes);
-          const uint32_t aa = base, bb = base + kABytes, bl = bb + kBBytes;
+          const uint32_t aa = smem_u32(ring + s * kStageBytes), bb = aa + kABytes;
 #pragma unroll
           for (int kk = 0; kk < kKHalves / 16; ++kk) {
             const uint32_t off = kk * 32;  // 16 halves
             mma_f16(acc, smem_desc(aa + off), smem_desc(bb + off), idesc, (kb == 0 && kk == 0) ? 0u : 1u);
-            mma_f16(acc, smem_desc(aa + off), smem_desc(bl + off), idesc, 1u);
           }
           mma_commit(&bars->empty[s]);
         }
@@ -313,8 +446,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else {
-    // ---------------- epilogue: warps 8..11 = TMEM lanes 0..127 ----------------
-    const int ew = warp - 8;
+    // ---------------- epilogue: warps 2..5, each on the 32 TMEM lanes that it may read ----------------
+    const int ew = warp & 3;
     long long local = 0;
     for (long long item = blockIdx.x; item < a.nitems; item += gridDim.x, ++local) {
       const int b = (int)(local & 1);
@@ -323,40 +456,46 @@ __global__ void __launch_bounds__(kThreads, 1)
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      int blk, mt, pos0, cnt, rt;
-      decode<MULTI>(a, item, blk, mt, pos0, cnt, rt);
+      int blk, mt, v0, cnt;
+      decode<COLS>(a, item, blk, mt, v0, cnt);
       const int row = mt * kTileM + ew * 32 + lane;
-      const uint32_t taddr = tmem + ((uint32_t)(ew * 32) << 16) + (uint32_t)(b * kTileN);
+      const uint32_t taddr = tmem + ((uint32_t)(ew * 32) << 16) + (uint32_t)(b * S::kN);
       const float ks = (row < a.nint) ? a.kscale[(long long)a.kc_slot_begin[blk] * a.q2 + row] : 0.f;
-      float re[32], im[32];
-      for (int half = 0; half < 2; ++half) {
-        tmem_ld32(taddr + half * 32, re);
-        tmem_ld32(taddr + kCols + half * 32, im);
+      const int sl = row / a.q2, j = row - sl * a.q2;
+      const int* zo = a.zoff + sl;
+      for (int h0 = 0; h0 < cnt; h0 += 16) {
+        // offsets and scales of 16 vectors first (independent loads), then the accumulators
+        int off[16];
+        float f[16];
+        int pos = (v0 + h0) / a.nrhs, rhs = v0 + h0 - pos * a.nrhs;
+        const int first = rhs;
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+          const bool on = h0 + c < cnt && row < a.nint;
+          off[c] = on ? zo[pos * 24] : 0;
+          f[c] = on ? a.tmax[v0 + h0 + c] : 0.f;
+          if (++rhs == a.nrhs) {
+            rhs = 0;
+            ++pos;
+          }
+        }
+        uint32_t reh[16], imh[16], rel[16], iml[16];
+        tmem_ld16(taddr + h0, reh);
+        tmem_ld16(taddr + COLS + h0, imh);
+        tmem_ld16(taddr + 2 * COLS + h0, rel);
+        tmem_ld16(taddr + 3 * COLS + h0, iml);
+        tmem_wait_ld();
+        rhs = first;
         if (row < a.nint) {
-          const int sl = row / a.q2, j = row % a.q2;
-          if (MULTI) {
-            const int cl = a.members[pos0];
-            const int lf = a.slot_lf[a.cl_slot_begin[cl] + sl];
-            const long long o = (long long)(lf / 6) * a.nb + (long long)(lf % 6) * a.q2 + j;
 #pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              const int rhs = rt * kCols + half * 32 + c;
-              if (rhs < a.nrhs) {
-                const float f = ks * a.tmax[(long long)rhs * a.ncl + cl];
-                a.z[(long long)rhs * a.nf + o] = make_float2(re[c] * f, im[c] * f);
-              }
+          for (int c = 0; c < 16; ++c) {
+            if (h0 + c < cnt) {
+              const float w = ks * f[c];
+              a.z[(long long)rhs * a.nf + off[c] + j] =
+                  make_float2((__uint_as_float(reh[c]) + __uint_as_float(rel[c])) * w,
+                              (__uint_as_float(imh[c]) + __uint_as_float(iml[c])) * w);
             }
-          } else {
-#pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              const int m = half * 32 + c;
-              if (m < cnt) {
-                const int cl = a.members[pos0 + m];
-                const int lf = a.slot_lf[a.cl_slot_begin[cl] + sl];
-                const float f = ks * a.tmax[cl];
-                a.z[(long long)(lf / 6) * a.nb + (long long)(lf % 6) * a.q2 + j] = make_float2(re[c] * f, im[c] * f);
-              }
-            }
+            if (++rhs == a.nrhs) rhs = 0;
           }
         }
       }
@@ -375,90 +514,83 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 }  // namespace
 
+int tc16_members_per_item(int cols, int nrhs) { return nrhs >= cols ? 1 : cols / nrhs; }
+
 bool precond_tc16_eligible(const hps_handle* h, int nrhs) {
-  return h->has_precond && h->opt.tc_apply && h->Kc16 && h->Kc16s && h->tc_error && h->tmax && h->ct.uniform &&
-         h->ct.nslots > 0 && (h->ct.nint0 % 32 == 0) && nrhs <= h->tmax_rhs &&
-         (nrhs == 1 || (nrhs >= kCols && nrhs % kCols == 0));
+  return h->has_precond && h->opt.tc_apply && h->Kc16 && h->Kc16s && h->tc_error && h->tmax && h->op16 &&
+         h->ct.uniform && h->ct.nslots > 0 && (h->ct.nint0 % 32 == 0) && nrhs <= h->tmax_rhs;
 }
 
-// z_int = K_c t for every cluster (FP16 blocks, FP16 t scaled per cluster by tmax), one launch.
-cudaError_t launch_precond_tc16(const hps_handle* h, const float2* t, float2* z, int nrhs, cudaStream_t st) {
+cudaError_t launch_precond_b16(const hps_handle* h, VType tin, const void* r, float2* z, float2* t32, int nrhs,
+                               cudaStream_t st) {
+  if (!precond_tc16_eligible(h, nrhs)) return cudaErrorInvalidValue;
+  if (tin == VType::C64) return stage_b16(h, (const float2*)r, z, t32, nrhs, st);
+  if (tin == VType::DF) return stage_b16(h, (const float4*)r, z, t32, nrhs, st);
+  return stage_b16(h, (const double2*)r, z, t32, nrhs, st);
+}
+
+cudaError_t launch_precond_tc16(const hps_handle* h, float2* z, int nrhs, bool skip_tc, cudaStream_t st) {
   const ClusterTables& ct = h->ct;
   if (!precond_tc16_eligible(h, nrhs)) return cudaErrorInvalidValue;
   auto encode = encoder();
   if (!encode) return cudaErrorNotSupported;
-  const int q2 = h->q * h->q;
   const int nint = ct.nint0;
-  const long long tstride = ct.tsize;
   // TMA: 16-byte aligned bases and strides (checked, not assumed)
-  if ((reinterpret_cast<uintptr_t>(h->Kc16) | reinterpret_cast<uintptr_t>(t)) % 16 != 0 || (4LL * nint) % 16 != 0 ||
-      (8LL * nint) % 16 != 0 || (8LL * tstride) % 16 != 0)
+  if ((reinterpret_cast<uintptr_t>(h->Kc16) | reinterpret_cast<uintptr_t>(h->op16)) % 16 != 0 || (4LL * nint) % 16 != 0)
     return cudaErrorInvalidValue;
-  const bool multi = nrhs > 1;
-  const int smem = kStages * kStageBytes + (int)sizeof(Bars) + 1024;
-  auto kern = multi ? tc_precond16_kernel<true> : tc_precond16_kernel<false>;
-  cudaError_t e = allow_dynamic_smem((const void*)kern, smem);
-  if (e != cudaSuccess) return e;
-  CUtensorMap mapA, mapT;
-  {
-    // FP16 blocks [block][row][2 nint halves], rows nint complex apart
-    cuuint64_t dims[3] = {(cuuint64_t)(2 * nint), (cuuint64_t)nint, (cuuint64_t)ct.nkc};
-    cuuint64_t strides[2] = {(cuuint64_t)nint * 4, (cuuint64_t)nint * nint * 4};
-    cuuint32_t box[3] = {kKHalves, kTileM, 1};
+  // Items of 16 vectors unless that takes more than twice as many items as 64 would (blocks shared
+  // by many vectors).  Measured per application of stage K at p = 8:
+  // 12^3 leaves of a bump medium, one right-hand side (few blocks, up to ~190 members) 18.9 us at 16
+  // against 51 us at 64 columns; 8^3 leaves, 12 right-hand sides (45 blocks) 37 against 73 us.
+  auto count_of = [&](int cols) {
+    const int p = tc16_members_per_item(cols, nrhs);
+    return (long long)(skip_tc ? ct.tc16_ntc[p] : ct.tc16_count[p]) * ((nrhs + cols - 1) / cols);
+  };
+  const int cols = count_of(16) <= 2 * count_of(64) ? 16 : 64;
+  const int P = tc16_members_per_item(cols, nrhs);
+  CUtensorMap mapA, mapB;
+  // three-dimensional FP16 arrays [d2][d1][2 nint halves] in boxes of 64 halves x b1 rows x b2
+  auto map3 = [&](CUtensorMap* m, void* base, cuuint64_t d1, cuuint64_t d2, cuuint32_t b1, cuuint32_t b2) {
+    cuuint64_t dims[3] = {(cuuint64_t)(2 * nint), d1, d2};
+    cuuint64_t strides[2] = {(cuuint64_t)nint * 4, (cuuint64_t)nint * 4 * d1};
+    cuuint32_t box[3] = {kKHalves, b1, b2};
     cuuint32_t es[3] = {1, 1, 1};
-    if (encode(&mapA, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, (void*)h->Kc16, dims, strides, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cudaErrorInvalidValue;
-  }
-  if (multi) {
-    // t [rhs][position][2 nint floats]; box 32 floats x 1 member x 64 right-hand sides
-    cuuint64_t dims[3] = {(cuuint64_t)(2 * nint), (cuuint64_t)ct.ncl, (cuuint64_t)nrhs};
-    cuuint64_t strides[2] = {(cuuint64_t)nint * 8, (cuuint64_t)tstride * 8};
-    cuuint32_t box[3] = {32, 1, kCols};
-    cuuint32_t es[3] = {1, 1, 1};
-    if (encode(&mapT, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, (void*)t, dims, strides, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cudaErrorInvalidValue;
-  } else {
-    // t [position][2 nint floats]; box 32 floats x 64 members
-    cuuint64_t dims[2] = {(cuuint64_t)(2 * nint), (cuuint64_t)ct.ncl};
-    cuuint64_t strides[1] = {(cuuint64_t)nint * 8};
-    cuuint32_t box[2] = {32, kCols};
-    cuuint32_t es[2] = {1, 1};
-    if (encode(&mapT, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, (void*)t, dims, strides, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cudaErrorInvalidValue;
-  }
+    return encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  };
+  if (!map3(&mapA, (void*)h->Kc16, (cuuint64_t)nint, (cuuint64_t)ct.nkc, kTileM, 1) ||
+      !map3(&mapB, (void*)h->op16, (cuuint64_t)ct.ncl * nrhs, 4, (cuuint32_t)cols, 4))
+    return cudaErrorInvalidValue;
   Pk16Args a;
   a.nint = nint;
-  a.mtiles = (nint + kTileM - 1) / kTileM;
   a.kblocks = 2 * nint / kKHalves;
-  a.q2 = q2;
+  a.q2 = h->q * h->q;
   a.nb = h->nb;
-  a.ncl = ct.ncl;
-  a.items = h->dct.tc16_items;
-  a.members = h->dct.kc_members;
-  a.pos_class = h->dct.pos_class;
+  a.items = h->dct.tc16_items + ct.tc16_begin[P];
+  a.rtiles = (nrhs + cols - 1) / cols;
+  a.nrhs = nrhs;
   a.kc_slot_begin = h->dct.kc_slot_begin;
-  a.cl_slot_begin = h->dct.cl_slot_begin;
-  a.slot_lf = h->dct.slot_lf;
+  a.zoff = h->dct.zoff;
   a.kscale = h->Kc16s;
   a.tmax = h->tmax;
-  a.rtiles = multi ? nrhs / kCols : 1;
-  a.nrhs = nrhs;
   a.nf = h->nf;
   a.z = z;
   a.error = h->tc_error;
   a.gate = h->gate;
-  a.nitems = multi ? (long long)ct.ncl * a.mtiles * a.rtiles : (long long)ct.tc16_items.size();
+  a.nitems = count_of(cols);
   if (a.nitems == 0) return cudaSuccess;
-  const int grid = (int)std::min<long long>(a.nitems, h->nsm);
-  kern<<<grid, kThreads, smem, st>>>(mapA, mapT, a);
-  ++h->prof.launches;
-  return cudaGetLastError();
+  auto run = [&](auto kern, int stage_bytes, int per_sm) -> cudaError_t {
+    const int smem = kStages * stage_bytes + (int)sizeof(Bars) + 1024;
+    const cudaError_t e = allow_dynamic_smem((const void*)kern, smem);
+    if (e != cudaSuccess) return e;
+    const int grid = (int)std::min<long long>(a.nitems, (long long)per_sm * h->nsm);
+    kern<<<grid, kThreads, smem, st>>>(mapA, mapB, a);
+    ++h->prof.launches;
+    return cudaGetLastError();
+  };
+  return cols == 16 ? run(tc_precond16_kernel<16>, Shape<16>::kStageBytes, 2)
+                    : run(tc_precond16_kernel<64>, Shape<64>::kStageBytes, 1);
 }
 
 }  // namespace hps
