@@ -431,7 +431,7 @@ size_t hps_setup_bytes(const hps_grid* g, const hps_options* opt, int nrhs) {
   const long long nblk = (h.nf + 1023) / 1024;
   bytes += vb * (M1 + 5) + tsize * nrhs * c16 + (size_t)nrhs * nblk * M1 * c16 +
            (size_t)o.max_rhs * (h.nint + h.nf) * c16 + (size_t)nrhs * (3 * M1 + 4 * o.restart + 8) * c16 +
-           (size_t)nrhs * std::max<long long>(256, nblk) * sizeof(double);
+           (size_t)nrhs * std::max<long long>(256, 8 * nblk) * sizeof(double);
   // transient setup workspace (largest phase) + medium staging
   const size_t cap = workspace_cap(&h);
   size_t trans = exact_maps_workspace(&h, cap, nullptr);

@@ -67,6 +67,14 @@ struct VecArgs {
   int self_dot;      // mdot: also w^H w (= ||w||^2) in slot nvec
 };
 
+// Vectors [g0, g1) of this CTA: blockIdx.z splits the groups of kG vectors (the partial sums are
+// the same whatever the split).
+__device__ __forceinline__ void vector_range(int nv, int& g0, int& g1) {
+  const int groups = (nv + kG - 1) / kG, per = (groups + (int)gridDim.z - 1) / (int)gridDim.z;
+  g0 = (int)blockIdx.z * per * kG;
+  g1 = min(nv, g0 + per * kG);
+}
+
 // part = block partials of V_{0..nvec-1}^H w
 __global__ void __launch_bounds__(kT) mdot_kernel(VecArgs a) {
   const int rhs = blockIdx.y, blk = blockIdx.x;
@@ -80,8 +88,9 @@ __global__ void __launch_bounds__(kT) mdot_kernel(VecArgs a) {
     wv[e] = (i < a.nf) ? w[i] : make_double2(0.0, 0.0);
   }
   double2* out = a.part + ((long long)rhs * a.nblk + blk) * a.M1;
-  const int nv = a.nvec + a.self_dot;
-  for (int g0 = 0; g0 < nv; g0 += kG) {
+  int gb, nv;
+  vector_range(a.nvec + a.self_dot, gb, nv);
+  for (int g0 = gb; g0 < nv; g0 += kG) {
     const int ng = min(kG, nv - g0);
     double2 acc[kG];
 #pragma unroll
@@ -105,8 +114,8 @@ __global__ void __launch_bounds__(kT) mdot_kernel(VecArgs a) {
   }
 }
 
-// w -= V coef; then (mode 1) partial dots V^H w, or (mode 2) partial ||w||^2.
-__global__ void __launch_bounds__(kT) axpy_kernel(VecArgs a, int mode) {
+// w -= V coef, then partial dots V^H w.
+__global__ void __launch_bounds__(kT) axpy_dot_kernel(VecArgs a) {
   const int rhs = blockIdx.y, blk = blockIdx.x;
   if (a.active && !a.active[rhs]) return;
   __shared__ double2 cf[64];
@@ -140,37 +149,84 @@ __global__ void __launch_bounds__(kT) axpy_kernel(VecArgs a, int mode) {
     if (i < a.nf) w[i] = wv[e];
   }
   double2* out = a.part + ((long long)rhs * a.nblk + blk) * a.M1;
-  if (mode == 1) {
-    for (int g0 = 0; g0 < a.nvec; g0 += kG) {
-      const int ng = min(kG, a.nvec - g0);
-      double2 acc[kG];
-#pragma unroll
-      for (int g = 0; g < kG; ++g) acc[g] = make_double2(0.0, 0.0);
-#pragma unroll
-      for (int g = 0; g < kG; ++g) {
-        if (g < ng) {
-          const double2* v = a.V + ((long long)(g0 + g) * a.nrhs + rhs) * a.nf;
-#pragma unroll
-          for (int e = 0; e < kE; ++e) {
-            const long long i = base + (long long)e * kT;
-            if (i < a.nf) {
-              const double2 vv = v[i];
-              acc[g].x += vv.x * wv[e].x + vv.y * wv[e].y;
-              acc[g].y += vv.x * wv[e].y - vv.y * wv[e].x;
-            }
-          }
-        }
-      }
-      block_reduce_store(acc, ng, out + g0);
-    }
-  } else if (mode == 2) {
+  for (int g0 = 0; g0 < a.nvec; g0 += kG) {
+    const int ng = min(kG, a.nvec - g0);
     double2 acc[kG];
 #pragma unroll
     for (int g = 0; g < kG; ++g) acc[g] = make_double2(0.0, 0.0);
 #pragma unroll
-    for (int e = 0; e < kE; ++e) acc[0].x += wv[e].x * wv[e].x + wv[e].y * wv[e].y;
-    block_reduce_store(acc, 1, out);
+    for (int g = 0; g < kG; ++g) {
+      if (g < ng) {
+        const double2* v = a.V + ((long long)(g0 + g) * a.nrhs + rhs) * a.nf;
+#pragma unroll
+        for (int e = 0; e < kE; ++e) {
+          const long long i = base + (long long)e * kT;
+          if (i < a.nf) {
+            const double2 vv = v[i];
+            acc[g].x += vv.x * wv[e].x + vv.y * wv[e].y;
+            acc[g].y += vv.x * wv[e].y - vv.y * wv[e].x;
+          }
+        }
+      }
+    }
+    block_reduce_store(acc, ng, out + g0);
   }
+}
+
+// Sum of one double per thread over the block in a fixed order; the result is valid in thread 0.
+template <int T>
+__device__ __forceinline__ double block_sum(double v) {
+  __shared__ double red[T / 32];
+  v = warp_sum(v);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < T / 32; ++w) t += red[w];
+  return t;
+}
+
+// w -= V coef, then the block's partial of ||w||^2 into npart.  E entries per thread in blocks of T
+// threads: one entry per thread of small blocks where a vector is short, since the update runs at
+// the pace of the SMs that hold its blocks (FP64: 2 fused multiply-adds per SM and clock).
+template <int E, int T>
+__global__ void __launch_bounds__(T) axpy_norm_kernel(VecArgs a, double* npart) {
+  const int rhs = blockIdx.y;
+  if (a.active && !a.active[rhs]) return;
+  __shared__ double2 cf[64];
+  for (int j = threadIdx.x; j < a.nvec; j += T) cf[j] = a.coef[(long long)rhs * a.cstride + j];
+  __syncthreads();
+  const long long base = (long long)blockIdx.x * (E * T) + threadIdx.x;
+  double2* w = a.w + rhs * a.nf;
+  double2 wv[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const long long i = base + (long long)e * T;
+    wv[e] = (i < a.nf) ? w[i] : make_double2(0.0, 0.0);
+  }
+#pragma unroll(E == 1 ? 8 : 4)
+  for (int j = 0; j < a.nvec; ++j) {
+    const double2* v = a.V + ((long long)j * a.nrhs + rhs) * a.nf;
+    const double2 c = cf[j];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const long long i = base + (long long)e * T;
+      if (i < a.nf) {
+        const double2 vv = v[i];
+        wv[e].x -= c.x * vv.x - c.y * vv.y;
+        wv[e].y -= c.x * vv.y + c.y * vv.x;
+      }
+    }
+  }
+  double n2 = 0.0;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const long long i = base + (long long)e * T;
+    if (i < a.nf) w[i] = wv[e];
+    n2 += wv[e].x * wv[e].x + wv[e].y * wv[e].y;
+  }
+  n2 = block_sum<T>(n2);
+  if (threadIdx.x == 0) npart[(long long)rhs * gridDim.x + blockIdx.x] = n2;
 }
 
 // ---------------------------------------------------------------------------
@@ -217,41 +273,6 @@ __device__ __forceinline__ void conjdot_acc(acc2& re, acc2& im, dfc v, dfc w) {
   acc2_msub(im, v.im, w.re);
 }
 
-// Block sums of kG double-float complex partials per thread: the partials go
-// through shared memory transposed, so each thread finishes with one warp
-// reduction for the whole group.  Result per vector as complex double.
-__device__ __forceinline__ void block_reduce_store_df(dfc (&part)[kG], int ng, double2* out) {
-  __shared__ dfc red[kG][kT];
-  __shared__ dfc red2[kG][kT / 32 / kG > 0 ? kT / 32 / kG : 1];
-  static_assert(kT % (32 * kG) == 0, "block must split into kG groups of whole warps");
-  constexpr int kPer = kT / kG;  // threads per vector in the transposed sum
-  const int tid = threadIdx.x, lane = tid & 31;
-#pragma unroll
-  for (int g = 0; g < kG; ++g) red[g][tid] = part[g];
-  __syncthreads();
-  const int g = tid / kPer, k = tid % kPer;
-  dfc a = dfc_zero();
-#pragma unroll
-  for (int m = 0; m < kT / kPer; ++m) a = dfc_add(a, red[g][k + kPer * m]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    dfc other;
-    other.re.h = __shfl_xor_sync(0xffffffffu, a.re.h, o);
-    other.re.l = __shfl_xor_sync(0xffffffffu, a.re.l, o);
-    other.im.h = __shfl_xor_sync(0xffffffffu, a.im.h, o);
-    other.im.l = __shfl_xor_sync(0xffffffffu, a.im.l, o);
-    a = dfc_add(a, other);
-  }
-  if (lane == 0) red2[g][k / 32] = a;
-  __syncthreads();
-  if (k == 0 && g < ng) {
-    dfc t = red2[g][0];
-    for (int w = 1; w < kPer / 32; ++w) t = dfc_add(t, red2[g][w]);
-    out[g] = dfc_to_double2(t);
-  }
-  __syncthreads();
-}
-
 __device__ __forceinline__ dfc shfl_xor_dfc(dfc a, int o) {
   dfc r;
   r.re.h = __shfl_xor_sync(0xffffffffu, a.re.h, o);
@@ -281,15 +302,15 @@ __device__ __forceinline__ dfc warp_reduce_groups(const dfc (&part)[kG]) {
   return k;
 }
 
-// Partial dots V^H w of this block (one per basis vector, complex double; with nv = nvec + 1
+// Partial dots V_j^H w of this block for gb <= j < nv (complex double; with nv = nvec + 1
 // the last "basis vector" is w itself, giving ||w||^2): per group of kG vectors each warp
 // reduces its lanes' partials on its own; one barrier at the end sums the warps in order.
 // nv <= 64 (restart <= 60).
 __device__ __forceinline__ void df_dots(const DfArgs& a, int rhs, long long base, const dfc (&wv)[kE], double2* out,
-                                        int nv) {
+                                        int gb, int nv) {
   __shared__ dfc wred[kT / 32][64];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int g0 = 0; g0 < nv; g0 += kG) {
+  for (int g0 = gb; g0 < nv; g0 += kG) {
     const int ng = min(kG, nv - g0);
     dfc part[kG];
 #pragma unroll
@@ -313,7 +334,7 @@ __device__ __forceinline__ void df_dots(const DfArgs& a, int rhs, long long base
     if ((lane & 7) == 0 && (lane >> 3) < ng) wred[warp][g0 + (lane >> 3)] = sum;
   }
   __syncthreads();
-  for (int j = threadIdx.x; j < nv; j += kT) {
+  for (int j = gb + threadIdx.x; j < nv; j += kT) {
     dfc t = wred[0][j];
 #pragma unroll
     for (int w = 1; w < kT / 32; ++w) t = dfc_add(t, wred[w][j]);
@@ -332,11 +353,13 @@ __global__ void __launch_bounds__(kT, 4) mdot_df_kernel(DfArgs a) {
     const long long i = base + (long long)e * kT;
     wv[e] = (i < a.nf) ? dfc_load(w[i]) : dfc_zero();
   }
-  df_dots(a, rhs, base, wv, a.part + ((long long)rhs * a.nblk + blk) * a.M1, a.nvec + a.self_dot);
+  int g0, g1;
+  vector_range(a.nvec + a.self_dot, g0, g1);
+  df_dots(a, rhs, base, wv, a.part + ((long long)rhs * a.nblk + blk) * a.M1, g0, g1);
 }
 
-// w -= V coef; then (mode 1) partial dots V^H w, or (mode 2) partial ||w||^2.
-__global__ void __launch_bounds__(kT, 4) axpy_df_kernel(DfArgs a, int mode) {
+// w -= V coef, then partial dots V^H w.
+__global__ void __launch_bounds__(kT, 4) axpy_dot_df_kernel(DfArgs a) {
   const int rhs = blockIdx.y, blk = blockIdx.x;
   if (a.active && !a.active[rhs]) return;
   __shared__ dfc cf[64];
@@ -380,21 +403,59 @@ __global__ void __launch_bounds__(kT, 4) axpy_df_kernel(DfArgs a, int mode) {
     if (i < a.nf) w[i] = dfc_store(wv[e]);
   }
   double2* out = a.part + ((long long)rhs * a.nblk + blk) * a.M1;
-  if (mode == 1) {
-    df_dots(a, rhs, base, wv, out, a.nvec);
-  } else if (mode == 2) {
-    dfc part[kG];
+  df_dots(a, rhs, base, wv, out, 0, a.nvec);
+}
+
+// w -= V coef, then the block's partial of ||w||^2 (complex double) into npart; E, T as in
+// axpy_norm_kernel.
+template <int E, int T>
+__global__ void __launch_bounds__(T) axpy_norm_df_kernel(DfArgs a, double* npart) {
+  const int rhs = blockIdx.y;
+  if (a.active && !a.active[rhs]) return;
+  __shared__ dfc cf[64];
+  for (int j = threadIdx.x; j < a.nvec; j += T) cf[j] = dfc_from(a.coef[(long long)rhs * a.cstride + j]);
+  __syncthreads();
+  const long long base = (long long)blockIdx.x * (E * T) + threadIdx.x;
+  float4* w = a.w + rhs * a.nf;
+  acc2 wr[E], wi[E];
 #pragma unroll
-    for (int g = 0; g < kG; ++g) part[g] = dfc_zero();
-    acc2 n2{0.f, 0.f};
-#pragma unroll
-    for (int e = 0; e < kE; ++e) {
-      acc2_madd(n2, wv[e].re, wv[e].re);
-      acc2_madd(n2, wv[e].im, wv[e].im);
-    }
-    part[0].re = acc2_value(n2);
-    block_reduce_store_df(part, 1, out);
+  for (int e = 0; e < E; ++e) {
+    const long long i = base + (long long)e * T;
+    const dfc x = (i < a.nf) ? dfc_load(w[i]) : dfc_zero();
+    wr[e] = {x.re.h, x.re.l};
+    wi[e] = {x.im.h, x.im.l};
   }
+#pragma unroll(E == 1 ? 8 : 2)
+  for (int j = 0; j < a.nvec; ++j) {
+    const float4* v = a.V + ((long long)j * a.nrhs + rhs) * a.nf;
+    const dfc c = cf[j];
+    float4 vv[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const long long i = base + (long long)e * T;
+      vv[e] = (i < a.nf) ? v[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const dfc x = dfc_load(vv[e]);
+      // w -= c x:  re -= c.re x.re - c.im x.im,  im -= c.re x.im + c.im x.re
+      acc2_msub(wr[e], c.re, x.re);
+      acc2_madd(wr[e], c.im, x.im);
+      acc2_msub(wi[e], c.re, x.im);
+      acc2_msub(wi[e], c.im, x.re);
+    }
+  }
+  acc2 n2{0.f, 0.f};
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const dfc x = {acc2_value(wr[e]), acc2_value(wi[e])};
+    const long long i = base + (long long)e * T;
+    if (i < a.nf) w[i] = dfc_store(x);
+    acc2_madd(n2, x.re, x.re);
+    acc2_madd(n2, x.im, x.im);
+  }
+  const double n = block_sum<T>(df_to_double(acc2_value(n2)));
+  if (threadIdx.x == 0) npart[(long long)rhs * gridDim.x + blockIdx.x] = n;
 }
 
 // w <- w * invn[rhs] in double-float; c32 (if given) receives the result rounded to complex FP32
@@ -433,17 +494,20 @@ __global__ void combine_df_kernel(const float4* V, int nrhs, long long nf, const
   __syncthreads();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nf; i += (long long)gridDim.x * blockDim.x) {
     dfc s = dfc_zero();
+#pragma unroll 8
     for (int j = 0; j < kmax; ++j) s = dfc_add(s, dfc_mul(ys[j], dfc_load(V[((long long)j * nrhs + rhs) * nf + i])));
     u[rhs * nf + i] = dfc_to_double2(s);
   }
 }
 
-// out[rhs][i] (=|+=) sum over blocks of part[rhs][blk][i].  One CTA per
+// out[rhs][i] = sum over blocks of part[rhs][blk][i].  One CTA per
 // (i, rhs): thread t sums blocks t, t+256, ... in order, then a fixed shuffle
 // tree and a fixed sum over warps, so the result is the same on every run.
+// clear (optional): a word set to 0 (the step's any_active, which the kernels before have read).
 __global__ void __launch_bounds__(kT) reduce_kernel(const double2* part, int nblk, int M1, double2* out, int ostride,
-                                                    int accumulate, const int* active) {
+                                                    const int* active, int* clear) {
   const int i = blockIdx.x, rhs = blockIdx.y;
+  if (clear && i == 0 && rhs == 0 && threadIdx.x == 0) *clear = 0;
   if (active && !active[rhs]) return;
   const double2* p = part + (long long)rhs * nblk * M1 + i;
   double2 s = make_double2(0.0, 0.0);
@@ -456,16 +520,27 @@ __global__ void __launch_bounds__(kT) reduce_kernel(const double2* part, int nbl
   if (threadIdx.x == 0) {
     double2 t = red[0];
     for (int w = 1; w < kT / 32; ++w) t = cadd(t, red[w]);
-    double2* o = out + (long long)rhs * ostride + i;
-    *o = accumulate ? cadd(*o, t) : t;
+    out[(long long)rhs * ostride + i] = t;
   }
 }
 
-struct GivensArgs {
-  int nrhs, m, j, M1, nblk;
-  const double2* part;  // norm^2 partials in slot 0
-  double2* hcol;        // [rhs][M1+1]: h1 (CGS pass 1)
-  const double2* h2;    // [rhs][M1]: CGS pass 2
+// End of an Arnoldi step for one right-hand side (one CTA each): ||w'||^2 from the block
+// partials, the decision on a second Gram-Schmidt pass, and, unless that is still to come,
+// column j of the Hessenberg matrix with its Givens rotation.
+//
+// First (the one pass is over): classical Gram-Schmidt leaves w' orthogonal to V up to about
+// eps ||w|| / ||w'||, so a second pass is taken when the first cancelled most of w --
+// Rutishauser's criterion (1967), ||w'|| < ||w|| / 10, which bounds the loss of orthogonality per
+// step by ~10 eps.  (The stricter DGKS threshold 1/sqrt(2) would fire at every step here: w = A v_j
+// = v_j + Pi R v_j, and removing the v_j component alone takes about half of the energy.)
+// hcol[j+1] holds ||w||^2 from the dot pass.  Second: only right-hand sides that took the second
+// pass, whose coefficients h2 are added.  Always: both passes were made (cgs2).
+enum class Finish { First, Second, Always };
+struct FinishArgs {
+  int m, j, M1, nblk;
+  const double* npart;  // [rhs][nblk] partials of ||w'||^2
+  double2* hcol;        // [rhs][M1+1]: coefficients of the first pass
+  const double2* h2;    // [rhs][M1]: second pass
   double2* H;           // [rhs][M1][m]
   double* cs;           // [rhs][m]
   double2* sn;          // [rhs][m]
@@ -474,43 +549,59 @@ struct GivensArgs {
   double* invn;         // [rhs]
   int* active;          // [rhs]
   int* kcount;          // [rhs]
+  int* reorth;          // [rhs]
+  int* nreorth;
   const double* target; // [rhs]
   int* any_active;
 };
 
-// Finish column j of the Hessenberg matrix, apply the previous rotations, make
-// the new one, update g.  One block of 64 threads per right-hand side: the new
-// column and the stored rotations are staged in shared memory in parallel,
-// thread 0 applies the rotations (a dependent chain) there, and the column is
-// written back in parallel.  Requires m + 1 < 64 (restart <= 60).
-__global__ void givens_kernel(GivensArgs a) {
-  const int rhs = blockIdx.x;
-  if (rhs >= a.nrhs || !a.active[rhs]) return;
+// The new column and the stored rotations are staged in shared memory in parallel, thread 0
+// applies the rotations (a dependent chain) there, and the column is written back in parallel.
+// Requires m + 1 < 64 (restart <= 60).
+template <Finish F>
+__global__ void __launch_bounds__(kT) finish_kernel(FinishArgs a) {
+  const int rhs = blockIdx.x, j = a.j, t = threadIdx.x;
+  if (F == Finish::Second ? !a.reorth[rhs] : !a.active[rhs]) {
+    if (F == Finish::First && t == 0) a.reorth[rhs] = 0;
+    return;
+  }
   __shared__ double2 col[64];
   __shared__ double csv[64];
   __shared__ double2 snv[64];
-  const int j = a.j, t = threadIdx.x;
+  __shared__ int again;
   const double2* hc = a.hcol + (long long)rhs * (a.M1 + 1);
   const double2* h2 = a.h2 + (long long)rhs * a.M1;
   double* cs = a.cs + (long long)rhs * a.m;
   double2* sn = a.sn + (long long)rhs * a.m;
-  if (t <= j) col[t] = cadd(hc[t], h2[t]);
+  double n2 = 0.0;
+  for (int b = t; b < a.nblk; b += kT) n2 += a.npart[(long long)rhs * a.nblk + b];
+  if (t <= j) col[t] = F == Finish::First ? hc[t] : cadd(hc[t], h2[t]);
   if (t < j) {
     csv[t] = cs[t];
     snv[t] = sn[t];
   }
-  __syncthreads();
+  n2 = block_sum<kT>(n2);
   if (t == 0) {
-    // ||w||^2 was reduced into the spare last slot of hcol
-    const double hn = sqrt(hc[a.M1].x);
-    col[j + 1] = make_double2(hn, 0.0);
+    again = 0;
+    if (F == Finish::First) {
+      again = n2 < 0.01 * hc[j + 1].x;
+      a.reorth[rhs] = again;
+      if (again) atomicAdd(a.nreorth, 1);
+    }
+  }
+  __syncthreads();
+  if (again) return;
+  if (t == 0) {
+    const double hn = sqrt(n2);
+    // the rotations in registers: x carries the entry that the next rotation needs
+    double2 x = col[0];
     for (int i = 0; i < j; ++i) {
-      const double2 x = col[i], y = col[i + 1];
+      const double2 y = col[i + 1];
       col[i] = cadd(cscale(x, csv[i]), cmul(snv[i], y));
       const double2 sc = make_double2(snv[i].x, -snv[i].y);
-      col[i + 1] = csub(cscale(y, csv[i]), cmul(sc, x));
+      x = csub(cscale(y, csv[i]), cmul(sc, x));
     }
-    const double2 x = col[j], y = col[j + 1];
+    const double2 y = make_double2(hn, 0.0);
     const double ax = sqrt(cabs2(x)), den = sqrt(cabs2(x) + cabs2(y));
     double c;
     double2 sv;
@@ -528,9 +619,10 @@ __global__ void givens_kernel(GivensArgs a) {
     col[j + 1] = make_double2(0.0, 0.0);
     double2* g = a.g + (long long)rhs * a.M1;
     const double2 gj = g[j];
-    g[j + 1] = make_double2(-(sv.x * gj.x + sv.y * gj.y), -(sv.x * gj.y - sv.y * gj.x));  // -conj(s) g_j
+    const double2 gn = make_double2(-(sv.x * gj.x + sv.y * gj.y), -(sv.x * gj.y - sv.y * gj.x));  // -conj(s) g_j
+    g[j + 1] = gn;
     g[j] = cscale(gj, c);
-    const double e = sqrt(cabs2(g[j + 1]));
+    const double e = sqrt(cabs2(gn));
     a.est[rhs] = e;
     a.kcount[rhs] = j + 1;
     const bool breakdown = !(hn > 1e-300 * fmax(1.0, den));
@@ -564,20 +656,31 @@ __global__ void scale_copy_kernel(const double2* src, double2* dst, long long nf
     dst[rhs * nf + i] = cscale(src[rhs * nf + i], s);
 }
 
-// y = H(0:k,0:k)^{-1} g(0:k) per rhs (upper triangular after the rotations).
-__global__ void lsq_kernel(int nrhs, int m, int M1, const double2* H, const double2* g, const int* kcount, double2* y) {
-  const int rhs = blockIdx.x * blockDim.x + threadIdx.x;
-  if (rhs >= nrhs) return;
+// y = H(0:k,0:k)^{-1} g(0:k) per rhs (upper triangular after the rotations): column by column
+// from the last, thread l holding row l's remaining right-hand side.  One thread per right-hand
+// side (k^2 / 2 dependent steps through global memory) took 400 us at k = 50.
+__global__ void __launch_bounds__(64) lsq_kernel(int m, int M1, const double2* H, const double2* g, const int* kcount,
+                                                 double2* y) {
+  const int rhs = blockIdx.x, l = threadIdx.x;
   const int k = kcount[rhs];
   const double2* Hc = H + (long long)rhs * M1 * m;
-  double2* yr = y + (long long)rhs * m;
-  for (int i = 0; i < m; ++i) yr[i] = make_double2(0.0, 0.0);
-  for (int i = k - 1; i >= 0; --i) {
-    double2 s = g[(long long)rhs * M1 + i];
-    for (int l = i + 1; l < k; ++l) s = csub(s, cmul(Hc[i * m + l], yr[l]));
-    const double2 d = Hc[i * m + i];
-    yr[i] = (d.x == 0.0 && d.y == 0.0) ? make_double2(0.0, 0.0) : cmul(s, cinv(d));
+  __shared__ double2 ys[64];
+  double2 s = make_double2(0.0, 0.0), dinv = s, h = s;
+  if (l < k) {
+    s = g[(long long)rhs * M1 + l];
+    const double2 d = Hc[l * m + l];
+    if (d.x != 0.0 || d.y != 0.0) dinv = cinv(d);
+    if (l < k - 1) h = Hc[l * m + k - 1];
   }
+  for (int i = k - 1; i >= 0; --i) {
+    const double2 next = (l < i - 1) ? Hc[l * m + i - 1] : make_double2(0.0, 0.0);
+    if (l == i) ys[i] = cmul(s, dinv);
+    __syncthreads();
+    if (l < i) s = csub(s, cmul(h, ys[i]));
+    h = next;
+  }
+  __syncthreads();
+  if (l < m) y[(long long)rhs * m + l] = l < k ? ys[l] : make_double2(0.0, 0.0);
 }
 
 // u = sum_{j<kmax} y_j v_j, kmax = kcount[rhs]
@@ -590,6 +693,7 @@ __global__ void combine_kernel(const double2* V, int nrhs, long long nf, const i
   __syncthreads();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nf; i += (long long)gridDim.x * blockDim.x) {
     double2 s = make_double2(0.0, 0.0);
+#pragma unroll 8
     for (int j = 0; j < kmax; ++j) {
       const double2 v = V[((long long)j * nrhs + rhs) * nf + i];
       cfma(s, ys[j], v);
@@ -602,26 +706,6 @@ template <class T>
 __global__ void xpy_kernel(double2* x, const T* z, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     x[i] = cadd(x[i], cvt<double2>(z[i]));
-}
-
-// Second Gram-Schmidt pass only where needed: after one classical pass w' = w - V h, the
-// computed w' is orthogonal to V up to about eps ||w|| / ||w'||, so a second pass is taken when
-// the first cancelled most of w -- Rutishauser's criterion (1967), ||w'|| < ||w|| / 10, which
-// bounds the loss of orthogonality per step by ~10 eps.  (The stricter DGKS threshold 1/sqrt(2)
-// would fire at every step here: w = A v_j = v_j + Pi R v_j, and removing the v_j component
-// alone takes about half of the energy.)  hcol[j+1] holds ||w||^2 (from the first dot pass),
-// hcol[M1] ||w'||^2.  Steps that skip the second pass get h2 = 0.
-__global__ void reorth_kernel(int nrhs, int j, int M1, const double2* hcol, const int* active, int* reorth, double2* h2,
-                            int* nreorth) {
-  const int rhs = blockIdx.x * blockDim.x + threadIdx.x;
-  if (rhs >= nrhs) return;
-  const double2* hc = hcol + (long long)rhs * (M1 + 1);
-  const bool act = active[rhs] != 0;
-  const bool need = act && hc[M1].x < 0.01 * hc[j + 1].x;
-  reorth[rhs] = need ? 1 : 0;
-  if (need) atomicAdd(nreorth, 1);
-  else if (act)
-    for (int t = 0; t <= j; ++t) h2[(long long)rhs * M1 + t] = make_double2(0.0, 0.0);
 }
 
 // norms[rhs] = ||x_rhs||_2 from block partials
@@ -699,7 +783,7 @@ int krylov_alloc(hps_handle* h, int nrhs, long long nvec) {
   if ((rc = alloc((void**)&k.sn, (size_t)nrhs * m * sizeof(double2)))) return rc;
   if ((rc = alloc((void**)&k.g, (size_t)nrhs * M1 * sizeof(double2)))) return rc;
   if ((rc = alloc((void**)&k.est, (size_t)nrhs * 4 * sizeof(double)))) return rc;  // est, invn, target, norms
-  if ((rc = alloc((void**)&k.nrm, (size_t)nrhs * std::max(256, k.nblk) * sizeof(double)))) return rc;
+  if ((rc = alloc((void**)&k.nrm, (size_t)nrhs * std::max(256, 8 * k.nblk) * sizeof(double)))) return rc;
   // active[nrhs], kcount[nrhs], any_active, status, reorth[nrhs], nreorth
   if ((rc = alloc((void**)&k.active, (size_t)(3 * nrhs + 3) * sizeof(int)))) return rc;
   k.status = k.active + 2 * nrhs + 1;
@@ -833,74 +917,89 @@ int gmres_core(hps_handle* h, const GmresOps& ops, bool mixed, const double2* b,
     da.active = active;
     da.self_dot = 0;
     const dim3 bgrid(k.nblk, nrhs);
+    // dots: the vectors split over more CTAs where the blocks of one vector leave SMs idle (4 CTAs
+    // per SM wanted); update: one entry per thread there
+    const int zmax = std::max(1, (int)std::min<long long>(16, 4LL * h->nsm / std::max<long long>(1, (long long)k.nblk * nrhs)));
+    const bool fine = (long long)k.nblk * nrhs < 4LL * h->nsm;
+    constexpr int kFineT = 128;
+    const int nblk_axpy = fine ? (int)((nf + kFineT - 1) / kFineT) : k.nblk;
     auto mdot = [&](const int* act, int self) {
       va.active = da.active = act;
       va.self_dot = da.self_dot = self;
-      if (mixed) mdot_df_kernel<<<bgrid, kT, 0, s>>>(da);
-      else mdot_kernel<<<bgrid, kT, 0, s>>>(va);
+      const dim3 grid(k.nblk, nrhs, std::min(zmax, (j + 1 + self + kG - 1) / kG));
+      if (mixed) mdot_df_kernel<<<grid, kT, 0, s>>>(da);
+      else mdot_kernel<<<grid, kT, 0, s>>>(va);
       va.self_dot = da.self_dot = 0;
     };
-    auto axpy = [&](const int* act, const double2* coef, int cstride, int mode) {
+    auto set_coef = [&](const int* act, const double2* coef, int cstride) {
       va.active = da.active = act;
       va.coef = da.coef = coef;
       va.cstride = da.cstride = cstride;
-      if (mixed) axpy_df_kernel<<<bgrid, kT, 0, s>>>(da, mode);
-      else axpy_kernel<<<bgrid, kT, 0, s>>>(va, mode);
     };
-    auto reduce = [&](int n, double2* out, int ostride, const int* act) {
-      reduce_kernel<<<dim3(n, nrhs), kT, 0, s>>>(k.part, k.nblk, M1, out, ostride, 0, act);
+    auto axpy_norm = [&](const int* act, const double2* coef, int cstride) {
+      set_coef(act, coef, cstride);
+      const dim3 grid(nblk_axpy, nrhs);
+      if (mixed) {
+        if (fine) axpy_norm_df_kernel<1, kFineT><<<grid, kFineT, 0, s>>>(da, k.nrm);
+        else axpy_norm_df_kernel<kE, kT><<<grid, kT, 0, s>>>(da, k.nrm);
+      } else {
+        if (fine) axpy_norm_kernel<1, kFineT><<<grid, kFineT, 0, s>>>(va, k.nrm);
+        else axpy_norm_kernel<kE, kT><<<grid, kT, 0, s>>>(va, k.nrm);
+      }
     };
+    auto reduce = [&](int n, double2* out, int ostride, const int* act, int* clear) {
+      reduce_kernel<<<dim3(n, nrhs), kT, 0, s>>>(k.part, k.nblk, M1, out, ostride, act, clear);
+    };
+    FinishArgs fa;
+    fa.m = m;
+    fa.j = j;
+    fa.M1 = M1;
+    fa.nblk = nblk_axpy;
+    fa.npart = k.nrm;
+    fa.hcol = k.hcol;
+    fa.h2 = h2;
+    fa.H = k.H;
+    fa.cs = k.cs;
+    fa.sn = k.sn;
+    fa.g = k.g;
+    fa.est = est;
+    fa.invn = invn;
+    fa.active = active;
+    fa.kcount = kcount;
+    fa.reorth = reorth;
+    fa.nreorth = nreorth;
+    fa.target = target;
+    fa.any_active = any_active;
     cudaEvent_t ev_arn = h->prof.begin(s);
     if (cgs2) {
       // classical Gram-Schmidt twice: dots; update + dots; update + norm
       mdot(active, 0);
-      reduce(j + 1, k.hcol, M1 + 1, active);
-      axpy(active, k.hcol, M1 + 1, 1);
-      reduce(j + 1, h2, M1, active);
-      axpy(active, h2, M1, 2);
-      reduce(1, k.hcol + M1, M1 + 1, active);
+      reduce(j + 1, k.hcol, M1 + 1, active, any_active);
+      set_coef(active, k.hcol, M1 + 1);
+      if (mixed) axpy_dot_df_kernel<<<bgrid, kT, 0, s>>>(da);
+      else axpy_dot_kernel<<<bgrid, kT, 0, s>>>(va);
+      reduce(j + 1, h2, M1, active, nullptr);
+      axpy_norm(active, h2, M1);
+      finish_kernel<Finish::Always><<<nrhs, kT, 0, s>>>(fa);
       h->prof.launches += 6;
     } else {
       // one pass (dots and ||w||^2; update + norm), the second only where the norm test asks
       mdot(active, 1);
-      reduce(j + 2, k.hcol, M1 + 1, active);
-      axpy(active, k.hcol, M1 + 1, 2);
-      reduce(1, k.hcol + M1, M1 + 1, active);
-      reorth_kernel<<<(nrhs + 63) / 64, 64, 0, s>>>(nrhs, j, M1, k.hcol, active, reorth, h2, nreorth);
+      reduce(j + 2, k.hcol, M1 + 1, active, any_active);
+      axpy_norm(active, k.hcol, M1 + 1);
+      finish_kernel<Finish::First><<<nrhs, kT, 0, s>>>(fa);
       mdot(reorth, 0);
-      reduce(j + 1, h2, M1, reorth);
-      axpy(reorth, h2, M1, 2);
-      reduce(1, k.hcol + M1, M1 + 1, reorth);
-      h->prof.launches += 9;
+      reduce(j + 1, h2, M1, reorth, nullptr);
+      axpy_norm(reorth, h2, M1);
+      finish_kernel<Finish::Second><<<nrhs, kT, 0, s>>>(fa);
+      h->prof.launches += 8;
     }
-    HPS_CUDA_TRY(cudaGetLastError());
-    HPS_CUDA_TRY(cudaMemsetAsync(any_active, 0, sizeof(int), s));
-    GivensArgs ga;
-    ga.nrhs = nrhs;
-    ga.m = m;
-    ga.j = j;
-    ga.M1 = M1;
-    ga.nblk = k.nblk;
-    ga.part = k.part;
-    ga.hcol = k.hcol;
-    ga.h2 = h2;
-    ga.H = k.H;
-    ga.cs = k.cs;
-    ga.sn = k.sn;
-    ga.g = k.g;
-    ga.est = est;
-    ga.invn = invn;
-    ga.active = active;
-    ga.kcount = kcount;
-    ga.target = target;
-    ga.any_active = any_active;
-    givens_kernel<<<nrhs, 64, 0, s>>>(ga);
     HPS_CUDA_TRY(cudaGetLastError());
     if (mixed) scale_df_kernel<<<vgrid, 256, 0, s>>>((float4*)w, nf, invn, vc32, active);
     else scale_kernel<<<vgrid, 256, 0, s>>>(w, nf, nrhs, invn, active);
     HPS_CUDA_TRY(cudaGetLastError());
     h->prof.end(HPS_PHASE_ARNOLDI, ev_arn, s);
-    h->prof.launches += 2;
+    h->prof.launches += 1;
     h->prof.step = -1;
     return HPS_OK;
   };
@@ -1029,7 +1128,7 @@ int gmres_core(hps_handle* h, const GmresOps& ops, bool mixed, const double2* b,
     }
     // x += M^{-1} (V y)
     cudaEvent_t ev_up = h->prof.begin(st);
-    lsq_kernel<<<(nrhs + 31) / 32, 32, 0, st>>>(nrhs, m, M1, k.H, k.g, kcount, k.y);
+    lsq_kernel<<<nrhs, 64, 0, st>>>(m, M1, k.H, k.g, kcount, k.y);
     HPS_CUDA_TRY(cudaGetLastError());
     if (mixed) combine_df_kernel<<<vgrid, 256, 0, st>>>((const float4*)k.V, nrhs, nf, kcount, m, k.y, k.u);
     else combine_kernel<<<vgrid, 256, 0, st>>>(k.V, nrhs, nf, kcount, m, k.y, k.u);
