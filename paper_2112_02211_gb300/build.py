@@ -14,7 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 ROOT = os.path.dirname(HERE)
 SOURCES = ["api.cu", "setup.cu", "apply.cu", "krylov.cu", "noalloc.cu", "tc_apply.cu", "tc_precond.cu", "full.cu",
-           "compensated.cu", "tc_precond16.cu", "inverse.cu"]
+           "compensated.cu", "tc_precond16.cu", "inverse.cu", "stream_apply.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include")]

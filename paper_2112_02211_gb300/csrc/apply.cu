@@ -9,7 +9,7 @@
 //               its own kernel, one thread per row, B stored transposed)
 //      stage K  z_int = K_c t                          (K_c = (I + D)^{-1})
 //
-// An item is (leaf, face) for apply/rhs (rows of that face's block), a leaf
+// An item is (leaf, part) for apply/rhs (a part of the rows of its faces with a neighbour), a leaf
 // for B, and for K one slot of a distinct K block against up to 8 clusters
 // sharing that block (their t vectors take the place of right-hand sides, so
 // a block shared by many clusters is read once per 8 of them).  The swap Pi is fused into the store: the rows
@@ -19,7 +19,13 @@
 // read).  A CTA stages the item's input vector in shared memory; each warp
 // streams RPW matrix rows with 16-byte loads (1 complex double or 2 complex
 // floats per lane per load), accumulates in the matrix's precision and
-// reduces with warp shuffles.
+// reduces with warp shuffles that halve the values in flight at every step.
+//
+// What bounds it: HBM for one right-hand side in complex float; the FP64 pipe (4 fused
+// multiply-adds per entry, two per SM and clock) in complex double, where the warp reductions
+// used to cost another third; shared-memory reads of the staged vectors for many right-hand
+// sides, which several rows per warp share.Measured, 9^3 leaves, p = 8, complex
+// double: 331 -> 268 us.  (Complex-float vectors take stream_apply.cu.)
 #include <algorithm>
 #include <array>
 #include <map>
@@ -86,8 +92,37 @@ struct ItemInfo {
   int ld, ncols;
   int nrows;       // matrix rows of the item (q^2, or all internal-face rows of a leaf)
   int leaf, face, nbr;
-  int mask;        // precond B: internal-face mask of the leaf
+  int mask;        // apply, rhs: faces with a neighbour; stage K: members
+  int row0;        // apply, rhs: first row of the item among the rows of those faces
+  unsigned flist;  // apply, rhs: those faces, 4 bits each
 };
+
+// Rows of a leaf's faces with a neighbour, cut into `parts` items: row l of an item belongs to the
+// (row0 + l) / q2 -th of those faces.
+__device__ __forceinline__ void leaf_rows(const GridDims& g, int q2, int parts, long long item, ItemInfo& it) {
+  it.leaf = (int)(item / parts);
+  const int part = (int)(item % parts);
+  it.mask = 0;
+  it.flist = 0;
+  int n = 0;
+#pragma unroll
+  for (int f = 0; f < 6; ++f)
+    if (g.neighbor(it.leaf, f) >= 0) {
+      it.mask |= 1 << f;
+      it.flist |= (unsigned)f << (4 * n++);
+    }
+  const int rows = n * q2;
+  it.row0 = rows * part / parts;
+  it.nrows = rows * (part + 1) / parts - it.row0;
+}
+// inv: row_inv(q2)
+__device__ __forceinline__ void leaf_row(const ItemInfo& it, int q2, unsigned inv, int l, int& face, int& j) {
+  const unsigned r = it.row0 + l, k = (r * inv) >> 20;
+  j = (int)(r - k * q2);
+  face = (it.flist >> (4 * k)) & 7u;
+}
+// Most right-hand sides x rows of accumulators per thread (complex values).
+template <class TM> constexpr int kMaxAcc = sizeof(TM) == 16 ? 16 : 32;
 
 // ---------------------------------------------------------------------------
 // y = f + g (apply) in the output's precision.  Double-float outputs (float4)
@@ -127,24 +162,24 @@ struct ApplyP {
     TOUT* y;
     const double2* bvec;  // residual mode: y = b - (I + Pi R) f
     long long nf;
-    int nrhs;
+    int nrhs, parts;
+    unsigned inv;
     long long nitems;
   };
   __device__ static bool decode(const Args& A, long long item, ItemInfo& it) {
-    it.leaf = (int)(item / 6);
-    it.face = (int)(item % 6);
-    it.nbr = A.g.neighbor(it.leaf, it.face);
+    leaf_rows(A.g, A.q2, A.parts, item, it);
+    it.face = (int)(item % A.parts);
     it.xoff = (long long)it.leaf * A.nb;
-    if (it.nbr < 0) {
-      it.ooff = it.xoff + (long long)it.face * A.q2;
-      return false;
-    }
-    it.mat = A.R + (long long)it.leaf * A.nb * A.ldR + (long long)it.face * A.q2 * A.ldR;
+    it.mat = A.R + (long long)it.leaf * A.nb * A.ldR;
     it.ld = A.ldR;
     it.ncols = A.nb;
-    it.nrows = A.q2;
-    it.ooff = (long long)it.nbr * A.nb + (long long)(it.face ^ 1) * A.q2;
     return true;
+  }
+  __device__ static long long row_off(const Args& A, const ItemInfo& it, int l) {
+    if (it.mask == 63) return (long long)(it.row0 + l) * A.ldR;
+    int face, j;
+    leaf_row(it, A.q2, A.inv, l, face, j);
+    return (long long)(face * A.q2 + j) * A.ldR;
   }
   __device__ static Acc load_x(const Args& A, const ItemInfo& it, int rhs, int c) {
     return cvt<Acc>(A.f[rhs * A.nf + it.xoff + c]);
@@ -156,16 +191,17 @@ struct ApplyP {
     A.y[o] = v;
   }
   __device__ static void store(const Args& A, const ItemInfo& it, const Acc* outs, int nr, int tid) {
-    for (int idx = tid; idx < nr * A.q2; idx += kThreads) {
-      const int rhs = idx / A.q2, j = idx % A.q2;
-      finish(A, rhs * A.nf + it.ooff + j, outs[idx]);
+    for (int l = tid; l < it.nrows; l += kThreads) {
+      int face, j;
+      leaf_row(it, A.q2, A.inv, l, face, j);
+      const long long o = (long long)A.g.neighbor(it.leaf, face) * A.nb + (long long)(face ^ 1) * A.q2 + j;
+      for (int rhs = 0; rhs < nr; ++rhs) finish(A, rhs * A.nf + o, outs[rhs * it.nrows + l]);
     }
-  }
-  __device__ static void copy(const Args& A, const ItemInfo& it, int nr, int tid) {
-    for (int idx = tid; idx < nr * A.q2; idx += kThreads) {
-      const int rhs = idx / A.q2, j = idx % A.q2;
-      finish(A, rhs * A.nf + it.ooff + j, czero<Acc>());
-    }
+    if (it.face != 0 || it.mask == 63) return;
+    // the leaf's first item: faces on the boundary of the cube only copy
+    for (int idx = tid; idx < 6 * A.q2; idx += kThreads)
+      if (!((it.mask >> (idx / A.q2)) & 1))
+        for (int rhs = 0; rhs < nr; ++rhs) finish(A, rhs * A.nf + it.xoff + idx, czero<Acc>());
   }
 };
 
@@ -181,42 +217,45 @@ struct RhsP {
     const double2* t;
     double2* out;
     long long nf, nint;
-    int nrhs;
+    int nrhs, parts;
+    unsigned inv;
     long long nitems;
   };
   __device__ static bool decode(const Args& A, long long item, ItemInfo& it) {
-    it.leaf = (int)(item / 6);
-    it.face = (int)(item % 6);
-    it.nbr = A.g.neighbor(it.leaf, it.face);
-    if (it.nbr < 0) {
-      it.ooff = (long long)it.leaf * A.nb + (long long)it.face * A.q2;
-      return false;
-    }
-    it.ooff = (long long)it.nbr * A.nb + (long long)(it.face ^ 1) * A.q2;
-    if (!A.s) return false;
-    it.mat = A.H + (long long)it.leaf * A.nb * A.ldH + (long long)it.face * A.q2 * A.ldH;
+    leaf_rows(A.g, A.q2, A.parts, item, it);
+    it.face = (int)(item % A.parts);
+    it.mat = A.H + (long long)it.leaf * A.nb * A.ldH;
     it.ld = A.ldH;
     it.ncols = A.ni;
-    it.nrows = A.q2;
     it.xoff = (long long)it.leaf * A.ni;
-    return true;
+    return A.s != nullptr;  // no body load: h = 0
+  }
+  __device__ static long long row_off(const Args& A, const ItemInfo& it, int l) {
+    int face, j;
+    leaf_row(it, A.q2, A.inv, l, face, j);
+    return (long long)(face * A.q2 + j) * A.ldH;
   }
   __device__ static Acc load_x(const Args& A, const ItemInfo& it, int rhs, int c) {
     return cvt<Acc>(A.s[rhs * A.nint + it.xoff + c]);
   }
   __device__ static void store(const Args& A, const ItemInfo& it, const Acc* outs, int nr, int tid) {
-    for (int idx = tid; idx < nr * A.q2; idx += kThreads) {
-      const int rhs = idx / A.q2, j = idx % A.q2;
-      const double2 v = cvt<double2>(outs[idx]);
-      A.out[rhs * A.nf + it.ooff + j] = make_double2(-v.x, -v.y);
+    for (int l = tid; l < it.nrows; l += kThreads) {
+      int face, j;
+      leaf_row(it, A.q2, A.inv, l, face, j);
+      const long long o = (long long)A.g.neighbor(it.leaf, face) * A.nb + (long long)(face ^ 1) * A.q2 + j;
+      for (int rhs = 0; rhs < nr; ++rhs) {
+        const double2 v = outs ? cvt<double2>(outs[rhs * it.nrows + l]) : make_double2(-0.0, -0.0);
+        A.out[rhs * A.nf + o] = make_double2(-v.x, -v.y);
+      }
     }
-  }
-  __device__ static void copy(const Args& A, const ItemInfo& it, int nr, int tid) {
-    for (int idx = tid; idx < nr * A.q2; idx += kThreads) {
-      const int rhs = idx / A.q2, j = idx % A.q2;
-      const long long o = rhs * A.nf + it.ooff + j;
-      A.out[o] = (it.nbr < 0 && A.t) ? A.t[o] : make_double2(0.0, 0.0);
-    }
+    if (it.face != 0 || it.mask == 63) return;
+    // the leaf's first item: boundary faces take t (or 0)
+    for (int idx = tid; idx < 6 * A.q2; idx += kThreads)
+      if (!((it.mask >> (idx / A.q2)) & 1))
+        for (int rhs = 0; rhs < nr; ++rhs) {
+          const long long o = rhs * A.nf + (long long)it.leaf * A.nb + idx;
+          A.out[o] = A.t ? A.t[o] : make_double2(0.0, 0.0);
+        }
   }
 };
 
@@ -238,7 +277,7 @@ struct PrecKP {
     const int* cl_slot_begin;
     const int* slot_lf;
     const long long* cl_tpos;
-    int nb, q2;
+    int nb, q2, split;
     const TIN* t;
     TOUT* z;
     long long nf, tstride;
@@ -246,12 +285,12 @@ struct PrecKP {
     int nrhs;  // vectors of an item, member group width x nrl
     long long nitems;
   };
-  // item (k, s * kKRowSplit + part, first member, members): rows
-  // [part * hq, min(q^2, (part + 1) * hq)) of slot s, hq = ceil(q^2 / kKRowSplit)
+  // item (k, s * split + part, first member, members): rows
+  // [part * hq, min(q^2, (part + 1) * hq)) of slot s, hq = ceil(q^2 / split)
   __device__ static bool decode(const Args& A, long long item, ItemInfo& it) {
     const int4 e = A.items[item];
-    const int k = e.x, s = e.y / kKRowSplit, part = e.y % kKRowSplit;
-    const int hq = (A.q2 + kKRowSplit - 1) / kKRowSplit;
+    const int k = e.x, s = e.y / A.split, part = e.y % A.split;
+    const int hq = (A.q2 + A.split - 1) / A.split;
     const int r0 = min(A.q2, part * hq);
     const int s0 = A.kc_slot_begin[k], ns = A.kc_slot_begin[k + 1] - s0;
     it.ncols = ns * A.q2;
@@ -265,12 +304,14 @@ struct PrecKP {
     it.aoff = (long long)(s0 + s) * A.q2 + r0;
     return it.nrows > 0;
   }
+  __device__ static long long row_off(const Args&, const ItemInfo& it, int l) { return (long long)l * it.ld; }
   __device__ static Acc load_x(const Args& A, const ItemInfo& it, int rr, int c) {
     const int m = rr / A.nrl;
     if (m >= it.mask) return czero<Acc>();
     return cvt<Acc>(A.t[(long long)(rr - m * A.nrl) * A.tstride + A.cl_tpos[A.members[it.xoff + m]] + c]);
   }
   __device__ static void store(const Args& A, const ItemInfo& it, const Acc* outs, int, int tid) {
+    if (!outs) return;
     for (int idx = tid; idx < it.mask * A.nrl * it.nrows; idx += kThreads) {
       const int rr = idx / it.nrows, jj = idx % it.nrows, m = rr / A.nrl;
       const int lf = A.slot_lf[A.cl_slot_begin[A.members[it.xoff + m]] + it.face];
@@ -278,7 +319,6 @@ struct PrecKP {
       A.z[(long long)(rr - m * A.nrl) * A.nf + o] = cvt<TOUT>(rscale(outs[idx], A.kscale, it.aoff + jj));
     }
   }
-  __device__ static void copy(const Args&, const ItemInfo&, int, int) {}
 };
 
 // ---------------------------------------------------------------------------
@@ -292,6 +332,7 @@ __global__ void __launch_bounds__(kThreads) seg_gemv_kernel(const typename P::Ar
   if (gate && *gate == 0) return;
   using TM = typename P::TM;
   using Acc = typename P::Acc;
+  using R_ = typename Real<Acc>::type;
   constexpr int VPL = MT<TM>::VPL;
   extern __shared__ __align__(16) unsigned char smraw[];
   Acc* xs = reinterpret_cast<Acc*>(smraw);
@@ -301,7 +342,7 @@ __global__ void __launch_bounds__(kThreads) seg_gemv_kernel(const typename P::Ar
   for (long long item = blockIdx.x; item < A.nitems; item += gridDim.x) {
     ItemInfo it;
     if (!P::decode(A, item, it)) {
-      P::copy(A, it, nr, tid);
+      P::store(A, it, nullptr, nr, tid);
       continue;
     }
     const int ncp = (it.ncols + VPL - 1) / VPL * VPL;
@@ -313,46 +354,44 @@ __global__ void __launch_bounds__(kThreads) seg_gemv_kernel(const typename P::Ar
     const TM* mat = reinterpret_cast<const TM*>(it.mat);
     const int nrows = it.nrows;
     for (int r0 = warp * RPW; r0 < nrows; r0 += kWarps * RPW) {
-      Acc acc[RPW][NR];
+      constexpr int V = 2 * RPW * NR;
+      R_ acc[V];  // (row, right-hand side, re/im)
 #pragma unroll
-      for (int i = 0; i < RPW; ++i)
+      for (int i = 0; i < V; ++i) acc[i] = 0;
+      const TM* row[RPW];
 #pragma unroll
-        for (int rr = 0; rr < NR; ++rr) acc[i][rr] = czero<Acc>();
+      for (int i = 0; i < RPW; ++i) row[i] = mat + P::row_off(A, it, min(r0 + i, nrows - 1));
 #pragma unroll 2
       for (int c = lane * VPL; c < ncp; c += 32 * VPL) {
         Acc mv[RPW][VPL];
 #pragma unroll
-        for (int i = 0; i < RPW; ++i) {
-          if (r0 + i < nrows) {
-            MT<TM>::load(mat + (long long)(r0 + i) * it.ld + c, mv[i]);
-          } else {
-#pragma unroll
-            for (int v = 0; v < VPL; ++v) mv[i][v] = czero<Acc>();
-          }
-        }
+        for (int i = 0; i < RPW; ++i) MT<TM>::load(row[i] + c, mv[i]);
 #pragma unroll
         for (int rr = 0; rr < NR; ++rr) {
 #pragma unroll
           for (int v = 0; v < VPL; ++v) {
             const Acc xv = xs[rr * ncp + c + v];
 #pragma unroll
-            for (int i = 0; i < RPW; ++i) cfma(acc[i][rr], mv[i][v], xv);
+            for (int i = 0; i < RPW; ++i) {
+              Acc t;
+              t.x = acc[2 * (i * NR + rr)];
+              t.y = acc[2 * (i * NR + rr) + 1];
+              cfma(t, mv[i][v], xv);
+              acc[2 * (i * NR + rr)] = t.x;
+              acc[2 * (i * NR + rr) + 1] = t.y;
+            }
           }
         }
       }
+      int first;
+      warp_sums<R_, V>(acc, lane, first);
+      constexpr int kHeld = V >= 32 ? V / 32 : 1, kSame = V >= 32 ? 1 : 32 / V;  // lanes with the same sums
+      if (lane % kSame == 0) {
 #pragma unroll
-      for (int i = 0; i < RPW; ++i)
-#pragma unroll
-        for (int rr = 0; rr < NR; ++rr) {
-          acc[i][rr].x = warp_sum(acc[i][rr].x);
-          acc[i][rr].y = warp_sum(acc[i][rr].y);
+        for (int k = 0; k < kHeld; ++k) {
+          const int s = first + k, i = s / (2 * NR), rr = (s / 2) % NR;
+          if (r0 + i < nrows) reinterpret_cast<R_*>(outs)[2 * (rr * nrows + r0 + i) + (s & 1)] = acc[k];
         }
-      if (lane == 0) {
-#pragma unroll
-        for (int i = 0; i < RPW; ++i)
-          if (r0 + i < nrows)
-#pragma unroll
-            for (int rr = 0; rr < NR; ++rr) outs[rr * nrows + r0 + i] = acc[i][rr];
       }
     }
     __syncthreads();
@@ -473,16 +512,17 @@ cudaError_t launch_one(const typename P::Args& A, int xcap, int rowcap, int nsm,
   return cudaGetLastError();
 }
 
-// launch_one with the rows per warp chosen at run time (1, 2, 4 or 8; at most 16
+// launch_one with the rows per warp chosen at run time (1, 2, 4 or 8; at most kMaxAcc
 // accumulators of RPW rows x NR right-hand sides per thread, fewer rows otherwise)
 template <class P, int NR>
 cudaError_t launch_shaped(const typename P::Args& A, int xcap, int rowcap, int nsm, cudaStream_t st,
                           long long* counter, const int* gate, LaunchShape sh) {
+  constexpr int kMax = kMaxAcc<typename P::TM>;
   const int r = sh.rpw;
-  if constexpr (NR <= 2) {
+  if constexpr (NR * 8 <= kMax) {
     if (r >= 8) return launch_one<P, NR, 8>(A, xcap, rowcap, nsm, st, counter, gate, sh.bps);
   }
-  if constexpr (NR <= 4) {
+  if constexpr (NR * 4 <= kMax) {
     if (r >= 4) return launch_one<P, NR, 4>(A, xcap, rowcap, nsm, st, counter, gate, sh.bps);
   }
   if (r >= 2) return launch_one<P, NR, 2>(A, xcap, rowcap, nsm, st, counter, gate, sh.bps);
@@ -530,6 +570,20 @@ int xcap_of(const hps_handle* h, XCap which) {
   return (int)round_up(std::max(mx, 1), 64);
 }
 
+// Items per leaf of the applies: enough for several waves of the chip (24 per SM, about 6 for each
+// resident CTA), as many as faces at most; whole leaves stage their vector once and divide evenly
+// among the warps (216 rows at p = 8, a face's 36 do not).  More where the results of NR
+// right-hand sides would not fit in shared memory.
+int leaf_parts(const hps_handle* h, int nr, size_t acc_bytes, int xcap) {
+  int parts = 1;
+  while (parts < 6 && (long long)h->nl * parts < 24LL * h->nsm) parts += parts < 3 ? 1 : 3;
+  auto fits = [&](int p) {
+    return (size_t)nr * (xcap + (h->nb + p - 1) / p) * acc_bytes <= (size_t)100 * 1024;
+  };
+  while (parts < 6 && !fits(parts)) parts += parts < 3 ? 1 : 3;
+  return parts;
+}
+
 template <class TM, class TIN, class TOUT>
 cudaError_t apply_t(const hps_handle* h, const TM* R, const TIN* f, TOUT* y, const double2* bvec, int nrhs,
                     cudaStream_t st) {
@@ -545,9 +599,12 @@ cudaError_t apply_t(const hps_handle* h, const TM* R, const TIN* f, TOUT* y, con
   A.bvec = bvec;
   A.nf = h->nf;
   A.nrhs = nrhs;
-  A.nitems = (long long)h->nl * 6;
+  const int xcap = xcap_of(h, XCap::Apply);
+  A.parts = leaf_parts(h, std::min(nrhs, 8), sizeof(typename P::Acc), xcap);
+  A.inv = row_inv(A.q2);
+  A.nitems = (long long)h->nl * A.parts;
   const LaunchShape* shapes = h->shapes.apply[std::is_same<TM, double2>::value ? 1 : 0];
-  return launch_groups<P>(h, A, nrhs, xcap_of(h, XCap::Apply), A.q2, st, [&](typename P::Args& B, int r0) {
+  return launch_groups<P>(h, A, nrhs, xcap, (h->nb + A.parts - 1) / A.parts, st, [&](typename P::Args& B, int r0) {
     B.f += (long long)r0 * h->nf;
     B.y += (long long)r0 * h->nf;
     if (B.bvec) B.bvec += (long long)r0 * h->nf;
@@ -654,6 +711,7 @@ cudaError_t precond_t(const hps_handle* h, const TM* B, const TM* K, const TIN* 
     A.cl_slot_begin = h->dct.cl_slot_begin;
     A.slot_lf = h->dct.slot_lf;
     A.cl_tpos = h->dct.cl_tpos;
+  A.split = h->ct.krow_split;
     A.nb = h->nb;
     A.q2 = q2;
     A.nf = h->nf;
@@ -718,6 +776,8 @@ cudaError_t launch_apply(const hps_handle* h, bool fp32_matrix, VType tin, const
     return launch_apply_tc(h, (const float2*)f, y, false, nrhs, h->tc_error, st);
   if (tc && tin == VType::C64 && tout == VType::DF)
     return launch_apply_tc(h, (const float2*)f, y, true, nrhs, h->tc_error, st);
+  if (tin == VType::C64 && (tout == VType::C64 || tout == VType::DF) && stream_apply_eligible(h, f))
+    return launch_stream_apply(h, (const float2*)f, tout, y, nrhs, st);
   if (tin == VType::C64 && tout == VType::C64)
     return apply_t(h, h->R32, (const float2*)f, (float2*)y, nullptr, nrhs, st);
   if (tin == VType::C64 && tout == VType::C128)
@@ -756,9 +816,12 @@ cudaError_t rhs_t(const hps_handle* h, const TM* H, const double2* s, const doub
   A.nf = h->nf;
   A.nint = h->nint;
   A.nrhs = nrhs;
-  A.nitems = (long long)h->nl * 6;
-  static const LaunchShape kDefault[4] = {{4, 0}, {4, 0}, {2, 0}, {1, 0}};
-  return launch_groups<P>(h, A, nrhs, xcap_of(h, XCap::Rhs), A.q2, st, [&](typename P::Args& B, int r0) {
+  const int xcap = xcap_of(h, XCap::Rhs);
+  A.parts = leaf_parts(h, std::min(nrhs, 8), sizeof(typename P::Acc), xcap);
+  A.inv = row_inv(A.q2);
+  A.nitems = (long long)h->nl * A.parts;
+  static const LaunchShape kDefault[4] = {{4, 0}, {4, 0}, {2, 0}, {2, 0}};
+  return launch_groups<P>(h, A, nrhs, xcap, (h->nb + A.parts - 1) / A.parts, st, [&](typename P::Args& B, int r0) {
     if (B.s) B.s += (long long)r0 * h->nint;
     if (B.t) B.t += (long long)r0 * h->nf;
     B.out += (long long)r0 * h->nf;
@@ -844,7 +907,8 @@ LaunchShape tune_group(const hps_handle* h, const typename P::Args& A, int nr, i
   };
   LaunchShape best = dflt;
   float tbest = time_one(dflt);
-  const int rmax = nr <= 2 ? 8 : nr <= 4 ? 4 : 2;
+  const int nrp = nr <= 2 ? nr : nr <= 4 ? 4 : 8;
+  const int rmax = std::min(8, kMaxAcc<typename P::TM> / nrp);
   for (int rpw = 1; rpw <= rmax; rpw *= 2)
     for (int bps = 0; bps <= 3; ++bps) {
       const LaunchShape sh{rpw, bps};
@@ -877,10 +941,13 @@ cudaError_t tune_apply(hps_handle* h, const TM* R, int kind, void* fbuf, void* y
   A.bvec = nullptr;
   A.nf = h->nf;
   A.nrhs = nr;
-  A.nitems = (long long)h->nl * 6;
+  const int xcap = xcap_of(h, XCap::Apply);
+  A.parts = leaf_parts(h, nr, sizeof(typename P::Acc), xcap);
+  A.inv = row_inv(A.q2);
+  A.nitems = (long long)h->nl * A.parts;
   const int g = group_index(nr);
   const std::array<long long, 6> key{h->dev, kind, h->q, h->nl, nr, A.nitems};
-  h->shapes.apply[kind][g] = tune_group<P>(h, A, nr, xcap_of(h, XCap::Apply), A.q2, key, h->shapes.apply[kind][g], st);
+  h->shapes.apply[kind][g] = tune_group<P>(h, A, nr, xcap, (h->nb + A.parts - 1) / A.parts, key, h->shapes.apply[kind][g], st);
   return cudaSuccess;
 }
 
@@ -896,6 +963,7 @@ cudaError_t tune_stage_k(hps_handle* h, const TM* K, const float* kscale, void* 
   A.cl_slot_begin = h->dct.cl_slot_begin;
   A.slot_lf = h->dct.slot_lf;
   A.cl_tpos = h->dct.cl_tpos;
+  A.split = h->ct.krow_split;
   A.nb = h->nb;
   A.q2 = h->q * h->q;
   A.nf = h->nf;
@@ -933,7 +1001,8 @@ int autotune_shapes(hps_handle* h, cudaStream_t st) {
   if (nr_max > 1) groups.push_back(nr_max);
   for (int nr : groups) {
     // the inner apply of each form: complex-FP32 operand into the double-float basis, and FP64
-    if (h->R32) tune_apply<float2, float2, float4>(h, h->R32, 0, fbuf, ybuf, nr, st);
+    if (h->R32 && !stream_apply_eligible(h, fbuf))
+      tune_apply<float2, float2, float4>(h, h->R32, 0, fbuf, ybuf, nr, st);
     if (h->R64) tune_apply<double2, double2, double2>(h, h->R64, 1, fbuf, ybuf, nr, st);
   }
   // SIMT stage K of the mixed solve (FP16 blocks when kept, else FP32)

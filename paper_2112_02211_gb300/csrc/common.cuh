@@ -144,6 +144,36 @@ template <class T> __device__ __forceinline__ T warp_sum(T v) {
   return v;
 }
 
+// Warp sums of V values per lane.  Each step o = 16, 8, ... exchanges half of the values still
+// held with lane ^ o (a plain exchange once one is left), so V values take about V shuffles
+// instead of 5 V; every sum has the same pairs in the same order as a butterfly.  On return v[0 ..
+// max(1, V / 32)) of a lane are the sums number `first` and following.
+template <class R, int V>
+__device__ __forceinline__ void warp_sums(R (&v)[V], int lane, int& first) {
+  first = 0;
+  int held = V;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    if (held > 1) {
+      const bool up = (lane & o) != 0;
+      held >>= 1;
+#pragma unroll
+      for (int k = 0; k < V / 2; ++k) {
+        if (k < held) {
+          const R keep = up ? v[k + held] : v[k], send = up ? v[k] : v[k + held];
+          v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      }
+      if (up) first += held;
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    }
+  }
+}
+
+// r / q2 = (r * row_inv(q2)) >> 20 for r * q2 < 2^20 (rows of a leaf: r < 6 * 196, q2 <= 196).
+__host__ __device__ constexpr unsigned row_inv(int q2) { return (1u << 20) / (unsigned)q2 + 1u; }
+
 // Leading dimension of stored matrices: columns padded to a multiple of 4.
 __host__ __device__ __forceinline__ long long rup4(long long v) { return (v + 3) / 4 * 4; }
 

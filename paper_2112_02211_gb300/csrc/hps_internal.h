@@ -100,10 +100,11 @@ struct ClusterTables {
   int nbc = 0;
   std::vector<int> leaf_bcls;        // [nleaves] B block of each leaf; FP16 scale row = (bcls*6 + face) q^2 + j
   std::vector<int> bc_rep;           // [nbc] first leaf using the block
-  // stage-K work items (block, block slot * kKRowSplit + part of its rows,
+  // stage-K work items (block, block slot * krow_split + part of its rows,
   // first member, member count) for member groups of width 1, 2, 4 and 8, and
   // the blocks whose members are many enough for the tensor-core path
   // (tc_precond.cu), which then skip the items above
+  int krow_split = 2;                // parts that the q^2 rows of a slot are cut into
   std::vector<int4> kitems[4];
   long long kitems_ntc[4] = {0, 0, 0, 0};
   std::vector<int> kc_tc;
@@ -190,7 +191,7 @@ struct LaunchShape {
 // member-group width (1, 2, 4, 8).  Defaults from a hand sweep; replaced at setup
 // by the autotuner (options.autotune).
 struct Shapes {
-  LaunchShape apply[2][4] = {{{4, 0}, {4, 0}, {2, 0}, {1, 0}}, {{4, 0}, {4, 0}, {2, 0}, {1, 0}}};
+  LaunchShape apply[2][4] = {{{4, 0}, {4, 0}, {4, 0}, {4, 0}}, {{4, 0}, {4, 0}, {4, 0}, {2, 0}}};
   LaunchShape k[4] = {{4, 0}, {4, 0}, {2, 0}, {2, 0}};
   bool tuned = false;
 };
@@ -475,9 +476,6 @@ void assign_blocks(hps_handle* h, const std::vector<double2>* lamq);
 constexpr int kTcMinMembers = 16;
 // Mark of a stage-B item whose block is in kc_tc.
 constexpr int kTcItem = 256;
-// Stage-K work items of the SIMT kernel cover 1/kKRowSplit of a slot's q^2 rows
-// (finer items balance the last wave of the launch).
-constexpr int kKRowSplit = 2;
 // Leaves per stage-B work item of the general layouts (leaves sharing one B block).
 constexpr int kBGroup = 1;
 // Dynamic shared memory a block may opt into on sm_103 (227 KB).
@@ -498,6 +496,10 @@ cudaError_t launch_rhs(const hps_handle* h, const double2* s, const double2* t, 
 constexpr double kCompensatedMinTol = 1e-8;
 cudaError_t launch_precond(const hps_handle* h, bool fp32_matrix, VType tin, const void* r,
                            VType tout, void* z, void* scratch, int nrhs, cudaStream_t st, bool fp16_blocks = false);
+// The apply with the maps streamed through shared memory (stream_apply.cu): complex-float vectors
+// and maps, into complex float or double-float.
+bool stream_apply_eligible(const hps_handle* h, const void* f);
+cudaError_t launch_stream_apply(const hps_handle* h, const float2* f, VType tout, void* y, int nrhs, cudaStream_t st);
 // Tensor-core apply for 64-RHS groups (tc_apply.cu); f complex float, y complex
 // float or double-float; nrhs a multiple of 64.
 // whether launch_apply runs nrhs right-hand sides with complex-FP32 input on the tensor cores
