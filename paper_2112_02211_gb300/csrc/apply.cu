@@ -427,6 +427,7 @@ struct PrecBArgs {
   const int2* groups;
   const int* gleaves;
   int ngroups;
+  int parts;  // CTAs per item, each a part of the rows (the first one also writes z_ext)
 };
 
 template <class TM> __device__ __forceinline__ typename MT<TM>::Acc load_one(const TM* p);
@@ -444,7 +445,8 @@ __global__ void __launch_bounds__(kThreads) prec_b_kernel(const PrecBArgs<TM, TI
   // item: a group of leaves sharing one B block (same block, same internal-face mask); the
   // vectors of a pass are NR (leaf of the group, right-hand side) pairs, so every entry of B
   // loaded from L2 serves NR independent accumulations
-  for (int item = blockIdx.x; item < A.ngroups; item += gridDim.x) {
+  for (int idx_i = blockIdx.x; idx_i < A.ngroups * A.parts; idx_i += gridDim.x) {
+    const int item = idx_i / A.parts, part = idx_i - item * A.parts;
     const int2 grp = A.groups[item];
     const int leaf0 = A.gleaves[grp.x];
     const int nint = __popc((unsigned)A.int_mask[leaf0]);
@@ -455,27 +457,50 @@ __global__ void __launch_bounds__(kThreads) prec_b_kernel(const PrecBArgs<TM, TI
     for (int v0 = 0; v0 < nvec; v0 += NR) {
       const int nr = min(NR, nvec - v0);
       __syncthreads();
-      for (int idx = threadIdx.x; idx < nr * ncols; idx += kThreads) {
+      for (int idx = threadIdx.x; idx < nr * ncols; idx += blockDim.x) {
         const int rr = idx / ncols, c = idx - rr * ncols;
         const int vid = v0 + rr, leaf = A.gleaves[grp.x + vid / A.nrhs], rhs = vid % A.nrhs;
         const int k = c / q2;
         const long long o = (long long)rhs * A.vstride + A.brd[leaf * 6 + nint + k] + (c - k * q2);
         const Acc v = cvt<Acc>(A.r[o]);
         xs[rr * ncols + c] = v;
-        A.z[o] = cvt<TOUT>(v);
+        if (part == 0) A.z[o] = cvt<TOUT>(v);
       }
       __syncthreads();
       if (nint == 0) continue;
-      for (int row = threadIdx.x; row < nrows; row += kThreads) {
-        Acc acc[NR];
+      const int row_end = nrows * (part + 1) / A.parts;
+      for (int row = nrows * part / A.parts + threadIdx.x; row < row_end; row += blockDim.x) {
+        // few right-hand sides in complex double: four sums per row, since one sum is a chain of two
+        // dependent FP64 operations per column (216 of them at p = 8)
+        constexpr int kS = sizeof(TM) == sizeof(double2) && NR <= 2 ? 4 : 1;
+        Acc acc[NR], sum[kS][NR];
 #pragma unroll
-        for (int rr = 0; rr < NR; ++rr) acc[rr] = czero<Acc>();
-#pragma unroll 4
-        for (int c = 0; c < ncols; ++c) {
+        for (int i = 0; i < kS; ++i)
+#pragma unroll
+          for (int rr = 0; rr < NR; ++rr) sum[i][rr] = czero<Acc>();
+        int c = 0;
+#pragma unroll(kS == 4 ? 3 : 1)
+        for (; c + 3 < ncols; c += 4) {
+          Acc bv[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) bv[i] = load_one<TM>(Bm + (long long)(c + i) * ldr + row);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int rr = 0; rr < NR; ++rr)
+              if (rr < nr) cfma(sum[i % kS][rr], bv[i], xs[rr * ncols + c + i]);
+        }
+        for (; c < ncols; ++c) {
           const Acc bv = load_one<TM>(Bm + (long long)c * ldr + row);
 #pragma unroll
           for (int rr = 0; rr < NR; ++rr)
-            if (rr < nr) cfma(acc[rr], bv, xs[rr * ncols + c]);
+            if (rr < nr) cfma(sum[0][rr], bv, xs[rr * ncols + c]);
+        }
+#pragma unroll
+        for (int rr = 0; rr < NR; ++rr) {
+          acc[rr] = sum[0][rr];
+#pragma unroll
+          for (int i = 1; i < kS; ++i) acc[rr] = cadd(acc[rr], sum[i][rr]);
         }
         const int k = row / q2, j = row - k * q2;
 #pragma unroll
@@ -665,8 +690,15 @@ cudaError_t precond_t(const hps_handle* h, const TM* B, const TM* K, const TIN* 
       int occ = 0;
       if (e2 == cudaSuccess) e2 = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, smem);
       if (e2 != cudaSuccess) return e2;
-      const int grid = (int)std::min<long long>(A.ngroups, (long long)h->nsm * std::max(occ, 1));
-      kern<<<grid, kThreads, smem, st>>>(A);
+      // Where the items leave SMs idle, each is cut by rows into CTAs of a warp or more (64 leaves
+      // at p = 8 in complex double: 32.5 us with one CTA and one sum per row, 28.5 us with 4 CTAs
+      // and four sums; both with the timer's own ~8 us).
+      PrecBArgs<TM, TIN, TOUT> C = A;
+      const int rows = 3 * q2;
+      C.parts = std::max(1, std::min((rows + 31) / 32, 2 * h->nsm / std::max(1, A.ngroups)));
+      const int threads = C.parts > 1 ? (int)round_up((rows + C.parts - 1) / C.parts, 32) : kThreads;
+      const int grid = (int)std::min<long long>((long long)A.ngroups * C.parts, (long long)h->nsm * std::max(occ, 1));
+      kern<<<grid, threads, smem, st>>>(C);
       ++h->prof.launches;
       return cudaGetLastError();
     };
@@ -744,7 +776,12 @@ cudaError_t precond_t(const hps_handle* h, const TM* B, const TM* K, const TIN* 
         A.nrhs = A.nrl << g;
         A.t = t + (long long)r0 * tstride;
         A.z = z + (long long)r0 * h->nf;
-        e = launch_group<P>(A, A.nrhs, xcap, q2, h->nsm, st, counter, h->gate, h->shapes.k[group_index(A.nrhs)]);
+        // shapes are tuned for single right-hand sides of the float kernels; otherwise as many rows
+        // per warp as leave work for all 8 warps of an item
+        const bool tuned = h->shapes.tuned && A.nrl == 1 && sizeof(TM) != sizeof(double2);
+        const int rows = (q2 + A.split - 1) / A.split;
+        const LaunchShape sh = tuned ? h->shapes.k[g] : LaunchShape{rows >= 32 ? 4 : rows >= 16 ? 2 : 1, 0};
+        e = launch_group<P>(A, A.nrhs, xcap, q2, h->nsm, st, counter, h->gate, sh);
       }
     }
     h->prof.end(HPS_PHASE_PRECOND_K, ev, st);
@@ -1003,10 +1040,10 @@ int autotune_shapes(hps_handle* h, cudaStream_t st) {
     // the inner apply of each form: complex-FP32 operand into the double-float basis, and FP64
     if (h->R32 && !stream_apply_eligible(h, fbuf))
       tune_apply<float2, float2, float4>(h, h->R32, 0, fbuf, ybuf, nr, st);
-    if (h->R64) tune_apply<double2, double2, double2>(h, h->R64, 1, fbuf, ybuf, nr, st);
+    if (h->R64 && (h->opt.forms & HPS_FORM_FP64)) tune_apply<double2, double2, double2>(h, h->R64, 1, fbuf, ybuf, nr, st);
   }
   // SIMT stage K of the mixed solve (FP16 blocks when kept, else FP32)
-  if (h->has_precond && h->ct.nslots > 0 && h->pc_scratch) {
+  if (h->has_precond && h->ct.nslots > 0 && h->pc_scratch && !precond_tc16_eligible(h, 1)) {
     cudaMemsetAsync(h->pc_scratch, 0, (size_t)h->ct.tsize * sizeof(float2), st);
     const bool tc = h->opt.tc_apply && h->Kc32 && h->tc_error && !h->ct.kc_tc.empty();
     if (h->Kc16) tune_stage_k<__half2>(h, h->Kc16, h->Kc16s, h->pc_scratch, ybuf, tc, st);

@@ -18,11 +18,11 @@
 // Kernel (one CTA per SM, persistent over items = (leaf, 128-row tile)):
 //   warp 0       TMA producer: A tile (128 rows x 32 floats) and F tile
 //                (64 rhs x 32 floats), 128-byte swizzle, into a 3-stage ring
-//   warps 2..7   split the stage: A -> A_hi (in place) + A_lo, F -> B_hi, B_lo
+//   warps 2..15  split the stage: A -> A_hi (in place) + A_lo, F -> B_hi, B_lo
 //   warp 1       tcgen05.alloc of 256 TMEM columns (two accumulators); one lane
 //                issues 12 tcgen05.mma (4 K-steps x 3 products) per stage and
 //                commits to mbarriers
-//   warps 8..11  epilogue: tcgen05.ld of the 128 x 128 FP32 accumulator,
+//   warps 16..19 epilogue: tcgen05.ld of the 128 x 128 FP32 accumulator,
 //                y = f + G written to the neighbour across the row's face (the
 //                swap Pi fused into the store)
 // Every wait is bounded: after a limit the CTA raises an error word, stops
@@ -53,7 +53,9 @@ constexpr int kFBytes = kRhs * kTileK * 4;    // 8 KB
 constexpr int kBBytes = kTileN * kTileK * 4;  // 16 KB
 // stage layout (each part 1024-byte aligned): Ahi(=A) | Alo | Bhi | Blo | F
 constexpr int kStageBytes = 2 * kABytes + 2 * kBBytes + kFBytes;  // 72 KB
-constexpr int kThreads = 384;  // 12 warps
+constexpr int kSplitWarps = 14;  // conversion warps (6: 4 % slower)
+constexpr int kSplitThreads = 32 * kSplitWarps;
+constexpr int kThreads = 32 * (6 + kSplitWarps);
 constexpr int kTmemCols = 256;
 
 struct TcArgs {
@@ -93,7 +95,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&bars->full[s], 1);
-      mbar_init(&bars->split[s], 6);  // one arrival per transform warp
+      mbar_init(&bars->split[s], kSplitWarps);  // one arrival per transform warp
       mbar_init(&bars->empty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -144,9 +146,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (long long j = (it > kStages ? it - kStages : 0); j < it; ++j)
         if (!mbar_wait(&bars->full[(int)(j % kStages)], (uint32_t)((j / kStages) & 1), a.spin)) fail();
     }
-  } else if (warp >= 2 && warp < 8) {
+  } else if (warp >= 2 && warp < 2 + kSplitWarps) {
     // ---------------- split into TF32 hi/lo operands ----------------
-    const int t = threadIdx.x - 64;  // 0..191
+    const int t = threadIdx.x - 64;  // 0..kSplitThreads - 1
     long long it = 0;
     for (long long item = blockIdx.x; item < nitems; item += gridDim.x) {
       for (int kb = 0; kb < a.kblocks; ++kb, ++it) {
@@ -162,7 +164,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         float4* Bhi = reinterpret_cast<float4*>(st + 2 * kABytes);
         float4* Blo = reinterpret_cast<float4*>(st + 2 * kABytes + kBBytes);
         const float4* F = reinterpret_cast<const float4*>(st + 2 * kABytes + 2 * kBBytes);
-        for (int c = t; c < kABytes / 16; c += 192) {
+        for (int c = t; c < kABytes / 16; c += kSplitThreads) {
           const float4 v = Ahi[c];
           const float4 h = make_float4(tf32_hi(v.x), tf32_hi(v.y), tf32_hi(v.z), tf32_hi(v.w));
           Ahi[c] = h;
@@ -170,7 +172,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         // F rows s (64 x 128 bytes): B row s = conj(f_s), B row 64+s = swap(f_s); the
         // 16-byte chunk positions (and so the swizzle) are the same in both halves.
-        for (int c = t; c < kFBytes / 16; c += 192) {
+        for (int c = t; c < kFBytes / 16; c += kSplitThreads) {
           const float4 v = F[c];
           const float4 cj = make_float4(v.x, -v.y, v.z, -v.w);
           const float4 sw = make_float4(v.y, v.x, v.w, v.z);
@@ -238,8 +240,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else {
-    // ---------------- epilogue: warps 8..11 = TMEM lanes 0..127 ----------------
-    const int ew = warp - 8;  // TMEM lane quarter
+    // ---------------- epilogue: the last 4 warps, each on the TMEM lanes that it may read ----------------
+    const int ew = warp & 3;  // TMEM lane quarter
     long long local = 0;
     for (long long item = blockIdx.x; item < nitems; item += gridDim.x, ++local) {
       const int b = (int)(local & 1);
@@ -251,34 +253,34 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int leaf = (int)(item / a.mtiles), mt = (int)(item % a.mtiles);
       const int row = mt * kTileM + ew * 32 + lane;
       const uint32_t taddr = tmem + ((uint32_t)(ew * 32) << 16) + (uint32_t)(b * kTileN);
-      float re[32], im[32];
-      // columns 0..63 = Re G for rhs 0..63, 64..127 = Im G
-      for (int half = 0; half < 2; ++half) {
-        tmem_ld32(taddr + half * 32, re);
-        tmem_ld32(taddr + 64 + half * 32, im);
-        if (row < a.nb) {
-          const int face = row / a.q2, j = row % a.q2;
-          const int ix = leaf % a.nx, iy = (leaf / a.nx) % a.ny, iz = leaf / (a.nx * a.ny);
-          int nx_ = ix, ny_ = iy, nz_ = iz;
-          const int d = (face & 1) ? 1 : -1;
-          bool inside = true;
-          if ((face >> 1) == 0) { nx_ += d; inside = nx_ >= 0 && nx_ < a.nx; }
-          else if ((face >> 1) == 1) { ny_ += d; inside = ny_ >= 0 && ny_ < a.ny; }
-          else { nz_ += d; inside = nz_ >= 0 && nz_ < a.nz; }
-          if (inside) {
-            const int nbr = nx_ + a.nx * (ny_ + a.ny * nz_);
-            const long long dst = (long long)nbr * a.nb + (long long)(face ^ 1) * a.q2 + j;
+      // the row's slot in the neighbour's data (rows of boundary faces are not used)
+      long long dst = -1;
+      if (row < a.nb) {
+        const int face = row / a.q2, j = row % a.q2;
+        const int nbr = GridDims{a.nx, a.ny, a.nz}.neighbor(leaf, face);
+        if (nbr >= 0) dst = (long long)nbr * a.nb + (long long)(face ^ 1) * a.q2 + j;
+      }
+      // columns 0..63 = Re G for rhs 0..63, 64..127 = Im G, 16 right-hand sides at a time: their f
+      // first (independent loads; one load, add and store after the other took 25 us an item)
+#pragma unroll 1
+      for (int r0 = 0; r0 < kRhs; r0 += 16) {
+        float2 fv[16];
 #pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              const int rhs = half * 32 + c;
-              const long long o = rhs * a.nf + dst;
-              const float2 fv = a.f[o];
-              if (a.out_df) {
-                const dfr r1 = df_two_sum(fv.x, re[c]), r2 = df_two_sum(fv.y, im[c]);
-                reinterpret_cast<float4*>(a.y)[o] = make_float4(r1.h, r2.h, r1.l, r2.l);
-              } else {
-                reinterpret_cast<float2*>(a.y)[o] = make_float2(fv.x + re[c], fv.y + im[c]);
-              }
+        for (int c = 0; c < 16; ++c) fv[c] = dst >= 0 ? __ldg(a.f + (r0 + c) * a.nf + dst) : make_float2(0.f, 0.f);
+        uint32_t re[16], im[16];
+        tmem_ld16(taddr + r0, re);
+        tmem_ld16(taddr + 64 + r0, im);
+        tmem_wait_ld();
+        if (dst >= 0) {
+#pragma unroll
+          for (int c = 0; c < 16; ++c) {
+            const long long o = (r0 + c) * a.nf + dst;
+            const float gr = __uint_as_float(re[c]), gi = __uint_as_float(im[c]);
+            if (a.out_df) {
+              const dfr r1 = df_two_sum(fv[c].x, gr), r2 = df_two_sum(fv[c].y, gi);
+              reinterpret_cast<float4*>(a.y)[o] = make_float4(r1.h, r2.h, r1.l, r2.l);
+            } else {
+              reinterpret_cast<float2*>(a.y)[o] = make_float2(fv[c].x + gr, fv[c].y + gi);
             }
           }
         }

@@ -29,10 +29,10 @@
 // Kernel (one CTA per SM, persistent over items = (128-row tile, 64-member tile)):
 //   warp 0       TMA producer: A tile (128 rows x 32 floats) and T tile
 //                (64 members x 32 floats), 128-byte swizzle, 5-stage ring
-//   warps 2..7   round A to TF32 in place, build the conj/swap rows of B
+//   warps 2..15  round A to TF32 in place, build the conj/swap rows of B
 //   warp 1       TMEM allocation (256 columns, two accumulators); one lane
 //                issues the MMAs and commits to mbarriers
-//   warps 8..11  epilogue: TMEM -> registers -> z at each member cluster's
+//   warps 16..19 epilogue: TMEM -> registers -> z at each member cluster's
 //                internal face slots
 // Every wait is bounded: after a limit the CTA raises the error word, stops
 // issuing work, waits (bounded) for its own tensor-core work, frees TMEM and
@@ -62,7 +62,9 @@ constexpr int kTBytes = kMem * kTileK * 4;    // 8 KB
 constexpr int kBBytes = kTileN * kTileK * 4;  // 16 KB
 // stage layout (each part 1024-byte aligned): A | B | T
 constexpr int kStageBytes = kABytes + kBBytes + kTBytes;  // 40 KB
-constexpr int kThreads = 384;
+constexpr int kSplitWarps = 14;
+constexpr int kSplitThreads = 32 * kSplitWarps;
+constexpr int kThreads = 32 * (6 + kSplitWarps);
 constexpr int kTmemCols = 256;
 
 struct PkArgs {
@@ -112,7 +114,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&bars->full[s], 1);
-      mbar_init(&bars->split[s], 6);
+      mbar_init(&bars->split[s], kSplitWarps);
       mbar_init(&bars->empty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -187,9 +189,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (long long j = (it > kStages ? it - kStages : 0); j < it; ++j)
         if (!mbar_wait(&bars->full[(int)(j % kStages)], (uint32_t)((j / kStages) & 1))) fail();
     }
-  } else if (warp >= 2 && warp < 8) {
+  } else if (warp >= 2 && warp < 2 + kSplitWarps) {
     // ---------------- split into TF32 hi/lo operands ----------------
-    const int t = threadIdx.x - 64;  // 0..191
+    const int t = threadIdx.x - 64;  // 0..kSplitThreads - 1
     long long it = 0;
     for (long long item = blockIdx.x; item < nitems; item += gridDim.x) {
       for (int kb = 0; kb < a.kblocks; ++kb, ++it) {
@@ -203,12 +205,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         float4* A = reinterpret_cast<float4*>(st);
         float4* B = reinterpret_cast<float4*>(st + kABytes);
         const float4* T = reinterpret_cast<const float4*>(st + kABytes + kBBytes);
-        for (int c = t; c < kABytes / 16; c += 192) {
+        for (int c = t; c < kABytes / 16; c += kSplitThreads) {
           const float4 v = A[c];
           A[c] = make_float4(tf32_hi(v.x), tf32_hi(v.y), tf32_hi(v.z), tf32_hi(v.w));
         }
         // B row m = conj(t_m), B row 64 + m = swap(t_m): same 16-byte chunk positions
-        for (int c = t; c < kTBytes / 16; c += 192) {
+        for (int c = t; c < kTBytes / 16; c += kSplitThreads) {
           const float4 v = T[c];
           B[c] = make_float4(tf32_hi(v.x), tf32_hi(-v.y), tf32_hi(v.z), tf32_hi(-v.w));
           B[c + kTBytes / 16] = make_float4(tf32_hi(v.y), tf32_hi(v.x), tf32_hi(v.w), tf32_hi(v.z));
@@ -261,8 +263,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else {
-    // ---------------- epilogue: warps 8..11 = TMEM lanes 0..127 ----------------
-    const int ew = warp - 8;
+    // ---------------- epilogue: the last 4 warps, each on the TMEM lanes that it may read ----------------
+    const int ew = warp & 3;
     long long local = 0;
     for (long long item = blockIdx.x; item < nitems; item += gridDim.x, ++local) {
       const int b = (int)(local & 1);
@@ -302,7 +304,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             int p = v0 / a.nrhs, rhs = v0 - p * a.nrhs;
 #pragma unroll
             for (int c = 0; c < 32; ++c) {
-              if (c < n) a.z[(long long)rhs * a.nf + a.zoff[p * 24 + sl] + j] = make_float2(re[c], im[c]);
+              if (c < n) a.z[(long long)rhs * a.nf + __ldg(a.zoff + p * 24 + sl) + j] = make_float2(re[c], im[c]);
               if (++rhs == a.nrhs) {
                 rhs = 0;
                 ++p;
