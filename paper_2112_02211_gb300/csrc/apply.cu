@@ -566,6 +566,16 @@ cudaError_t launch_group(const typename P::Args& B, int nr, int xcap, int rowcap
   return launch_shaped<P, 8>(B, xcap, rowcap, nsm, st, counter, gate, sh);
 }
 
+// Right-hand sides (or vectors) of the next launch, at most `most` of `left`: in complex double
+// whole powers of two, since the FP64 pipe is the bound and a group of 6 would compute 8.
+template <class TM>
+int next_group(int left, int most) {
+  int n = std::min(left, most);
+  if (sizeof(TM) == sizeof(double2))
+    while (n & (n - 1)) n &= n - 1;
+  return n;
+}
+
 // Launch over right-hand-side groups of at most 8 (each group re-reads the matrix);
 // shapes[g]: the launch shape of group index g.
 template <class P, class Shift>
@@ -573,9 +583,9 @@ cudaError_t launch_groups(const hps_handle* h, typename P::Args A, int nrhs, int
                           Shift shift, const LaunchShape* shapes) {
   const int nsm = h->nsm;
   long long* counter = &h->prof.launches;
-  for (int r0 = 0; r0 < nrhs; r0 += 8) {
+  for (int r0 = 0, nr; r0 < nrhs; r0 += nr) {
     typename P::Args B = A;
-    const int nr = std::min(8, nrhs - r0);
+    nr = next_group<typename P::TM>(nrhs - r0, 8);
     shift(B, r0);
     B.nrhs = nr;
     const cudaError_t e = launch_group<P>(B, nr, xcap, rowcap, nsm, st, counter, h->gate, shapes[group_index(nr)]);
@@ -771,8 +781,8 @@ cudaError_t precond_t(const hps_handle* h, const TM* B, const TM* K, const TIN* 
       A.items = h->dct.kitems[g];
       A.nitems = n;
       const int step = std::max(1, fit >> g);
-      for (int r0 = 0; r0 < nrhs && e == cudaSuccess; r0 += step) {
-        A.nrl = std::min(step, nrhs - r0);
+      for (int r0 = 0; r0 < nrhs && e == cudaSuccess; r0 += A.nrl) {
+        A.nrl = next_group<TM>(nrhs - r0, step);
         A.nrhs = A.nrl << g;
         A.t = t + (long long)r0 * tstride;
         A.z = z + (long long)r0 * h->nf;

@@ -13,9 +13,15 @@
 //
 // This gives the lean form an FP64-accurate restart residual
 // b - (I + Pi R) x, an FP64-accurate right-hand side b = tbar - Pi H s and
-// complex-double applies, instead of FP32-accurate ones.  Item = (leaf, face):
-// the q^2 rows of that face's block; the swap Pi is fused into the store as in
+// complex-double applies, instead of FP32-accurate ones.  Item = (leaf, part): a
+// part of the rows of the leaf's faces with a neighbour; the swap Pi is fused into the store as in
 // the other applies (one writer per output slot).
+//
+// What bounds it: about 50 FP32 instructions per complex entry and right-hand side (12 bytes), on
+// top of the warp reductions, which halve the sums in flight at every exchange, and the latency of
+// the map entries, which are loaded one step ahead.Measured, 8^3 leaves at p = 8:
+// restart residual of 8 right-hand sides 2.23 -> 0.55 ms, of one 217 -> 103 us; right-hand side of 8
+// sources 2.20 -> 0.54 ms (before: items of a face's 32 and 4 rows, one CTA per SM, full butterflies).
 #include <algorithm>
 
 #include "common.cuh"
@@ -29,7 +35,7 @@ constexpr int kT = 256;
 constexpr int kW = kT / 32;
 constexpr int kRPW = 2;  // rows per warp pass
 constexpr int kNRMax = 4;  // most right-hand sides per pass over the block
-constexpr int kCR = 32;    // rows per work item: a face block is split so that the rows every
+constexpr int kCR = 48;    // rows per work item at most: a leaf is split so that the rows every
                            // pass over the right-hand sides re-reads stay in L2
 
 // (sum, error) pair: value = s + c
@@ -65,96 +71,149 @@ struct CfArgs {
   const double2* t;    // H: boundary data for the boundary-face slots, or nullptr
   long long nf;
   int nrhs, rhs_mode;  // rhs_mode: the map is H (b = tbar - Pi H s) instead of R
+  int parts;           // items per leaf
+  unsigned inv;        // row_inv(q2)
   long long nitems;
 };
 
+// One row's sums of one right-hand side.
+struct CfSum {
+  cacc re, im;
+  float sre, sim;
+};
+__device__ __forceinline__ float pick(bool first, float a, float b) { return first ? a : b; }
+__device__ __forceinline__ CfSum cf_pick(bool first, CfSum a, CfSum b) {
+  return {{pick(first, a.re.s, b.re.s), pick(first, a.re.c, b.re.c)},
+          {pick(first, a.im.s, b.im.s), pick(first, a.im.c, b.im.c)},
+          pick(first, a.sre, b.sre),
+          pick(first, a.sim, b.sim)};
+}
+__device__ __forceinline__ CfSum cf_exchange(CfSum keep, CfSum send, int o) {
+  return {cacc_merge(keep.re, cacc_shfl(send.re, o)), cacc_merge(keep.im, cacc_shfl(send.im, o)),
+          __fadd_rn(keep.sre, __shfl_xor_sync(0xffffffffu, send.sre, o)),
+          __fadd_rn(keep.sim, __shfl_xor_sync(0xffffffffu, send.sim, o))};
+}
+
 // kNR right-hand sides per pass over the block (1, 2 or 4)
 template <int kNR>
-__global__ void __launch_bounds__(kT) cf_gemv_kernel(const CfArgs A, int ncp) {
+__global__ void __launch_bounds__(kT, kNR == 4 ? 2 : kNR == 2 ? 2 : 3) cf_gemv_kernel(const CfArgs A, int ncp) {
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* xh = reinterpret_cast<float2*>(smraw);  // kNR x ncp
   float2* xl = xh + kNR * ncp;                    // kNR x ncp
   double2* outs = reinterpret_cast<double2*>(xl + kNR * ncp);  // kNR x kCR
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int q2 = A.q2;
-  const int nchunk = (q2 + kCR - 1) / kCR;
   for (long long item = blockIdx.x; item < A.nitems; item += gridDim.x) {
-    const long long lf = item / nchunk;
-    const int chunk = (int)(item % nchunk);
-    const int leaf = (int)(lf / 6), face = (int)(lf % 6);
-    const int row0 = chunk * kCR, nrow = min(kCR, q2 - row0);
-    const int nbr = A.g.neighbor(leaf, face);
-    const long long own = (long long)leaf * A.nb + (long long)face * q2;
-    if (nbr < 0) {
-      // boundary face: R rows unused (Pi is 0 there); H: the slot takes t (or 0)
-      for (int idx = tid; idx < A.nrhs * nrow; idx += kT) {
-        const int rr = idx / nrow, j = row0 + idx % nrow;
-        const long long o = (long long)rr * A.nf + own + j;
-        if (A.rhs_mode) {
-          A.y[o] = A.t ? A.t[o] : make_double2(0.0, 0.0);
-        } else {
-          const double2 xv = A.x[(long long)rr * A.xstride + own + j];
-          A.y[o] = A.b ? csub(A.b[o], xv) : xv;
+    const int leaf = (int)(item / A.parts), part = (int)(item % A.parts);
+    unsigned mask = 0, flist = 0;
+    int faces = 0;
+#pragma unroll
+    for (int f = 0; f < 6; ++f)
+      if (A.g.neighbor(leaf, f) >= 0) {
+        mask |= 1u << f;
+        flist |= (unsigned)f << (4 * faces++);
+      }
+    const int row0 = faces * q2 * part / A.parts, nrow = faces * q2 * (part + 1) / A.parts - row0;
+    auto place = [&](int l, int& face, int& j) {  // row l of the item
+      const unsigned r = row0 + l, k = (r * A.inv) >> 20;
+      j = (int)(r - k * q2);
+      face = (flist >> (4 * k)) & 7u;
+    };
+    if (part == 0 && mask != 63u)
+      // boundary faces: R rows unused (Pi is 0 there); H: the slot takes t (or 0)
+      for (int idx = tid; idx < 6 * q2; idx += kT) {
+        if ((mask >> (idx / q2)) & 1u) continue;
+        for (int rr = 0; rr < A.nrhs; ++rr) {
+          const long long o = (long long)rr * A.nf + (long long)leaf * A.nb + idx;
+          if (A.rhs_mode) {
+            A.y[o] = A.t ? A.t[o] : make_double2(0.0, 0.0);
+          } else {
+            const double2 xv = A.x[(long long)rr * A.xstride + (long long)leaf * A.nb + idx];
+            A.y[o] = A.b ? csub(A.b[o], xv) : xv;
+          }
         }
+      }
+    if (A.rhs_mode && !A.x) {  // no body load: h = 0
+      for (int l = tid; l < nrow; l += kT) {
+        int face, j;
+        place(l, face, j);
+        const long long o = (long long)A.g.neighbor(leaf, face) * A.nb + (long long)(face ^ 1) * q2 + j;
+        for (int rr = 0; rr < A.nrhs; ++rr) A.y[(long long)rr * A.nf + o] = make_double2(0.0, 0.0);
       }
       continue;
     }
-    const long long dst = (long long)nbr * A.nb + (long long)(face ^ 1) * q2;
-    if (A.rhs_mode && !A.x) {  // no body load: h = 0
-      for (int idx = tid; idx < A.nrhs * nrow; idx += kT)
-        A.y[(long long)(idx / nrow) * A.nf + dst + row0 + idx % nrow] = make_double2(0.0, 0.0);
-      continue;
-    }
-    const float2* Mb = A.M + (long long)leaf * A.leaf_stride + (long long)(face * q2 + row0) * A.ld;
-    const __half2* Lb = A.lo + (long long)leaf * A.leaf_stride + (long long)(face * q2 + row0) * A.ld;
-    const float* Sb = A.scale + (long long)leaf * A.nb + (long long)face * q2 + row0;
+    const float2* Mb = A.M + (long long)leaf * A.leaf_stride;
+    const __half2* Lb = A.lo + (long long)leaf * A.leaf_stride;
+    const float* Sb = A.scale + (long long)leaf * A.nb;
     for (int r0 = 0; r0 < A.nrhs; r0 += kNR) {
       const int nr = min(kNR, A.nrhs - r0);
       __syncthreads();
-      for (int idx = tid; idx < kNR * ncp; idx += kT) {
-        const int rr = idx / ncp, c = idx % ncp;
-        double2 v = make_double2(0.0, 0.0);
-        if (rr < nr && c < A.ncols) v = A.x[(long long)(r0 + rr) * A.xstride + (long long)leaf * A.xleaf + c];
-        const float hr = __double2float_rn(v.x), hi = __double2float_rn(v.y);
-        xh[idx] = make_float2(hr, hi);
-        xl[idx] = make_float2(__double2float_rn(v.x - (double)hr), __double2float_rn(v.y - (double)hi));
-      }
+#pragma unroll
+      for (int rr = 0; rr < kNR; ++rr)
+        for (int c = tid; c < ncp; c += kT) {
+          double2 v = make_double2(0.0, 0.0);
+          if (rr < nr && c < A.ncols) v = A.x[(long long)(r0 + rr) * A.xstride + (long long)leaf * A.xleaf + c];
+          const float hr = __double2float_rn(v.x), hi = __double2float_rn(v.y);
+          xh[rr * ncp + c] = make_float2(hr, hi);
+          xl[rr * ncp + c] = make_float2(__double2float_rn(v.x - (double)hr), __double2float_rn(v.y - (double)hi));
+        }
       __syncthreads();
       for (int rw = warp * kRPW; rw < nrow; rw += kW * kRPW) {
-        cacc are[kRPW][kNR], aim[kRPW][kNR];
-        float sre[kRPW][kNR], sim[kRPW][kNR];
+        constexpr int V = kRPW * kNR;
+        CfSum acc[V];  // (row, right-hand side)
         float sig[kRPW];
+        const float2* mrow[kRPW];
+        const __half2* lrow[kRPW];
 #pragma unroll
         for (int i = 0; i < kRPW; ++i) {
-          sig[i] = (rw + i < nrow) ? Sb[rw + i] : 0.f;
-#pragma unroll
-          for (int rr = 0; rr < kNR; ++rr) {
-            are[i][rr] = {0.f, 0.f};
-            aim[i][rr] = {0.f, 0.f};
-            sre[i][rr] = 0.f;
-            sim[i][rr] = 0.f;
-          }
+          int face, j;
+          place(min(rw + i, nrow - 1), face, j);
+          const int r = face * q2 + j;
+          sig[i] = Sb[r];
+          mrow[i] = Mb + (long long)r * A.ld;
+          lrow[i] = Lb + (long long)r * A.ld;
         }
-        for (int c = lane * 2; c < ncp; c += 64) {
+#pragma unroll
+        for (int i = 0; i < V; ++i) acc[i] = {{0.f, 0.f}, {0.f, 0.f}, 0.f, 0.f};
+        // entries one step ahead
+        float4 m[kRPW];
+        uint2 lraw[kRPW];
+        int c = lane * 2;
+        auto fetch = [&](int cc) {
+          if (cc >= ncp) return;
 #pragma unroll
           for (int i = 0; i < kRPW; ++i) {
-            if (rw + i >= nrow) continue;
-            const float4 m = __ldg(reinterpret_cast<const float4*>(Mb + (long long)(rw + i) * A.ld + c));
-            const uint2 lraw = __ldg(reinterpret_cast<const uint2*>(Lb + (long long)(rw + i) * A.ld + c));
-            const float2 l0 = __half22float2(*reinterpret_cast<const __half2*>(&lraw.x));
-            const float2 l1 = __half22float2(*reinterpret_cast<const __half2*>(&lraw.y));
-            const float2 mv[2] = {make_float2(m.x, m.y), make_float2(m.z, m.w)};
+            m[i] = __ldg(reinterpret_cast<const float4*>(mrow[i] + cc));
+            lraw[i] = __ldg(reinterpret_cast<const uint2*>(lrow[i] + cc));
+          }
+        };
+        fetch(c);
+        for (; c < ncp; c += 64) {
+          float4 mc[kRPW];
+          uint2 lc[kRPW];
+#pragma unroll
+          for (int i = 0; i < kRPW; ++i) {
+            mc[i] = m[i];
+            lc[i] = lraw[i];
+          }
+          fetch(c + 64);
+#pragma unroll
+          for (int i = 0; i < kRPW; ++i) {
+            const float2 l0 = __half22float2(*reinterpret_cast<const __half2*>(&lc[i].x));
+            const float2 l1 = __half22float2(*reinterpret_cast<const __half2*>(&lc[i].y));
+            const float2 mv[2] = {make_float2(mc[i].x, mc[i].y), make_float2(mc[i].z, mc[i].w)};
             const float2 lv[2] = {make_float2(l0.x * sig[i], l0.y * sig[i]), make_float2(l1.x * sig[i], l1.y * sig[i])};
 #pragma unroll
             for (int v = 0; v < 2; ++v) {
 #pragma unroll
               for (int rr = 0; rr < kNR; ++rr) {
+                CfSum& a = acc[i * kNR + rr];
                 const float2 h = xh[rr * ncp + c + v], l = xl[rr * ncp + c + v];
                 // main part, exactly: (a + ib)(xr + i xi) with the high parts of x
-                cacc_prod(are[i][rr], mv[v].x, h.x);
-                cacc_prod(are[i][rr], -mv[v].y, h.y);
-                cacc_prod(aim[i][rr], mv[v].x, h.y);
-                cacc_prod(aim[i][rr], mv[v].y, h.x);
+                cacc_prod(a.re, mv[v].x, h.x);
+                cacc_prod(a.re, -mv[v].y, h.y);
+                cacc_prod(a.im, mv[v].x, h.y);
+                cacc_prod(a.im, mv[v].y, h.x);
                 // small part: M32 x_lo + sigma lo x_hi
                 float tr = __fmaf_rn(mv[v].x, l.x, -__fmul_rn(mv[v].y, l.y));
                 tr = __fmaf_rn(lv[v].x, h.x, tr);
@@ -162,50 +221,51 @@ __global__ void __launch_bounds__(kT) cf_gemv_kernel(const CfArgs A, int ncp) {
                 float ti = __fmaf_rn(mv[v].x, l.y, __fmul_rn(mv[v].y, l.x));
                 ti = __fmaf_rn(lv[v].x, h.y, ti);
                 ti = __fmaf_rn(lv[v].y, h.x, ti);
-                sre[i][rr] = __fadd_rn(sre[i][rr], tr);
-                sim[i][rr] = __fadd_rn(sim[i][rr], ti);
+                a.sre = __fadd_rn(a.sre, tr);
+                a.sim = __fadd_rn(a.sim, ti);
               }
             }
           }
         }
-        // warp sums in a fixed order, then value = s + c + small
+        // warp sums: each step exchanges half of the sums still held (plain once one is left)
+        int held = V, first = 0;
 #pragma unroll
-        for (int i = 0; i < kRPW; ++i)
+        for (int o = 16; o > 0; o >>= 1) {
+          if (held > 1) {
+            held >>= 1;
+            const bool up = (lane & o) != 0;
 #pragma unroll
-          for (int rr = 0; rr < kNR; ++rr) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-              are[i][rr] = cacc_merge(are[i][rr], cacc_shfl(are[i][rr], o));
-              aim[i][rr] = cacc_merge(aim[i][rr], cacc_shfl(aim[i][rr], o));
-              sre[i][rr] = __fadd_rn(sre[i][rr], __shfl_xor_sync(0xffffffffu, sre[i][rr], o));
-              sim[i][rr] = __fadd_rn(sim[i][rr], __shfl_xor_sync(0xffffffffu, sim[i][rr], o));
-            }
+            for (int k = 0; k < V / 2; ++k)
+              if (k < held) acc[k] = cf_exchange(cf_pick(up, acc[k + held], acc[k]), cf_pick(up, acc[k], acc[k + held]), o);
+            if (up) first += held;
+          } else {
+            acc[0] = cf_exchange(acc[0], acc[0], o);
           }
-        if (lane == 0) {
-#pragma unroll
-          for (int i = 0; i < kRPW; ++i)
-            if (rw + i < nrow)
-#pragma unroll
-              for (int rr = 0; rr < kNR; ++rr)
-                outs[rr * kCR + rw + i] =
-                    make_double2((double)are[i][rr].s + (double)are[i][rr].c + (double)sre[i][rr],
-                                 (double)aim[i][rr].s + (double)aim[i][rr].c + (double)sim[i][rr]);
         }
+        const int i = first / kNR, rr = first % kNR;
+        if (lane % (32 / V) == 0 && rw + i < nrow)
+          outs[rr * kCR + rw + i] = make_double2((double)acc[0].re.s + (double)acc[0].re.c + (double)acc[0].sre,
+                                                 (double)acc[0].im.s + (double)acc[0].im.c + (double)acc[0].sim);
       }
       __syncthreads();
-      for (int idx = tid; idx < nr * nrow; idx += kT) {
-        const int rr = idx / nrow, jj = idx % nrow, j = row0 + jj;
-        const long long o = (long long)(r0 + rr) * A.nf + dst + j;
-        const double2 gv = outs[rr * kCR + jj];
-        if (A.rhs_mode) {
-          A.y[o] = make_double2(-gv.x, -gv.y);
-        } else {
-          const double2 xv = A.x[(long long)(r0 + rr) * A.xstride + dst + j];
-          const double2 yv = cadd(xv, gv);
-          A.y[o] = A.b ? csub(A.b[o], yv) : yv;
+      for (int l = tid; l < nrow; l += kT) {
+        int face, j;
+        place(l, face, j);
+        const long long dst = (long long)A.g.neighbor(leaf, face) * A.nb + (long long)(face ^ 1) * q2 + j;
+        for (int rr = 0; rr < nr; ++rr) {
+          const long long o = (long long)(r0 + rr) * A.nf + dst;
+          const double2 gv = outs[rr * kCR + l];
+          if (A.rhs_mode) {
+            A.y[o] = make_double2(-gv.x, -gv.y);
+          } else {
+            const double2 xv = A.x[(long long)(r0 + rr) * A.xstride + dst];
+            const double2 yv = cadd(xv, gv);
+            A.y[o] = A.b ? csub(A.b[o], yv) : yv;
+          }
         }
       }
     }
+    __syncthreads();
   }
 }
 
@@ -292,7 +352,9 @@ cudaError_t launch_apply_cf(const hps_handle* h, const double2* x, double2* y, c
   A.nf = h->nf;
   A.nrhs = nrhs;
   A.rhs_mode = 0;
-  A.nitems = (long long)h->nl * 6 * ((A.q2 + kCR - 1) / kCR);
+  A.parts = (6 * A.q2 + kCR - 1) / kCR;
+  A.inv = row_inv(A.q2);
+  A.nitems = (long long)h->nl * A.parts;
   return launch_cf(h, A, (int)round_up(h->ldR, 2), st);
 }
 
@@ -319,7 +381,9 @@ cudaError_t launch_rhs_cf(const hps_handle* h, const double2* s, const double2* 
   A.nf = h->nf;
   A.nrhs = nrhs;
   A.rhs_mode = 1;
-  A.nitems = (long long)h->nl * 6 * ((A.q2 + kCR - 1) / kCR);
+  A.parts = (6 * A.q2 + kCR - 1) / kCR;
+  A.inv = row_inv(A.q2);
+  A.nitems = (long long)h->nl * A.parts;
   return launch_cf(h, A, (int)round_up(h->ldH, 2), st);
 }
 
