@@ -654,7 +654,10 @@ cudaError_t precond_t(const hps_handle* h, const TM* B, const TM* K, const TIN* 
   const long long tstride = h->ct.tsize;
   // FP16 blocks with complex-float output on the uniform layout: both stages in tc_precond16.cu
   if constexpr (std::is_same<TM, __half2>::value && std::is_same<TOUT, float2>::value) {
-    if (precond_tc16_eligible(h, nrhs)) {
+    // (2..63 right-hand sides and ragged multiples only with the handle's own scratch: a caller's
+    // array may be in use while another call on the handle fills its operand rows)
+    const bool own = t == h->pc_scratch || t == h->ks.zt;
+    if (precond_tc16_eligible(h, nrhs) && (own || nrhs == 1 || nrhs % 64 == 0)) {
       constexpr VType kIn = std::is_same<TIN, float2>::value ? VType::C64
                             : std::is_same<TIN, float4>::value ? VType::DF : VType::C128;
       // blocks shared by many clusters: their complex-FP32 copies where they are kept, except for
@@ -753,7 +756,7 @@ cudaError_t precond_t(const hps_handle* h, const TM* B, const TM* K, const TIN* 
     A.cl_slot_begin = h->dct.cl_slot_begin;
     A.slot_lf = h->dct.slot_lf;
     A.cl_tpos = h->dct.cl_tpos;
-  A.split = h->ct.krow_split;
+    A.split = h->ct.krow_split;
     A.nb = h->nb;
     A.q2 = q2;
     A.nf = h->nf;
