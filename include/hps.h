@@ -158,9 +158,10 @@ int hps_nodes(const hps_grid* grid, double* interior_xyz, double* face_xyz, doub
 
 /*
  * Builds the leaf ItI maps R^tau (Gauss basis), the body-load maps H^tau and
- * the preconditioner for one medium.  Per leaf this assembles the leaf system
- * of eq. (leaf) and eliminates it with partial pivoting in FP64 on the
- * device: R_C = I - 2 i eta (A^{-1})_bb, H_C = -2 i eta (A^{-1})_bi, then
+ * the preconditioner for one medium.  Per leaf this solves the leaf system of
+ * eq. (leaf) in FP64 on the device (face unknowns eliminated line by line, the
+ * interior operator inverted with partial pivoting):
+ * R_C = I - 2 i eta (A^{-1})_bb, H_C = -2 i eta (A^{-1})_bi, then
  * R = P R_C P^{-1}, H = P H_C with P the Chebyshev-to-Gauss face
  * interpolation.  The preconditioner uses the same construction with
  * C = kappa^2 (1 - b) replaced by lambda^tau = (max + min)/2 of C over the
@@ -214,8 +215,9 @@ int hps_precond(hps_handle* h, int dtype, const void* r, void* z, int nrhs, void
  * (internal face slots) * q^2 * nrhs * sizeof(element) bytes of it (for the
  * 16^3-leaf, p = 10 grid: 12.6 MB per complex-double right-hand side) and
  * returns HPS_EINVAL with a message when that exceeds the array.  nrhs is not
- * limited by options.max_rhs (the handle's scratch is not used), only by the
- * array.  Every call looks up the array's device address on the current device
+ * limited by options.max_rhs, only by the array.  With FP16 blocks, one
+ * right-hand side or a multiple of 64 up to max_rhs also uses the handle's
+ * operand scratch and must not overlap other calls on the handle.  Every call looks up the array's device address on the current device
  * (a host-side symbol lookup that allocates nothing); the first call on a
  * device may load the library's device code, so make it before any stream
  * capture begins.  The array keeps whatever the last call left in it; nothing
@@ -278,8 +280,8 @@ int hps_gmres_solve(hps_handle* h, int form, const double* s, const double* t, i
  * u_out: nrhs interior vectors (layout of hps_nodes' interior points);
  * u_face_out: NULL or nrhs face-layout vectors of u at the Chebyshev face
  * nodes (hps_nodes' cheb_face_xyz), the rest of the leaf's unknowns.  All
- * device pointers, complex double; one FP64 elimination per leaf and call
- * (cost comparable to hps_setup's).  Synchronous.
+ * device pointers, complex double; one FP64 elimination per leaf and call.
+ * Synchronous.
  */
 int hps_recover(hps_handle* h, const double* s, const double* f, int nrhs, double* u_out,
                 double* u_face_out, void* stream);

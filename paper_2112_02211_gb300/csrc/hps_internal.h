@@ -131,7 +131,6 @@ struct ClusterTables {
   bool uniform = false;
   int nint0 = 0;                     // internal values of every cluster when uniform
   std::vector<int> pos_class;        // [ncl] K block of the member at stage-K position m
-  std::vector<int> leaf_cluster;     // [nleaves] cluster of each leaf
   // FP16 tensor-core stage K (uniform layout): items (block, 128-row tile, first member position,
   // members <= P) for every P = members per item that some number of right-hand sides up to
   // max_rhs needs; list P is [tc16_begin[P], + tc16_count[P]), the blocks of kc_tc last (from
@@ -170,7 +169,6 @@ struct DeviceClusterTables {
   int* bto = nullptr;
   int* bsc = nullptr;
   int* pos_class = nullptr;
-  int* leaf_cluster = nullptr;
   int4* tc16_items = nullptr;
   int* cl_leaves = nullptr;
   int* zoff = nullptr;

@@ -1171,9 +1171,6 @@ void build_cluster_tables(hps_handle* h, int width) {
       }
   ct.max_ext = 0;
   for (int leaf = 0; leaf < h->nl; ++leaf) ct.max_ext = std::max(ct.max_ext, 6 - __builtin_popcount(ct.int_mask[leaf]));
-  ct.leaf_cluster.assign(h->nl, 0);
-  for (int c = 0; c < ct.ncl; ++c)
-    for (int l = ct.cl_leaf_begin[c]; l < ct.cl_leaf_begin[c + 1]; ++l) ct.leaf_cluster[ct.cl_leaves[l]] = c;
   assign_blocks(h, nullptr);
 }
 
@@ -1703,7 +1700,6 @@ int classify_preconditioner(hps_handle* h, const double2* cdiag, cudaStream_t st
   if ((rc = upload(h, h->dct.bto, ct.bto, st))) return rc;
   if ((rc = upload(h, h->dct.bsc, ct.bsc, st))) return rc;
   if ((rc = upload(h, h->dct.pos_class, ct.pos_class, st))) return rc;
-  if ((rc = upload(h, h->dct.leaf_cluster, ct.leaf_cluster, st))) return rc;
   if ((rc = upload(h, h->dct.tc16_items, ct.tc16_items, st))) return rc;
   if ((rc = upload(h, h->dct.cl_leaves, ct.cl_leaves, st))) return rc;
   if ((rc = upload(h, h->dct.zoff, ct.zoff, st))) return rc;
