@@ -366,13 +366,12 @@ def run_gpu(args, dist):
     # double-float (16-byte) input to stage B
     kb, bb = precond_bytes(L, q, 4, 8, in_bytes=16, scale_bytes=4, k_blocks=k_blocks, b_blocks=b_blocks)
     phases = {"apply": a_bytes, "precond_k": kb, "precond_b": bb}
-    rpw = shapes["apply_rows_per_warp"][0][0]
-    kernels = {"apply": f"seg_gemv_kernel<ApplyP<float2,float2,float4>,1,{rpw}> (rows per warp chosen at setup)",
-               "precond_k": "tc_precond16_kernel<false> (every cluster block on the tensor cores, kind::f16, "
+    kernels = {"apply": "stream_apply_kernel<float2,float4,1,R> (maps streamed through shared memory)",
+               "precond_k": "tc_precond16_kernel<16|64> (every cluster block on the tensor cores, kind::f16, "
                             "t scaled per cluster as two FP16 terms) when the clusters are uniform, else "
                             "seg_gemv_kernel<PrecKP<__half2,float2,float2>,1,R>",
-               "precond_b": "prec_b_kernel<__half2,float4,float2,1> (one leaf per item, one thread per row, "
-                            "B transposed)"}
+               "precond_b": "prec_b16_kernel (t written as FP16 operand rows) when the clusters are uniform, else "
+                            "prec_b_kernel<__half2,float4,float2,NR>"}
     roof = {}
     for ph, by in phases.items():
         cnt = prof["count"][ph]
