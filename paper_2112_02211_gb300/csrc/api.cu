@@ -348,7 +348,7 @@ int hps_setup(const hps_grid* g, double kappa, double eta, const double* b, cons
       }
       const size_t ts = (size_t)ct.tsize * o.max_rhs * sizeof(double2);
       if ((r = dalloc(h, &h->pc_scratch, ts))) return r;
-      if (fp16 && o.tc_apply && ct.uniform && ct.nint0 % 32 == 0) {  // operand of the FP16 tensor-core stage K
+      if (fp16 && o.tc_apply && ct.tc16) {  // operand of the FP16 tensor-core stage K
         if ((r = dalloc(h, (void**)&h->op16, (size_t)4 * ct.ncl * o.max_rhs * ct.nint0 * sizeof(__half2)))) return r;
         if ((r = dalloc(h, (void**)&h->tmax, (size_t)ct.ncl * o.max_rhs * sizeof(float)))) return r;
         h->tmax_rhs = o.max_rhs;

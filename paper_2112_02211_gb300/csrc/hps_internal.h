@@ -130,8 +130,12 @@ struct ClusterTables {
   // side, so the multi-RHS tensor-core stage K runs every block in one launch.
   bool uniform = false;
   int nint0 = 0;                     // internal values of every cluster when uniform
+  // Uniform and every cluster 2x2x2 (8 leaves of 3 internal faces), 24 q^2 a multiple of 32: what
+  // tc_precond16.cu and its tables below are written for.  Flat grids (an axis of one leaf) are
+  // uniform too, with 2x2x1 or 2x1x1 clusters; they take the general kernels.
+  bool tc16 = false;
   std::vector<int> pos_class;        // [ncl] K block of the member at stage-K position m
-  // FP16 tensor-core stage K (uniform layout): items (block, 128-row tile, first member position,
+  // FP16 tensor-core stage K (tc16): items (block, 128-row tile, first member position,
   // members <= P) for every P = members per item that some number of right-hand sides up to
   // max_rhs needs; list P is [tc16_begin[P], + tc16_count[P]), the blocks of kc_tc last (from
   // tc16_ntc[P] on)
@@ -140,7 +144,7 @@ struct ClusterTables {
   std::vector<int2> b16_items;       // its stage B: (first position, members <= P, + kTcItem in kc_tc), P = 1, 2, 4
   int b16_begin[5] = {}, b16_count[5] = {};
   int max_members = 0;               // most members of any K block
-  std::vector<int> zoff;             // uniform: [position][24] face-vector offset of each slot
+  std::vector<int> zoff;             // tc16: [position][24] face-vector offset of each slot
   // stage-B work items: leaves sorted by B block, in groups of at most kBGroup that share one
   // block (first index into bgroup_leaves, count)
   std::vector<int> bgroup_leaves;

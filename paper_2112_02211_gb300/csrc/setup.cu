@@ -1354,6 +1354,7 @@ void assign_blocks(hps_handle* h, const std::vector<double2>* lamq) {
     for (int m = 0; m < ct.ncl && ct.uniform; ++m)
       if (ct.cl_tpos[ct.kc_members[m]] != m * nint0) ct.uniform = false;
     ct.nint0 = ct.uniform ? (int)nint0 : 0;
+    ct.tc16 = ct.uniform && nint0 == 24LL * q2 && nint0 % 32 == 0;
   }
   // blocks for the tensor-core path: many members, an even row length (16-byte
   // aligned member rows of complex floats)
@@ -1389,7 +1390,7 @@ void assign_blocks(hps_handle* h, const std::vector<double2>* lamq) {
   for (int k = 0; k < ct.nkc; ++k) ct.max_members = std::max(ct.max_members, ct.kc_mem_begin[k + 1] - ct.kc_mem_begin[k]);
   std::fill(ct.tc16_begin, ct.tc16_begin + 65, 0);
   std::fill(ct.tc16_count, ct.tc16_count + 65, 0);
-  if (ct.uniform && ct.nint0 % 32 == 0) {
+  if (ct.tc16) {
     const int mtiles = (ct.nint0 + 127) / 128;
     for (int m = 0; m < ct.ncl; ++m)
       for (int sl = 0; sl < 24; ++sl) {

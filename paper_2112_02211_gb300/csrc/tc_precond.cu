@@ -424,7 +424,7 @@ cudaError_t launch_precond_tc(const hps_handle* h, const float2* t, float2* z, i
 cudaError_t launch_precond_tc_vec(const hps_handle* h, const float2* t32, float2* z, int nrhs, int* d_error,
                                   cudaStream_t st) {
   const ClusterTables& ct = h->ct;
-  if (!h->Kc32 || !d_error || !ct.uniform) return cudaErrorInvalidValue;
+  if (!h->Kc32 || !d_error || !ct.tc16) return cudaErrorInvalidValue;
   const int P = tc16_members_per_item(kMem, nrhs);
   PkArgs a = {};
   a.nitems = ct.tc16_count[P] - ct.tc16_ntc[P];

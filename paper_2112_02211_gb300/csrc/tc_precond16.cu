@@ -518,7 +518,7 @@ int tc16_members_per_item(int cols, int nrhs) { return nrhs >= cols ? 1 : cols /
 
 bool precond_tc16_eligible(const hps_handle* h, int nrhs) {
   return h->has_precond && h->opt.tc_apply && h->Kc16 && h->Kc16s && h->tc_error && h->tmax && h->op16 &&
-         h->ct.uniform && h->ct.nslots > 0 && (h->ct.nint0 % 32 == 0) && nrhs <= h->tmax_rhs;
+         h->ct.tc16 && nrhs <= h->tmax_rhs;
 }
 
 cudaError_t launch_precond_b16(const hps_handle* h, VType tin, const void* r, float2* z, float2* t32, int nrhs,
