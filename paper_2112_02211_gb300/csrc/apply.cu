@@ -280,7 +280,7 @@ struct PrecKP {
     int nb, q2, split;
     const TIN* t;
     TOUT* z;
-    long long nf, tstride;
+    long long nf, tstride, tmul;  // t of (rhs, cluster) at rhs * tstride + cl_tpos * tmul
     int nrl;   // right-hand sides of the launch: vector rr = member * nrl + rhs
     int nrhs;  // vectors of an item, member group width x nrl
     long long nitems;
@@ -308,7 +308,7 @@ struct PrecKP {
   __device__ static Acc load_x(const Args& A, const ItemInfo& it, int rr, int c) {
     const int m = rr / A.nrl;
     if (m >= it.mask) return czero<Acc>();
-    return cvt<Acc>(A.t[(long long)(rr - m * A.nrl) * A.tstride + A.cl_tpos[A.members[it.xoff + m]] + c]);
+    return cvt<Acc>(A.t[(long long)(rr - m * A.nrl) * A.tstride + A.cl_tpos[A.members[it.xoff + m]] * A.tmul + c]);
   }
   __device__ static void store(const Args& A, const ItemInfo& it, const Acc* outs, int, int tid) {
     if (!outs) return;
@@ -646,30 +646,85 @@ cudaError_t apply_t(const hps_handle* h, const TM* R, const TIN* f, TOUT* y, con
   }, shapes);
 }
 
+// Stage K of every block that the tensor cores do not take (use_tc: all but those of kc_tc), by the
+// batched GEMV.  t of right-hand side r at t + r * rstride, cluster c's part at cl_tpos[c] * tmul.
+template <class TM, class TT>
+cudaError_t stage_k_simt(const hps_handle* h, const TM* K, const float* kscale, const TT* t, long long rstride,
+                         long long tmul, TT* z, int nrhs, bool use_tc, cudaStream_t st) {
+  const int q2 = h->q * h->q;
+  using P = PrecKP<TM, TT, TT>;
+  typename P::Args A;
+  A.K = K;
+  A.kscale = kscale;
+  A.kc_off = h->dct.kc_off;
+  A.kc_slot_begin = h->dct.kc_slot_begin;
+  A.members = h->dct.kc_members;
+  A.cl_slot_begin = h->dct.cl_slot_begin;
+  A.slot_lf = h->dct.slot_lf;
+  A.cl_tpos = h->dct.cl_tpos;
+  A.split = h->ct.krow_split;
+  A.nb = h->nb;
+  A.q2 = q2;
+  A.nf = h->nf;
+  A.tstride = rstride;
+  A.tmul = tmul;
+  const int xcap = xcap_of(h, XCap::StageK);
+  // member groups of width w take 8 / w right-hand sides per launch (fewer where the staged
+  // vectors do not fit in shared memory)
+  int fit = 8;
+  while (fit > 1 && (size_t)fit * (xcap + q2) * sizeof(typename MT<TM>::Acc) > (size_t)220 * 1024) fit >>= 1;
+  for (int g = 0; g < 4; ++g) {
+    const long long n = use_tc ? h->ct.kitems_ntc[g] : (long long)h->ct.kitems[g].size();
+    if (n == 0) continue;
+    A.items = h->dct.kitems[g];
+    A.nitems = n;
+    const int step = std::max(1, fit >> g);
+    for (int r0 = 0; r0 < nrhs; r0 += A.nrl) {
+      A.nrl = next_group<TM>(nrhs - r0, step);
+      A.nrhs = A.nrl << g;
+      A.t = t + (long long)r0 * rstride;
+      A.z = z + (long long)r0 * h->nf;
+      // shapes are tuned for single right-hand sides of the float kernels; otherwise as many rows
+      // per warp as leave work for all 8 warps of an item
+      const bool tuned = h->shapes.tuned && A.nrl == 1 && sizeof(TM) != sizeof(double2);
+      const int rows = (q2 + A.split - 1) / A.split;
+      const LaunchShape sh = tuned ? h->shapes.k[g] : LaunchShape{rows >= 32 ? 4 : rows >= 16 ? 2 : 1, 0};
+      const cudaError_t e = launch_group<P>(A, A.nrhs, xcap, q2, h->nsm, st, &h->prof.launches, h->gate, sh);
+      if (e != cudaSuccess) return e;
+    }
+  }
+  return cudaSuccess;
+}
+
 template <class TM, class TIN, class TOUT>
 cudaError_t precond_t(const hps_handle* h, const TM* B, const TM* K, const TIN* r, TOUT* z, TOUT* t, int nrhs,
                       cudaStream_t st, const float* bscale = nullptr, const float* kscale = nullptr,
                       bool use_tc = false) {
   const int q2 = h->q * h->q;
   const long long tstride = h->ct.tsize;
-  // FP16 blocks with complex-float output on the uniform layout: both stages in tc_precond16.cu
+  // FP16 blocks with complex-float output on 2x2x2 clusters: stage B in tc_precond16.cu, and stage K
+  // there too for one right-hand side and multiples of 64.  In between (and for ragged multiples)
+  // the widely shared blocks take their complex-FP32 copies on the tensor cores and the others the
+  // FP32 kernel: error against the exact product of the same blocks at p = 10 1.9e-7, on the FP16
+  // tensor-core kernel 4.0e-7 (3.5e-6 with one sum per row), which is 103 instead of 514 us for 12
+  // right-hand sides at 8^3 leaves, p = 8, but less than the FP32 that these calls have promised.
   if constexpr (std::is_same<TM, __half2>::value && std::is_same<TOUT, float2>::value) {
-    // (2..63 right-hand sides and ragged multiples only with the handle's own scratch: a caller's
-    // array may be in use while another call on the handle fills its operand rows)
-    const bool own = t == h->pc_scratch || t == h->ks.zt;
-    if (precond_tc16_eligible(h, nrhs) && (own || nrhs == 1 || nrhs % 64 == 0)) {
+    const bool tc16 = precond_tc16_eligible(h, nrhs);
+    if (precond_b16_eligible(h) && (tc16 || !precond_tc_multi_eligible(h, nrhs))) {
       constexpr VType kIn = std::is_same<TIN, float2>::value ? VType::C64
                             : std::is_same<TIN, float4>::value ? VType::DF : VType::C128;
-      // blocks shared by many clusters: their complex-FP32 copies where they are kept, except for
-      // one right-hand side and multiples of 64
-      const bool tc32 = use_tc && nrhs > 1 && nrhs % 64 != 0;
       cudaEvent_t ev = h->prof.begin(st);
-      cudaError_t e = launch_precond_b16(h, kIn, r, z, tc32 ? t : nullptr, nrhs, st);
+      cudaError_t e = launch_precond_b16(h, kIn, r, z, tc16 ? nullptr : t, nrhs, st);
       h->prof.end(HPS_PHASE_PRECOND_B, ev, st);
       if (e != cudaSuccess) return e;
       ev = h->prof.begin(st);
-      e = launch_precond_tc16(h, z, nrhs, tc32, st);
-      if (e == cudaSuccess && tc32) e = launch_precond_tc_vec(h, t, z, nrhs, h->tc_error, st);
+      if (tc16) {
+        e = launch_precond_tc16(h, z, nrhs, st);
+      } else {
+        // t as [position][right-hand side][nint0]; position p is cl_tpos / nint0
+        if (use_tc) e = launch_precond_tc_vec(h, t, z, nrhs, h->tc_error, st);
+        if (e == cudaSuccess) e = stage_k_simt(h, K, kscale, t, h->ct.nint0, nrhs, z, nrhs, use_tc, st);
+      }
       h->prof.end(HPS_PHASE_PRECOND_K, ev, st);
       return e;
     }
@@ -736,70 +791,21 @@ cudaError_t precond_t(const hps_handle* h, const TM* B, const TM* K, const TIN* 
     if (e != cudaSuccess) return e;
   }
   if (h->ct.nslots == 0) return cudaSuccess;
+  cudaEvent_t ev = h->prof.begin(st);
+  cudaError_t e = cudaSuccess;
   if constexpr (std::is_same<TOUT, float2>::value) {
     // many right-hand sides: every block once per 64 of them, on the tensor cores
     if (precond_tc_multi_eligible(h, nrhs)) {
-      cudaEvent_t ev = h->prof.begin(st);
-      const cudaError_t e = launch_precond_tc_multi(h, (const float2*)t, (float2*)z, nrhs, h->tc_error, st);
+      e = launch_precond_tc_multi(h, t, z, nrhs, h->tc_error, st);
       h->prof.end(HPS_PHASE_PRECOND_K, ev, st);
       return e;
     }
+    for (int rhs = 0; use_tc && rhs < nrhs && e == cudaSuccess; ++rhs)
+      e = launch_precond_tc(h, t + (long long)rhs * tstride, z + (long long)rhs * h->nf, h->tc_error, st);
   }
-  {
-    using P = PrecKP<TM, TOUT, TOUT>;
-    typename P::Args A;
-    A.K = K;
-    A.kscale = kscale;
-    A.kc_off = h->dct.kc_off;
-    A.kc_slot_begin = h->dct.kc_slot_begin;
-    A.members = h->dct.kc_members;
-    A.cl_slot_begin = h->dct.cl_slot_begin;
-    A.slot_lf = h->dct.slot_lf;
-    A.cl_tpos = h->dct.cl_tpos;
-    A.split = h->ct.krow_split;
-    A.nb = h->nb;
-    A.q2 = q2;
-    A.nf = h->nf;
-    A.tstride = tstride;
-    const int xcap = xcap_of(h, XCap::StageK);
-    long long* counter = &h->prof.launches;
-    cudaEvent_t ev = h->prof.begin(st);
-    cudaError_t e = cudaSuccess;
-    if (use_tc) {
-      for (int rhs = 0; rhs < nrhs && e == cudaSuccess; ++rhs) {
-        if constexpr (std::is_same<TOUT, float2>::value)
-          e = launch_precond_tc(h, (const float2*)t + (long long)rhs * tstride, (float2*)z + (long long)rhs * h->nf,
-                                h->tc_error, st);
-        else
-          e = cudaErrorInvalidValue;
-      }
-    }
-    // member groups of width w take 8 / w right-hand sides per launch (fewer where the staged
-    // vectors do not fit in shared memory)
-    int fit = 8;
-    while (fit > 1 && (size_t)fit * (xcap + q2) * sizeof(typename MT<TM>::Acc) > (size_t)220 * 1024) fit >>= 1;
-    for (int g = 0; g < 4 && e == cudaSuccess; ++g) {
-      const long long n = use_tc ? h->ct.kitems_ntc[g] : (long long)h->ct.kitems[g].size();
-      if (n == 0) continue;
-      A.items = h->dct.kitems[g];
-      A.nitems = n;
-      const int step = std::max(1, fit >> g);
-      for (int r0 = 0; r0 < nrhs && e == cudaSuccess; r0 += A.nrl) {
-        A.nrl = next_group<TM>(nrhs - r0, step);
-        A.nrhs = A.nrl << g;
-        A.t = t + (long long)r0 * tstride;
-        A.z = z + (long long)r0 * h->nf;
-        // shapes are tuned for single right-hand sides of the float kernels; otherwise as many rows
-        // per warp as leave work for all 8 warps of an item
-        const bool tuned = h->shapes.tuned && A.nrl == 1 && sizeof(TM) != sizeof(double2);
-        const int rows = (q2 + A.split - 1) / A.split;
-        const LaunchShape sh = tuned ? h->shapes.k[g] : LaunchShape{rows >= 32 ? 4 : rows >= 16 ? 2 : 1, 0};
-        e = launch_group<P>(A, A.nrhs, xcap, q2, h->nsm, st, counter, h->gate, sh);
-      }
-    }
-    h->prof.end(HPS_PHASE_PRECOND_K, ev, st);
-    return e;
-  }
+  if (e == cudaSuccess) e = stage_k_simt(h, K, kscale, t, tstride, 1, z, nrhs, use_tc, st);
+  h->prof.end(HPS_PHASE_PRECOND_K, ev, st);
+  return e;
 }
 
 }  // namespace
@@ -1018,6 +1024,7 @@ cudaError_t tune_stage_k(hps_handle* h, const TM* K, const float* kscale, void* 
   A.q2 = h->q * h->q;
   A.nf = h->nf;
   A.tstride = h->ct.tsize;
+  A.tmul = 1;
   A.t = (const float2*)t;
   A.z = (float2*)z;
   for (int g = 0; g < 4; ++g) {

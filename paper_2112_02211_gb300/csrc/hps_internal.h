@@ -136,12 +136,14 @@ struct ClusterTables {
   bool tc16 = false;
   std::vector<int> pos_class;        // [ncl] K block of the member at stage-K position m
   // FP16 tensor-core stage K (tc16): items (block, 128-row tile, first member position,
-  // members <= P) for every P = members per item that some number of right-hand sides up to
-  // max_rhs needs; list P is [tc16_begin[P], + tc16_count[P]), the blocks of kc_tc last (from
-  // tc16_ntc[P] on)
+  // members <= P) for P = members per item of one right-hand side (16, 64) and of multiples of 64
+  // (1); list P is [tc16_begin[P], + tc16_count[P])
   std::vector<int4> tc16_items;
-  int tc16_begin[65] = {}, tc16_count[65] = {}, tc16_ntc[65] = {};
-  std::vector<int2> b16_items;       // its stage B: (first position, members <= P, + kTcItem in kc_tc), P = 1, 2, 4
+  int tc16_begin[65] = {}, tc16_count[65] = {};
+  // the blocks of kc_tc for other numbers of right-hand sides (tc_precond.cu): the same items, list
+  // P = 64 / nrhs of at least one member
+  int vec_begin[65] = {}, vec_count[65] = {};
+  std::vector<int2> b16_items;       // their stage B: (first position, members <= P), P = 1, 2, 4
   int b16_begin[5] = {}, b16_count[5] = {};
   int max_members = 0;               // most members of any K block
   std::vector<int> zoff;             // tc16: [position][24] face-vector offset of each slot
@@ -403,7 +405,7 @@ struct hps_handle {
   __half2* B16 = nullptr;   // FP16 copies of B, rows scaled by 1/B16s[(bcls*6+face)*q^2 + j]
   float* B16s = nullptr;
   void* pc_scratch = nullptr;  // nslots*q^2*max_rhs complex double (precond t buffer)
-  // FP16 tensor-core stage K: stage B's t of each vector (position * nrhs + rhs), scaled by its
+  // FP16 tensor-core stage K (one right-hand side, multiples of 64): stage B's t of each vector (position * nrhs + rhs), scaled by its
   // largest |component| tmax and split into FP16 operand rows [4][vector][nint0] (tc_precond16.cu)
   __half2* op16 = nullptr;
   float* tmax = nullptr;
@@ -476,8 +478,6 @@ void build_cluster_tables(hps_handle* h, int width);
 void assign_blocks(hps_handle* h, const std::vector<double2>* lamq);
 // Shared K blocks with at least this many member clusters run on the tensor cores.
 constexpr int kTcMinMembers = 16;
-// Mark of a stage-B item whose block is in kc_tc.
-constexpr int kTcItem = 256;
 // Leaves per stage-B work item of the general layouts (leaves sharing one B block).
 constexpr int kBGroup = 1;
 // Dynamic shared memory a block may opt into on sm_103 (227 KB).
@@ -519,15 +519,16 @@ cudaError_t launch_precond_tc(const hps_handle* h, const float2* t, float2* z, i
 // in one launch (complex-FP32 blocks, one TF32 product): the GEMM of each K_c against the
 // columns (member cluster, right-hand side).  Needs ct.uniform.  t: [rhs][tsize], z: [rhs][nf].
 bool precond_tc_multi_eligible(const hps_handle* h, int nrhs);
-// The preconditioner with FP16 blocks on the uniform layout (tc_precond16.cu): stage B into
-// FP16 operand rows, stage K of every cluster block on the tensor cores; any nrhs up to max_rhs.
+// The preconditioner with FP16 blocks on 2x2x2 clusters (tc_precond16.cu).  Stage B for any nrhs:
+// with t32 the vectors t themselves, [vector][nint0], without it the FP16 operand rows of stage K,
+// which runs every cluster block on the tensor cores for one right-hand side or a multiple of 64
+// (up to max_rhs).
+bool precond_b16_eligible(const hps_handle* h);
 bool precond_tc16_eligible(const hps_handle* h, int nrhs);
 int tc16_members_per_item(int cols, int nrhs);
-// t32: where stage B leaves t itself, [vector][nint0], for the blocks of kc_tc (or nullptr);
-// skip_tc: without those blocks (launch_precond_tc_vec applies them).
 cudaError_t launch_precond_b16(const hps_handle* h, VType tin, const void* r, float2* z, float2* t32, int nrhs,
                                cudaStream_t st);
-cudaError_t launch_precond_tc16(const hps_handle* h, float2* z, int nrhs, bool skip_tc, cudaStream_t st);
+cudaError_t launch_precond_tc16(const hps_handle* h, float2* z, int nrhs, cudaStream_t st);
 // Stage K of the shared blocks ct.kc_tc (complex-FP32 blocks, one TF32 product) for nrhs right-hand
 // sides in one launch; uniform layout, t32 [vector][nint0].
 cudaError_t launch_precond_tc_vec(const hps_handle* h, const float2* t32, float2* z, int nrhs, int* d_error,

@@ -1381,15 +1381,15 @@ void assign_blocks(hps_handle* h, const std::vector<double2>* lamq) {
   for (auto& v : ct.kitems) v.clear();
   std::vector<char> is_tc(ct.nkc, 0);
   for (int k : ct.kc_tc) is_tc[k] = 1;
-  // FP16 tensor-core stage K items: per block, per 128-row tile, its members P at a time
+  // tensor-core stage K items: per block, per 128-row tile, its members P at a time
   // (consecutive items reuse the block's row tile from L2)
   ct.tc16_items.clear();
   ct.zoff.clear();
   ct.b16_items.clear();
   ct.max_members = 0;
   for (int k = 0; k < ct.nkc; ++k) ct.max_members = std::max(ct.max_members, ct.kc_mem_begin[k + 1] - ct.kc_mem_begin[k]);
-  std::fill(ct.tc16_begin, ct.tc16_begin + 65, 0);
   std::fill(ct.tc16_count, ct.tc16_count + 65, 0);
+  std::fill(ct.vec_count, ct.vec_count + 65, 0);
   if (ct.tc16) {
     const int mtiles = (ct.nint0 + 127) / 128;
     for (int m = 0; m < ct.ncl; ++m)
@@ -1401,22 +1401,23 @@ void assign_blocks(hps_handle* h, const std::vector<double2>* lamq) {
       ct.b16_begin[P] = (int)ct.b16_items.size();
       for (int k = 0; k < ct.nkc; ++k)
         for (int p0 = ct.kc_mem_begin[k]; p0 < ct.kc_mem_begin[k + 1]; p0 += P)
-          ct.b16_items.push_back(make_int2(p0, std::min(P, ct.kc_mem_begin[k + 1] - p0) + (is_tc[k] ? kTcItem : 0)));
+          ct.b16_items.push_back(make_int2(p0, std::min(P, ct.kc_mem_begin[k + 1] - p0)));
       ct.b16_count[P] = (int)ct.b16_items.size() - ct.b16_begin[P];
     }
-    for (int e = 0; e < 2 * std::min(64, h->opt.max_rhs); ++e) {
-      const int P = tc16_members_per_item(e & 1 ? 64 : 16, e / 2 + 1);
-      if (ct.tc16_count[P]) continue;
-      ct.tc16_begin[P] = (int)ct.tc16_items.size();
-      for (int pass = 0; pass < 2; ++pass) {
-        for (int k = 0; k < ct.nkc; ++k)
-          for (int mt = 0; is_tc[k] == pass && mt < mtiles; ++mt)
-            for (int p0 = ct.kc_mem_begin[k]; p0 < ct.kc_mem_begin[k + 1]; p0 += P)
-              ct.tc16_items.push_back(make_int4(k, mt, p0, std::min(P, ct.kc_mem_begin[k + 1] - p0)));
-        if (pass == 0) ct.tc16_ntc[P] = (int)ct.tc16_items.size() - ct.tc16_begin[P];
-      }
-      ct.tc16_count[P] = (int)ct.tc16_items.size() - ct.tc16_begin[P];
+    auto add = [&](int P, bool tc_only, int* begin, int* count) {
+      if (count[P]) return;
+      begin[P] = (int)ct.tc16_items.size();
+      for (int k = 0; k < ct.nkc; ++k)
+        for (int mt = 0; (!tc_only || is_tc[k]) && mt < mtiles; ++mt)
+          for (int p0 = ct.kc_mem_begin[k]; p0 < ct.kc_mem_begin[k + 1]; p0 += P)
+            ct.tc16_items.push_back(make_int4(k, mt, p0, std::min(P, ct.kc_mem_begin[k + 1] - p0)));
+      count[P] = (int)ct.tc16_items.size() - begin[P];
+    };
+    for (int cols : {16, 64}) {
+      add(tc16_members_per_item(cols, 1), false, ct.tc16_begin, ct.tc16_count);
+      add(tc16_members_per_item(cols, 64), false, ct.tc16_begin, ct.tc16_count);
     }
+    for (int nrhs = 2; nrhs <= 64; ++nrhs) add(tc16_members_per_item(64, nrhs), true, ct.vec_begin, ct.vec_count);
   }
   for (int pass = 0; pass < 2; ++pass) {
     for (int k = 0; k < ct.nkc; ++k) {

@@ -23,8 +23,8 @@
 //
 // Several right-hand sides on the uniform layout (VEC): the vectors (member, right-hand side) of a
 // block are consecutive rows of t ([position][rhs][nint]), so an item is (block, 128-row tile, up
-// to 64 vectors) from the list of the FP16 path (tc_precond16.cu) and all blocks and right-hand
-// sides run in one launch; one launch per block and right-hand side took 8 us each.
+// to 64 vectors) and all blocks and right-hand sides run in one launch; one launch per block and
+// right-hand side took 8 us each.
 //
 // Kernel (one CTA per SM, persistent over items = (128-row tile, 64-member tile)):
 //   warp 0       TMA producer: A tile (128 rows x 32 floats) and T tile
@@ -427,7 +427,7 @@ cudaError_t launch_precond_tc_vec(const hps_handle* h, const float2* t32, float2
   if (!h->Kc32 || !d_error || !ct.tc16) return cudaErrorInvalidValue;
   const int P = tc16_members_per_item(kMem, nrhs);
   PkArgs a = {};
-  a.nitems = ct.tc16_count[P] - ct.tc16_ntc[P];
+  a.nitems = ct.vec_count[P];
   if (a.nitems == 0) return cudaSuccess;
   auto encode = encoder();
   if (!encode) return cudaErrorNotSupported;
@@ -463,7 +463,7 @@ cudaError_t launch_precond_tc_vec(const hps_handle* h, const float2* t32, float2
   a.kblocks = (2 * nint + kTileK - 1) / kTileK;
   a.q2 = h->q * h->q;
   a.nb = h->nb;
-  a.items = h->dct.tc16_items + ct.tc16_begin[P] + ct.tc16_ntc[P];
+  a.items = h->dct.tc16_items + ct.vec_begin[P];
   a.zoff = h->dct.zoff;
   a.rtiles = (nrhs + kMem - 1) / kMem;
   a.nrhs = nrhs;

@@ -1,20 +1,26 @@
-// The cluster preconditioner on the uniform layout with FP16 blocks (z = J^{-1} r, Sec. 4,
-// Algorithm 4 in face form), for any number of right-hand sides, in two launches:
+// The cluster preconditioner with FP16 blocks where every cluster is 2x2x2 (z = J^{-1} r, Sec. 4,
+// Algorithm 4 in face form):
 //
-// * stage B (prec_b16_kernel): a thread-block cluster of 4 CTAs per up to 4 vectors that share
-//   their B blocks (right-hand sides, or members of one K block), two of the 8 leaves a CTA, forms
-//   t = r_int - B r_ext (SIMT, two rows per thread, B stored transposed), finds the largest component t_max through distributed shared memory and
-//   writes t / t_max as the tensor cores' operand: two FP16 terms hi + lo (~22 bits), each as the
-//   rows conj(t) and the re/im swap of t.  Doing this here, once, replaces the conversion that
+// * stage B (prec_b16_kernel), any number of right-hand sides: a thread-block cluster of 4 CTAs per
+//   up to 4 vectors that share their B blocks (right-hand sides, or members of one K block), two of
+//   the 8 leaves a CTA, forms t = r_int - B r_ext (SIMT, two rows per thread, B stored transposed).
+//   For the tensor-core stage K it finds the largest component t_max through distributed shared
+//   memory and writes t / t_max as the tensor cores' operand: two FP16 terms hi + lo (~22 bits), each
+//   as the rows conj(t) and the re/im swap of t.  Doing this here, once, replaces the conversion that
 //   every 128-row tile of stage K would repeat (7 times at p = 8) on its way through shared memory.
-// * stage K (tc_precond16_kernel): z_int = K_c t on the 5th-generation tensor cores
+//   Otherwise it writes t itself, for the SIMT stage K and the TF32 one of widely shared blocks.
+// * stage K (tc_precond16_kernel), one right-hand side or a multiple of 64:
+//   z_int = K_c t on the 5th-generation tensor cores
 //   (tcgen05.mma.kind::f16, FP32 accumulation in TMEM).  A = K_c's FP16 copy (each row divided by
 //   its FP32 scale s_row) as a real n x 2n matrix of interleaved (re, im) halves; B = the operand
 //   rows; A B_hi + A B_lo = [Re | Im] of K_c t / (s_row t_max), multiplied back by s_row and t_max
 //   in the epilogue.  K_c carries 2^-11 relative rounding (a fixed matrix); t is kept to ~2^-22,
 //   so the result stays linear in t to FP32 level.  GMRES applies the preconditioner to V y in its
 //   update and assumes that this equals sum_j y_j M^{-1} v_j; with one FP16 rounding of t (2^-11,
-//   input-dependent) that would hold only to ~2e-4.
+//   input-dependent) that would hold only to ~2e-4.  The tensor cores' sums truncate, so they are
+//   kept short and added up in FP32 (kChunk); that is still 2e-7 to 4e-7 of the exact product of the
+//   same blocks (p = 4 .. 12) where FP32 products and sums stay within 0.7e-7 to 2.4e-7, so other
+//   numbers of right-hand sides take those (apply.cu).
 //
 // Vector v = position * nrhs + rhs (position: place of the member cluster in stage-K order), so
 // the vectors of the clusters that share a block are consecutive.  A stage-K item is (block,
@@ -30,7 +36,7 @@
 // MMA issuer, warps 2..5 the epilogue.  Every wait is bounded; on a time-out the CTA sets the error
 // word, waits (bounded) for its own copies and MMAs, frees TMEM and returns.
 //
-// Needs the uniform layout (every cluster 2x2x2, 24 q^2 a multiple of 32).
+// Needs ClusterTables::tc16 (every cluster 2x2x2, 24 q^2 a multiple of 32).
 #include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -61,10 +67,10 @@ struct PrecB16Args {
   const int* bsc;         // per leaf, internal faces: row-scale bases
   const int* members;     // clusters in stage-K position order
   const int* leaves;      // 8 leaves of each cluster
-  const int2* items;      // (first position, members), members of one K block; + kTcItem: a block of kc_tc
+  const int2* items;      // (first position, members), members of one K block
   const TIN* r;
   float2* z;
-  float2* t32;            // optional [vector][n]: t itself for the vectors of kc_tc blocks
+  float2* t32;            // [vector][n]: t itself, or nullptr: op and tmax
   __half2* op;            // operand rows [4][ncl * nrhs][n]: conj hi, swap hi, conj lo, swap lo
   float* tmax;            // [ncl * nrhs]
   int q2, n, ncl, nrhs, rtiles;
@@ -90,9 +96,7 @@ __global__ void __cluster_dims__(kBCluster, 1, 1) __maxnreg__(80) prec_b16_kerne
   __shared__ long long roff[NR];
   __shared__ int vpos[NR];
   const int item = blockIdx.x / kBCluster, l0 = (blockIdx.x % kBCluster) * 2;
-  int2 it = A.items[item / A.rtiles];
-  const bool keep = A.t32 && it.y >= kTcItem;
-  it.y &= kTcItem - 1;
+  const int2 it = A.items[item / A.rtiles];
   const int first = (item % A.rtiles) * NR;
   const int nr = min(NR, it.y * A.nrhs - first), v0 = it.x * A.nrhs + first;
   const int tid = threadIdx.x, nt = blockDim.x;
@@ -190,10 +194,11 @@ __global__ void __cluster_dims__(kBCluster, 1, 1) __maxnreg__(80) prec_b16_kerne
 #pragma unroll
       for (int rr = 0; rr < NR; ++rr) {
         tv[i][rr] = csub(tv[i][rr], make_float2(acc[i][rr].x * sc[i], acc[i][rr].y * sc[i]));
-        if (keep && rr < nr) A.t32[(long long)(v0 + rr) * n + to[i][rr]] = tv[i][rr];
+        if (A.t32 && rr < nr) A.t32[(long long)(v0 + rr) * n + to[i][rr]] = tv[i][rr];
         if (rr < nr) mx[rr] = fmaxf(mx[rr], fmaxf(fabsf(tv[i][rr].x), fabsf(tv[i][rr].y)));
       }
   }
+  if (A.t32) return;  // the same for every CTA of the cluster
 #pragma unroll
   for (int rr = 0; rr < NR; ++rr) {
 #pragma unroll
@@ -294,6 +299,12 @@ constexpr int kStages = 4;
 constexpr int kTileM = 128;
 constexpr int kKHalves = 64;            // K extent of a stage (128 bytes of FP16)
 constexpr int kABytes = kTileM * 128;   // 16 KB
+// Stages whose products the tensor cores add up before the sums move to FP32 registers.  The
+// accumulation truncates, a loss of about one unit in the last place per step in one direction, so
+// long sums drift.  Measured against the exact product of the same FP16 blocks, 2^3 leaves at p = 10
+// (48 stages): 3.5e-6 with one sum, 4.0e-7 with 12 of 4 stages; 12^3 leaves at p = 8, both stages of
+// one right-hand side: 39.7 us and 39.3 us.
+constexpr int kChunk = 4;
 constexpr int kThreads = 192;
 
 template <int COLS> struct Shape {
@@ -412,16 +423,18 @@ __global__ void __launch_bounds__(kThreads, COLS == 16 ? 2 : 1)
       long long it = 0;
       long long local = 0;
       bool ok = true;
-      for (long long item = blockIdx.x; item < a.nitems && ok; item += gridDim.x, ++local) {
-        const int b = (int)(local & 1);
-        const uint32_t acc = tmem + (uint32_t)(b * S::kN);
-        if (local >= 2 && !mbar_wait(&bars->acc_empty[b], (uint32_t)(((local >> 1) - 1) & 1))) {
-          fail();
-          ok = false;
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      for (long long item = blockIdx.x; item < a.nitems && ok; item += gridDim.x) {
         for (int kb = 0; kb < a.kblocks; ++kb, ++it) {
+          const int b = (int)(local & 1);
+          const uint32_t acc = tmem + (uint32_t)(b * S::kN);
+          if (kb % kChunk == 0) {
+            if (local >= 2 && !mbar_wait(&bars->acc_empty[b], (uint32_t)(((local >> 1) - 1) & 1))) {
+              fail();
+              ok = false;
+              break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          }
           const int s = (int)(it % kStages);
           const uint32_t ph = (uint32_t)((it / kStages) & 1);
           if (bars->abort || !mbar_wait(&bars->full[s], ph)) {
@@ -434,12 +447,14 @@ __global__ void __launch_bounds__(kThreads, COLS == 16 ? 2 : 1)
 #pragma unroll
           for (int kk = 0; kk < kKHalves / 16; ++kk) {
             const uint32_t off = kk * 32;  // 16 halves
-            mma_f16(acc, smem_desc(aa + off), smem_desc(bb + off), idesc, (kb == 0 && kk == 0) ? 0u : 1u);
+            mma_f16(acc, smem_desc(aa + off), smem_desc(bb + off), idesc, (kb % kChunk == 0 && kk == 0) ? 0u : 1u);
           }
           mma_commit(&bars->empty[s]);
+          if (kb % kChunk == kChunk - 1 || kb == a.kblocks - 1) {
+            mma_commit(&bars->acc_full[b]);
+            ++local;
+          }
         }
-        if (!ok) break;
-        mma_commit(&bars->acc_full[b]);
       }
       mma_commit(&bars->drain);
       if (!mbar_wait(&bars->drain, 0)) fail();
@@ -448,27 +463,19 @@ __global__ void __launch_bounds__(kThreads, COLS == 16 ? 2 : 1)
   } else {
     // ---------------- epilogue: warps 2..5, each on the 32 TMEM lanes that it may read ----------------
     const int ew = warp & 3;
+    const int chunks = (a.kblocks + kChunk - 1) / kChunk;
     long long local = 0;
-    for (long long item = blockIdx.x; item < a.nitems; item += gridDim.x, ++local) {
-      const int b = (int)(local & 1);
-      if (bars->abort || !mbar_wait(&bars->acc_full[b], (uint32_t)((local >> 1) & 1))) {
-        fail();
-        break;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    bool ok = true;
+    for (long long item = blockIdx.x; item < a.nitems && ok; item += gridDim.x) {
       int blk, mt, v0, cnt;
       decode<COLS>(a, item, blk, mt, v0, cnt);
       const int row = mt * kTileM + ew * 32 + lane;
-      const uint32_t taddr = tmem + ((uint32_t)(ew * 32) << 16) + (uint32_t)(b * S::kN);
       const float ks = (row < a.nint) ? a.kscale[(long long)a.kc_slot_begin[blk] * a.q2 + row] : 0.f;
       const int sl = row / a.q2, j = row - sl * a.q2;
       const int* zo = a.zoff + sl;
-      for (int h0 = 0; h0 < cnt; h0 += 16) {
-        // offsets and scales of 16 vectors first (independent loads), then the accumulators
-        int off[16];
-        float f[16];
+      // offsets and scales of 16 vectors
+      auto place = [&](int h0, int (&off)[16], float (&f)[16]) {
         int pos = (v0 + h0) / a.nrhs, rhs = v0 + h0 - pos * a.nrhs;
-        const int first = rhs;
 #pragma unroll
         for (int c = 0; c < 16; ++c) {
           const bool on = h0 + c < cnt && row < a.nint;
@@ -479,29 +486,58 @@ __global__ void __launch_bounds__(kThreads, COLS == 16 ? 2 : 1)
             ++pos;
           }
         }
-        uint32_t reh[16], imh[16], rel[16], iml[16];
-        tmem_ld16(taddr + h0, reh);
-        tmem_ld16(taddr + COLS + h0, imh);
-        tmem_ld16(taddr + 2 * COLS + h0, rel);
-        tmem_ld16(taddr + 3 * COLS + h0, iml);
-        tmem_wait_ld();
-        rhs = first;
+      };
+      int off[16];
+      float f[16];
+      if (COLS == 16) place(0, off, f);  // in flight during the sums
+      float re[COLS], im[COLS];
+#pragma unroll
+      for (int c = 0; c < COLS; ++c) re[c] = im[c] = 0.f;
+      for (int ch = 0; ch < chunks; ++ch, ++local) {
+        const int b = (int)(local & 1);
+        if (bars->abort || !mbar_wait(&bars->acc_full[b], (uint32_t)((local >> 1) & 1))) {
+          fail();
+          ok = false;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t taddr = tmem + ((uint32_t)(ew * 32) << 16) + (uint32_t)(b * S::kN);
+#pragma unroll
+        for (int h0 = 0; h0 < COLS; h0 += 16) {
+          if (h0 >= cnt) break;
+          uint32_t reh[16], imh[16], rel[16], iml[16];
+          tmem_ld16(taddr + h0, reh);
+          tmem_ld16(taddr + COLS + h0, imh);
+          tmem_ld16(taddr + 2 * COLS + h0, rel);
+          tmem_ld16(taddr + 3 * COLS + h0, iml);
+          tmem_wait_ld();
+#pragma unroll
+          for (int c = 0; c < 16; ++c) {
+            re[h0 + c] += __uint_as_float(reh[c]) + __uint_as_float(rel[c]);
+            im[h0 + c] += __uint_as_float(imh[c]) + __uint_as_float(iml[c]);
+          }
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->acc_empty[b]);
+      }
+      if (!ok) break;
+#pragma unroll
+      for (int h0 = 0; h0 < COLS; h0 += 16) {
+        if (h0 >= cnt) break;
+        if (COLS > 16) place(h0, off, f);
+        int rhs = (v0 + h0) % a.nrhs;
         if (row < a.nint) {
 #pragma unroll
           for (int c = 0; c < 16; ++c) {
             if (h0 + c < cnt) {
               const float w = ks * f[c];
-              a.z[(long long)rhs * a.nf + off[c] + j] =
-                  make_float2((__uint_as_float(reh[c]) + __uint_as_float(rel[c])) * w,
-                              (__uint_as_float(imh[c]) + __uint_as_float(iml[c])) * w);
+              a.z[(long long)rhs * a.nf + off[c] + j] = make_float2(re[h0 + c] * w, im[h0 + c] * w);
             }
             if (++rhs == a.nrhs) rhs = 0;
           }
         }
       }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&bars->acc_empty[b]);
     }
   }
 
@@ -516,20 +552,23 @@ __global__ void __launch_bounds__(kThreads, COLS == 16 ? 2 : 1)
 
 int tc16_members_per_item(int cols, int nrhs) { return nrhs >= cols ? 1 : cols / nrhs; }
 
+bool precond_b16_eligible(const hps_handle* h) {
+  return h->has_precond && h->opt.tc_apply && h->Kc16 && h->Kc16s && h->tc_error && h->ct.tc16;
+}
+
 bool precond_tc16_eligible(const hps_handle* h, int nrhs) {
-  return h->has_precond && h->opt.tc_apply && h->Kc16 && h->Kc16s && h->tc_error && h->tmax && h->op16 &&
-         h->ct.tc16 && nrhs <= h->tmax_rhs;
+  return precond_b16_eligible(h) && h->tmax && h->op16 && nrhs <= h->tmax_rhs && (nrhs == 1 || nrhs % 64 == 0);
 }
 
 cudaError_t launch_precond_b16(const hps_handle* h, VType tin, const void* r, float2* z, float2* t32, int nrhs,
                                cudaStream_t st) {
-  if (!precond_tc16_eligible(h, nrhs)) return cudaErrorInvalidValue;
+  if (!(t32 ? precond_b16_eligible(h) : precond_tc16_eligible(h, nrhs))) return cudaErrorInvalidValue;
   if (tin == VType::C64) return stage_b16(h, (const float2*)r, z, t32, nrhs, st);
   if (tin == VType::DF) return stage_b16(h, (const float4*)r, z, t32, nrhs, st);
   return stage_b16(h, (const double2*)r, z, t32, nrhs, st);
 }
 
-cudaError_t launch_precond_tc16(const hps_handle* h, float2* z, int nrhs, bool skip_tc, cudaStream_t st) {
+cudaError_t launch_precond_tc16(const hps_handle* h, float2* z, int nrhs, cudaStream_t st) {
   const ClusterTables& ct = h->ct;
   if (!precond_tc16_eligible(h, nrhs)) return cudaErrorInvalidValue;
   auto encode = encoder();
@@ -539,12 +578,10 @@ cudaError_t launch_precond_tc16(const hps_handle* h, float2* z, int nrhs, bool s
   if ((reinterpret_cast<uintptr_t>(h->Kc16) | reinterpret_cast<uintptr_t>(h->op16)) % 16 != 0 || (4LL * nint) % 16 != 0)
     return cudaErrorInvalidValue;
   // Items of 16 vectors unless that takes more than twice as many items as 64 would (blocks shared
-  // by many vectors).  Measured per application of stage K at p = 8:
-  // 12^3 leaves of a bump medium, one right-hand side (few blocks, up to ~190 members) 18.9 us at 16
-  // against 51 us at 64 columns; 8^3 leaves, 12 right-hand sides (45 blocks) 37 against 73 us.
+  // by many vectors).  Measured per application of stage K at p = 8: 12^3 leaves of a bump medium,
+  // one right-hand side (few blocks, up to ~190 members) 18.9 us at 16 against 51 us at 64 columns.
   auto count_of = [&](int cols) {
-    const int p = tc16_members_per_item(cols, nrhs);
-    return (long long)(skip_tc ? ct.tc16_ntc[p] : ct.tc16_count[p]) * ((nrhs + cols - 1) / cols);
+    return (long long)ct.tc16_count[tc16_members_per_item(cols, nrhs)] * ((nrhs + cols - 1) / cols);
   };
   const int cols = count_of(16) <= 2 * count_of(64) ? 16 : 64;
   const int P = tc16_members_per_item(cols, nrhs);
@@ -579,7 +616,6 @@ cudaError_t launch_precond_tc16(const hps_handle* h, float2* z, int nrhs, bool s
   a.error = h->tc_error;
   a.gate = h->gate;
   a.nitems = count_of(cols);
-  if (a.nitems == 0) return cudaSuccess;
   auto run = [&](auto kern, int stage_bytes, int per_sm) -> cudaError_t {
     const int smem = kStages * stage_bytes + (int)sizeof(Bars) + 1024;
     const cudaError_t e = allow_dynamic_smem((const void*)kern, smem);
