@@ -215,9 +215,10 @@ int hps_precond(hps_handle* h, int dtype, const void* r, void* z, int nrhs, void
  * (internal face slots) * q^2 * nrhs * sizeof(element) bytes of it (for the
  * 16^3-leaf, p = 10 grid: 12.6 MB per complex-double right-hand side) and
  * returns HPS_EINVAL with a message when that exceeds the array.  nrhs is not
- * limited by options.max_rhs, only by the array.  With FP16 blocks, one
- * right-hand side or a multiple of 64 up to max_rhs also uses the handle's
- * operand scratch and must not overlap other calls on the handle.  Every call looks up the array's device address on the current device
+ * limited by options.max_rhs (the handle's scratch is not used), only by the
+ * array.  (FP16 blocks, one right-hand side or a multiple of 64: the tensor-core
+ * kernel needs 16 bytes per value; where only sizeof(element) fit, the call runs
+ * in FP32.)  Every call looks up the array's device address on the current device
  * (a host-side symbol lookup that allocates nothing); the first call on a
  * device may load the library's device code, so make it before any stream
  * capture begins.  The array keeps whatever the last call left in it; nothing

@@ -116,7 +116,7 @@ void free_handle(hps_handle* h) {
                   h->dct.int_mask, h->dct.b_off, h->dct.leaf_bcls, h->dct.bc_rep, h->dct.kc_off,
                   h->dct.kc_slot_begin, h->dct.kslot_class, h->dct.kc_members, h->dct.kitems[0], h->dct.kitems[1],
                   h->dct.kitems[2], h->dct.kitems[3], h->dct.cl_tpos, h->dct.lf_tpos, h->dct.brd, h->dct.bto,
-                  h->dct.bsc, h->dct.pos_class, h->dct.tc16_items, h->dct.cl_leaves, h->dct.zoff, h->dct.b16_items, h->op16, h->dct.bgroup_leaves, h->dct.bgroups, h->tmax, h->fs.d_cls, h->fs.Sinv64, h->fs.Sinv32, h->fs.eig};
+                  h->dct.bsc, h->dct.pos_class, h->dct.tc16_items, h->dct.cl_leaves, h->dct.zoff, h->dct.b16_items, h->dct.bgroup_leaves, h->dct.bgroups, h->fs.d_cls, h->fs.Sinv64, h->fs.Sinv32, h->fs.eig};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (h->stream) cudaStreamDestroy(h->stream);
@@ -346,13 +346,7 @@ int hps_setup(const hps_grid* g, double kappa, double eta, const double* b, cons
         HPS_CUDA_TRY(cudaMemsetAsync(h->Kc16, 0, ke * sizeof(__half2), st));
         HPS_CUDA_TRY(cudaMemsetAsync(h->B16, 0, be * sizeof(__half2), st));
       }
-      const size_t ts = (size_t)ct.tsize * o.max_rhs * sizeof(double2);
-      if ((r = dalloc(h, &h->pc_scratch, ts))) return r;
-      if (fp16 && o.tc_apply && ct.tc16) {  // operand of the FP16 tensor-core stage K
-        if ((r = dalloc(h, (void**)&h->op16, (size_t)4 * ct.ncl * o.max_rhs * ct.nint0 * sizeof(__half2)))) return r;
-        if ((r = dalloc(h, (void**)&h->tmax, (size_t)ct.ncl * o.max_rhs * sizeof(float)))) return r;
-        h->tmax_rhs = o.max_rhs;
-      }
+      if ((r = dalloc(h, &h->pc_scratch, precond_scratch_bytes(ct, o.max_rhs)))) return r;
       if ((r = build_preconditioner(h, dc, st))) return r;
       if (fp16 && (r = build_precond_fp16(h, st))) return r;
     }
@@ -392,7 +386,7 @@ size_t hps_setup_bytes(const hps_grid* g, const hps_options* opt, int nrhs) {
   if (want32)  // FP16 remainders of R and H and their row scales; FP32 H beside FP64 H
     bytes += (rel + hel) * sizeof(__half2) + (size_t)2 * h.nl * h.nb * sizeof(float) + (o.lean ? 0 : hel * c8);
   const int q2 = h.q * h.q;
-  size_t nslots = 0, tsize = 1;
+  size_t nslots = 0;
   if (o.cluster == 2) {
     build_cluster_tables(&h, 2);
     const ClusterTables& ct = h.ct;
@@ -412,14 +406,12 @@ size_t hps_setup_bytes(const hps_grid* g, const hps_options* opt, int nrhs) {
       bytes += (o.tc_apply && ct.uniform && o.max_rhs >= 64) ? (size_t)ct.kc_elems * c8
                                                               : std::min<size_t>((size_t)ct.kc_elems * c8, (size_t)4 << 30);
     bytes += (size_t)ct.ncl * sizeof(int) +                                  // position -> block
-             (size_t)ct.ncl * o.max_rhs * (sizeof(float) + (size_t)4 * ct.nint0 * sizeof(__half2)) +  // FP16 operand
              ct.tc16_items.size() * sizeof(int4) + (ct.cl_leaves.size() + ct.zoff.size() + 2 * ct.b16_items.size()) * sizeof(int) +
              (size_t)h.nl * (sizeof(int) + sizeof(int2));  // stage-B groups
     if (want32 && (o.precond_fp16 || o.lean))
       bytes += (size_t)(ct.kc_elems + ct.b_elems) * sizeof(__half2) + nslots * q2 * sizeof(float) +
                (size_t)h.nl * 6 * q2 * sizeof(float);
-    bytes += (size_t)ct.tsize * o.max_rhs * c16;
-    tsize = ct.tsize;
+    bytes += precond_scratch_bytes(ct, o.max_rhs);
   }
   bytes += (size_t)h.nint * c16 + sizeof(int);  // medium C kept for recovery, error word
   if (o.full_system)  // S~^{-1} per leaf at most, class index, lambda values, Algorithm 3 tables
@@ -429,7 +421,7 @@ size_t hps_setup_bytes(const hps_grid* g, const hps_options* opt, int nrhs) {
   const int M1 = o.restart + 1;
   const size_t vb = (size_t)nrhs * h.nf * c16;
   const long long nblk = (h.nf + 1023) / 1024;
-  bytes += vb * (M1 + 5) + tsize * nrhs * c16 + (size_t)nrhs * nblk * M1 * c16 +
+  bytes += vb * (M1 + 5) + precond_scratch_bytes(h.ct, nrhs) + (size_t)nrhs * nblk * M1 * c16 +
            (size_t)o.max_rhs * (h.nint + h.nf) * c16 + (size_t)nrhs * (3 * M1 + 4 * o.restart + 8) * c16 +
            (size_t)nrhs * std::max<long long>(256, 8 * nblk) * sizeof(double);
   // transient setup workspace (largest phase) + medium staging
@@ -579,25 +571,26 @@ int hps_precond(hps_handle* h, int dtype, const void* r, void* z, int nrhs, void
     HPS_CUDA_TRY(cudaMemcpyAsync(z, r, (size_t)nrhs * h->nf * es, cudaMemcpyDeviceToDevice, st));
     return HPS_OK;
   }
+  const size_t scratch_bytes = precond_scratch_bytes(h->ct, h->opt.max_rhs);
   if (dtype == HPS_C128) {
     if (!h->Kc64) {
       set_error("hps_precond: FP64 preconditioner was not built (HPS_FORM_FP64)");
       return HPS_EINVAL;
     }
-    HPS_CUDA_TRY(launch_precond(h, false, VType::C128, r, VType::C128, z, h->pc_scratch, nrhs, st));
+    HPS_CUDA_TRY(launch_precond(h, false, VType::C128, r, VType::C128, z, h->pc_scratch, scratch_bytes, nrhs, st));
   } else if (dtype == HPS_C64_H16) {
     if (!h->Kc16) {
       set_error("hps_precond: FP16 preconditioner blocks were not built (options.precond_fp16)");
       return HPS_EINVAL;
     }
-    HPS_CUDA_TRY(launch_precond(h, true, VType::C64, r, VType::C64, z, h->pc_scratch, nrhs, st, true));
+    HPS_CUDA_TRY(launch_precond(h, true, VType::C64, r, VType::C64, z, h->pc_scratch, scratch_bytes, nrhs, st, true));
   } else {
     if (!h->Kc32 && !h->Kc16) {
       set_error("hps_precond: FP32 preconditioner was not built (HPS_FORM_MIXED)");
       return HPS_EINVAL;
     }
     // lean mode keeps the cluster inverses in FP16 only
-    HPS_CUDA_TRY(launch_precond(h, true, VType::C64, r, VType::C64, z, h->pc_scratch, nrhs, st, !h->Kc32));
+    HPS_CUDA_TRY(launch_precond(h, true, VType::C64, r, VType::C64, z, h->pc_scratch, scratch_bytes, nrhs, st, !h->Kc32));
   }
   return HPS_OK;
 }

@@ -697,8 +697,8 @@ cudaError_t stage_k_simt(const hps_handle* h, const TM* K, const float* kscale, 
 }
 
 template <class TM, class TIN, class TOUT>
-cudaError_t precond_t(const hps_handle* h, const TM* B, const TM* K, const TIN* r, TOUT* z, TOUT* t, int nrhs,
-                      cudaStream_t st, const float* bscale = nullptr, const float* kscale = nullptr,
+cudaError_t precond_t(const hps_handle* h, const TM* B, const TM* K, const TIN* r, TOUT* z, TOUT* t,
+                      size_t scratch_bytes, int nrhs, cudaStream_t st, const float* bscale = nullptr, const float* kscale = nullptr,
                       bool use_tc = false) {
   const int q2 = h->q * h->q;
   const long long tstride = h->ct.tsize;
@@ -709,17 +709,17 @@ cudaError_t precond_t(const hps_handle* h, const TM* B, const TM* K, const TIN* 
   // tensor-core kernel 4.0e-7 (3.5e-6 with one sum per row), which is 103 instead of 514 us for 12
   // right-hand sides at 8^3 leaves, p = 8, but less than the FP32 that these calls have promised.
   if constexpr (std::is_same<TM, __half2>::value && std::is_same<TOUT, float2>::value) {
-    const bool tc16 = precond_tc16_eligible(h, nrhs);
+    const bool tc16 = precond_tc16_eligible(h, nrhs, scratch_bytes);
     if (precond_b16_eligible(h) && (tc16 || !precond_tc_multi_eligible(h, nrhs))) {
       constexpr VType kIn = std::is_same<TIN, float2>::value ? VType::C64
                             : std::is_same<TIN, float4>::value ? VType::DF : VType::C128;
       cudaEvent_t ev = h->prof.begin(st);
-      cudaError_t e = launch_precond_b16(h, kIn, r, z, tc16 ? nullptr : t, nrhs, st);
+      cudaError_t e = launch_precond_b16(h, kIn, r, z, t, tc16, nrhs, st);
       h->prof.end(HPS_PHASE_PRECOND_B, ev, st);
       if (e != cudaSuccess) return e;
       ev = h->prof.begin(st);
       if (tc16) {
-        e = launch_precond_tc16(h, z, nrhs, st);
+        e = launch_precond_tc16(h, t, z, nrhs, st);
       } else {
         // t as [position][right-hand side][nint0]; position p is cl_tpos / nint0
         if (use_tc) e = launch_precond_tc_vec(h, t, z, nrhs, h->tc_error, st);
@@ -893,10 +893,10 @@ cudaError_t launch_rhs(const hps_handle* h, const double2* s, const double2* t, 
 }
 
 cudaError_t launch_precond(const hps_handle* h, bool fp32_matrix, VType tin, const void* r, VType tout, void* z,
-                           void* scratch, int nrhs, cudaStream_t st, bool fp16_blocks) {
+                           void* scratch, size_t scratch_bytes, int nrhs, cudaStream_t st, bool fp16_blocks) {
   if (!fp32_matrix) {
     if (tin == VType::C128 && tout == VType::C128)
-      return precond_t(h, h->B64, h->Kc64, (const double2*)r, (double2*)z, (double2*)scratch, nrhs, st);
+      return precond_t(h, h->B64, h->Kc64, (const double2*)r, (double2*)z, (double2*)scratch, scratch_bytes, nrhs, st);
     return cudaErrorInvalidValue;
   }
   if (tout != VType::C64) return cudaErrorInvalidValue;
@@ -904,22 +904,20 @@ cudaError_t launch_precond(const hps_handle* h, bool fp32_matrix, VType tin, con
   const bool tc = h->opt.tc_apply && h->Kc32 && h->tc_error && !h->ct.kc_tc.empty();
   if (fp16_blocks) {
     if (!h->Kc16 || !h->B16) return cudaErrorInvalidValue;
-    if (tin == VType::C64)
-      return precond_t(h, h->B16, h->Kc16, (const float2*)r, (float2*)z, (float2*)scratch, nrhs, st, h->B16s, h->Kc16s,
-                       tc);
-    if (tin == VType::DF)
-      return precond_t(h, h->B16, h->Kc16, (const float4*)r, (float2*)z, (float2*)scratch, nrhs, st, h->B16s, h->Kc16s,
-                       tc);
-    return precond_t(h, h->B16, h->Kc16, (const double2*)r, (float2*)z, (float2*)scratch, nrhs, st, h->B16s, h->Kc16s,
-                     tc);
+    auto run = [&](auto* in) {
+      return precond_t(h, h->B16, h->Kc16, in, (float2*)z, (float2*)scratch, scratch_bytes, nrhs, st, h->B16s, h->Kc16s, tc);
+    };
+    if (tin == VType::C64) return run((const float2*)r);
+    if (tin == VType::DF) return run((const float4*)r);
+    return run((const double2*)r);
   }
-  if (tin == VType::C64)
-    return precond_t(h, h->B32, h->Kc32, (const float2*)r, (float2*)z, (float2*)scratch, nrhs, st, nullptr, nullptr,
-                     tc);
-  if (tin == VType::DF)
-    return precond_t(h, h->B32, h->Kc32, (const float4*)r, (float2*)z, (float2*)scratch, nrhs, st, nullptr, nullptr,
-                     tc);
-  return precond_t(h, h->B32, h->Kc32, (const double2*)r, (float2*)z, (float2*)scratch, nrhs, st, nullptr, nullptr, tc);
+  auto run = [&](auto* in) {
+    return precond_t(h, h->B32, h->Kc32, in, (float2*)z, (float2*)scratch, scratch_bytes, nrhs, st, (const float*)nullptr,
+                     (const float*)nullptr, tc);
+  };
+  if (tin == VType::C64) return run((const float2*)r);
+  if (tin == VType::DF) return run((const float4*)r);
+  return run((const double2*)r);
 }
 
 // ---------------------------------------------------------------------------
@@ -1068,7 +1066,7 @@ int autotune_shapes(hps_handle* h, cudaStream_t st) {
     if (h->R64 && (h->opt.forms & HPS_FORM_FP64)) tune_apply<double2, double2, double2>(h, h->R64, 1, fbuf, ybuf, nr, st);
   }
   // SIMT stage K of the mixed solve (FP16 blocks when kept, else FP32)
-  if (h->has_precond && h->ct.nslots > 0 && h->pc_scratch && !precond_tc16_eligible(h, 1)) {
+  if (h->has_precond && h->ct.nslots > 0 && h->pc_scratch && !precond_b16_eligible(h)) {
     cudaMemsetAsync(h->pc_scratch, 0, (size_t)h->ct.tsize * sizeof(float2), st);
     const bool tc = h->opt.tc_apply && h->Kc32 && h->tc_error && !h->ct.kc_tc.empty();
     if (h->Kc16) tune_stage_k<__half2>(h, h->Kc16, h->Kc16s, h->pc_scratch, ybuf, tc, st);

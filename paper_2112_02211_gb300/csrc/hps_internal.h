@@ -404,12 +404,7 @@ struct hps_handle {
   float* Kc16s = nullptr;
   __half2* B16 = nullptr;   // FP16 copies of B, rows scaled by 1/B16s[(bcls*6+face)*q^2 + j]
   float* B16s = nullptr;
-  void* pc_scratch = nullptr;  // nslots*q^2*max_rhs complex double (precond t buffer)
-  // FP16 tensor-core stage K (one right-hand side, multiples of 64): stage B's t of each vector (position * nrhs + rhs), scaled by its
-  // largest |component| tmax and split into FP16 operand rows [4][vector][nint0] (tc_precond16.cu)
-  __half2* op16 = nullptr;
-  float* tmax = nullptr;
-  int tmax_rhs = 0;            // right-hand sides they hold
+  void* pc_scratch = nullptr;  // precond_scratch_bytes(ct, max_rhs): hps_precond's t
 
   int* tc_error = nullptr;  // device error word of the tensor-core kernels
   // While a GMRES cycle is captured: the device word that the per-step kernels
@@ -496,8 +491,12 @@ cudaError_t launch_rhs(const hps_handle* h, const double2* s, const double2* t, 
 // Smallest solve tolerance at which the mixed form forms its restart residual and right-hand
 // side from the compensated FP32 maps (~3e-11 from the FP64 maps) instead of the FP64 maps.
 constexpr double kCompensatedMinTol = 1e-8;
-cudaError_t launch_precond(const hps_handle* h, bool fp32_matrix, VType tin, const void* r,
-                           VType tout, void* z, void* scratch, int nrhs, cudaStream_t st, bool fp16_blocks = false);
+// scratch holds t (values of tout) or, where scratch_bytes leave room for them, the operand rows of
+// the FP16 tensor-core stage K.
+cudaError_t launch_precond(const hps_handle* h, bool fp32_matrix, VType tin, const void* r, VType tout, void* z,
+                           void* scratch, size_t scratch_bytes, int nrhs, cudaStream_t st, bool fp16_blocks = false);
+// Scratch of nrhs right-hand sides with room for every form of t.
+size_t precond_scratch_bytes(const ClusterTables& ct, int nrhs);
 // The apply with the maps streamed through shared memory (stream_apply.cu): complex-float vectors
 // and maps, into complex float or double-float.
 bool stream_apply_eligible(const hps_handle* h, const void* f);
@@ -520,15 +519,16 @@ cudaError_t launch_precond_tc(const hps_handle* h, const float2* t, float2* z, i
 // columns (member cluster, right-hand side).  Needs ct.uniform.  t: [rhs][tsize], z: [rhs][nf].
 bool precond_tc_multi_eligible(const hps_handle* h, int nrhs);
 // The preconditioner with FP16 blocks on 2x2x2 clusters (tc_precond16.cu).  Stage B for any nrhs:
-// with t32 the vectors t themselves, [vector][nint0], without it the FP16 operand rows of stage K,
-// which runs every cluster block on the tensor cores for one right-hand side or a multiple of 64
-// (up to max_rhs).
+// the vectors t themselves, [vector][nint0], or (operand) the FP16 operand rows of stage K in their
+// place, which runs every cluster block on the tensor cores for one right-hand side or a multiple
+// of 64.  Both in t; precond_tc16_eligible: the operand rows fit in scratch_bytes.
 bool precond_b16_eligible(const hps_handle* h);
-bool precond_tc16_eligible(const hps_handle* h, int nrhs);
+bool precond_tc16_eligible(const hps_handle* h, int nrhs, size_t scratch_bytes);
+size_t tc16_operand_bytes(const ClusterTables& ct, int nrhs);
 int tc16_members_per_item(int cols, int nrhs);
-cudaError_t launch_precond_b16(const hps_handle* h, VType tin, const void* r, float2* z, float2* t32, int nrhs,
-                               cudaStream_t st);
-cudaError_t launch_precond_tc16(const hps_handle* h, float2* z, int nrhs, cudaStream_t st);
+cudaError_t launch_precond_b16(const hps_handle* h, VType tin, const void* r, float2* z, float2* t, bool operand,
+                               int nrhs, cudaStream_t st);
+cudaError_t launch_precond_tc16(const hps_handle* h, const void* t, float2* z, int nrhs, cudaStream_t st);
 // Stage K of the shared blocks ct.kc_tc (complex-FP32 blocks, one TF32 product) for nrhs right-hand
 // sides in one launch; uniform layout, t32 [vector][nint0].
 cudaError_t launch_precond_tc_vec(const hps_handle* h, const float2* t32, float2* z, int nrhs, int* d_error,

@@ -773,8 +773,7 @@ int krylov_alloc(hps_handle* h, int nrhs, long long nvec) {
   if ((rc = alloc((void**)&k.b, vb))) return rc;
   if ((rc = alloc((void**)&k.u, vb))) return rc;
   if ((rc = alloc(&k.z, vb))) return rc;
-  const size_t ts = (size_t)std::max<long long>(1, h->ct.tsize) * nrhs * sizeof(double2);
-  if ((rc = alloc(&k.zt, ts))) return rc;
+  if ((rc = alloc(&k.zt, precond_scratch_bytes(h->ct, nrhs)))) return rc;
   if ((rc = alloc((void**)&k.part, (size_t)nrhs * k.nblk * M1 * sizeof(double2)))) return rc;
   if ((rc = alloc((void**)&k.hcol, (size_t)nrhs * (M1 + 1) * sizeof(double2)))) return rc;
   if ((rc = alloc((void**)&k.y, (size_t)nrhs * M1 * sizeof(double2)))) return rc;  // also h2
@@ -1200,7 +1199,8 @@ int gmres_solve(hps_handle* h, int form, const double2* b, double2* x, int nrhs,
     return timed_apply(h, HPS_PHASE_APPLY, mixed, tin, in, tout, out, nullptr, nrhs, false, s);
   };
   ops.precond = [h, mixed](VType tin, const void* in, VType tout, void* out, int nrhs, cudaStream_t s) {
-    return launch_precond(h, mixed, tin, in, tout, out, h->ks.zt, nrhs, s, mixed && h->Kc16 != nullptr);
+    return launch_precond(h, mixed, tin, in, tout, out, h->ks.zt, precond_scratch_bytes(h->ct, h->ks.nrhs), nrhs, s,
+                          mixed && h->Kc16 != nullptr);
   };
   // restart residual: FP64 maps, or the compensated FP32 maps (lean mode; the mixed form at
   // tolerances >= 1e-8)

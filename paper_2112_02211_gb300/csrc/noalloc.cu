@@ -18,7 +18,8 @@ namespace {
 
 // The scratch holds the cluster-internal right-hand sides t (stage B output,
 // stage K input): tsize * nrhs complex values of the call's type (tsize: the
-// internal-face values of all clusters, blocks padded to 16 values).
+// internal-face values of all clusters, blocks padded to 16 values), or their
+// operand rows for the FP16 tensor-core stage K where those fit too.
 // Every device that loads the library reserves these bytes until the process exits.
 constexpr size_t kNoAllocScratchBytes = HPS_PRECOND_NOALLOC_MAX_BYTES;
 
@@ -96,8 +97,8 @@ int hps_precond_noalloc(hps_handle* h, int dtype, const void* r, void* z, int nr
   // complex float: the FP16 copies for HPS_C64_H16, and for HPS_C64 when the handle keeps the
   // cluster inverses in FP16 only (lean mode), as hps_precond does
   cudaError_t e = (dtype == HPS_C128)
-                      ? launch_precond(h, false, VType::C128, r, VType::C128, z, scratch, nrhs, st)
-                      : launch_precond(h, true, VType::C64, r, VType::C64, z, scratch, nrhs, st,
+                      ? launch_precond(h, false, VType::C128, r, VType::C128, z, scratch, kNoAllocScratchBytes, nrhs, st)
+                      : launch_precond(h, true, VType::C64, r, VType::C64, z, scratch, kNoAllocScratchBytes, nrhs, st,
                                        dtype == HPS_C64_H16 || !h->Kc32);
   h->prof.on = prof_on;
   HPS_CUDA_TRY(e);

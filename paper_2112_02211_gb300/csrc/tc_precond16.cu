@@ -70,7 +70,7 @@ struct PrecB16Args {
   const int2* items;      // (first position, members), members of one K block
   const TIN* r;
   float2* z;
-  float2* t32;            // [vector][n]: t itself, or nullptr: op and tmax
+  float2* t32;            // [vector][n]: t itself; nullptr: op and tmax
   __half2* op;            // operand rows [4][ncl * nrhs][n]: conj hi, swap hi, conj lo, swap lo
   float* tmax;            // [ncl * nrhs]
   int q2, n, ncl, nrhs, rtiles;
@@ -243,8 +243,14 @@ __global__ void __cluster_dims__(kBCluster, 1, 1) __maxnreg__(80) prec_b16_kerne
   cl.sync();  // no CTA leaves while another may read its maximum
 }
 
+// The operand rows [4][vector][nint0] lie at the start of the scratch, the maxima behind them.
+float* operand_tmax(const ClusterTables& ct, const void* t, int nrhs) {
+  return (float*)((__half2*)t + (size_t)4 * ct.ncl * nrhs * ct.nint0);
+}
+
 template <class TIN>
-cudaError_t stage_b16(const hps_handle* h, const TIN* r, float2* z, float2* t32, int nrhs, cudaStream_t st) {
+cudaError_t stage_b16(const hps_handle* h, const TIN* r, float2* z, float2* t, bool operand, int nrhs,
+                      cudaStream_t st) {
   const ClusterTables& ct = h->ct;
   PrecB16Args<TIN> a;
   a.B = h->B16;
@@ -257,9 +263,9 @@ cudaError_t stage_b16(const hps_handle* h, const TIN* r, float2* z, float2* t32,
   a.leaves = h->dct.cl_leaves;
   a.r = r;
   a.z = z;
-  a.t32 = t32;
-  a.op = h->op16;
-  a.tmax = h->tmax;
+  a.t32 = operand ? nullptr : t;
+  a.op = (__half2*)t;
+  a.tmax = operand_tmax(ct, t, nrhs);
   a.q2 = h->q * h->q;
   a.n = ct.nint0;
   a.ncl = ct.ncl;
@@ -556,26 +562,35 @@ bool precond_b16_eligible(const hps_handle* h) {
   return h->has_precond && h->opt.tc_apply && h->Kc16 && h->Kc16s && h->tc_error && h->ct.tc16;
 }
 
-bool precond_tc16_eligible(const hps_handle* h, int nrhs) {
-  return precond_b16_eligible(h) && h->tmax && h->op16 && nrhs <= h->tmax_rhs && (nrhs == 1 || nrhs % 64 == 0);
+bool precond_tc16_eligible(const hps_handle* h, int nrhs, size_t scratch_bytes) {
+  return precond_b16_eligible(h) && (nrhs == 1 || nrhs % 64 == 0) && tc16_operand_bytes(h->ct, nrhs) <= scratch_bytes;
 }
 
-cudaError_t launch_precond_b16(const hps_handle* h, VType tin, const void* r, float2* z, float2* t32, int nrhs,
-                               cudaStream_t st) {
-  if (!(t32 ? precond_b16_eligible(h) : precond_tc16_eligible(h, nrhs))) return cudaErrorInvalidValue;
-  if (tin == VType::C64) return stage_b16(h, (const float2*)r, z, t32, nrhs, st);
-  if (tin == VType::DF) return stage_b16(h, (const float4*)r, z, t32, nrhs, st);
-  return stage_b16(h, (const double2*)r, z, t32, nrhs, st);
+size_t tc16_operand_bytes(const ClusterTables& ct, int nrhs) {
+  return (size_t)ct.ncl * nrhs * ((size_t)4 * ct.nint0 * sizeof(__half2) + sizeof(float));
 }
 
-cudaError_t launch_precond_tc16(const hps_handle* h, float2* z, int nrhs, cudaStream_t st) {
+size_t precond_scratch_bytes(const ClusterTables& ct, int nrhs) {
+  const size_t t = (size_t)std::max<long long>(1, ct.tsize) * nrhs * sizeof(double2);
+  return ct.tc16 ? std::max(t, tc16_operand_bytes(ct, nrhs)) : t;
+}
+
+cudaError_t launch_precond_b16(const hps_handle* h, VType tin, const void* r, float2* z, float2* t, bool operand,
+                               int nrhs, cudaStream_t st) {
+  if (!precond_b16_eligible(h)) return cudaErrorInvalidValue;
+  if (tin == VType::C64) return stage_b16(h, (const float2*)r, z, t, operand, nrhs, st);
+  if (tin == VType::DF) return stage_b16(h, (const float4*)r, z, t, operand, nrhs, st);
+  return stage_b16(h, (const double2*)r, z, t, operand, nrhs, st);
+}
+
+cudaError_t launch_precond_tc16(const hps_handle* h, const void* t, float2* z, int nrhs, cudaStream_t st) {
   const ClusterTables& ct = h->ct;
-  if (!precond_tc16_eligible(h, nrhs)) return cudaErrorInvalidValue;
+  if (!precond_b16_eligible(h) || (nrhs != 1 && nrhs % 64 != 0)) return cudaErrorInvalidValue;
   auto encode = encoder();
   if (!encode) return cudaErrorNotSupported;
   const int nint = ct.nint0;
   // TMA: 16-byte aligned bases and strides (checked, not assumed)
-  if ((reinterpret_cast<uintptr_t>(h->Kc16) | reinterpret_cast<uintptr_t>(h->op16)) % 16 != 0 || (4LL * nint) % 16 != 0)
+  if ((reinterpret_cast<uintptr_t>(h->Kc16) | reinterpret_cast<uintptr_t>(t)) % 16 != 0 || (4LL * nint) % 16 != 0)
     return cudaErrorInvalidValue;
   // Items of 16 vectors unless that takes more than twice as many items as 64 would (blocks shared
   // by many vectors).  Measured per application of stage K at p = 8: 12^3 leaves of a bump medium,
@@ -597,7 +612,7 @@ cudaError_t launch_precond_tc16(const hps_handle* h, float2* z, int nrhs, cudaSt
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
   };
   if (!map3(&mapA, (void*)h->Kc16, (cuuint64_t)nint, (cuuint64_t)ct.nkc, kTileM, 1) ||
-      !map3(&mapB, (void*)h->op16, (cuuint64_t)ct.ncl * nrhs, 4, (cuuint32_t)cols, 4))
+      !map3(&mapB, const_cast<void*>(t), (cuuint64_t)ct.ncl * nrhs, 4, (cuuint32_t)cols, 4))
     return cudaErrorInvalidValue;
   Pk16Args a;
   a.nint = nint;
@@ -610,7 +625,7 @@ cudaError_t launch_precond_tc16(const hps_handle* h, float2* z, int nrhs, cudaSt
   a.kc_slot_begin = h->dct.kc_slot_begin;
   a.zoff = h->dct.zoff;
   a.kscale = h->Kc16s;
-  a.tmax = h->tmax;
+  a.tmax = operand_tmax(ct, t, nrhs);
   a.nf = h->nf;
   a.z = z;
   a.error = h->tc_error;
