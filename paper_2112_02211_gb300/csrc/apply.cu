@@ -576,16 +576,16 @@ int next_group(int left, int most) {
   return n;
 }
 
-// Launch over right-hand-side groups of at most 8 (each group re-reads the matrix);
+// Launch over right-hand-side groups of at most `most` (each group re-reads the matrix);
 // shapes[g]: the launch shape of group index g.
 template <class P, class Shift>
-cudaError_t launch_groups(const hps_handle* h, typename P::Args A, int nrhs, int xcap, int rowcap, cudaStream_t st,
-                          Shift shift, const LaunchShape* shapes) {
+cudaError_t launch_groups(const hps_handle* h, typename P::Args A, int nrhs, int most, int xcap, int rowcap,
+                          cudaStream_t st, Shift shift, const LaunchShape* shapes) {
   const int nsm = h->nsm;
   long long* counter = &h->prof.launches;
   for (int r0 = 0, nr; r0 < nrhs; r0 += nr) {
     typename P::Args B = A;
-    nr = next_group<typename P::TM>(nrhs - r0, 8);
+    nr = next_group<typename P::TM>(nrhs - r0, most);
     shift(B, r0);
     B.nrhs = nr;
     const cudaError_t e = launch_group<P>(B, nr, xcap, rowcap, nsm, st, counter, h->gate, shapes[group_index(nr)]);
@@ -605,18 +605,27 @@ int xcap_of(const hps_handle* h, XCap which) {
   return (int)round_up(std::max(mx, 1), 64);
 }
 
+// Accumulators of a launch of n right-hand sides: 1, 2, 4 or 8.
+int round_up2(int n) { return n <= 2 ? n : n <= 4 ? 4 : 8; }
+
 // Items per leaf of the applies: enough for several waves of the chip (24 per SM, about 6 for each
 // resident CTA), as many as faces at most; whole leaves stage their vector once and divide evenly
-// among the warps (216 rows at p = 8, a face's 36 do not).  More where the results of NR
-// right-hand sides would not fit in shared memory.
-int leaf_parts(const hps_handle* h, int nr, size_t acc_bytes, int xcap) {
-  int parts = 1;
-  while (parts < 6 && (long long)h->nl * parts < 24LL * h->nsm) parts += parts < 3 ? 1 : 3;
-  auto fits = [&](int p) {
-    return (size_t)nr * (xcap + (h->nb + p - 1) / p) * acc_bytes <= (size_t)100 * 1024;
+// among the warps (216 rows at p = 8, a face's 36 do not).  More parts where the results of the
+// right-hand sides of a launch would take more than 100 KB of shared memory beside their vectors,
+// and fewer right-hand sides per launch (`most`) where the vectors themselves do not fit (body loads
+// of 12^3 values and more in complex double).
+struct LeafPlan {
+  int parts, most;
+};
+LeafPlan leaf_plan(const hps_handle* h, int nrhs, size_t acc_bytes, int xcap) {
+  LeafPlan l{1, 8};
+  while (l.parts < 6 && (long long)h->nl * l.parts < 24LL * h->nsm) l.parts += l.parts < 3 ? 1 : 3;
+  auto smem = [&]() {
+    return (size_t)std::min(round_up2(nrhs), l.most) * (xcap + (h->nb + l.parts - 1) / l.parts) * acc_bytes;
   };
-  while (parts < 6 && !fits(parts)) parts += parts < 3 ? 1 : 3;
-  return parts;
+  while (l.parts < 6 && smem() > (size_t)100 * 1024) l.parts += l.parts < 3 ? 1 : 3;
+  while (l.most > 1 && smem() > (size_t)220 * 1024) l.most >>= 1;
+  return l;
 }
 
 template <class TM, class TIN, class TOUT>
@@ -635,11 +644,12 @@ cudaError_t apply_t(const hps_handle* h, const TM* R, const TIN* f, TOUT* y, con
   A.nf = h->nf;
   A.nrhs = nrhs;
   const int xcap = xcap_of(h, XCap::Apply);
-  A.parts = leaf_parts(h, std::min(nrhs, 8), sizeof(typename P::Acc), xcap);
+  const LeafPlan plan = leaf_plan(h, nrhs, sizeof(typename P::Acc), xcap);
+  A.parts = plan.parts;
   A.inv = row_inv(A.q2);
   A.nitems = (long long)h->nl * A.parts;
   const LaunchShape* shapes = h->shapes.apply[std::is_same<TM, double2>::value ? 1 : 0];
-  return launch_groups<P>(h, A, nrhs, xcap, (h->nb + A.parts - 1) / A.parts, st, [&](typename P::Args& B, int r0) {
+  return launch_groups<P>(h, A, nrhs, plan.most, xcap, (h->nb + A.parts - 1) / A.parts, st, [&](typename P::Args& B, int r0) {
     B.f += (long long)r0 * h->nf;
     B.y += (long long)r0 * h->nf;
     if (B.bvec) B.bvec += (long long)r0 * h->nf;
@@ -873,11 +883,12 @@ cudaError_t rhs_t(const hps_handle* h, const TM* H, const double2* s, const doub
   A.nint = h->nint;
   A.nrhs = nrhs;
   const int xcap = xcap_of(h, XCap::Rhs);
-  A.parts = leaf_parts(h, std::min(nrhs, 8), sizeof(typename P::Acc), xcap);
+  const LeafPlan plan = leaf_plan(h, nrhs, sizeof(typename P::Acc), xcap);
+  A.parts = plan.parts;
   A.inv = row_inv(A.q2);
   A.nitems = (long long)h->nl * A.parts;
   static const LaunchShape kDefault[4] = {{4, 0}, {4, 0}, {2, 0}, {2, 0}};
-  return launch_groups<P>(h, A, nrhs, xcap, (h->nb + A.parts - 1) / A.parts, st, [&](typename P::Args& B, int r0) {
+  return launch_groups<P>(h, A, nrhs, plan.most, xcap, (h->nb + A.parts - 1) / A.parts, st, [&](typename P::Args& B, int r0) {
     if (B.s) B.s += (long long)r0 * h->nint;
     if (B.t) B.t += (long long)r0 * h->nf;
     B.out += (long long)r0 * h->nf;
@@ -996,7 +1007,9 @@ cudaError_t tune_apply(hps_handle* h, const TM* R, int kind, void* fbuf, void* y
   A.nf = h->nf;
   A.nrhs = nr;
   const int xcap = xcap_of(h, XCap::Apply);
-  A.parts = leaf_parts(h, nr, sizeof(typename P::Acc), xcap);
+  const LeafPlan plan = leaf_plan(h, nr, sizeof(typename P::Acc), xcap);
+  if (plan.most < nr) return cudaSuccess;  // such groups are not launched
+  A.parts = plan.parts;
   A.inv = row_inv(A.q2);
   A.nitems = (long long)h->nl * A.parts;
   const int g = group_index(nr);
