@@ -774,7 +774,7 @@ cudaError_t precond_t(const hps_handle* h, const TM* B, const TM* K, const TIN* 
       PrecBArgs<TM, TIN, TOUT> C = A;
       const int rows = 3 * q2;
       C.parts = std::max(1, std::min((rows + 31) / 32, 2 * h->nsm / std::max(1, A.ngroups)));
-      const int threads = C.parts > 1 ? (int)round_up((rows + C.parts - 1) / C.parts, 32) : kThreads;
+      const int threads = C.parts > 1 ? std::min(kThreads, (int)round_up((rows + C.parts - 1) / C.parts, 32)) : kThreads;
       const int grid = (int)std::min<long long>((long long)A.ngroups * C.parts, (long long)h->nsm * std::max(occ, 1));
       kern<<<grid, threads, smem, st>>>(C);
       ++h->prof.launches;
