@@ -189,7 +189,8 @@ size_t hps_setup_bytes(const hps_grid* grid, const hps_options* opt, int nrhs);
  * Sec. 3.1).  f, y: device, nrhs*N_f complex of the given dtype (HPS_C128
  * needs HPS_FORM_FP64 operators, HPS_C64 needs HPS_FORM_MIXED ones), must not
  * overlap.  stream: a cudaStream_t (NULL = legacy default stream).  The call
- * is asynchronous with respect to the host.
+ * is asynchronous with respect to the host; hps_status reports what went wrong
+ * on the device.
  */
 int hps_apply(hps_handle* h, int dtype, const void* f, void* y, int nrhs, void* stream);
 
@@ -267,8 +268,8 @@ int hps_rhs(hps_handle* h, const double* s, const double* t, int nrhs, double* b
  * Errors: HPS_ENOCONV when maxit iterations did not reach tol (f_out holds
  * the last iterate, info the last residual); HPS_EBREAKDOWN when a residual
  * norm is not finite (NaN or Inf in the data or a non-finite intermediate),
- * found at the start or at a restart; HPS_ETIMEOUT when a tensor-core
- * kernel's bounded wait gave up; HPS_ECUDA for a CUDA error.
+ * found at the start or at a restart; HPS_ETIMEOUT when a kernel's bounded
+ * wait gave up; HPS_ECUDA for a CUDA error.
  */
 int hps_gmres_solve(hps_handle* h, int form, const double* s, const double* t, int nrhs,
                     double tol, double* f_out, hps_solve_info* info, void* stream);
@@ -379,17 +380,28 @@ long long hps_export(hps_handle* h, int what, int index, double* host_out);
 int hps_import_map(hps_handle* h, int what, int index, const double* host_in);
 
 /*
+ * Outcome of the asynchronous calls on a handle: waits for `stream` and returns
+ * HPS_ETIMEOUT when a kernel's bounded wait gave up since the last report, so
+ * that the output of an hps_apply, hps_precond or hps_precond_noalloc call is
+ * incomplete; HPS_OK otherwise.  Calls on other streams are seen once they have
+ * run.  A report clears the error.  Solves report their own time-outs and keep
+ * an earlier call's for this function.
+ */
+int hps_status(hps_handle* h, void* stream);
+
+/*
  * Test hook for the bounded device waits (no counterpart in the paper).  Every
- * wait of the tensor-core kernels on an mbarrier is bounded: after a limit the
- * CTA sets the handle's error word, stops issuing work, waits (bounded) for its
- * own copies and tensor-core operations, frees its tensor memory and returns,
- * and the solve returns HPS_ETIMEOUT with the GPU context intact.  With
- * what = HPS_INJECT_SKIP_ARRIVAL, one warp of CTA 0 of the multi-RHS
- * tensor-core apply leaves out one arrival, so that the MMA-issuing thread's
- * wait runs out; spin_limit (> 0) replaces the wait limit (tries of
- * mbarrier.try_wait) of that kernel, 0 keeps the default.  HPS_INJECT_NONE
- * with spin_limit 0 restores normal operation.  Drops the handle's captured
- * GMRES cycle.  For tests of the time-out path only.
+ * wait on an mbarrier (tensor-core kernels, streamed applies) is bounded: after
+ * a limit the CTA sets the handle's error word, stops issuing work, waits
+ * (bounded) for its own copies and tensor-core operations, frees its tensor
+ * memory and returns; the solve, or hps_status after other calls, returns
+ * HPS_ETIMEOUT with the GPU context intact.  With what =
+ * HPS_INJECT_SKIP_ARRIVAL, one warp of CTA 0 of the complex-float applies (64,
+ * 128, ... right-hand sides on the tensor cores; the streamed ones) leaves out
+ * one arrival, so that another warp's wait runs out; spin_limit (> 0) replaces
+ * the wait limit (tries of mbarrier.try_wait) of those kernels, 0 keeps the
+ * default.  HPS_INJECT_NONE with spin_limit 0 restores normal operation.  Drops
+ * the handle's captured GMRES cycle.  For tests of the time-out path only.
  */
 #define HPS_INJECT_NONE 0
 #define HPS_INJECT_SKIP_ARRIVAL 1

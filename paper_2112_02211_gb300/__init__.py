@@ -154,6 +154,11 @@ class Solver:
         N.check(self.lib.hps_precond(self.handle, dt, _ptr(r), _ptr(z), self._nrhs(r), _stream(stream)))
         return z
 
+    def check(self, stream=None):
+        """Wait for the stream; raise HPSError (HPS_ETIMEOUT) when a kernel of an earlier apply or
+        preconditioner call gave up a bounded wait, so that its result is incomplete."""
+        N.check(self.lib.hps_status(self.handle, _stream(stream)))
+
     def rhs(self, s=None, t=None, nrhs=1, stream=None):
         """b = tbar - Pi (H s) on the GPU (complex128 tensors)."""
         torch = _torch()

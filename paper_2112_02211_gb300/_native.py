@@ -81,6 +81,7 @@ SIGNATURES = {
     "hps_recover": (ctypes.c_int, [_P, _P, _P, ctypes.c_int, _P, _P, _P]),
     "hps_export": (ctypes.c_longlong, [_P, ctypes.c_int, ctypes.c_int, _P]),
     "hps_import_map": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_int, _P]),
+    "hps_status": (ctypes.c_int, [_P, _P]),
     "hps_test_inject": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_longlong]),
     "hps_get_launch_shapes": (ctypes.c_int, [_P, ctypes.POINTER(LaunchShapes)]),
     "hps_full_apply": (ctypes.c_int, [_P, ctypes.c_int, _P, _P, ctypes.c_int, _P]),

@@ -869,6 +869,23 @@ int hps_test_inject(hps_handle* h, int what, long long spin_limit) {
   return HPS_OK;
 }
 
+int hps_status(hps_handle* h, void* stream) {
+  if (!h) {
+    set_error("hps_status: NULL handle");
+    return HPS_EINVAL;
+  }
+  HPS_CUDA_TRY(cudaSetDevice(h->dev));
+  cudaStream_t st = (cudaStream_t)stream;
+  int err = 0;
+  HPS_CUDA_TRY(cudaMemcpyAsync(&err, h->tc_error, sizeof(int), cudaMemcpyDeviceToHost, st));
+  HPS_CUDA_TRY(cudaStreamSynchronize(st));
+  if (!err && !h->timed_out) return HPS_OK;
+  h->timed_out = false;
+  HPS_CUDA_TRY(cudaMemsetAsync(h->tc_error, 0, sizeof(int), st));
+  set_error("a bounded device wait gave up: the result of an earlier call on the handle is incomplete");
+  return HPS_ETIMEOUT;
+}
+
 int hps_get_launch_shapes(const hps_handle* h, hps_launch_shapes* out) {
   if (!h || !out) {
     set_error("hps_get_launch_shapes: bad arguments");

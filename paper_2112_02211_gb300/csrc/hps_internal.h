@@ -406,7 +406,8 @@ struct hps_handle {
   float* B16s = nullptr;
   void* pc_scratch = nullptr;  // precond_scratch_bytes(ct, max_rhs): hps_precond's t
 
-  int* tc_error = nullptr;  // device error word of the tensor-core kernels
+  int* tc_error = nullptr;  // device error word of the kernels with bounded waits
+  bool timed_out = false;   // it was set before a solve cleared it; hps_status reports it
   // While a GMRES cycle is captured: the device word that the per-step kernels
   // (apply, preconditioner) read first, returning at once when it is 0 (no
   // right-hand side still active).  nullptr otherwise.

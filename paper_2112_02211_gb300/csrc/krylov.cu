@@ -1003,10 +1003,15 @@ int gmres_core(hps_handle* h, const GmresOps& ops, bool mixed, const double2* b,
     return HPS_OK;
   };
 
-  // the tensor-core kernels' error word starts clear for every solve
-  if (h->tc_error) HPS_CUDA_TRY(cudaMemsetAsync(h->tc_error, 0, sizeof(int), st));
+  // the error word of the bounded waits starts clear for every solve; an earlier call's error is
+  // kept for hps_status
   std::vector<double> bnorm, rnorm;
-  if ((rc = vec_norms(h, b, nrhs, bnorm, st))) return rc;
+  int terr = 0;
+  if ((rc = vec_norms(h, b, nrhs, bnorm, st, h->tc_error, &terr, 1))) return rc;
+  if (terr) {
+    h->timed_out = true;
+    HPS_CUDA_TRY(cudaMemsetAsync(h->tc_error, 0, sizeof(int), st));
+  }
   if (fl.x0) {
     HPS_CUDA_TRY(ops.residual(x, b, k.r, nrhs, st));
     if ((rc = vec_norms(h, k.r, nrhs, rnorm, st))) return rc;
@@ -1154,17 +1159,16 @@ int gmres_core(hps_handle* h, const GmresOps& ops, bool mixed, const double2* b,
     int done = 0;
     for (int r = 0; r < nrhs; ++r) done = std::max(done, hread[nrhs + r]);
     nre_total += hread[3 * nrhs + 2];
+    // before the norms: a time-out leaves vectors incomplete
+    HPS_CUDA_TRY(cudaMemcpy(&terr, h->tc_error, sizeof(int), cudaMemcpyDeviceToHost));
+    if (terr) {
+      HPS_CUDA_TRY(cudaMemsetAsync(h->tc_error, 0, sizeof(int), st));
+      set_error("GMRES: a bounded device wait gave up");
+      return HPS_ETIMEOUT;
+    }
     if ((rc = finite_norms("restart residual"))) return rc;
     if (replayed && h->prof.on) h->prof.read_recs(k.graph.recs, done);
     its += done;
-    if (h->tc_error) {
-      int terr = 0;
-      HPS_CUDA_TRY(cudaMemcpy(&terr, h->tc_error, sizeof(int), cudaMemcpyDeviceToHost));
-      if (terr) {
-        set_error("tensor-core apply: a bounded wait gave up");
-        return HPS_ETIMEOUT;
-      }
-    }
     ++cycles;
     if (done == 0) break;  // nothing was active: no progress possible
   }

@@ -20,8 +20,9 @@
 // 122 -> 114 us (5.2 TB/s).  In complex double the FP64 pipe is the bound and seg_gemv_kernel, with
 // more warps resident, is the faster one (9^3, p = 8: 268 against 277 us).
 //
-// Every wait is bounded: on a time-out the CTA sets the error word, waits (bounded) for its own
-// copies and returns.
+// Every wait is bounded: on a time-out the CTA sets the error word, its producer stops, waits
+// (bounded) for the copies in flight and returns, and its consumers go through their remaining chunks
+// without waiting, on whatever the ring holds (hps_status and the solves report it).
 #include <algorithm>
 
 #include "common.cuh"
@@ -53,6 +54,8 @@ struct StreamArgs {
   void* y;
   long long nf, rows;   // values per right-hand side; matrix rows that are read
   int nrhs, stages;
+  long long spin;    // tries per bounded wait
+  int skip_arrival;  // test hook: CTA 0's first warp does not give back the first chunk
   int* error;
   const int* gate;
 };
@@ -192,7 +195,7 @@ __global__ void __launch_bounds__(32 * (kGroups<NR> * kGroup + 1), 1) stream_app
     for (bool ok = true; w.more() && ok; ++it) {
       if (fresh) {  // the leaf's vectors
         const int b = nx & 1;
-        if (nx >= 2 && !mbar_wait(&bars->xempty[b], (uint32_t)(((nx >> 1) - 1) & 1))) {
+        if (nx >= 2 && !mbar_wait(&bars->xempty[b], (uint32_t)(((nx >> 1) - 1) & 1), a.spin)) {
           fail();
           break;
         }
@@ -203,7 +206,7 @@ __global__ void __launch_bounds__(32 * (kGroups<NR> * kGroup + 1), 1) stream_app
         ++nx;
       }
       const int s = (int)(it % a.stages), n = w.count(kChunk);
-      if (*abort || (it >= a.stages && !mbar_wait(&bars->empty[s], (uint32_t)((it / a.stages - 1) & 1)))) {
+      if (*abort || (it >= a.stages && !mbar_wait(&bars->empty[s], (uint32_t)((it / a.stages - 1) & 1), a.spin))) {
         fail();
         break;
       }
@@ -222,12 +225,20 @@ __global__ void __launch_bounds__(32 * (kGroups<NR> * kGroup + 1), 1) stream_app
     }
     // copies in flight land before the CTA leaves (bounded)
     for (long long j = it > a.stages ? it - a.stages : 0; j < it; ++j)
-      if (!mbar_wait(&bars->full[(int)(j % a.stages)], (uint32_t)((j / a.stages) & 1))) fail();
+      if (!mbar_wait(&bars->full[(int)(j % a.stages)], (uint32_t)((j / a.stages) & 1), a.spin)) fail();
     for (int j = nx > 2 ? nx - 2 : 0; j < nx; ++j)
-      if (!mbar_wait(&bars->xfull[j & 1], (uint32_t)((j >> 1) & 1))) fail();
+      if (!mbar_wait(&bars->xfull[j & 1], (uint32_t)((j >> 1) & 1), a.spin)) fail();
     return;
   }
   // ---------------- consumers ----------------
+  // After a time-out no branch depends on it: the lanes of a warp may leave a wait differently, and
+  // they meet again in warp_sums.
+  auto wait = [&](uint64_t* bar, uint32_t parity) {
+    if (mbar_wait(bar, parity, 1)) return;
+    for (long long i = 1; i < a.spin; ++i)
+      if (*abort || mbar_wait(bar, parity, 1)) return;
+    fail();
+  };
   constexpr int V = 2 * RPW * NR;
   constexpr int kHeld = V >= 32 ? V / 32 : 1, kSame = V >= 32 ? 1 : 32 / V;
   constexpr int kMine = kHeld >= 2 ? kHeld / 2 : 1;  // complex results per lane
@@ -237,10 +248,7 @@ __global__ void __launch_bounds__(32 * (kGroups<NR> * kGroup + 1), 1) stream_app
   for (long long it = 0; w.more(); ++it) {
     const int s = (int)(it % a.stages), n = w.count(kChunk), leaf = w.leaf;
     if (fresh) {
-      if (*abort || !mbar_wait(&bars->xfull[nx & 1], (uint32_t)((nx >> 1) & 1))) {
-        fail();
-        return;
-      }
+      wait(&bars->xfull[nx & 1], (uint32_t)((nx >> 1) & 1));
       ++nx;
       // the leaf's first rows are this CTA's: its faces on the boundary of the cube only copy
       if (w.lrow == 0 && w.mask != 63u)
@@ -257,10 +265,7 @@ __global__ void __launch_bounds__(32 * (kGroups<NR> * kGroup + 1), 1) stream_app
       continue;
     }
     const T* x = xs + (size_t)((nx - 1) & 1) * nrhs * nb;
-    if (*abort || !mbar_wait(&bars->full[s], (uint32_t)((it / a.stages) & 1))) {
-      fail();
-      return;
-    }
+    wait(&bars->full[s], (uint32_t)((it / a.stages) & 1));
     const int l0 = warp % kGroup * RPW;
     if (l0 < n) {
       const T* row[RPW];
@@ -334,7 +339,7 @@ __global__ void __launch_bounds__(32 * (kGroups<NR> * kGroup + 1), 1) stream_app
       }
     }
     __syncwarp();
-    if (lane == 0) mbar_arrive(&bars->empty[s]);
+    if (lane == 0 && !(a.skip_arrival && blockIdx.x == 0 && warp == 0 && it == 0)) mbar_arrive(&bars->empty[s]);
     fresh = w.advance(a.g, q2, n);
     if (fresh && lane == 0) mbar_arrive(&bars->xempty[(nx - 1) & 1]);
   }
@@ -387,6 +392,8 @@ cudaError_t run(const hps_handle* h, const T* R, const T* f, TOUT* y, int nrhs, 
   a.nf = h->nf;
   const long long nx = h->nx, ny = h->ny, nz = h->nz;
   a.rows = (6 * nx * ny * nz - 2 * (nx * ny + nx * nz + ny * nz)) * a.q2;
+  a.spin = h->test_spin > 0 ? h->test_spin : kSpinLimit;
+  a.skip_arrival = h->test_skip_arrival;
   a.error = h->tc_error;
   a.gate = h->gate;
   // as many right-hand sides per launch as fit beside the ring
