@@ -457,8 +457,12 @@ __global__ void __launch_bounds__(kThreads) prec_b_kernel(const PrecBArgs<TM, TI
     for (int v0 = 0; v0 < nvec; v0 += NR) {
       const int nr = min(NR, nvec - v0);
       __syncthreads();
-      for (int idx = threadIdx.x; idx < nr * ncols; idx += blockDim.x) {
+      for (int idx = threadIdx.x; idx < NR * ncols; idx += blockDim.x) {
         const int rr = idx / ncols, c = idx - rr * ncols;
+        if (rr >= nr) {  // summed all the same: a test per product costs more
+          xs[idx] = czero<Acc>();
+          continue;
+        }
         const int vid = v0 + rr, leaf = A.gleaves[grp.x + vid / A.nrhs], rhs = vid % A.nrhs;
         const int k = c / q2;
         const long long o = (long long)rhs * A.vstride + A.brd[leaf * 6 + nint + k] + (c - k * q2);
@@ -488,13 +492,13 @@ __global__ void __launch_bounds__(kThreads) prec_b_kernel(const PrecBArgs<TM, TI
           for (int i = 0; i < 4; ++i)
 #pragma unroll
             for (int rr = 0; rr < NR; ++rr)
-              if (rr < nr) cfma(sum[i % kS][rr], bv[i], xs[rr * ncols + c + i]);
+              cfma(sum[i % kS][rr], bv[i], xs[rr * ncols + c + i]);
         }
         for (; c < ncols; ++c) {
           const Acc bv = load_one<TM>(Bm + (long long)c * ldr + row);
 #pragma unroll
           for (int rr = 0; rr < NR; ++rr)
-            if (rr < nr) cfma(sum[0][rr], bv, xs[rr * ncols + c]);
+            cfma(sum[0][rr], bv, xs[rr * ncols + c]);
         }
 #pragma unroll
         for (int rr = 0; rr < NR; ++rr) {
@@ -503,14 +507,25 @@ __global__ void __launch_bounds__(kThreads) prec_b_kernel(const PrecBArgs<TM, TI
           for (int i = 1; i < kS; ++i) acc[rr] = cadd(acc[rr], sum[i][rr]);
         }
         const int k = row / q2, j = row - k * q2;
+        // the loads of up to 8 vectors, then their stores (one after the other waited for each load:
+        // 64 right-hand sides at 4^3 leaves, p = 8, both stages 114 us, so 102 us)
+        constexpr int kIn = NR < 8 ? NR : 8;
 #pragma unroll
-        for (int rr = 0; rr < NR; ++rr) {
-          if (rr >= nr) break;
-          const int vid = v0 + rr, leaf = A.gleaves[grp.x + vid / A.nrhs], rhs = vid % A.nrhs;
-          const int e = leaf * 6 + k;
-          const Acc g = rscale(acc[rr], A.bscale, (long long)A.bsc[e] + j);
-          const Acc v = csub(cvt<Acc>(A.r[(long long)rhs * A.vstride + A.brd[e] + j]), g);
-          A.t[(long long)rhs * A.tstride + A.bto[e] + j] = cvt<TOUT>(v);
+        for (int r0 = 0; r0 < NR; r0 += kIn) {
+          if (r0 >= nr) break;
+          Acc rv[kIn];
+          long long to[kIn];
+#pragma unroll
+          for (int i = 0; i < kIn; ++i) {
+            const int vid = v0 + min(r0 + i, nr - 1), leaf = A.gleaves[grp.x + vid / A.nrhs], rhs = vid % A.nrhs;
+            const int e = leaf * 6 + k;
+            to[i] = (long long)rhs * A.tstride + A.bto[e] + j;
+            rv[i] = csub(cvt<Acc>(A.r[(long long)rhs * A.vstride + A.brd[e] + j]),
+                         rscale(acc[r0 + i], A.bscale, (long long)A.bsc[e] + j));
+          }
+#pragma unroll
+          for (int i = 0; i < kIn; ++i)
+            if (r0 + i < nr) A.t[to[i]] = cvt<TOUT>(rv[i]);
         }
       }
     }
@@ -770,10 +785,12 @@ cudaError_t precond_t(const hps_handle* h, const TM* B, const TM* K, const TIN* 
       if (e2 != cudaSuccess) return e2;
       // Where the items leave SMs idle, each is cut by rows into CTAs of a warp or more (64 leaves
       // at p = 8 in complex double: 32.5 us with one CTA and one sum per row, 28.5 us with 4 CTAs
-      // and four sums; both with the timer's own ~8 us).
+      // and four sums; both with the timer's own ~8 us).  Not with many vectors per pass, which
+      // every part would stage again: 64 right-hand sides, complex float, both stages at 4^3 leaves,
+      // p = 8, 305 us in parts and 102 us whole; 2^3 leaves, p = 6, 86 and 52 us.
       PrecBArgs<TM, TIN, TOUT> C = A;
       const int rows = 3 * q2;
-      C.parts = std::max(1, std::min((rows + 31) / 32, 2 * h->nsm / std::max(1, A.ngroups)));
+      C.parts = nr > 8 ? 1 : std::max(1, std::min((rows + 31) / 32, 2 * h->nsm / std::max(1, A.ngroups)));
       const int threads = C.parts > 1 ? std::min(kThreads, (int)round_up((rows + C.parts - 1) / C.parts, 32)) : kThreads;
       const int grid = (int)std::min<long long>((long long)A.ngroups * C.parts, (long long)h->nsm * std::max(occ, 1));
       kern<<<grid, threads, smem, st>>>(C);
