@@ -695,9 +695,12 @@ cudaError_t stage_k_simt(const hps_handle* h, const TM* K, const float* kscale, 
   A.tmul = tmul;
   const int xcap = xcap_of(h, XCap::StageK);
   // member groups of width w take 8 / w right-hand sides per launch (fewer where the staged
-  // vectors do not fit in shared memory)
+  // vectors do not fit in shared memory: in complex double twice per SM, since one CTA's warps leave
+  // the FP64 pipe idle between their items; 64 blocks of one cluster at p = 8, 8 right-hand sides: 4.4
+  // ms with 8 vectors and one CTA per SM, 3.4 ms with 4 and two)
+  constexpr bool k64 = sizeof(TM) == sizeof(double2);
   int fit = 8;
-  while (fit > 1 && (size_t)fit * (xcap + q2) * sizeof(typename MT<TM>::Acc) > (size_t)220 * 1024) fit >>= 1;
+  while (fit > 1 && (size_t)fit * (xcap + q2) * sizeof(typename MT<TM>::Acc) > (size_t)(k64 ? 110 : 220) * 1024) fit >>= 1;
   for (int g = 0; g < 4; ++g) {
     const long long n = use_tc ? h->ct.kitems_ntc[g] : (long long)h->ct.kitems[g].size();
     if (n == 0) continue;
@@ -711,7 +714,7 @@ cudaError_t stage_k_simt(const hps_handle* h, const TM* K, const float* kscale, 
       A.z = z + (long long)r0 * h->nf;
       // shapes are tuned for single right-hand sides of the float kernels; otherwise as many rows
       // per warp as leave work for all 8 warps of an item
-      const bool tuned = h->shapes.tuned && A.nrl == 1 && sizeof(TM) != sizeof(double2);
+      const bool tuned = h->shapes.tuned && A.nrl == 1 && !k64;
       const int rows = (q2 + A.split - 1) / A.split;
       const LaunchShape sh = tuned ? h->shapes.k[g] : LaunchShape{rows >= 32 ? 4 : rows >= 16 ? 2 : 1, 0};
       const cudaError_t e = launch_group<P>(A, A.nrhs, xcap, q2, h->nsm, st, &h->prof.launches, h->gate, sh);
