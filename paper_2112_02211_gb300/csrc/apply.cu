@@ -712,9 +712,9 @@ cudaError_t stage_k_simt(const hps_handle* h, const TM* K, const float* kscale, 
       A.nrhs = A.nrl << g;
       A.t = t + (long long)r0 * rstride;
       A.z = z + (long long)r0 * h->nf;
-      // shapes are tuned for single right-hand sides of the float kernels; otherwise as many rows
-      // per warp as leave work for all 8 warps of an item
-      const bool tuned = h->shapes.tuned && A.nrl == 1 && !k64;
+      // shapes are tuned for single right-hand sides of the float kernels, on handles whose solves
+      // run them; otherwise as many rows per warp as leave work for all 8 warps of an item
+      const bool tuned = h->shapes.k_tuned && A.nrl == 1 && !k64;
       const int rows = (q2 + A.split - 1) / A.split;
       const LaunchShape sh = tuned ? h->shapes.k[g] : LaunchShape{rows >= 32 ? 4 : rows >= 16 ? 2 : 1, 0};
       const cudaError_t e = launch_group<P>(A, A.nrhs, xcap, q2, h->nsm, st, &h->prof.launches, h->gate, sh);
@@ -1104,6 +1104,7 @@ int autotune_shapes(hps_handle* h, cudaStream_t st) {
     const bool tc = h->opt.tc_apply && h->Kc32 && h->tc_error && !h->ct.kc_tc.empty();
     if (h->Kc16) tune_stage_k<__half2>(h, h->Kc16, h->Kc16s, h->pc_scratch, ybuf, tc, st);
     else if (h->Kc32) tune_stage_k<float2>(h, h->Kc32, nullptr, h->pc_scratch, ybuf, tc, st);
+    h->shapes.k_tuned = true;
   }
   cudaStreamSynchronize(st);
   cudaGetLastError();

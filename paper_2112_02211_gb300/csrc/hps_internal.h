@@ -197,7 +197,7 @@ struct LaunchShape {
 struct Shapes {
   LaunchShape apply[2][4] = {{{4, 0}, {4, 0}, {4, 0}, {4, 0}}, {{4, 0}, {4, 0}, {4, 0}, {2, 0}}};
   LaunchShape k[4] = {{4, 0}, {4, 0}, {2, 0}, {2, 0}};
-  bool tuned = false;
+  bool tuned = false, k_tuned = false;  // the tuner ran; it timed stage K
 };
 
 // Per-phase CUDA-event timing and a launch counter (see hps_profile).  Events
