@@ -100,20 +100,24 @@ struct ItemInfo {
 // Rows of a leaf's faces with a neighbour, cut into `parts` items: row l of an item belongs to the
 // (row0 + l) / q2 -th of those faces.
 __device__ __forceinline__ void leaf_rows(const GridDims& g, int q2, int parts, long long item, ItemInfo& it) {
-  it.leaf = (int)(item / parts);
-  const int part = (int)(item % parts);
-  it.mask = 0;
+  it.leaf = (int)item / parts;
+  const int part = (int)item - it.leaf * parts;
+  const int line = it.leaf / g.nx, ix = it.leaf - line * g.nx, iz = line / g.ny, iy = line - iz * g.ny;
+  it.mask = (ix > 0 ? 1 : 0) | (ix + 1 < g.nx ? 2 : 0) | (iy > 0 ? 4 : 0) | (iy + 1 < g.ny ? 8 : 0) | (iz > 0 ? 16 : 0) |
+            (iz + 1 < g.nz ? 32 : 0);
   it.flist = 0;
   int n = 0;
 #pragma unroll
   for (int f = 0; f < 6; ++f)
-    if (g.neighbor(it.leaf, f) >= 0) {
-      it.mask |= 1 << f;
-      it.flist |= (unsigned)f << (4 * n++);
-    }
+    if ((it.mask >> f) & 1) it.flist |= (unsigned)f << (4 * n++);
   const int rows = n * q2;
   it.row0 = rows * part / parts;
   it.nrows = rows * (part + 1) / parts - it.row0;
+}
+// The leaf across a face that has one.
+__device__ __forceinline__ int across(const GridDims& g, int leaf, int face) {
+  const int step = face >> 1 == 0 ? 1 : face >> 1 == 1 ? g.nx : g.nx * g.ny;
+  return leaf + (face & 1 ? step : -step);
 }
 // inv: row_inv(q2)
 __device__ __forceinline__ void leaf_row(const ItemInfo& it, int q2, unsigned inv, int l, int& face, int& j) {
@@ -194,7 +198,7 @@ struct ApplyP {
     for (int l = tid; l < it.nrows; l += kThreads) {
       int face, j;
       leaf_row(it, A.q2, A.inv, l, face, j);
-      const long long o = (long long)A.g.neighbor(it.leaf, face) * A.nb + (long long)(face ^ 1) * A.q2 + j;
+      const long long o = (long long)across(A.g, it.leaf, face) * A.nb + (long long)(face ^ 1) * A.q2 + j;
       for (int rhs = 0; rhs < nr; ++rhs) finish(A, rhs * A.nf + o, outs[rhs * it.nrows + l]);
     }
     if (it.face != 0 || it.mask == 63) return;
@@ -242,7 +246,7 @@ struct RhsP {
     for (int l = tid; l < it.nrows; l += kThreads) {
       int face, j;
       leaf_row(it, A.q2, A.inv, l, face, j);
-      const long long o = (long long)A.g.neighbor(it.leaf, face) * A.nb + (long long)(face ^ 1) * A.q2 + j;
+      const long long o = (long long)across(A.g, it.leaf, face) * A.nb + (long long)(face ^ 1) * A.q2 + j;
       for (int rhs = 0; rhs < nr; ++rhs) {
         const double2 v = outs ? cvt<double2>(outs[rhs * it.nrows + l]) : make_double2(-0.0, -0.0);
         A.out[rhs * A.nf + o] = make_double2(-v.x, -v.y);
@@ -582,28 +586,43 @@ cudaError_t launch_group(const typename P::Args& B, int nr, int xcap, int rowcap
 }
 
 // Right-hand sides (or vectors) of the next launch, at most `most` of `left`: in complex double
-// whole powers of two, since the FP64 pipe is the bound and a group of 6 would compute 8.
+// whole powers of two, since the FP64 pipe is the bound and a group of 6 would compute 8 -- unless
+// the whole product (entries of the matrices) takes no longer than the other launch does: 3 right-hand
+// sides at 3^3 leaves, p = 5, 17.6 us as 2 + 1 and 12.5 us in one launch; 4^3 leaves, p = 10 (8.8
+// million entries) 210 and 280 us.
+constexpr long long kSplitEntries = 1000000;
 template <class TM>
-int next_group(int left, int most) {
+int next_group(int left, int most, long long entries) {
   int n = std::min(left, most);
-  if (sizeof(TM) == sizeof(double2))
+  if (sizeof(TM) == sizeof(double2) && entries >= kSplitEntries)
     while (n & (n - 1)) n &= n - 1;
   return n;
 }
 
 // Launch over right-hand-side groups of at most `most` (each group re-reads the matrix);
-// shapes[g]: the launch shape of group index g.
+// shapes[g]: the launch shape of group index g, tuned[g]: chosen by the tuner.  The defaults suit
+// items of many rows; items of a face's few take no more rows per warp than give every warp some, and
+// two with four right-hand sides in complex float where there are several per SM.  Measured: 3^3
+// leaves, p = 5, complex double, 4 right-hand sides (9 rows): 25.4 us with 4 rows per warp, 12.9 us
+// with 2; complex float, 4 right-hand sides: 6^3 leaves, p = 7 (25 rows) 23.1 us with 4, 18.9 us with
+// 2; 3^3 leaves, p = 10 (one item per SM) 11.0 and 13.8 us.
 template <class P, class Shift>
 cudaError_t launch_groups(const hps_handle* h, typename P::Args A, int nrhs, int most, int xcap, int rowcap,
-                          cudaStream_t st, Shift shift, const LaunchShape* shapes) {
+                          cudaStream_t st, Shift shift, const LaunchShape* shapes, const bool* tuned) {
   const int nsm = h->nsm;
   long long* counter = &h->prof.launches;
   for (int r0 = 0, nr; r0 < nrhs; r0 += nr) {
     typename P::Args B = A;
-    nr = next_group<typename P::TM>(nrhs - r0, most);
+    nr = next_group<typename P::TM>(nrhs - r0, most, (long long)h->nl * h->nb * xcap);
     shift(B, r0);
     B.nrhs = nr;
-    const cudaError_t e = launch_group<P>(B, nr, xcap, rowcap, nsm, st, counter, h->gate, shapes[group_index(nr)]);
+    const int g = group_index(nr);
+    LaunchShape sh = shapes[g];
+    if (!tuned || !tuned[g]) {
+      if (g == 2 && sizeof(typename P::Acc) == sizeof(float2) && rowcap < 128 && A.nitems >= 2LL * nsm) sh.rpw = std::min(sh.rpw, 2);
+      while (sh.rpw > 1 && kWarps * (sh.rpw / 2) >= rowcap) sh.rpw >>= 1;
+    }
+    const cudaError_t e = launch_group<P>(B, nr, xcap, rowcap, nsm, st, counter, h->gate, sh);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -625,7 +644,9 @@ int round_up2(int n) { return n <= 2 ? n : n <= 4 ? 4 : 8; }
 
 // Items per leaf of the applies: enough for several waves of the chip (24 per SM, about 6 for each
 // resident CTA), as many as faces at most; whole leaves stage their vector once and divide evenly
-// among the warps (216 rows at p = 8, a face's 36 do not).  More parts where the results of the
+// among the warps (216 rows at p = 8, a face's 36 do not).  In complex double, where the SM with the
+// most rows sets the pace, finer ones down to 16 rows while there are fewer than 4 per SM: 3^3 leaves,
+// p = 10, 40.2 us with 162 items, 33.6 us with 648.  More parts where the results of the
 // right-hand sides of a launch would take more than 100 KB of shared memory beside their vectors,
 // and fewer right-hand sides per launch (`most`) where the vectors themselves do not fit (body loads
 // of 12^3 values and more in complex double).
@@ -635,6 +656,8 @@ struct LeafPlan {
 LeafPlan leaf_plan(const hps_handle* h, int nrhs, size_t acc_bytes, int xcap) {
   LeafPlan l{1, 8};
   while (l.parts < 6 && (long long)h->nl * l.parts < 24LL * h->nsm) l.parts += l.parts < 3 ? 1 : 3;
+  if (acc_bytes == sizeof(double2))
+    while (l.parts < 24 && (long long)h->nl * l.parts < 4LL * h->nsm && h->nb >= 32 * l.parts) l.parts *= 2;
   auto smem = [&]() {
     return (size_t)std::min(round_up2(nrhs), l.most) * (xcap + (h->nb + l.parts - 1) / l.parts) * acc_bytes;
   };
@@ -668,7 +691,7 @@ cudaError_t apply_t(const hps_handle* h, const TM* R, const TIN* f, TOUT* y, con
     B.f += (long long)r0 * h->nf;
     B.y += (long long)r0 * h->nf;
     if (B.bvec) B.bvec += (long long)r0 * h->nf;
-  }, shapes);
+  }, shapes, h->shapes.apply_tuned[std::is_same<TM, double2>::value ? 1 : 0]);
 }
 
 // Stage K of every block that the tensor cores do not take (use_tc: all but those of kc_tc), by the
@@ -708,7 +731,7 @@ cudaError_t stage_k_simt(const hps_handle* h, const TM* K, const float* kscale, 
     A.nitems = n;
     const int step = std::max(1, fit >> g);
     for (int r0 = 0; r0 < nrhs; r0 += A.nrl) {
-      A.nrl = next_group<TM>(nrhs - r0, step);
+      A.nrl = next_group<TM>(nrhs - r0, step, kSplitEntries);
       A.nrhs = A.nrl << g;
       A.t = t + (long long)r0 * rstride;
       A.z = z + (long long)r0 * h->nf;
@@ -912,7 +935,7 @@ cudaError_t rhs_t(const hps_handle* h, const TM* H, const double2* s, const doub
     if (B.s) B.s += (long long)r0 * h->nint;
     if (B.t) B.t += (long long)r0 * h->nf;
     B.out += (long long)r0 * h->nf;
-  }, kDefault);
+  }, kDefault, nullptr);
 }
 
 cudaError_t launch_rhs(const hps_handle* h, const double2* s, const double2* t, double2* b, int nrhs,
@@ -1034,6 +1057,7 @@ cudaError_t tune_apply(hps_handle* h, const TM* R, int kind, void* fbuf, void* y
   A.nitems = (long long)h->nl * A.parts;
   const int g = group_index(nr);
   const std::array<long long, 6> key{h->dev, kind, h->q, h->nl, nr, A.nitems};
+  h->shapes.apply_tuned[kind][g] = true;
   h->shapes.apply[kind][g] = tune_group<P>(h, A, nr, xcap, (h->nb + A.parts - 1) / A.parts, key, h->shapes.apply[kind][g], st);
   return cudaSuccess;
 }

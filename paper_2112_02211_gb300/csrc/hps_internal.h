@@ -198,6 +198,7 @@ struct Shapes {
   LaunchShape apply[2][4] = {{{4, 0}, {4, 0}, {4, 0}, {4, 0}}, {{4, 0}, {4, 0}, {4, 0}, {2, 0}}};
   LaunchShape k[4] = {{4, 0}, {4, 0}, {2, 0}, {2, 0}};
   bool tuned = false, k_tuned = false;  // the tuner ran; it timed stage K
+  bool apply_tuned[2][4] = {};          // and these applies
 };
 
 // Per-phase CUDA-event timing and a launch counter (see hps_profile).  Events
