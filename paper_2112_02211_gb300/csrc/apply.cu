@@ -885,7 +885,7 @@ cudaError_t launch_apply(const hps_handle* h, bool fp32_matrix, VType tin, const
     return launch_apply_tc(h, (const float2*)f, y, false, nrhs, h->tc_error, st);
   if (tc && tin == VType::C64 && tout == VType::DF)
     return launch_apply_tc(h, (const float2*)f, y, true, nrhs, h->tc_error, st);
-  if (tin == VType::C64 && (tout == VType::C64 || tout == VType::DF) && stream_apply_eligible(h, f))
+  if (tin == VType::C64 && (tout == VType::C64 || tout == VType::DF) && stream_apply_eligible(h, f, tout, nrhs))
     return launch_stream_apply(h, (const float2*)f, tout, y, nrhs, st);
   if (tin == VType::C64 && tout == VType::C64)
     return apply_t(h, h->R32, (const float2*)f, (float2*)y, nullptr, nrhs, st);
@@ -1117,7 +1117,7 @@ int autotune_shapes(hps_handle* h, cudaStream_t st) {
     // what is left for the FP32 maps.  A 16^3-leaf, p = 10 solve: 209.8 ms with the default
     // shapes, 202.1 ms with the tuned ones.
     if (h->R32) {
-      if (stream_apply_eligible(h, fbuf)) tune_apply<float2, float4, float4>(h, h->R32, 0, fbuf, ybuf, nr, st);
+      if (stream_apply_eligible(h, fbuf, VType::DF, nr)) tune_apply<float2, float4, float4>(h, h->R32, 0, fbuf, ybuf, nr, st);
       else tune_apply<float2, float2, float4>(h, h->R32, 0, fbuf, ybuf, nr, st);
     }
     if (h->R64 && (h->opt.forms & HPS_FORM_FP64)) tune_apply<double2, double2, double2>(h, h->R64, 1, fbuf, ybuf, nr, st);

@@ -501,7 +501,8 @@ cudaError_t launch_precond(const hps_handle* h, bool fp32_matrix, VType tin, con
 size_t precond_scratch_bytes(const ClusterTables& ct, int nrhs);
 // The apply with the maps streamed through shared memory (stream_apply.cu): complex-float vectors
 // and maps, into complex float or double-float.
-bool stream_apply_eligible(const hps_handle* h, const void* f);
+// Whether it takes the call: f 16-byte aligned, the ring fits, and it is the faster kernel there.
+bool stream_apply_eligible(const hps_handle* h, const void* f, VType tout, int nrhs);
 cudaError_t launch_stream_apply(const hps_handle* h, const float2* f, VType tout, void* y, int nrhs, cudaStream_t st);
 // Tensor-core apply for 64-RHS groups (tc_apply.cu); f complex float, y complex
 // float or double-float; nrhs a multiple of 64.

@@ -415,12 +415,31 @@ cudaError_t run(const hps_handle* h, const T* R, const T* f, TOUT* y, int nrhs, 
   return cudaSuccess;
 }
 
+// The batched GEMV (apply.cu) is the faster one for up to 8 right-hand sides where the maps come from
+// L2 and its items fill the chip: maps of at most half of L2 inside a solve (double-float results),
+// which applies them at every step, and of a third in single calls, whose maps may have left it; faces
+// of at most 256 KB, so that few CTAs do not work long at one item; and leaves for an item per SM,
+// unless their rows are short.  Measured, us, GEMV and streamed, maps in L2: 4^3 leaves, p = 8, one
+// right-hand side 9.2 and 12.9; 6^3, p = 7, one 12.4 and 18.9; 8^3, p = 6, one 17.1 and 23.1, eight
+// 39.8 and 37.4; 6^3, p = 8 (67 MB), one 15.0 and 22.9, after an L2 flush 35.5 and 27.3.  On the other
+// side: 7^3, p = 8 (110 MB), two 49 and 34; 2^3, p = 12 (faces of 480 KB), one 10.7 and 8.8; 4^3,
+// p = 8, 16 right-hand sides 35 and 25.
+bool stream_apply_better(const hps_handle* h, VType tout, int nrhs) {
+  if (nrhs > 8) return true;
+  const double row = h->ldR * sizeof(float2);
+  const double bytes = (6.0 * h->nl - 2.0 * (h->nx * h->ny + h->nx * h->nz + h->ny * h->nz)) * h->q * h->q * row;
+  const bool in_l2 = bytes <= (tout == VType::DF ? 64.0 : 40.0) * (1 << 20);
+  const bool short_items = h->q * h->q * row <= 256.0 * 1024 && (6LL * h->nl >= h->nsm || h->nb <= 96);
+  return !(in_l2 && short_items);
+}
+
 }  // namespace
 
-bool stream_apply_eligible(const hps_handle* h, const void* f) {
+bool stream_apply_eligible(const hps_handle* h, const void* f, VType tout, int nrhs) {
   int rpw, stages;
   size_t smem;
-  return h->tc_error && h->nl > 1 && reinterpret_cast<uintptr_t>(f) % 16 == 0 && plan(h, 1, rpw, stages, smem);
+  return h->tc_error && h->nl > 1 && reinterpret_cast<uintptr_t>(f) % 16 == 0 && plan(h, 1, rpw, stages, smem) &&
+         stream_apply_better(h, tout, nrhs);
 }
 
 cudaError_t launch_stream_apply(const hps_handle* h, const float2* f, VType tout, void* y, int nrhs, cudaStream_t st) {
