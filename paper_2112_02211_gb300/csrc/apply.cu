@@ -100,21 +100,22 @@ struct ItemInfo {
 // Rows of a leaf's faces with a neighbour, cut into `parts` items: row l of an item belongs to the
 // (row0 + l) / q2 -th of those faces.
 __device__ __forceinline__ void leaf_rows(const GridDims& g, int q2, int parts, long long item, ItemInfo& it) {
-  it.leaf = (int)item / parts;
-  const int part = (int)item - it.leaf * parts;
-  const int line = it.leaf / g.nx, ix = it.leaf - line * g.nx, iz = line / g.ny, iy = line - iz * g.ny;
-  it.mask = (ix > 0 ? 1 : 0) | (ix + 1 < g.nx ? 2 : 0) | (iy > 0 ? 4 : 0) | (iy + 1 < g.ny ? 8 : 0) | (iz > 0 ? 16 : 0) |
-            (iz + 1 < g.nz ? 32 : 0);
+  it.leaf = (int)(item / parts);
+  const int part = (int)(item % parts);
+  it.mask = 0;
   it.flist = 0;
   int n = 0;
 #pragma unroll
   for (int f = 0; f < 6; ++f)
-    if ((it.mask >> f) & 1) it.flist |= (unsigned)f << (4 * n++);
+    if (g.neighbor(it.leaf, f) >= 0) {
+      it.mask |= 1 << f;
+      it.flist |= (unsigned)f << (4 * n++);
+    }
   const int rows = n * q2;
   it.row0 = rows * part / parts;
   it.nrows = rows * (part + 1) / parts - it.row0;
 }
-// The leaf across a face that has one.
+// The leaf across a face that has one (for the stores of single rows; GridDims::neighbor divides).
 __device__ __forceinline__ int across(const GridDims& g, int leaf, int face) {
   const int step = face >> 1 == 0 ? 1 : face >> 1 == 1 ? g.nx : g.nx * g.ny;
   return leaf + (face & 1 ? step : -step);
