@@ -84,6 +84,21 @@ __device__ __forceinline__ float2 rscale(float2 v, const float* s, long long i) 
 }
 __device__ __forceinline__ double2 rscale(double2 v, const float*, long long) { return v; }
 
+// Staged vectors in shared memory, VPL entries per lane and load: column c of a vector lies at
+// staged(c), so that a warp's 16-byte reads take consecutive addresses (4 entries per lane in two
+// halves of a 128-column chunk; read 8 bytes at a time they conflict four ways).
+template <int VPL> __device__ __forceinline__ int staged(int c) {
+  return VPL == 4 ? (c & ~127) + ((c & 2) << 5) + ((c & 124) >> 1) + (c & 1) : c;
+}
+__device__ __forceinline__ void load_staged(const float2* x, int c, float2 (&v)[4]) {  // c a multiple of 4
+  const float2* p = x + staged<4>(c);
+  const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 64);
+  v[0] = make_float2(a.x, a.y);
+  v[1] = make_float2(a.z, a.w);
+  v[2] = make_float2(b.x, b.y);
+  v[3] = make_float2(b.z, b.w);
+}
+
 struct ItemInfo {
   const void* mat;
   long long xoff;  // base offset of the input vector (per rhs)
@@ -286,14 +301,17 @@ struct PrecKP {
     const TIN* t;
     TOUT* z;
     long long nf, tstride, tmul;  // t of (rhs, cluster) at rhs * tstride + cl_tpos * tmul
-    int nrl;   // right-hand sides of the launch: vector rr = member * nrl + rhs
-    int nrhs;  // vectors of an item, member group width x nrl
+    int nrl;    // right-hand sides of an item: vector rr = member * nrl + rhs
+    int nrhs;   // vectors of an item, member group width x nrl
+    int total;  // right-hand sides of the launch: `groups` of nrl, item = entry of items * groups + group
+    int groups;
     long long nitems;
   };
   // item (k, s * split + part, first member, members): rows
   // [part * hq, min(q^2, (part + 1) * hq)) of slot s, hq = ceil(q^2 / split)
   __device__ static bool decode(const Args& A, long long item, ItemInfo& it) {
-    const int4 e = A.items[item];
+    const int entry = (int)item / A.groups, grp = (int)item - entry * A.groups;
+    const int4 e = A.items[entry];
     const int k = e.x, s = e.y / A.split, part = e.y % A.split;
     const int hq = (A.q2 + A.split - 1) / A.split;
     const int r0 = min(A.q2, part * hq);
@@ -306,22 +324,24 @@ struct PrecKP {
     it.nbr = r0;    // first row within the slot
     it.xoff = e.z;  // first member
     it.mask = e.w;  // members
+    it.leaf = grp * A.nrl;  // first right-hand side
     it.aoff = (long long)(s0 + s) * A.q2 + r0;
     return it.nrows > 0;
   }
   __device__ static long long row_off(const Args&, const ItemInfo& it, int l) { return (long long)l * it.ld; }
   __device__ static Acc load_x(const Args& A, const ItemInfo& it, int rr, int c) {
-    const int m = rr / A.nrl;
-    if (m >= it.mask) return czero<Acc>();
-    return cvt<Acc>(A.t[(long long)(rr - m * A.nrl) * A.tstride + A.cl_tpos[A.members[it.xoff + m]] * A.tmul + c]);
+    const int m = rr / A.nrl, rhs = it.leaf + rr - m * A.nrl;
+    if (m >= it.mask || rhs >= A.total) return czero<Acc>();
+    return cvt<Acc>(A.t[(long long)rhs * A.tstride + A.cl_tpos[A.members[it.xoff + m]] * A.tmul + c]);
   }
   __device__ static void store(const Args& A, const ItemInfo& it, const Acc* outs, int, int tid) {
     if (!outs) return;
     for (int idx = tid; idx < it.mask * A.nrl * it.nrows; idx += kThreads) {
-      const int rr = idx / it.nrows, jj = idx % it.nrows, m = rr / A.nrl;
+      const int rr = idx / it.nrows, jj = idx % it.nrows, m = rr / A.nrl, rhs = it.leaf + rr - m * A.nrl;
+      if (rhs >= A.total) continue;
       const int lf = A.slot_lf[A.cl_slot_begin[A.members[it.xoff + m]] + it.face];
       const long long o = (long long)(lf / 6) * A.nb + (long long)(lf % 6) * A.q2 + it.nbr + jj;
-      A.z[(long long)(rr - m * A.nrl) * A.nf + o] = cvt<TOUT>(rscale(outs[idx], A.kscale, it.aoff + jj));
+      A.z[(long long)rhs * A.nf + o] = cvt<TOUT>(rscale(outs[idx], A.kscale, it.aoff + jj));
     }
   }
 };
@@ -350,10 +370,10 @@ __global__ void __launch_bounds__(kThreads) seg_gemv_kernel(const typename P::Ar
       P::store(A, it, nullptr, nr, tid);
       continue;
     }
-    const int ncp = (it.ncols + VPL - 1) / VPL * VPL;
+    const int ncp = (it.ncols + VPL - 1) / VPL * VPL, ncs = VPL == 4 ? (ncp + 127) & ~127 : ncp;
     for (int idx = tid; idx < NR * ncp; idx += kThreads) {
       const int rr = idx / ncp, c = idx % ncp;
-      xs[rr * ncp + c] = (rr < nr && c < it.ncols) ? P::load_x(A, it, rr, c) : czero<Acc>();
+      xs[rr * ncs + staged<VPL>(c)] = (rr < nr && c < it.ncols) ? P::load_x(A, it, rr, c) : czero<Acc>();
     }
     __syncthreads();
     const TM* mat = reinterpret_cast<const TM*>(it.mat);
@@ -373,9 +393,11 @@ __global__ void __launch_bounds__(kThreads) seg_gemv_kernel(const typename P::Ar
         for (int i = 0; i < RPW; ++i) MT<TM>::load(row[i] + c, mv[i]);
 #pragma unroll
         for (int rr = 0; rr < NR; ++rr) {
+          Acc xq[4];
+          if constexpr (VPL == 4) load_staged(xs + rr * ncs, c, xq);
 #pragma unroll
           for (int v = 0; v < VPL; ++v) {
-            const Acc xv = xs[rr * ncp + c + v];
+            const Acc xv = VPL == 4 ? xq[v] : xs[rr * ncs + c + v];
 #pragma unroll
             for (int i = 0; i < RPW; ++i) {
               Acc t;
@@ -637,7 +659,7 @@ int xcap_of(const hps_handle* h, XCap which) {
   if (which == XCap::StageK && h->has_precond)
     for (int c = 0; c < h->ct.ncl; ++c)
       mx = std::max(mx, (h->ct.cl_slot_begin[c + 1] - h->ct.cl_slot_begin[c]) * h->q * h->q);
-  return (int)round_up(std::max(mx, 1), 64);
+  return (int)round_up(std::max(mx, 1), which == XCap::StageK ? 128 : 64);
 }
 
 // Accumulators of a launch of n right-hand sides: 1, 2, 4 or 8.
@@ -718,29 +740,37 @@ cudaError_t stage_k_simt(const hps_handle* h, const TM* K, const float* kscale, 
   A.tstride = rstride;
   A.tmul = tmul;
   const int xcap = xcap_of(h, XCap::StageK);
-  // member groups of width w take 8 / w right-hand sides per launch (fewer where the staged
-  // vectors do not fit in shared memory: in complex double twice per SM, since one CTA's warps leave
-  // the FP64 pipe idle between their items; 64 blocks of one cluster at p = 8, 8 right-hand sides: 4.4
-  // ms with 8 vectors and one CTA per SM, 3.4 ms with 4 and two)
+  // An item of member groups of width w takes up to fit / w right-hand sides (fewer where the staged
+  // vectors do not fit in shared memory), and a launch all of them, the groups of one block's rows one
+  // after the other so that they find the rows in L2.  64 blocks of one cluster at p = 8 (8^3 leaves),
+  // both stages: complex float with FP16 blocks, 12 right-hand sides, 454 us with 8 and 4 vectors in
+  // two launches, 353 us with 4 at a time in one; complex double, 8 right-hand sides, 4.4 ms with 8
+  // vectors (119 KB, one CTA per SM), 3.4 ms with 4 and two CTAs per SM.
   constexpr bool k64 = sizeof(TM) == sizeof(double2);
-  int fit = 8;
+  int fit = k64 ? 8 : 4;
   while (fit > 1 && (size_t)fit * (xcap + q2) * sizeof(typename MT<TM>::Acc) > (size_t)(k64 ? 110 : 220) * 1024) fit >>= 1;
   for (int g = 0; g < 4; ++g) {
     const long long n = use_tc ? h->ct.kitems_ntc[g] : (long long)h->ct.kitems[g].size();
     if (n == 0) continue;
     A.items = h->dct.kitems[g];
-    A.nitems = n;
     const int step = std::max(1, fit >> g);
-    for (int r0 = 0; r0 < nrhs; r0 += A.nrl) {
+    for (int r0 = 0; r0 < nrhs; r0 += A.total) {
       A.nrl = next_group<TM>(nrhs - r0, step, kSplitEntries);
+      // all groups of one size in a launch; in complex float the last one may be smaller
+      A.total = k64 ? (nrhs - r0) / A.nrl * A.nrl : nrhs - r0;
+      A.groups = (A.total + A.nrl - 1) / A.nrl;
+      A.nitems = n * A.groups;
       A.nrhs = A.nrl << g;
       A.t = t + (long long)r0 * rstride;
       A.z = z + (long long)r0 * h->nf;
       // shapes are tuned for single right-hand sides of the float kernels, on handles whose solves
-      // run them; otherwise as many rows per warp as leave work for all 8 warps of an item
+      // run them; otherwise as many rows per warp as leave work for all 8 warps of an item, and with
+      // several vectors no second turn for a few rows left (18 rows, p = 8, 12 right-hand sides at
+      // 8^3 leaves: 418 us with 2 rows per warp, 353 us with 1)
       const bool tuned = h->shapes.k_tuned && A.nrl == 1 && !k64;
       const int rows = (q2 + A.split - 1) / A.split;
-      const LaunchShape sh = tuned ? h->shapes.k[g] : LaunchShape{rows >= 32 ? 4 : rows >= 16 ? 2 : 1, 0};
+      const int half = A.nrhs == 1 || k64 ? 16 : 24, full = A.nrhs == 1 || k64 ? 32 : 40;
+      const LaunchShape sh = tuned ? h->shapes.k[g] : LaunchShape{rows >= full ? 4 : rows >= half ? 2 : 1, 0};
       const cudaError_t e = launch_group<P>(A, A.nrhs, xcap, q2, h->nsm, st, &h->prof.launches, h->gate, sh);
       if (e != cudaSuccess) return e;
     }
@@ -1088,7 +1118,7 @@ cudaError_t tune_stage_k(hps_handle* h, const TM* K, const float* kscale, void* 
     if (n == 0) continue;
     A.items = h->dct.kitems[g];
     A.nitems = n;
-    A.nrl = 1;
+    A.nrl = A.total = A.groups = 1;
     A.nrhs = 1 << g;
     const std::array<long long, 6> key{h->dev, 10 + (long long)sizeof(TM), h->q, h->nl, g, n};
     h->shapes.k[g] = tune_group<P>(h, A, 1 << g, xcap_of(h, XCap::StageK), A.q2, key, h->shapes.k[g], st);
