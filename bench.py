@@ -225,13 +225,13 @@ def peaks():
 def committed_traffic(kernel):
     """ncu DRAM bytes per launch from profiles/, valid only for the current kernel source."""
     path = os.path.join(ROOT, "profiles", "traffic.json")
-    src = os.path.join(ROOT, "paper_2112_02211_gb300", "csrc", "apply.cu")
+    src = os.path.join(ROOT, "paper_2112_02211_gb300", "csrc", "stream_apply.cu")
     try:
         with open(path) as fh:
             d = json.load(fh)
         digest = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
         e = d.get(kernel)
-        if e and e.get("apply_cu_sha256_16") == digest:
+        if e and e.get("stream_apply_cu_sha256_16") == digest:
             return e["bytes_per_launch"]
     except Exception:
         pass
@@ -368,9 +368,9 @@ def run_gpu(args, dist):
     phases = {"apply": a_bytes, "precond_k": kb, "precond_b": bb}
     kernels = {"apply": "stream_apply_kernel<float2,float4,1,R> (maps streamed through shared memory)",
                "precond_k": "tc_precond16_kernel<16|64> (every cluster block on the tensor cores, kind::f16, "
-                            "t scaled per cluster as two FP16 terms) when the clusters are uniform, else "
+                            "t scaled per cluster as two FP16 terms) when every cluster is 2x2x2, else "
                             "seg_gemv_kernel<PrecKP<__half2,float2,float2>,1,R>",
-               "precond_b": "prec_b16_kernel (t written as FP16 operand rows) when the clusters are uniform, else "
+               "precond_b": "prec_b16_kernel (t written as FP16 operand rows) when every cluster is 2x2x2, else "
                             "prec_b_kernel<__half2,float4,float2,NR>"}
     roof = {}
     for ph, by in phases.items():

@@ -103,16 +103,18 @@ typedef struct {
   int tc_apply;       /* tensor cores (three TF32 products, FP32 accumulation) for the
                          complex-FP32 apply of 64, 128, ... right-hand sides (inside an
                          unpreconditioned mixed solve the Krylov vectors are also kept rounded
-                         to complex FP32 for it) and, with one TF32 product, for
-                         preconditioner blocks shared by >= 16 clusters (complex-FP32
-                         blocks; see lambda_bin); default 1 */
+                         to complex FP32 for it); with one TF32 product, for preconditioner
+                         blocks shared by >= 16 clusters (complex-FP32 blocks; see lambda_bin)
+                         and for 64, 128, ... right-hand sides; and with FP16 blocks on 2x2x2
+                         clusters, one right-hand side or 64, 128, ...: two FP16 terms of the
+                         vectors (22 bits), FP32 accumulation; default 1 */
   int lean;           /* memory-lean mixed form (forms must be HPS_FORM_MIXED): the exact leaf
                          maps R, H are eliminated in FP64 but kept only in FP32, the cluster
                          inverses only in FP16 (plus complex-FP32 copies of blocks shared by
-                         >= 16 clusters when they take <= 4 GiB, for the tensor-core path),
-                         and the restart residual uses the FP32 maps with
-                         FP64 vectors (about 1e-7 relative per apply, for tolerances >= 1e-5).
-                         HPS_C128 applies are then unavailable.  Default 0. */
+                         >= 16 clusters when they take <= 4 GiB, for the tensor-core path).
+                         FP16 remainders of the FP32 maps keep the restart residual, the
+                         right-hand side and HPS_C128 applies accurate to about 3e-11 per
+                         map entry.  Default 0. */
   double lambda_bin;  /* shared preconditioner blocks (Sec. 4.1 remark: one local solver for
                          leaves with nearly the same medium): each lambda^tau is rounded to the
                          nearest multiple of lambda_bin * max_tau |lambda^tau| (real and imaginary
@@ -122,9 +124,9 @@ typedef struct {
                          still shared where values are bitwise equal.  Finite, >= 0.  Changes the
                          preconditioner only, never the converged solution. */
   int autotune;       /* time the candidate launch shapes (rows per warp, resident CTAs per SM)
-                         of the ItI apply and of the preconditioner's stage K at setup and keep
-                         the fastest (hps_launch_shapes); shapes never change results.
-                         Default 1. */
+                         of the batched GEMV kernels of the ItI apply, and of the preconditioner's
+                         stage K where the solves run that kernel, at setup and keep the fastest
+                         (hps_launch_shapes); shapes never change results.  Default 1. */
   int full_system;    /* also build the paper's own iterative path on the global system
                          (Sec. 3-4; hps_full_apply, hps_full_precond, hps_full_solve): per
                          distinct homogenized constant the inverse Schur complement S~^{-1}, and
@@ -409,7 +411,11 @@ int hps_test_inject(hps_handle* h, int what, long long spin_limit);
 
 /* Launch shapes of a handle's batched GEMV kernels, per right-hand-side group
  * (1, 2, <= 4, <= 8 per launch): matrix rows per warp pass (1, 2, 4, 8) and a
- * cap on resident CTAs per SM (0 = the occupancy limit). */
+ * cap on resident CTAs per SM (0 = the occupancy limit).  The other kernels have
+ * no tuned shapes: the streamed and tensor-core applies in complex float, and
+ * stage K on the tensor cores; there the FP32-map entries are those of the
+ * double-float operands of solves without the preconditioner, and stage K's are
+ * the defaults. */
 typedef struct {
   int apply_rows_per_warp[2][4];   /* ItI apply with FP32 maps [0], FP64 maps [1] */
   int apply_ctas_per_sm[2][4];

@@ -347,7 +347,7 @@ int hps_setup(const hps_grid* g, double kappa, double eta, const double* b, cons
         HPS_CUDA_TRY(cudaMemsetAsync(h->B16, 0, be * sizeof(__half2), st));
       }
       if ((r = dalloc(h, &h->pc_scratch, precond_scratch_bytes(ct, o.max_rhs)))) return r;
-      if ((r = build_preconditioner(h, dc, st))) return r;
+      if ((r = build_preconditioner(h, st))) return r;
       if (fp16 && (r = build_precond_fp16(h, st))) return r;
     }
     if (o.full_system && (r = build_full_system(h, dc, st))) return r;

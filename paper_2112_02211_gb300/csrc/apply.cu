@@ -10,9 +10,9 @@
 //      stage K  z_int = K_c t                          (K_c = (I + D)^{-1})
 //
 // An item is (leaf, part) for apply/rhs (a part of the rows of its faces with a neighbour), a leaf
-// for B, and for K one slot of a distinct K block against up to 8 clusters
-// sharing that block (their t vectors take the place of right-hand sides, so
-// a block shared by many clusters is read once per 8 of them).  The swap Pi is fused into the store: the rows
+// or a part of its rows for B, and for K a part of one slot of a distinct K block against up to 8
+// vectors: clusters sharing that block and right-hand sides, so that a block shared by many is read
+// once per 8 or 4 of them.  The swap Pi is fused into the store: the rows
 // of leaf tau's face k produce the incoming data of the neighbour across k,
 // so every output slot has exactly one writer and no atomics are needed.
 // Faces on the boundary of the cube only copy (their rows of R are never
@@ -24,8 +24,8 @@
 // What bounds it: HBM for one right-hand side in complex float; the FP64 pipe (4 fused
 // multiply-adds per entry, two per SM and clock) in complex double, where the warp reductions
 // used to cost another third; shared-memory reads of the staged vectors for many right-hand
-// sides, which several rows per warp share.Measured, 9^3 leaves, p = 8, complex
-// double: 331 -> 268 us.  (Complex-float vectors take stream_apply.cu.)
+// sides, which several rows per warp share.  Measured, 9^3 leaves, p = 8, complex double: 331 -> 263
+// us.  (Complex-float vectors take stream_apply.cu where that is faster, see stream_apply_better.)
 #include <algorithm>
 #include <array>
 #include <map>

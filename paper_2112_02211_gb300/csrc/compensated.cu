@@ -19,7 +19,7 @@
 //
 // What bounds it: about 50 FP32 instructions per complex entry and right-hand side (12 bytes), on
 // top of the warp reductions, which halve the sums in flight at every exchange, and the latency of
-// the map entries, which are loaded one step ahead.Measured, 8^3 leaves at p = 8:
+// the map entries, which are loaded one step ahead.  Measured, 8^3 leaves at p = 8:
 // restart residual of 8 right-hand sides 2.23 -> 0.55 ms, of one 217 -> 103 us; right-hand side of 8
 // sources 2.20 -> 0.54 ms (before: items of a face's 32 and 4 rows, one CTA per SM, full butterflies).
 #include <algorithm>

@@ -55,10 +55,6 @@ __device__ __forceinline__ void cfms(double2& v, double2 m, double2 u) {
   v.x = fma(-m.x, u.x, fma(m.y, u.y, v.x));
   v.y = fma(-m.x, u.y, fma(-m.y, u.x, v.y));
 }
-__device__ __forceinline__ void cfms(float2& v, float2 m, float2 u) {
-  v.x = fmaf(-m.x, u.x, fmaf(m.y, u.y, v.x));
-  v.y = fmaf(-m.x, u.y, fmaf(-m.y, u.x, v.y));
-}
 
 // NT threads, RP rows per thread: N <= NT * RP.
 template <class T, int NB, int NT, int RP>

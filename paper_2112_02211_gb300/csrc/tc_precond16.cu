@@ -321,7 +321,7 @@ template <int COLS> struct Shape {
 };
 
 struct Pk16Args {
-  int nint, kblocks, q2, nb;
+  int nint, kblocks, q2;
   long long nitems;
   const int4* items;       // (block, row tile, first position, members)
   int rtiles;              // COLS-RHS tiles of one member (nrhs > COLS), else 1
@@ -618,7 +618,6 @@ cudaError_t launch_precond_tc16(const hps_handle* h, const void* t, float2* z, i
   a.nint = nint;
   a.kblocks = 2 * nint / kKHalves;
   a.q2 = h->q * h->q;
-  a.nb = h->nb;
   a.items = h->dct.tc16_items + ct.tc16_begin[P];
   a.rtiles = (nrhs + cols - 1) / cols;
   a.nrhs = nrhs;
